@@ -579,6 +579,14 @@ double dense_round_lower_bound_ms(const maxsat_ctx* ctx, int32_t B) {
   return 1e3 * (2.0 * m_pad * n_pad * Bp / (4.5e15 * scale) + 2.0 * Bp * scatter / (2.25e15 * scale));
 }
 
+// Places the chains in an ensemble of B_total from global chain 8 g8_off on.
+void set_ensemble(maxsat_ctx* ctx, int32_t g8_off, int32_t B_total) {
+  ctx->C.g8_off = g8_off;
+  ctx->C.B_total = B_total;
+  ctx->C.inv_B_total = 1.0f / (float)B_total;
+  ctx->C.nib = !ctx->dense && !ctx->wide_h && nib_patterns_supported(ctx->T, B_total) ? 1 : 0;
+}
+
 // Measured path choice (MAXSAT_PATH_AUTO): times a few Gibbs rounds of B
 // chains on the sparse path, then on the dense path unless its tensor-core
 // products alone (at nominal peaks) would take longer than the measured
@@ -619,9 +627,7 @@ int choose_path(maxsat_ctx* ctx, int32_t B) {
     rc = alloc_chains(ctx, B);
     if (rc != MAXSAT_OK) break;
     ctx->C.keys = philox_keys(0x5EEDu, 0u);
-    ctx->C.g8_off = 0;
-    ctx->C.B_total = B;
-    ctx->C.inv_B_total = 1.0f / (float)B;
+    set_ensemble(ctx, 0, B);
     cudaError_t e = ctx->dense ? launch_init_dense(ctx->C, ctx->dX, ctx->dnu, ctx->dbest_x, ctx->n,
                                                    ctx->n_pad, ctx->e5m2, ctx->stream)
                                : launch_init_sparse(ctx->F, ctx->C, ctx->n, ctx->stream);
@@ -690,9 +696,7 @@ int tune_blocks(maxsat_ctx* ctx, int32_t B) {
     int r0 = alloc_chains(ctx, B);
     if (r0 != MAXSAT_OK) return r0;
     ctx->C.keys = philox_keys(0x5EEDu, 0u);
-    ctx->C.g8_off = 0;
-    ctx->C.B_total = B;
-    ctx->C.inv_B_total = 1.0f / (float)B;
+    set_ensemble(ctx, 0, B);
     cudaError_t e = launch_init_sparse(ctx->F, ctx->C, ctx->n, ctx->stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "init");
     constexpr int kWarm = 2, kRounds = 6;
@@ -1162,6 +1166,65 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
         });
       }
     UP(order, F.var_order);
+    F.var_inc8 = nullptr;
+    F.var_slot = nullptr;
+    T.ptab = nullptr;
+    T.pva = nullptr;
+    if (T.one_chunk && ctx->tabs.gq_absmax <= kNibMaxContribution) {
+      const HostTables& H = ctx->tabs;
+      // rows {low bytes, high bytes} of contribution + bias per temperature,
+      // group, position and sign; row 0 of each temperature is zero
+      T.ptab_bias = H.gq_absmax;
+      T.ptab_stride = 16 * (1 + 6 * T.n_groups);
+      std::vector<uint32_t> rows((size_t)T.n_temps * T.ptab_stride / 4, 0u);
+      auto row_of = [](int g, int k, bool neg) { return 16 * (1 + (g * 3 + k) * 2 + (neg ? 1 : 0)); };
+      for (int e = 0; e < T.n_temps; ++e)
+        for (int g = 0; g < T.n_groups; ++g) {
+          const GroupMeta& gm = H.meta[g];
+          for (int k = 0; k < gm.len && k < 3; ++k)
+            for (int neg = 0; neg < 2; ++neg) {
+              uint8_t* row = reinterpret_cast<uint8_t*>(rows.data()) +
+                             (size_t)e * T.ptab_stride + row_of(g, k, neg != 0);
+              for (int hp = 0; hp < (1 << gm.nh); ++hp) {
+                const int v = H.gq[(size_t)gm.gq_off + ((size_t)e << gm.nh) * gm.len + hp * gm.len + k];
+                const int biased = (neg ? -v : v) + T.ptab_bias;
+                row[hp] = (uint8_t)(biased & 0xFF);
+                row[8 + hp] = (uint8_t)(biased >> 8);
+              }
+            }
+        }
+      UP(rows, T.ptab);
+      // nu's increment as the kernels round it: fl(alpha fl(P (65536 - P)) 2^-32)
+      std::vector<uint2> pva(H.pv.size());
+      const float alpha = (float)prm.alpha;
+      for (size_t q = 0; q < pva.size(); ++q) {
+        const uint32_t P = H.pv[q];
+        const float var = (float)(P * (65536u - P)) * 2.3283064365386963e-10f;
+        const float inc = alpha * var;
+        uint32_t bits;
+        std::memcpy(&bits, &inc, 4);
+        pva[q] = make_uint2(P, bits);
+      }
+      UP(pva, T.pva);
+      std::vector<int2> inc8(nnz);
+      {
+        std::vector<int32_t> fill(var_off.begin(), var_off.end() - 1);
+        for (int64_t c = 0; c < m; ++c)
+          for (int64_t j = off[c]; j < off[c + 1]; ++j) {
+            const int32_t l = lits[j];
+            inc8[fill[(l > 0 ? l : -l) - 1]++] =
+                make_int2((int32_t)c, row_of(cl_grp[c], (int)(j - off[c]), l < 0));
+          }
+      }
+      UP(inc8, F.var_inc8);
+      std::vector<int4> slots(n);
+      for (int k = 0; k < n_inst; ++k)
+        for (int s = var_base[k]; s < var_base[k + 1]; ++s) {
+          const int i = order[s];
+          slots[s] = make_int4(i, var_off[i], var_off[i + 1] - var_off[i], k);
+        }
+      UP(slots, F.var_slot);
+    }
   }
   F.cl4 = nullptr;
   if (T.one_chunk) {
@@ -1180,7 +1243,9 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
         lv[k] = l & 0x7FFFFFFF;
         if (l < 0) neg |= 1 << k;
       }
-      cl4[c] = make_int4(lv[0], lv[1], lv[2], len > 0 ? (cl_grp[c] << 8) | (neg << 2) | len : 0);
+      const int32_t sat = len > 0 && ctx->tabs.meta[cl_grp[c]].sat ? 1 << 5 : 0;
+      cl4[c] = make_int4(lv[0], lv[1], lv[2],
+                         len > 0 ? (cl_grp[c] << 8) | sat | (neg << 2) | len : 0);
     }
     UP(cl4, F.cl4);
   }
@@ -1195,8 +1260,9 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   T.rec3 = nullptr;
   T.rec3_words = 0;
   if (T.one_chunk && (int64_t)T.n_groups * T.n_temps * 256 <= 32 * 1024) {
-    // one 256-byte block per (group, temperature): the group's 2^K records,
-    // then its flags at word 32 (bit 8: a saturated hidden unit)
+    // one 256-byte block per (group, temperature): the group's 2^K records at
+    // that temperature, then from word 32 those at the next one (for octets of
+    // chains that lie across two temperatures)
     const int E = T.n_temps;
     std::vector<uint32_t> rec3((size_t)T.n_groups * E * 64, 0u);
     for (int g = 0; g < T.n_groups; ++g) {
@@ -1208,8 +1274,10 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
       }
       for (int e = 0; e < E; ++e) {
         uint32_t* blk = rec3.data() + ((size_t)g * E + e) * 64;
-        for (int w = 0; w < 4 * np; ++w) blk[w] = ctx->tabs.rec[(size_t)gm.rec_off + (size_t)e * 4 * np + w];
-        blk[32] = gm.sat ? 0x100u : 0u;
+        for (int w = 0; w < 4 * np; ++w) {
+          blk[w] = ctx->tabs.rec[(size_t)gm.rec_off + (size_t)e * 4 * np + w];
+          blk[32 + w] = ctx->tabs.rec[(size_t)gm.rec_off + (size_t)std::min(e + 1, E - 1) * 4 * np + w];
+        }
       }
     }
     UP(rec3, T.rec3);
@@ -1398,9 +1466,7 @@ int maxsat_reset_shard(maxsat_ctx* ctx, int32_t B, uint64_t seed, int32_t chain_
   ctx->C.key0 = (uint32_t)seed;
   ctx->C.key1 = (uint32_t)(seed >> 32);
   ctx->C.keys = philox_keys(ctx->C.key0, ctx->C.key1);
-  ctx->C.g8_off = chain_offset / 8;
-  ctx->C.B_total = total_chains;
-  ctx->C.inv_B_total = 1.0f / (float)total_chains;
+  set_ensemble(ctx, chain_offset / 8, total_chains);
   ctx->seed = seed;
   ctx->t = 0;
   ctx->d_t_synced = false;

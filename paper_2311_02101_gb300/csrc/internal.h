@@ -20,6 +20,7 @@ namespace rbmsat {
 enum : uint32_t { kPhaseInit = 1, kPhaseHidden = 2, kPhaseVisible = 3, kPhaseSwap = 4 };
 
 constexpr int kChainTile = 256;   // chains per block of the sparse kernels
+constexpr int kNibMaxContribution = 1023;  // largest |2^Q G| of the nibble update's rows
 constexpr int kClauseBlock = 64;  // clauses per block of the sparse gather
 
 // ---------------------------------------------------------------------------
@@ -53,10 +54,16 @@ struct DevFormula {
                            // table's negated half), clause length K,
                            // per-temperature stride 2^L K of gq}
   const int4* cl4;         // m clause records {0-based variable of literals
-                           // 0..2 (0 when absent), group << 8 | negated << 2 |
-                           // length}, bit k of `negated` set when literal k is
+                           // 0..2 (0 when absent), group << 8 | saturated << 5
+                           // | negated << 2 | length}, `saturated` when some
+                           // hidden probability of the group is 65536, bit k of `negated` set when literal k is
                            // negated, when every clause has at most 3
                            // literals (one-chunk tables); else NULL
+  // one-chunk tables only (else NULL): the incidences of a variable as
+  // {clause, byte offset of its row in a temperature's block of ptab}, and per
+  // position of var_order {variable, first incidence, incidences, instance}
+  const int2* var_inc8;
+  const int4* var_slot;
   const int32_t* var_order;  // n: the visible update's order: variables by
                              // degree, highest first (ties to the lower index),
                              // within windows of 512 variables of one formula
@@ -85,13 +92,20 @@ struct DevTables {
   const uint32_t* rec;
   // one-chunk tables only: the records of group g at temperature e as a
   // 256-byte block at word (g E + e) 64: the 2^K records of 4 words, then at
-  // word 32 the group's flags (bit 8: some hidden probability is 65536); NULL
-  // when not built (too large)
+  // word 32 those of temperature e + 1 (the last temperature: its own again);
+  // NULL when not built (too large)
   const uint32_t* rec3;
   int32_t rec3_words;
   const int16_t* gq;   // 2 gq_len entries: 2^Q G, then -2^Q G (a negated
                        // literal's incidence reads the second half)
   const uint32_t* pv;
+  // one-chunk tables only (else NULL): per temperature a block of ptab_stride
+  // bytes of 16-byte rows, row 0 zero, then one per (group, position, sign):
+  // the low bytes of contribution + ptab_bias for the 8 hidden patterns, then
+  // their high bytes
+  const uint32_t* ptab;
+  int32_t ptab_stride, ptab_bias;
+  const uint2* pva;  // pv_len: {P, float bits of fl(alpha fl(P (65536 - P)) 2^-32)}
 };
 
 // Lets kernel `kern` launch with `dyn` bytes of dynamic shared memory: when
@@ -121,6 +135,7 @@ struct DevChains {
   int32_t cost32;     // sparse gather: every clause block's weight sum < 2^31
   int32_t cost16;     // one-chunk gather: a thread's clauses of one block (its
                       // eighth of the block) weigh less than 2^16 in total
+  int32_t nib;        // hidden patterns as 4-bit fields, one word per clause and octet
   int32_t n_inst;     // formulas: best / cost / fe / improved are n_inst x Bp,
                       // tickets n_inst x (Bp / kChainTile)
   uint32_t key0, key1;
@@ -134,7 +149,8 @@ struct DevChains {
   uint8_t* improved;  // Bp flags of the last best-keep
   int64_t* cost_part; // [clause block][Bp]
   float* fe_part;     // [clause block][Bp]
-  void* H;            // m x Bp hidden patterns (uint8_t, or uint16_t when L > 8)
+  void* H;            // m x Bp hidden patterns (uint8_t, or uint16_t when L > 8;
+                      // nib: m x Bp / 8 words)
   int32_t* tickets;   // Bp / kChainTile arrival counters of the gather blocks
 };
 
@@ -295,6 +311,9 @@ cudaError_t launch_gather(GatherMode mode, const DevFormula& F, const DevTables&
 cudaError_t launch_visible(const DevFormula& F, const DevTables& T, const DevChains& C,
                            float alpha, const uint32_t* tdev, uint32_t t_rel, bool wide_h,
                            cudaStream_t st, int batch = 4);
+// whether hidden patterns of these tables and this ensemble are stored as
+// 4-bit fields (C.nib)
+bool nib_patterns_supported(const DevTables& T, int B_total);
 // the persistent round (one cooperative launch of `rounds` Gibbs rounds,
 // grid barriers between the phases) covers this context's sparse round:
 // clauses of at most 3 literals, single-temperature octets, byte patterns

@@ -304,7 +304,12 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
         else
           hidden_draws<true, ONE>(tab, row4, chunks, gm.nh, lc, octet, t, phase_h, C.keys, hp, fe);
         HT* H = static_cast<HT*>(C.H) + (size_t)c * Bp + b0;
-        if (sizeof(HT) == 1) {
+        if (ONE && C.nib) {
+          uint32_t v = 0;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v |= hp[q] << (4 * q);
+          static_cast<uint32_t*>(C.H)[(size_t)c * (Bp / 8) + g8] = v;
+        } else if (sizeof(HT) == 1) {
           uint64_t v = 0;
 #pragma unroll
           for (int q = 0; q < 8; ++q) v |= (uint64_t)hp[q] << (8 * q);
@@ -380,8 +385,8 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
 
 // ---------------------------------------------------------------------------
 // Step gather for formulas whose clauses all have at most 3 literals (one
-// 16-byte record per truth pattern) when every octet of chains has a single
-// temperature: the same results as k_gather<kStep, true, uint8_t, true> with
+// 16-byte record per truth pattern) when no octet of chains has more than two
+// temperatures: the same results as k_gather<kStep, true, uint8_t, true> with
 // fewer instructions per clause and 8 chains.
 //  - Philox4x32-10 rounds 0..2: unit h of chain octet o draws from counter
 //    (clause, o | h << 24, t, phase). Round 0's product of word z (= t) is
@@ -399,8 +404,8 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
 //    into the block's address.
 //  - Each draw is a compare and a predicated OR into the hidden pattern word
 //    (even chains move their draw into the high half first; groups with a
-//    saturated unit, P = 65536 stored as 0xFFFF0001, also clear the low half
-//    of odd chains' words).
+//    saturated unit, P = 65536 stored as 0xFFFF0001, bit 5 of the clause
+//    record, also clear the low half of odd chains' words).
 //  - The weighted unsatisfied costs stay in registers: each chain adds the
 //    clause weight times its 0/1 "no true literal" byte, without branches.
 //  - Latency: the state bytes and weight of the next clause are loaded while
@@ -460,50 +465,199 @@ __device__ __forceinline__ void load_clause_state(const uint8_t* xtb, int Bp, co
 }
 
 // Unit H's draw for chain Q of the octet against threshold word w: bit
-// 8 (Q & 3) + H of hw.
-template <bool SAT, int Q, int H>
+// 4 Q + H of hw (NIB), else bit 8 (Q & 3) + H.
+template <bool SAT, bool NIB, int Q, int H>
 __device__ __forceinline__ void unit_draw(const uint4 (&R)[3], uint32_t w, uint32_t& hw) {
   const uint32_t word = word_of(R[H], Q >> 1);
   const uint32_t x = (Q & 1) ? (SAT ? (word & 0xFFFF0000u) : word) : (word << 16);
-  or_if_below<(1u << (8 * (Q & 3) + H))>(hw, x, w);
+  or_if_below<(1u << ((NIB ? 4 * Q : 8 * (Q & 3)) + H))>(hw, x, w);
 }
 
 // Chain Q of the octet: its record (free energy, thresholds of units 0..2)
 // and its three draws.
-template <bool SAT, int Q>
+template <bool SAT, bool NIB, int Q>
 __device__ __forceinline__ void chain_draws(uint32_t addr_bytes, uint32_t rb, const uint4 (&R)[3],
                                             float& fe, uint32_t& hw) {
   const uint4 r = lds128(__byte_perm(addr_bytes, rb, 0x7650u | (Q & 3)));
   fe += __uint_as_float(r.x);
-  unit_draw<SAT, Q, 0>(R, r.y, hw);
-  unit_draw<SAT, Q, 1>(R, r.z, hw);
-  unit_draw<SAT, Q, 2>(R, r.w, hw);
+  unit_draw<SAT, NIB, Q, 0>(R, r.y, hw);
+  unit_draw<SAT, NIB, Q, 1>(R, r.z, hw);
+  unit_draw<SAT, NIB, Q, 2>(R, r.w, hw);
 }
 
-template <bool SAT>
+// The octet's hidden pattern: with NIB all 8 chains in h_lo, 4 bits each;
+// else chains 0..3 in the bytes of h_lo and 4..7 in those of h_hi.
+template <bool SAT, bool NIB>
 __device__ __forceinline__ void octet_draws(uint32_t a_lo, uint32_t a_hi, uint32_t rb,
                                             const uint4 (&R)[3], float (&fe)[8], uint32_t& h_lo,
                                             uint32_t& h_hi) {
-  chain_draws<SAT, 0>(a_lo, rb, R, fe[0], h_lo);
-  chain_draws<SAT, 1>(a_lo, rb, R, fe[1], h_lo);
-  chain_draws<SAT, 2>(a_lo, rb, R, fe[2], h_lo);
-  chain_draws<SAT, 3>(a_lo, rb, R, fe[3], h_lo);
-  chain_draws<SAT, 4>(a_hi, rb, R, fe[4], h_hi);
-  chain_draws<SAT, 5>(a_hi, rb, R, fe[5], h_hi);
-  chain_draws<SAT, 6>(a_hi, rb, R, fe[6], h_hi);
-  chain_draws<SAT, 7>(a_hi, rb, R, fe[7], h_hi);
+  chain_draws<SAT, NIB, 0>(a_lo, rb, R, fe[0], h_lo);
+  chain_draws<SAT, NIB, 1>(a_lo, rb, R, fe[1], h_lo);
+  chain_draws<SAT, NIB, 2>(a_lo, rb, R, fe[2], h_lo);
+  chain_draws<SAT, NIB, 3>(a_lo, rb, R, fe[3], h_lo);
+  chain_draws<SAT, NIB, 4>(a_hi, rb, R, fe[4], NIB ? h_lo : h_hi);
+  chain_draws<SAT, NIB, 5>(a_hi, rb, R, fe[5], NIB ? h_lo : h_hi);
+  chain_draws<SAT, NIB, 6>(a_hi, rb, R, fe[6], NIB ? h_lo : h_hi);
+  chain_draws<SAT, NIB, 7>(a_hi, rb, R, fe[7], NIB ? h_lo : h_hi);
 }
 
+// Where a thread's 8 chains read their records: the block of group 0 at the
+// first chain's temperature, the stride between groups, and 0x80 in the
+// address bytes of the chains that belong to the next temperature (the upper
+// half of a record block holds the next temperature's records).
+struct G3Tables {
+  uint32_t tab_e, gstride, up_lo, up_hi;
+};
+
+__device__ __forceinline__ G3Tables gather3_tables(const DevTables& T, const DevChains& C,
+                                                   uint32_t tab, int b0) {
+  const int E = T.n_temps, gb0 = C.g8_off * 8 + b0;
+  const int e0 = temp_of(gb0, E, C.B_total, C.inv_B_total);
+  G3Tables g;
+  g.tab_e = tab + (uint32_t)e0 * 256u;
+  g.gstride = (uint32_t)E * 256u;
+  g.up_lo = g.up_hi = 0u;
+  if (e0 != temp_of(gb0 + 7, E, C.B_total, C.inv_B_total)) {
+    const int split = (int)(((long long)(e0 + 1) * C.B_total + E - 1) / E) - gb0;  // 1 .. 7
+    const uint64_t up = 0x8080808080808080ull << (8 * split);
+    g.up_lo = (uint32_t)up;
+    g.up_hi = (uint32_t)(up >> 32);
+  }
+  return g;
+}
+
+// The clauses c_begin + warp, + 8, ... of a block for the thread's octet: cost
+// and free energy added into cost[] / fe[], hidden patterns stored.
 // PLAIN3: every clause has exactly 3 literals and no group has a saturated
 // hidden unit (T.plain3). COST16: a warp's clauses of its block weigh less
 // than 2^16 in total (C.cost16), so chains 2j and 2j + 1 keep their costs in
 // the low and high half of one register.
+// CG: the chain state is read from the L2 (a resident launch writes it).
+// NIB: the hidden patterns go out as one 32-bit word per clause and octet
+// (k_visible_nib's layout), else as 8 bytes.
+template <bool PLAIN3, bool COST16, bool CG, bool NIB>
+__device__ __forceinline__ void gather3_clauses(const DevFormula& F, const DevChains& C,
+                                                const G3Tables& G, int inst, int c_begin,
+                                                int c_end, int cl_base, uint32_t t, int g8,
+                                                int warp, int32_t (&cost)[8], float (&fe)[8]) {
+  const int Bp = C.Bp, b0 = g8 * 8;
+  const RoundKeys& K = C.keys;
+  const uint32_t octet = (uint32_t)(g8 + C.g8_off);
+  const uint32_t phase = kPhaseHidden | ((uint32_t)inst << 8);
+  // round 0, word z = t: common to every unit and clause
+  const uint64_t pt = (uint64_t)kPhiloxM1 * t;
+  const uint32_t u1 = (uint32_t)(pt >> 32) ^ K.k0[0];
+  const uint32_t u2 = (uint32_t)pt;
+  // round 1, word x = round 0's (octet | h << 24) ^ u1: per thread and unit
+  uint32_t th[3], sh[3];
+#pragma unroll
+  for (int h = 0; h < 3; ++h) {
+    const uint64_t p = (uint64_t)kPhiloxM0 * ((octet | ((uint32_t)h << 24)) ^ u1);
+    th[h] = (uint32_t)(p >> 32) ^ K.k1[1];
+    sh[h] = (uint32_t)p;
+  }
+  const uint8_t* xtb = C.xt + b0;
+  uint8_t* hb = static_cast<uint8_t*>(C.H) + (NIB ? b0 / 2 : b0);
+  const int hstride = NIB ? Bp / 2 : Bp;
+
+  // software pipeline: the state bytes of the next clause and the record of
+  // the one after it are loaded while the current clause is sampled
+  const int c0 = c_begin + warp;
+  int4 rec_n = make_int4(0, 0, 0, 0);
+  if (c0 < c_end) rec_n = __ldg(F.cl4 + c0);
+  uint2 xa, xb, xc;
+  uint32_t info = (uint32_t)rec_n.w;
+  int32_t wc = 0;
+  if (c0 < c_end) wc = (int32_t)__ldg(F.cl_w + c0);
+  load_clause_state<PLAIN3, CG>(xtb, Bp, rec_n, xa, xb, xc);
+  if (c0 + 8 < c_end) rec_n = __ldg(F.cl4 + c0 + 8);
+  for (int c = c0; c < c_end; c += 8) {
+    uint2 na = make_uint2(0u, 0u), nb = na, nc = na;
+    const uint32_t ninfo = (uint32_t)rec_n.w;
+    int32_t nwc = 0;
+    if (c + 8 < c_end) {
+      load_clause_state<PLAIN3, CG>(xtb, Bp, rec_n, na, nb, nc);
+      nwc = (int32_t)__ldg(F.cl_w + c + 8);
+    }
+    if (c + 16 < c_end) rec_n = __ldg(F.cl4 + c + 16);
+    const int len = info & 3;
+    // byte q: chain q's truth pattern (chains 0..3 | 4..7)
+    const uint32_t flip = ((info >> 2) & 7u) * 0x01010101u;
+    const uint32_t lo = (xa.x + 2u * xb.x + 4u * xc.x) ^ flip;
+    const uint32_t hi = (xa.y + 2u * xb.y + 4u * xc.y) ^ flip;
+    const uint32_t cinfo = info, grp = info >> 8;
+    const int32_t w_cur = wc;
+    xa = na;
+    xb = nb;
+    xc = nc;
+    info = ninfo;
+    wc = nwc;
+    // byte q is 1 when chain q has no true literal (pattern 0: 0x7F + p sets
+    // bit 7 for every p in 1..7 and never carries), else 0; each chain adds
+    // the clause weight times its byte, without branches
+    const uint32_t u_lo = (~(lo + 0x7F7F7F7Fu) & 0x80808080u) >> 7;
+    const uint32_t u_hi = (~(hi + 0x7F7F7F7Fu) & 0x80808080u) >> 7;
+    if (COST16) {
+      // bytes 2j, 2j + 1 -> 16-bit halves of one word
+      cost[0] += (int32_t)(__byte_perm(u_lo, 0u, 0x4140u) * (uint32_t)w_cur);
+      cost[1] += (int32_t)(__byte_perm(u_lo, 0u, 0x4342u) * (uint32_t)w_cur);
+      cost[2] += (int32_t)(__byte_perm(u_hi, 0u, 0x4140u) * (uint32_t)w_cur);
+      cost[3] += (int32_t)(__byte_perm(u_hi, 0u, 0x4342u) * (uint32_t)w_cur);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        cost[q] += (int32_t)__byte_perm(u_lo, 0u, 0x4440u | q) * w_cur;
+        cost[q + 4] += (int32_t)__byte_perm(u_hi, 0u, 0x4440u | q) * w_cur;
+      }
+    }
+    if (!PLAIN3 && len == 0) continue;  // an empty clause has no clause RBM
+
+    const uint32_t rb = G.tab_e + grp * G.gstride;
+    const bool sat = !PLAIN3 && ((cinfo >> 5) & 1u) != 0;
+    // Philox rounds 0..2: the clause's share, then each unit's
+    const uint32_t cl = (uint32_t)(c - cl_base);
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * cl;
+    const uint32_t c1 = (uint32_t)(p0 >> 32) ^ phase ^ K.k1[0];
+    const uint32_t c2 = (uint32_t)p0;
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * c1;
+    const uint32_t c3 = (uint32_t)(p1 >> 32) ^ u2 ^ K.k0[1];
+    const uint32_t c4 = (uint32_t)p1;
+    const uint64_t p2 = (uint64_t)kPhiloxM0 * c3;
+    const uint32_t c5 = (uint32_t)(p2 >> 32) ^ K.k1[2];
+    const uint32_t c6 = (uint32_t)p2;
+    uint4 R[3];
+#pragma unroll
+    for (int h = 0; h < 3; ++h) {
+      const uint64_t pz = (uint64_t)kPhiloxM1 * (th[h] ^ c2);
+      R[h] = philox_rounds<3>(
+          make_uint4((uint32_t)(pz >> 32) ^ c4 ^ K.k0[2], (uint32_t)pz, c5 ^ sh[h], c6), K);
+    }
+    uint32_t h_lo = 0, h_hi = 0;
+    if (!sat)
+      octet_draws<false, NIB>((lo << 4) | G.up_lo, (hi << 4) | G.up_hi, rb, R, fe, h_lo, h_hi);
+    else
+      octet_draws<true, NIB>((lo << 4) | G.up_lo, (hi << 4) | G.up_hi, rb, R, fe, h_lo, h_hi);
+    if constexpr (NIB)
+      *reinterpret_cast<uint32_t*>(hb + (size_t)c * hstride) = h_lo;
+    else
+      *reinterpret_cast<uint2*>(hb + (size_t)c * hstride) = make_uint2(h_lo, h_hi);
+  }
+
+  if (COST16) {
+#pragma unroll
+    for (int j = 3; j >= 0; --j) {
+      cost[2 * j + 1] = (int32_t)((uint32_t)cost[j] >> 16);
+      cost[2 * j] = cost[j] & 0xFFFF;
+    }
+  }
+}
+
 // One block of the gather: chain tile bx of gx, clause block by of gy.
 // PERSIST: a block of the persistent round (k_round_persistent), which has
 // staged the record blocks already, orders its phases by grid barriers
 // instead of programmatic dependent launch, and reads the chain state from
 // the L2.
-template <bool PLAIN3, bool COST16, bool PERSIST>
+template <bool PLAIN3, bool COST16, bool PERSIST, bool NIB>
 __device__ __forceinline__ void gather3_block(const DevFormula& F, const DevTables& T,
                                               const DevChains& C, const GatherPlan& P,
                                               const uint32_t* tdev, uint32_t t_rel,
@@ -532,10 +686,7 @@ __device__ __forceinline__ void gather3_block(const DevFormula& F, const DevTabl
     stage(smem + (tab - s0), T.rec3, T.rec3_words * 4);
     __syncthreads();
   }
-  const int E = T.n_temps;
-  const int e0 = temp_of(C.g8_off * 8 + b0, E, C.B_total, C.inv_B_total);
-  const uint32_t tab_e = tab + (uint32_t)e0 * 256u;  // group 0 at the thread's temperature
-  const uint32_t gstride = (uint32_t)E * 256u;       // from one group to the next
+  const G3Tables G = gather3_tables(T, C, tab, b0);
   // the weighted unsatisfied cost of the thread's 8 chains in registers:
   // the host runs this kernel only when every clause block's weight sum is
   // below 2^31 (C.cost32); with COST16, cost[j] packs chains 2j and 2j + 1
@@ -559,114 +710,12 @@ __device__ __forceinline__ void gather3_block(const DevFormula& F, const DevTabl
     if (w1 > w0) l2_prefetch(reinterpret_cast<const void*>(w0), (uint32_t)(w1 - w0));
   }
   const uint32_t t = step_index(tdev, t_rel);
-  const RoundKeys& K = C.keys;
-  const uint32_t octet = (uint32_t)(g8 + C.g8_off);
-  const uint32_t phase = kPhaseHidden | ((uint32_t)inst << 8);
-  // round 0, word z = t: common to every unit and clause
-  const uint64_t pt = (uint64_t)kPhiloxM1 * t;
-  const uint32_t u1 = (uint32_t)(pt >> 32) ^ K.k0[0];
-  const uint32_t u2 = (uint32_t)pt;
-  // round 1, word x = round 0's (octet | h << 24) ^ u1: per thread and unit
-  uint32_t th[3], sh[3];
-#pragma unroll
-  for (int h = 0; h < 3; ++h) {
-    const uint64_t p = (uint64_t)kPhiloxM0 * ((octet | ((uint32_t)h << 24)) ^ u1);
-    th[h] = (uint32_t)(p >> 32) ^ K.k1[1];
-    sh[h] = (uint32_t)p;
-  }
-  const uint8_t* xtb = C.xt + b0;
-  uint8_t* hb = static_cast<uint8_t*>(C.H) + b0;
-
-  // software pipeline: the state bytes of the next clause and the record of
-  // the one after it are loaded while the current clause is sampled
-  const int c0 = c_begin + warp;
-  int4 rec_n = make_int4(0, 0, 0, 0);
-  if (c0 < c_end) rec_n = __ldg(F.cl4 + c0);
-  uint2 xa, xb, xc;
-  uint32_t info = (uint32_t)rec_n.w;
-  int32_t wc = 0;
-  if (c0 < c_end) wc = (int32_t)__ldg(F.cl_w + c0);
-  load_clause_state<PLAIN3, PERSIST>(xtb, Bp, rec_n, xa, xb, xc);
-  if (c0 + 8 < c_end) rec_n = __ldg(F.cl4 + c0 + 8);
-  for (int c = c0; c < c_end; c += 8) {
-    uint2 na = make_uint2(0u, 0u), nb = na, nc = na;
-    const uint32_t ninfo = (uint32_t)rec_n.w;
-    int32_t nwc = 0;
-    if (c + 8 < c_end) {
-      load_clause_state<PLAIN3, PERSIST>(xtb, Bp, rec_n, na, nb, nc);
-      nwc = (int32_t)__ldg(F.cl_w + c + 8);
-    }
-    if (c + 16 < c_end) rec_n = __ldg(F.cl4 + c + 16);
-    const int len = info & 3;
-    // byte q: chain q's truth pattern (chains 0..3 | 4..7)
-    const uint32_t flip = ((info >> 2) & 7u) * 0x01010101u;
-    const uint32_t lo = (xa.x + 2u * xb.x + 4u * xc.x) ^ flip;
-    const uint32_t hi = (xa.y + 2u * xb.y + 4u * xc.y) ^ flip;
-    const uint32_t grp = info >> 8;
-    const int32_t w_cur = wc;
-    xa = na;
-    xb = nb;
-    xc = nc;
-    info = ninfo;
-    wc = nwc;
-    // byte q is 1 when chain q has no true literal (pattern 0: 0x7F + p sets
-    // bit 7 for every p in 1..7 and never carries), else 0; each chain adds
-    // the clause weight times its byte, without branches
-    const uint32_t u_lo = (~(lo + 0x7F7F7F7Fu) & 0x80808080u) >> 7;
-    const uint32_t u_hi = (~(hi + 0x7F7F7F7Fu) & 0x80808080u) >> 7;
-    if (COST16) {
-      // bytes 2j, 2j + 1 -> 16-bit halves of one word
-      cost[0] += (int32_t)(__byte_perm(u_lo, 0u, 0x4140u) * (uint32_t)w_cur);
-      cost[1] += (int32_t)(__byte_perm(u_lo, 0u, 0x4342u) * (uint32_t)w_cur);
-      cost[2] += (int32_t)(__byte_perm(u_hi, 0u, 0x4140u) * (uint32_t)w_cur);
-      cost[3] += (int32_t)(__byte_perm(u_hi, 0u, 0x4342u) * (uint32_t)w_cur);
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        cost[q] += (int32_t)__byte_perm(u_lo, 0u, 0x4440u | q) * w_cur;
-        cost[q + 4] += (int32_t)__byte_perm(u_hi, 0u, 0x4440u | q) * w_cur;
-      }
-    }
-    if (!PLAIN3 && len == 0) continue;  // an empty clause has no clause RBM
-
-    const uint32_t rb = tab_e + grp * gstride;
-    const bool sat = !PLAIN3 && (lds32(rb + 128u) & 0x100u) != 0;
-    // Philox rounds 0..2: the clause's share, then each unit's
-    const uint32_t cl = (uint32_t)(c - cl_base);
-    const uint64_t p0 = (uint64_t)kPhiloxM0 * cl;
-    const uint32_t c1 = (uint32_t)(p0 >> 32) ^ phase ^ K.k1[0];
-    const uint32_t c2 = (uint32_t)p0;
-    const uint64_t p1 = (uint64_t)kPhiloxM1 * c1;
-    const uint32_t c3 = (uint32_t)(p1 >> 32) ^ u2 ^ K.k0[1];
-    const uint32_t c4 = (uint32_t)p1;
-    const uint64_t p2 = (uint64_t)kPhiloxM0 * c3;
-    const uint32_t c5 = (uint32_t)(p2 >> 32) ^ K.k1[2];
-    const uint32_t c6 = (uint32_t)p2;
-    uint4 R[3];
-#pragma unroll
-    for (int h = 0; h < 3; ++h) {
-      const uint64_t pz = (uint64_t)kPhiloxM1 * (th[h] ^ c2);
-      R[h] = philox_rounds<3>(
-          make_uint4((uint32_t)(pz >> 32) ^ c4 ^ K.k0[2], (uint32_t)pz, c5 ^ sh[h], c6), K);
-    }
-    uint32_t h_lo = 0, h_hi = 0;
-    if (!sat)
-      octet_draws<false>(lo << 4, hi << 4, rb, R, fe, h_lo, h_hi);
-    else
-      octet_draws<true>(lo << 4, hi << 4, rb, R, fe, h_lo, h_hi);
-    *reinterpret_cast<uint2*>(hb + (size_t)c * Bp) = make_uint2(h_lo, h_hi);
-  }
+  gather3_clauses<PLAIN3, COST16, PERSIST, NIB>(F, C, G, inst, c_begin, c_end, cl_base, t, g8, warp,
+                                                cost, fe);
 
   // per-block partial sums; the block that arrives last among its instance's
   // blocks for this tile of 256 chains reduces them in block order and keeps
   // improvements (as k_gather)
-  if (COST16) {
-#pragma unroll
-    for (int j = 3; j >= 0; --j) {
-      cost[2 * j + 1] = (int32_t)((uint32_t)cost[j] >> 16);
-      cost[2 * j] = cost[j] & 0xFFFF;
-    }
-  }
   int32_t* my_cost32 = reinterpret_cast<int32_t*>(&s_cost[0][0]) + warp * 256 + lane * 8;
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
@@ -713,12 +762,12 @@ __device__ __forceinline__ void gather3_block(const DevFormula& F, const DevTabl
 #undef G3_GY
 }
 
-template <bool PLAIN3, bool COST16>
+template <bool PLAIN3, bool COST16, bool NIB>
 __global__ void __launch_bounds__(256, 2) k_gather3(DevFormula F, DevTables T, DevChains C,
                                                     GatherPlan P, const uint32_t* tdev,
                                                     uint32_t t_rel, int64_t* cost_part,
                                                     float* fe_part, int32_t* tickets) {
-  gather3_block<PLAIN3, COST16, false>(F, T, C, P, tdev, t_rel, cost_part, fe_part, tickets,
+  gather3_block<PLAIN3, COST16, false, NIB>(F, T, C, P, tdev, t_rel, cost_part, fe_part, tickets,
                                        blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
 }
 
@@ -909,6 +958,256 @@ __global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4) k_visible(DevFormula 
 }
 
 // ---------------------------------------------------------------------------
+// Visible update on nibble patterns (C.nib): formulas whose clause groups all
+// have at most 3 hidden units. The results are those of k_visible, bit for bit.
+//
+// The sum over a variable's incidences is what the update does most of: at
+// weighted 3-SAT n = 1000, m = 6000 and 4096 chains, 18000 incidences x 4096
+// chains a round. k_visible looks each (incidence, chain) up in a shared-memory
+// table: 78 warp instructions per incidence and 8 chains, 22.6 M a launch, issue
+// active 64 %. Here the gather stores an octet's patterns as one word of 4-bit
+// fields, and an incidence's contributions to its literal for the 8 patterns of
+// 3 hidden units are 8 low and 8 high bytes (four registers, read by one
+// broadcast from shared memory). A byte permute takes four 4-bit fields as its
+// selector and so looks up four chains in one instruction; two lookups (low and
+// high bytes) and two permutes give four chains' 16-bit contributions as pairs,
+// which are added as pairs: 13 instructions per incidence and 8 chains, and half
+// the pattern bytes to read. The table holds contribution + T.ptab_bias
+// (>= 0), so a pair's halves never borrow from one another; a window of 32
+// incidences stays below 2^16 (the host takes this kernel only for
+// |2^Q G| <= 1023), then the sums move to 32 bits.
+//
+// The blocks are resident (4 per SM) and each warp walks variables: the tables
+// are staged once per block instead of once per 8 variables, and the next
+// variable's record and incidences are loaded while the current one is summed.
+// ---------------------------------------------------------------------------
+struct VisPos {  // position in the walk over (chain tile, variable slot)
+  int fast, slow;
+};
+
+__device__ __forceinline__ VisPos vis_next(VisPos p, int dfast, int dslow, int nfast) {
+  p.fast += dfast;
+  p.slow += dslow;
+  if (p.fast >= nfast) {
+    p.fast -= nfast;
+    ++p.slow;
+  }
+  return p;
+}
+
+// the contributions of four chains (selector s, low 16 bits) as pairs
+__device__ __forceinline__ void nib_pairs(const uint4& tb, uint32_t s, uint32_t& p01,
+                                          uint32_t& p23) {
+  const uint32_t lo = __byte_perm(tb.x, tb.y, s), hi = __byte_perm(tb.z, tb.w, s);
+  p01 = __byte_perm(lo, hi, 0x5140u);
+  p23 = __byte_perm(lo, hi, 0x7362u);
+}
+
+// adds the contributions of the octet's 8 chains (pattern word h)
+__device__ __forceinline__ void nib_add(const uint4& tb, uint32_t h, uint32_t (&acc)[4]) {
+  uint32_t a, b;
+  nib_pairs(tb, h, a, b);
+  acc[0] += a;
+  acc[1] += b;
+  nib_pairs(tb, h >> 16, a, b);
+  acc[2] += a;
+  acc[3] += b;
+}
+
+// as nib_add for an octet across two temperatures: table ta, and tb for the
+// chains of mask mk (one 16-bit half per chain)
+__device__ __forceinline__ void nib_add2(const uint4& ta, const uint4& tb, uint32_t h,
+                                         const uint32_t (&mk)[4], uint32_t (&acc)[4]) {
+#pragma unroll
+  for (int w = 0; w < 4; w += 2) {
+    uint32_t a, b, a1, b1;
+    nib_pairs(ta, w ? h >> 16 : h, a, b);
+    nib_pairs(tb, w ? h >> 16 : h, a1, b1);
+    acc[w] += (a & ~mk[w]) | (a1 & mk[w]);
+    acc[w + 1] += (b & ~mk[w + 1]) | (b1 & mk[w + 1]);
+  }
+}
+
+// the masks of the chains from `split` on
+__device__ __forceinline__ void nib_masks(int split, uint32_t (&mk)[4]) {
+#pragma unroll
+  for (int w = 0; w < 4; ++w)
+    mk[w] = (2 * w >= split ? 0x0000FFFFu : 0u) | (2 * w + 1 >= split ? 0xFFFF0000u : 0u);
+}
+
+// the octet's temperatures: tab at the first chain's; returns the first chain
+// of the next temperature (8: none; octets have at most two)
+__device__ __forceinline__ int nib_split(const DevTables& T, const DevChains& C, int b0,
+                                         uint32_t tab0, uint32_t& tab) {
+  const int gb0 = C.g8_off * 8 + b0;
+  const int e0 = temp_of(gb0, T.n_temps, C.B_total, C.inv_B_total);
+  tab = tab0 + (uint32_t)(e0 * T.ptab_stride);
+  if (e0 == temp_of(gb0 + 7, T.n_temps, C.B_total, C.inv_B_total)) return 8;
+  return (int)(((long long)(e0 + 1) * C.B_total + T.n_temps - 1) / T.n_temps) - gb0;
+}
+
+// moves a window's sums (with cw biases) to 32 bits
+__device__ __forceinline__ void nib_flush(const uint32_t (&acc)[4], int bias, int (&z)[8]) {
+#pragma unroll
+  for (int w = 0; w < 4; ++w) {
+    z[2 * w] += (int)(acc[w] & 0xFFFFu) - bias;
+    z[2 * w + 1] += (int)(acc[w] >> 16) - bias;
+  }
+}
+
+// The end of a visible update, as visible_tail: best-so-far of the chains
+// flagged in imp, the visible draws (Eq. 3) and nu (Sec. 4.4); an entry of pva
+// holds P and alpha rho (1 - rho) as visible_tail rounds it.
+__device__ __forceinline__ void nib_tail(const DevTables& T, const DevChains& C, const uint2* pva,
+                                         float keep, uint32_t t, int inst, int local, int g8,
+                                         size_t o, uint64_t xold, uint64_t imp, const float4& n0,
+                                         const float4& n1, const int (&z)[8]) {
+  if (imp) {
+    const uint64_t mask = imp * 0xFFull;  // 0x01 flags -> 0xFF byte masks
+    uint64_t* bx = reinterpret_cast<uint64_t*>(C.best_xt + o);
+    *bx = (*bx & ~mask) | (xold & mask);
+  }
+  const uint4 r = philox4x32_10(make_uint4((uint32_t)local, (uint32_t)(g8 + C.g8_off), t,
+                                           kPhaseVisible | ((uint32_t)inst << 8)),
+                                C.keys);
+  float nu[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
+  uint32_t x_lo = 0, x_hi = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const uint2 pv = pva[__viaddmin_s32_relu(z[q], T.qmax, 2 * T.qmax)];
+    nu[q] = __fmaf_rn(keep, nu[q], __uint_as_float(pv.y));
+    const uint32_t bit = lane16(r, q) < pv.x ? 1u << (8 * (q & 3)) : 0u;
+    if (q < 4) x_lo |= bit;
+    else x_hi |= bit;
+  }
+  float4* nu4 = reinterpret_cast<float4*>(C.nu + o);
+  nu4[0] = make_float4(nu[0], nu[1], nu[2], nu[3]);
+  nu4[1] = make_float4(nu[4], nu[5], nu[6], nu[7]);
+  *reinterpret_cast<uint2*>(C.xt + o) = make_uint2(x_lo, x_hi);
+}
+
+// shared memory of k_visible_nib: contribution rows, then visible entries
+__host__ __device__ __forceinline__ int nib_rows_bytes(const DevTables& T) {
+  return T.n_temps * T.ptab_stride;
+}
+
+template <int BATCH>
+__global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4)
+    k_visible_nib(DevFormula F, DevTables T, DevChains C, float keep, const uint32_t* tdev,
+                  uint32_t t_rel, int tile_major) {
+  static_assert(32 % BATCH == 0, "incidence windows hold whole batches");
+  pdl_release();
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int2 s_inc[8][32];  // per warp: a window of its variable's incidences
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rows = nib_rows_bytes(T);
+  stage(smem, T.ptab, rows);
+  stage(smem + rows, T.pva, align16(T.pv_len * 8));
+  __syncthreads();
+  const uint32_t tab0 = (uint32_t)__cvta_generic_to_shared(smem);
+  const uint2* pva = reinterpret_cast<const uint2*>(smem + rows);
+  const int tiles = C.Bp / kChainTile;
+  // tile_major: every variable of one chain tile before the next tile (its
+  // patterns, m x 128 bytes, then stay in the L2)
+  const int nfast = tile_major ? F.n : tiles, nslow = tile_major ? tiles : F.n;
+  const int stride = (int)gridDim.x * 8;
+  const int dslow = stride / nfast, dfast = stride - dslow * nfast;
+  VisPos p;
+  {
+    const int first = blockIdx.x * 8 + warp;
+    p.slow = first / nfast;
+    p.fast = first - p.slow * nfast;
+  }
+  auto slot_of = [&](const VisPos& q) { return tile_major ? q.fast : q.slow; };
+  auto load_slot = [&](const VisPos& q) {
+    return q.slow < nslow ? __ldg(F.var_slot + slot_of(q)) : make_int4(0, 0, 0, 0);
+  };
+  // a window of up to 32 incidences; the padding reads clause 0 and the zero row
+  auto load_inc = [&](int j0, int cnt) {
+    return lane < cnt ? __ldg(F.var_inc8 + j0 + lane) : make_int2(0, 0);
+  };
+  int4 rec = load_slot(p);
+  VisPos p1 = vis_next(p, dfast, dslow, nfast);
+  int4 rec1 = load_slot(p1);
+  int2 win = load_inc(rec.y, rec.z);
+  pdl_wait();  // chain state from here on
+  const uint32_t t = step_index(tdev, t_rel);
+  int last_tile = -1, split = 8;
+  uint32_t tab = tab0;
+  bool two = false;
+  const size_t hstride = (size_t)(C.Bp / 8);
+
+  while (p.slow < nslow) {
+    const int tile = tile_major ? p.slow : p.fast;
+    const int g8 = tile * 32 + lane, b0 = g8 * 8;
+    __syncwarp();
+    s_inc[warp][lane] = win;
+    __syncwarp();
+    // this item's state and the next item's incidences go out first
+    const int i = rec.x, cnt = rec.z;
+    const size_t o = (size_t)i * C.Bp + b0;
+    const uint64_t xold = *reinterpret_cast<const uint64_t*>(C.xt + o);
+    const float4 n0 = reinterpret_cast<const float4*>(C.nu + o)[0];
+    const float4 n1 = reinterpret_cast<const float4*>(C.nu + o)[1];
+    const int local = F.var_inst ? __ldg(F.var_inst + i).y : i;
+    const VisPos p2 = vis_next(p1, dfast, dslow, nfast);
+    const int4 rec2 = load_slot(p2);
+    win = load_inc(rec1.y, rec1.z);
+    if (tile != last_tile) {
+      last_tile = tile;
+      split = nib_split(T, C, b0, tab0, tab);
+      two = __any_sync(0xFFFFFFFFu, split < 8);
+    }
+    const uint32_t* H = static_cast<const uint32_t*>(C.H) + g8;
+    int z[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) z[q] = 0;
+    for (int j = 0; j < cnt; j += 32) {
+      if (j > 0) {
+        const int2 w = load_inc(rec.y + j, cnt - j);
+        __syncwarp();
+        s_inc[warp][lane] = w;
+        __syncwarp();
+      }
+      const int cw = min(cnt - j, 32);
+      uint32_t acc[4] = {0u, 0u, 0u, 0u};
+      if (!two) {
+#pragma unroll 1
+        for (int k = 0; k < cw; k += BATCH) {
+          uint32_t h[BATCH];
+#pragma unroll
+          for (int u = 0; u < BATCH; ++u) h[u] = __ldg(H + (size_t)s_inc[warp][k + u].x * hstride);
+#pragma unroll
+          for (int u = 0; u < BATCH; ++u) {
+            nib_add(lds128(tab + (uint32_t)s_inc[warp][k + u].y), h[u], acc);
+          }
+        }
+      } else {
+        // some octet of the warp lies across two temperatures: both tables,
+        // the upper one for the chains from `split` on
+        uint32_t mk[4];
+        nib_masks(split, mk);
+        const uint32_t tab1 = split < 8 ? tab + (uint32_t)T.ptab_stride : tab;
+#pragma unroll 1
+        for (int k = 0; k < cw; ++k) {
+          const int2 inc = s_inc[warp][k];
+          nib_add2(lds128(tab + (uint32_t)inc.y), lds128(tab1 + (uint32_t)inc.y),
+                   __ldg(H + (size_t)inc.x * hstride), mk, acc);
+        }
+      }
+      nib_flush(acc, cw * T.ptab_bias, z);
+    }
+    const uint64_t imp = *reinterpret_cast<const unsigned long long*>(
+        C.improved + (size_t)rec.w * C.Bp + b0);
+    nib_tail(T, C, pva, keep, t, rec.w, local, g8, o, xold, imp, n0, n1, z);
+    p = p1;
+    p1 = p2;
+    rec = rec1;
+    rec1 = rec2;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Persistent round: `rounds` Gibbs rounds in one cooperative launch. Every
 // block walks the virtual blocks of the gather (chain tile fastest, as the
 // gather's grid), meets the other blocks at a grid barrier, walks the
@@ -986,7 +1285,7 @@ __global__ void __launch_bounds__(256, 2)
   for (int r = 0; r < rounds; ++r) {
     const uint32_t t = t0 + (uint32_t)r;
     for (uint32_t vb = blockIdx.x; vb < n_gather; vb += gridDim.x)
-      gather3_block<PLAIN3, COST16, true>(F, T, C, P, nullptr, t, C.cost_part, C.fe_part,
+      gather3_block<PLAIN3, COST16, true, false>(F, T, C, P, nullptr, t, C.cost_part, C.fe_part,
                                           C.tickets, vb % tiles, vb / tiles, tiles, n_blk);
     if (!grid_barrier(bar, target, err)) return;
     for (uint32_t vb = blockIdx.x; vb < n_visible; vb += gridDim.x) {
@@ -1036,6 +1335,8 @@ int visible_smem_bytes(const DevTables& T) {
 }
 
 constexpr int kSmemLimit = 160 * 1024;
+constexpr int kNibSmemLimit = 48 * 1024;
+int l2_bytes();
 constexpr int kMaxGridY = 65535;
 
 // a launch that may overlap its predecessor's tail (see pdl_wait)
@@ -1062,9 +1363,10 @@ int gather3_smem_bytes(const DevTables& T) { return T.rec3_words * 4 + 256; }
 using Gather3Fn = void (*)(DevFormula, DevTables, DevChains, GatherPlan, const uint32_t*,
                            uint32_t, int64_t*, float*, int32_t*);
 
+template <bool NIB>
 Gather3Fn gather3_kernel(const DevTables& T, const DevChains& C) {
-  if (T.plain3) return C.cost16 ? k_gather3<true, true> : k_gather3<true, false>;
-  return C.cost16 ? k_gather3<false, true> : k_gather3<false, false>;
+  if (T.plain3) return C.cost16 ? k_gather3<true, true, NIB> : k_gather3<true, false, NIB>;
+  return C.cost16 ? k_gather3<false, true, NIB> : k_gather3<false, false, NIB>;
 }
 
 // every octet of chains has one temperature: each temperature block starts
@@ -1077,6 +1379,12 @@ bool octets_single_temperature(const DevTables& T, const DevChains& C) {
   return true;
 }
 
+// no octet of chains has more than two temperatures, the second one the next
+// (temperature blocks of at least 8 chains, or blocks that begin with octets)
+bool octets_two_temperatures(const DevTables& T, const DevChains& C) {
+  return T.n_temps == 1 || C.B_total / T.n_temps >= 8 || octets_single_temperature(T, C);
+}
+
 template <int MODE, bool SM, typename HT>
 cudaError_t gather_variant(dim3 grid, int smem, cudaStream_t st, const DevFormula& F,
                            const DevTables& T, const DevChains& C, const uint8_t* xt, int B,
@@ -1084,9 +1392,9 @@ cudaError_t gather_variant(dim3 grid, int smem, cudaStream_t st, const DevFormul
                            int64_t* cost_part, float* fe_part, int32_t* tickets,
                            int64_t* eval_out) {
   if constexpr (MODE == kStep && SM && sizeof(HT) == 1) {
-    if (T.one_chunk && T.rec3 && F.cl4 && C.cost32 && octets_single_temperature(T, C)) {
+    if (T.one_chunk && T.rec3 && F.cl4 && C.cost32 && octets_two_temperatures(T, C)) {
       const int sm3 = gather3_smem_bytes(T);
-      auto kern = gather3_kernel(T, C);
+      auto kern = C.nib ? gather3_kernel<true>(T, C) : gather3_kernel<false>(T, C);
       const cudaError_t e = allow_dynamic_smem(kern, sm3);
       if (e != cudaSuccess) return e;
       return launch_pdl(kern, grid, sm3, st, F, T, C, P, tdev, t_rel, cost_part, fe_part,
@@ -1150,14 +1458,7 @@ cudaError_t visible_variant(dim3 grid, int smem, cudaStream_t st, const DevFormu
   }
   const int groups = (F.n + 7) / 8, tiles = (int)grid.x;
   // tile-major when the hidden patterns exceed half the L2
-  static int l2 = -1;
-  if (l2 < 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
-      l2 = 0;
-  }
-  const int tm = (double)F.m * C.Bp * sizeof(HT) > 0.5 * (double)l2 ? 1 : 0;
+  const int tm = (double)F.m * C.Bp * sizeof(HT) > 0.5 * (double)l2_bytes() ? 1 : 0;
   if (tm) {
     // x = variable groups, y = chain tiles (launches of at most kMaxGridY tiles)
     grid.x = (unsigned)groups;
@@ -1177,7 +1478,58 @@ cudaError_t visible_variant(dim3 grid, int smem, cudaStream_t st, const DevFormu
   return cudaGetLastError();
 }
 
+// L2 bytes of the current device (0 when unknown)
+int l2_bytes() {
+  static int l2 = -1;
+  if (l2 < 0) {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
+      v = 0;
+    l2 = v;
+  }
+  return l2;
+}
+
+int sm_count() {
+  static int sms = 0;
+  if (!sms) {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+      v = 1;
+    sms = v;
+  }
+  return sms;
+}
+
+int nib_smem_bytes(const DevTables& T) { return nib_rows_bytes(T) + align16(T.pv_len * 8); }
+
+cudaError_t visible_nib(const DevFormula& F, const DevTables& T, const DevChains& C, float alpha,
+                        const uint32_t* tdev, uint32_t t_rel, int batch, cudaStream_t st) {
+  auto kern = batch >= 8 ? k_visible_nib<8> : batch <= 2 ? k_visible_nib<2> : k_visible_nib<4>;
+  const int smem = nib_smem_bytes(T);
+  const cudaError_t e = allow_dynamic_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  const long long items = (long long)F.n * (C.Bp / kChainTile);
+  const long long grid = std::min<long long>((items + 7) / 8, (batch >= 8 ? 3LL : 4LL) * sm_count());
+  const int tm = (double)F.m * C.Bp * 0.5 > 0.5 * (double)l2_bytes() ? 1 : 0;
+  // 1 - alpha as the device's one rounding gives it
+  volatile float one = 1.0f;
+  const float keep = one - alpha;
+  return launch_pdl(kern, dim3((unsigned)grid), smem, st, F, T, C, keep, tdev, t_rel, tm);
+}
+
 }  // namespace
+
+// Nibble patterns: every group has at most 3 hidden units, the contribution
+// rows were built (|2^Q G| <= 1023, so a window of 32 incidences fits 16 bits)
+// and leave room for 4 blocks per SM, and no octet of chains spans more than
+// two temperatures (temperature blocks of at least 8 chains).
+bool nib_patterns_supported(const DevTables& T, int B_total) {
+  return T.one_chunk && T.ptab && nib_smem_bytes(T) <= kNibSmemLimit &&
+         (T.n_temps == 1 || B_total / T.n_temps >= 8);
+}
 
 int clause_block_for(int m) {
   const int per = (m + 255) / 256;
@@ -1227,9 +1579,10 @@ int gather_blocks_per_sm(const DevTables& T, bool wide) {
     // k_gather3 runs whenever the chains' octets have single temperatures
     // (the variant with the most registers stands for all four)
     const int sm3 = gather3_smem_bytes(T);
-    if (allow_dynamic_smem(k_gather3<false, false>, sm3) != cudaSuccess) return 1;
+    auto kern = k_gather3<false, false, true>;
+    if (allow_dynamic_smem(kern, sm3) != cudaSuccess) return 1;
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_gather3<false, false>, 256, sm3) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 256, sm3) !=
         cudaSuccess)
       return 1;
     return nb > 0 ? nb : 1;
@@ -1274,6 +1627,7 @@ cudaError_t launch_gather(GatherMode mode, const DevFormula& F, const DevTables&
 cudaError_t launch_visible(const DevFormula& F, const DevTables& T, const DevChains& C,
                            float alpha, const uint32_t* tdev, uint32_t t_rel, bool wide,
                            cudaStream_t st, int batch) {
+  if (C.nib && !wide) return visible_nib(F, T, C, alpha, tdev, t_rel, batch, st);
   dim3 grid(C.Bp / kChainTile, (F.n + 7) / 8);
   const int sm = visible_smem_bytes(T);
   const bool use_sm = sm <= kSmemLimit;

@@ -1,0 +1,91 @@
+"""Rounds on formulas of at most 3 literals per clause, where their kernels
+change form: variables in more than 32 clauses (several incidence windows),
+octets of chains across two temperatures, temperature blocks too small or
+contributions too large for 4-bit patterns, several chain tiles, formulas
+smaller than a block. Every case against the oracle, bit for bit (the free
+energy within the 1e-3 bar of the other parity tests)."""
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+FSTARS = [0.05, 0.068, 0.12, 0.25, 0.4, 0.528]
+
+
+@pytest.fixture(scope="module")
+def ms():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2311_02101_gb300 as m
+    return m
+
+
+_tables = {}
+
+
+def table_for(temps, Q):
+    if (temps, Q) not in _tables:
+        table = oracle.make_table([1, 2, 3], FSTARS[:temps], n_buckets=2, Q=Q, iters=1500)
+        for s in table.sets:
+            s["W"] = 6.0 * np.asarray(s["W"])  # on the grid, sized as converged fits are
+        _tables[temps, Q] = table
+    return _tables[temps, Q]
+
+
+def short_clauses(n, m, seed):
+    """m clauses of 0..3 literals, repeated and opposite literals included."""
+    rng = np.random.default_rng(seed)
+    cl = [list(rng.integers(1, n + 1, size=k) * (1 - 2 * rng.integers(0, 2, size=k)))
+          for k in rng.integers(0, 4, size=m)]
+    return oracle.Instance.from_clauses(n, cl, list(rng.integers(1, 9, size=m)))
+
+
+CASES = {
+    # name: (instance, chains, temperatures, quantisation bits)
+    "high-degree": (lambda: oracle.Instance(*workloads.random_ksat(9, 400, 3, 1)), 264, 2, 4),
+    "straddle": (lambda: oracle.Instance(*workloads.random_ksat(40, 171, 3, 2, 50)), 300, 3, 4),
+    "short": (lambda: short_clauses(23, 90, 3), 520, 6, 4),
+    "thin-temperatures": (lambda: short_clauses(23, 90, 4), 44, 6, 4),
+    "wide-contributions": (lambda: short_clauses(23, 90, 5), 256, 2, 8),
+    "one-clause": (lambda: short_clauses(3, 1, 6), 8, 1, 4),
+    "no-clause": (lambda: oracle.Instance.from_clauses(5, [], []), 40, 2, 4),
+    "tiles": (lambda: oracle.Instance(*workloads.random_ksat(70, 333, 3, 7, 30000)), 1300, 2, 4),
+    "more-variables-than-clauses": (lambda: oracle.Instance(*workloads.random_ksat(900, 20, 3, 8)),
+                                    256, 2, 4),
+}
+
+
+@pytest.mark.parametrize("profiled", [False, True])
+@pytest.mark.parametrize("case", list(CASES))
+def test_rounds_match_oracle(ms, case, profiled):
+    """`profiled` keeps the two-launch round (events around every launch)."""
+    import torch
+    make, B, temps, Q = CASES[case]
+    inst, table, alpha, seed = make(), table_for(temps, Q), 0.05, 21
+    p = ms.maxsat_default_params(sets=table.sets, n_temps=temps, n_buckets=2, alpha=alpha,
+                                 quant_bits=Q, path=ms.MAXSAT_PATH_SPARSE, steps_per_graph=4)
+    ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, torch.cuda.Stream())
+    ms.maxsat_reset(ctx, B, seed)
+    if profiled:
+        ms.maxsat_set_profiling(ctx, True)
+    for steps in (1, 7, 4):
+        ms.maxsat_step(ctx, steps)
+    g = ms.maxsat_get_state(ctx)
+    ms.maxsat_destroy(ctx)
+    st = oracle.init_chains(inst.n, B, seed)
+    oracle.gibbs(inst, table, st, 12, seed, n_temps=temps, n_buckets=2, alpha=alpha,
+                 threads=os.cpu_count() or 4)
+    assert g["t"] == 12
+    assert np.array_equal(g["x"], st.x)
+    assert np.array_equal(g["nu"], st.nu32)
+    for k in ("cost", "best_cost", "best_x"):
+        assert np.array_equal(g[k], getattr(st, k)), k
+    np.testing.assert_allclose(g["free_energy"], st.free_energy, rtol=1e-3, atol=1e-6)
