@@ -237,6 +237,11 @@ struct maxsat_ctx {
   int ev_buf = 0;                 // state buffer of the next evaluation
   int* d_err = nullptr;           // device wait-timeout code (0 = none)
   uint32_t* d_bar = nullptr;      // persistent round: grid-barrier arrivals and give-up flag
+  // resident rounds (k_rounds) of the current chains: blocks per chain tile (0:
+  // not used), its buffers, and what the next launch starts from
+  RoundsArgs rounds;
+  bool rounds_cost16 = false;
+  int rounds_slot_count = -1;     // resident blocks of k_rounds (-1: not queried)
   bool persist_ran = false;       // some maxsat_step ran persistent launches (read d_err)
   // dense scatter-add (GEMM2): block-diagonal variable x incidence matrix
   int tiles_v = 0, kmax = 0;
@@ -459,11 +464,78 @@ int upload_plan(maxsat_ctx* ctx, DevAllocs& A, int cb, GatherPlan* P, int64_t* w
   return MAXSAT_OK;
 }
 
+// Largest weight sum of a block, and of the clauses one warp of it takes
+// (every eighth), when one formula's clauses are split into nb blocks of whole
+// groups of 8, as even as possible.
+void split_weights(const maxsat_ctx* ctx, int nb, int64_t* wmax, int64_t* wmax8) {
+  const int m = ctx->m, groups = (m + 7) / 8;
+  *wmax = *wmax8 = 0;
+  for (int k = 0, c = 0; k < nb; ++k) {
+    const int e = std::min(m, c + 8 * (groups / nb + (k < groups % nb ? 1 : 0)));
+    int64_t sum = 0, part[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int q = c; q < e; ++q) {
+      sum += ctx->h_w[q];
+      part[(q - c) & 7] += ctx->h_w[q];
+    }
+    *wmax = std::max(*wmax, sum);
+    for (int64_t v : part) *wmax8 = std::max(*wmax8, v);
+    c = e;
+  }
+}
+
+// Sets up the resident rounds for the chains being allocated (Bp chains, the
+// gather's plan made): S blocks per chain tile, as many as the plan has when
+// they are all resident, else as many as are. S = 0 (two launches per round)
+// for a batch, for more chain tiles than half the resident blocks, or when
+// whole tiles would leave more than a sixth of them idle.
+int plan_rounds(maxsat_ctx* ctx, DevAllocs& A, int Bp) {
+  RoundsArgs& R = ctx->rounds;
+  R = RoundsArgs{};
+  if (ctx->n_inst != 1 || ctx->wide_h || !ctx->F.cl4) return MAXSAT_OK;
+  if (ctx->rounds_slot_count < 0) ctx->rounds_slot_count = rounds_slots(ctx->T);
+  const int slots = ctx->rounds_slot_count, tiles = Bp / kChainTile;
+  const int most = slots / tiles;
+  if (most < 2) return MAXSAT_OK;
+  const int S = std::min(most, std::max(1, ctx->plan.n_blk));
+  if (S == most && tiles * most < slots - slots / 6) return MAXSAT_OK;
+  int64_t w = 0, w8 = 0;
+  split_weights(ctx, S, &w, &w8);
+  if (w >= ((int64_t)1 << 31)) return MAXSAT_OK;
+  double fmax = 0.0;
+  for (const GroupMeta& gm : ctx->tabs.meta)
+    for (int k = 0; k < ctx->T.n_temps << gm.len; ++k) {
+      float f;
+      std::memcpy(&f, &ctx->tabs.rec[(size_t)gm.rec_off + (size_t)k * gm.stride], 4);
+      fmax = std::max(fmax, std::fabs((double)f));
+    }
+  const double sum = std::max(1.0, 2.0 * fmax * std::max(ctx->m, 1));
+  R.fe_scale = std::ldexp(1.0, std::min(40, 61 - (int)std::ceil(std::log2(sum))));
+  ctx->rounds_cost16 = w8 < 65536;
+  CK(ctx, A.alloc(&R.bar, (size_t)tiles * kBarStride));
+  CK(ctx, A.alloc(&R.acc, (size_t)6 * Bp));
+  R.err = ctx->d_err;
+  R.S = S;
+  return MAXSAT_OK;
+}
+
+// Fresh barrier counts and accumulators for the resident rounds.
+int clear_rounds(maxsat_ctx* ctx) {
+  RoundsArgs& R = ctx->rounds;
+  if (R.S == 0) return MAXSAT_OK;
+  const int Bp = ctx->C.Bp;
+  CK(ctx, cudaMemsetAsync(R.bar, 0, 4 * (size_t)(Bp / kChainTile) * kBarStride, ctx->stream));
+  CK(ctx, cudaMemsetAsync(R.acc, 0, 8 * (size_t)6 * Bp, ctx->stream));
+  R.bar0 = 0;
+  R.acc0 = 0;
+  return MAXSAT_OK;
+}
+
 int alloc_chains(maxsat_ctx* ctx, int32_t B) {
   if (ctx->have_chains && ctx->C.B == B && ctx->chains_dense == ctx->dense) return MAXSAT_OK;
   destroy_graph(ctx);
   ctx->chain_mem.release();
   ctx->have_chains = false;
+  ctx->rounds = RoundsArgs{};
   const int Bp = (B + kChainTile - 1) / kChainTile * kChainTile;
   const size_t nB = (size_t)ctx->n * Bp;
   if (ctx->gather_slots == 0) {
@@ -523,7 +595,7 @@ int alloc_chains(maxsat_ctx* ctx, int32_t B) {
   uint8_t* H = nullptr;
   CK(ctx, A.alloc(&H, (size_t)ctx->m * Bp * (ctx->wide_h ? 2 : 1)));
   C.H = H;
-  return MAXSAT_OK;
+  return plan_rounds(ctx, A, Bp);
 }
 
 // Copies h to a new device buffer padded with zeros to a multiple of 16 bytes
@@ -534,7 +606,7 @@ int check_device_error(maxsat_ctx* ctx) {
   CK(ctx, cudaMemcpy(&code, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost));
   if (code != 0)
     return fail(ctx, MAXSAT_ECUDA,
-                std::string(code == 16 ? "a grid barrier of the persistent round"
+                std::string(code == 16 ? "a block barrier of the resident or persistent rounds"
                                        : "a tensor-core pipeline wait") +
                     " timed out (code " + std::to_string(code) + "); results are invalid");
   return MAXSAT_OK;
@@ -1425,6 +1497,28 @@ static bool persistent_round_active(const maxsat_ctx* ctx) {
          persistent_round_supported(ctx->T, ctx->C, ctx->F, ctx->wide_h);
 }
 
+// The caller is capturing the context's stream: a resident launch carries the
+// barrier counts it starts from, so it cannot be replayed.
+static bool stream_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return s != cudaStreamCaptureStatusNone;
+}
+
+// rounds per launch of the resident rounds
+static constexpr int64_t kMaxResidentRounds = 1000;
+
+// maxsat_step runs resident rounds (k_rounds): planned for these chains, no
+// per-kernel profiling, no GPU unit propagation pending (it runs beside the
+// rounds on a side stream, and a cooperative launch would wait for its SMs)
+static bool resident_rounds_active(const maxsat_ctx* ctx) {
+  return ctx->have_chains && !ctx->dense && ctx->rounds.S > 0 && ctx->C.nib && !ctx->profiling &&
+         !(ctx->up_pending && ctx->up_on_gpu) && !stream_capturing(ctx->stream);
+}
+
 int maxsat_get_persistent_round(const maxsat_ctx* ctx) {
   if (!ctx) return MAXSAT_EINVAL;
   return persistent_round_active(ctx) ? 1 : 0;
@@ -1475,6 +1569,8 @@ int maxsat_reset_shard(maxsat_ctx* ctx, int32_t B, uint64_t seed, int32_t chain_
                               ctx->e5m2, ctx->stream));
   else
     CK(ctx, launch_init_sparse(ctx->F, ctx->C, ctx->n, ctx->stream));
+  rc = clear_rounds(ctx);
+  if (rc != MAXSAT_OK) return rc;
   ctx->have_chains = true;
   return MAXSAT_OK;
 }
@@ -1485,6 +1581,22 @@ int maxsat_step(maxsat_ctx* ctx, int64_t steps) {
   if (!ctx->have_chains) return fail(ctx, MAXSAT_ESTATE, "maxsat_step before maxsat_reset");
   if (steps < 0) return fail(ctx, MAXSAT_EINVAL, "steps must be >= 0");
   if ((uint64_t)ctx->t + (uint64_t)steps > 0xFFFFFFFFull) return fail(ctx, MAXSAT_EINVAL, "round index would exceed 2^32");
+  if (resident_rounds_active(ctx)) {
+    while (steps > 0) {
+      RoundsArgs& R = ctx->rounds;
+      R.t0 = ctx->t;
+      R.rounds = (int)std::min<int64_t>(steps, kMaxResidentRounds);
+      CK(ctx, launch_rounds(ctx->F, ctx->T, ctx->C, R, ctx->rounds_cost16, (float)ctx->prm.alpha,
+                            ctx->stream));
+      ctx->persist_ran = true;
+      R.bar0 += (uint32_t)R.S * (2u * (uint32_t)R.rounds - 1u);
+      R.acc0 = (R.acc0 + R.rounds) % 3;
+      ctx->t += (uint32_t)R.rounds;
+      ctx->d_t_synced = false;
+      steps -= R.rounds;
+    }
+    return MAXSAT_OK;
+  }
   if (persistent_round_active(ctx)) {
     const int64_t chunk = std::max(1, ctx->prm.steps_per_graph);
     while (steps > 0) {
@@ -1603,6 +1715,14 @@ static int ensure_eval_scratch(maxsat_ctx* ctx, int Bp) {
   CK(ctx, cudaMemsetAsync(ctx->ev_tickets, 0, sizeof(int32_t) * ntk, ctx->stream));
   ctx->ev_Bp = Bp;
   return MAXSAT_OK;
+}
+
+// variables of the context's largest formula
+static int max_formula_vars(const maxsat_ctx* ctx) {
+  int mx = 0;
+  for (int k = 0; k < ctx->n_inst; ++k)
+    mx = std::max(mx, ctx->inst_var_base[k + 1] - ctx->inst_var_base[k]);
+  return mx;
 }
 
 int maxsat_eval(maxsat_ctx* ctx, const uint8_t* assign_dev, int32_t B, int64_t* cost_dev) {
@@ -2003,14 +2123,6 @@ int maxsat_pt_swap(maxsat_ctx* ctx, int32_t parity, int32_t* accepted) {
     *accepted = h;
   }
   return MAXSAT_OK;
-}
-
-// variables of the context's largest formula
-static int max_formula_vars(const maxsat_ctx* ctx) {
-  int mx = 0;
-  for (int k = 0; k < ctx->n_inst; ++k)
-    mx = std::max(mx, ctx->inst_var_base[k + 1] - ctx->inst_var_base[k]);
-  return mx;
 }
 
 // the GPU form of unit propagation and of the merges applies: sparse path

@@ -314,6 +314,25 @@ cudaError_t launch_visible(const DevFormula& F, const DevTables& T, const DevCha
 // whether hidden patterns of these tables and this ensemble are stored as
 // 4-bit fields (C.nib)
 bool nib_patterns_supported(const DevTables& T, int B_total);
+// Resident rounds of one formula (k_rounds): `rounds` rounds from t0 in one
+// cooperative launch of S blocks per tile of 256 chains. bar: kBarStride words
+// per tile, counting arrivals from bar0 on (a launch adds S (2 rounds - 1) to
+// each tile's); acc: 3 buffers of 2 Bp 64-bit sums, buffer acc0 % 3 zero; err:
+// device error code (16 = a barrier wait gave up after about 2 s).
+constexpr int kBarStride = 32;
+struct RoundsArgs {
+  uint32_t t0 = 0;
+  int rounds = 0, S = 0, acc0 = 0;
+  uint32_t bar0 = 0;
+  uint32_t* bar = nullptr;
+  unsigned long long* acc = nullptr;
+  int* err = nullptr;
+  double fe_scale = 1.0;  // a power of two: block free energies as 64-bit fixed point
+  float keep = 0.f;       // 1 - alpha (set by the launch)
+};
+int rounds_slots(const DevTables& T);
+cudaError_t launch_rounds(const DevFormula& F, const DevTables& T, const DevChains& C,
+                          RoundsArgs A, bool cost16, float alpha, cudaStream_t st);
 // the persistent round (one cooperative launch of `rounds` Gibbs rounds,
 // grid barriers between the phases) covers this context's sparse round:
 // clauses of at most 3 literals, single-temperature octets, byte patterns

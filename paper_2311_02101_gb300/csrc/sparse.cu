@@ -1208,15 +1208,39 @@ __global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4)
 }
 
 // ---------------------------------------------------------------------------
-// Persistent round: `rounds` Gibbs rounds in one cooperative launch. Every
-// block walks the virtual blocks of the gather (chain tile fastest, as the
-// gather's grid), meets the other blocks at a grid barrier, walks the
-// virtual blocks of the visible update (the visible launch's order), and
-// meets them again before the next round. The blocks are the same as the
-// two-launch round's, so states, costs, draws and free energies are the
-// same bit for bit. Clauses of at most 3 literals on single-temperature
-// octets, byte hidden patterns, tables in shared memory (the k_gather3 and
-// k_visible<true, uint8_t, 4> case); the host checks this.
+// Resident rounds (one formula of clauses of at most 3 literals): many Gibbs
+// rounds in one cooperative launch, without a grid-wide barrier. Chains never
+// meet during a round, so each tile of 256 chains is given its own group of S
+// blocks (blocks tile, tile + tiles, ...) that runs the tile's rounds alone:
+// every block gathers its share of the clauses, the group meets at its own
+// barrier, every warp updates its share of the variables, the group meets
+// again. An SM holds two blocks, mostly of different tiles, so one computes
+// while the other waits. The states, costs and draws are those of the
+// two-launch round, bit for bit.
+//
+// What bounds the two-launch round is not its arithmetic alone (weighted 3-SAT
+// n = 1000, m = 6000, 4096 chains: 62.2 us a round, of which the warp
+// instructions take 33 us at full issue): each launch pays its start, its
+// tables and its last wave (a round of 256 chains of the same formula, 1/16 of
+// the work, takes 24.9 us; of n = 50, m = 215, 10.5 us), and the gather's last
+// block adds the partial sums of all blocks one after another (300 of them at
+// 256 chains).
+//  - Costs: each block adds its weighted costs to the tile's accumulators in
+//    the L2 (int64, exact in any order) before the first barrier; after it
+//    every block reads them back and keeps its own copy of the tile's best
+//    costs in shared memory. Three accumulator buffers take turns: round r
+//    adds to buffer r, reads it after the barrier, and clears buffer r + 1
+//    (last read two barriers ago).
+//  - The free energy is accumulated over clauses in every round as the
+//    two-launch round does; the last round of a launch, whose sum is the one
+//    that can be read, adds the block sums as 64-bit fixed point (order-free).
+//  - Visible update: k_visible_nib's sums, with the hidden patterns of the
+//    next variable copied into shared memory (cp.async, 16 bytes: four rows of
+//    the tile per warp instruction) while the current one is summed.
+//  - State that another block wrote is read from the L2 (ld.global.cg,
+//    cp.async.cg); the barrier's release and acquire order it.
+// Every barrier wait is bounded (about 2 s): a block that gives up records
+// kErrGridBarrier and leaves, and so do the others of its tile.
 // ---------------------------------------------------------------------------
 constexpr long long kBarrierWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 constexpr int kErrGridBarrier = 16;                    // device error code of a barrier timeout
@@ -1227,6 +1251,261 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
   return v;
 }
 
+// Barrier of a tile's blocks in two halves. bar counts arrivals and is never
+// cleared; target is the count at which every block of this phase has arrived.
+__device__ __forceinline__ void tile_arrive(uint32_t* bar) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+  }
+}
+
+__device__ __forceinline__ bool tile_wait(const uint32_t* bar, uint32_t target, int* err,
+                                          int* s_go) {
+  if (threadIdx.x == 0) {
+    int go = 1;
+    const long long t0 = clock64();
+    while ((int32_t)(ld_acquire_gpu(bar) - target) < 0) {
+      if (clock64() - t0 > kBarrierWaitCycles) {
+        atomicCAS(err, 0, kErrGridBarrier);
+        go = 0;
+        break;
+      }
+    }
+    __threadfence();
+    *s_go = go;
+  }
+  __syncthreads();
+  return *s_go != 0;
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// bytes of pattern rows per warp: two buffers of 32 rows of 128 bytes
+constexpr int kRowBuf = 32 * 128;
+
+template <bool PLAIN3, bool COST16>
+__global__ void __launch_bounds__(256, 2)
+    k_rounds(DevFormula F, DevTables T, DevChains C, RoundsArgs A) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int64_t s_best[256];
+  __shared__ __align__(8) uint8_t s_imp[256];
+  __shared__ __align__(16) uint32_t s_off[8][2][32];
+  __shared__ int s_go;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tiles = C.Bp / kChainTile;
+  const int tile = (int)blockIdx.x % tiles, rank = (int)blockIdx.x / tiles, S = A.S;
+  const int g8 = tile * 32 + lane, b0 = g8 * 8, b = tile * kChainTile + tid;
+  // shared memory: record blocks (256-byte aligned), contribution rows,
+  // visible entries, then the pattern rows (the gather's block sums share
+  // their space)
+  const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
+  const uint32_t rec_tab = (s0 + 255u) & ~255u;
+  const int rows_at = align16((int)(rec_tab - s0) + T.rec3_words * 4);
+  const int pva_at = rows_at + nib_rows_bytes(T);
+  const int buf_at = align16(pva_at + align16(T.pv_len * 8));
+  stage(smem + (rec_tab - s0), T.rec3, T.rec3_words * 4);
+  stage(smem + rows_at, T.ptab, nib_rows_bytes(T));
+  stage(smem + pva_at, T.pva, align16(T.pv_len * 8));
+  const uint2* pva = reinterpret_cast<const uint2*>(smem + pva_at);
+  int32_t* s_cost = reinterpret_cast<int32_t*>(smem + buf_at);       // [8][256]
+  float* s_fe = reinterpret_cast<float*>(smem + buf_at) + 8 * 256;   // [8][256]
+  const uint32_t* rows = reinterpret_cast<const uint32_t*>(smem + buf_at) + warp * (2 * kRowBuf / 4);
+  const uint32_t rows_s = s0 + (uint32_t)(buf_at + warp * 2 * kRowBuf);
+  s_best[tid] = C.best[b];
+  const G3Tables G = gather3_tables(T, C, rec_tab, b0);
+  uint32_t tab;
+  const int split = nib_split(T, C, b0, s0 + (uint32_t)rows_at, tab);
+  const bool two = __any_sync(0xFFFFFFFFu, split < 8);
+  // this block's clauses: whole groups of 8, as even as possible
+  int c_begin, c_end;
+  {
+    const int groups = (F.m + 7) / 8, per = groups / S, more = groups % S;
+    const int g0 = rank * per + min(rank, more);
+    c_begin = min(F.m, 8 * g0);
+    c_end = min(F.m, 8 * (g0 + per + (rank < more ? 1 : 0)));
+  }
+  uint32_t* bar = A.bar + tile * kBarStride;
+  uint32_t target = A.bar0;
+  const int n_warps = S * 8, first = rank * 8 + warp;
+  const uint32_t* H = static_cast<const uint32_t*>(C.H) + tile * 32 + (lane & 7) * 4;
+  const size_t hstride = (size_t)(C.Bp / 8);
+  auto load_slot = [&](int slot) {
+    return slot < F.n ? __ldg(F.var_slot + slot) : make_int4(0, 0, 0, 0);
+  };
+  // up to 32 incidences; the padding reads the zero row
+  auto load_inc = [&](int j0, int cnt) {
+    return lane < cnt ? __ldg(F.var_inc8 + j0 + lane) : make_int2(0, 0);
+  };
+  // copies the pattern rows of a window into buffer `buf`: lane / 8 picks one
+  // of four rows, lane % 8 its 16 bytes
+  auto copy_rows = [&](const int2& win, int cnt, int buf) {
+    s_off[warp][buf][lane] = (uint32_t)win.y;
+    for (int u = 0; u < cnt; u += 4) {
+      const int row = u + (lane >> 3);
+      const int c = __shfl_sync(0xFFFFFFFFu, win.x, row & 31);
+      if (row < cnt)
+        cp_async16(rows_s + (uint32_t)(buf * kRowBuf + row * 128 + (lane & 7) * 16),
+                   H + (size_t)c * hstride);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  __syncthreads();
+
+  for (int r = 0; r < A.rounds; ++r) {
+    const uint32_t t = A.t0 + (uint32_t)r;
+    const bool last = r + 1 == A.rounds;
+    const int buf = (A.acc0 + r) % 3, clear = (A.acc0 + r + 1) % 3;
+    unsigned long long* acc_cost = A.acc + (size_t)buf * 2 * C.Bp + b;
+    unsigned long long* acc_fe = acc_cost + C.Bp;
+    // ---- gather
+    int32_t cost[8];
+    float fe[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      cost[q] = 0;
+      fe[q] = 0.f;
+    }
+    gather3_clauses<PLAIN3, COST16, true, true>(F, C, G, 0, c_begin, c_end, 0, t, g8, warp, cost,
+                                                fe);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      s_cost[warp * 256 + lane * 8 + q] = cost[q];
+      s_fe[warp * 256 + lane * 8 + q] = fe[q];
+    }
+    __syncthreads();
+    int64_t tc = 0;
+    float tf = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      tc += s_cost[w * 256 + tid];
+      tf += s_fe[w * 256 + tid];
+    }
+    atomicAdd(acc_cost, (unsigned long long)tc);
+    if (last) atomicAdd(acc_fe, (unsigned long long)__double2ll_rn((double)tf * A.fe_scale));
+    if (rank == 0) {
+      unsigned long long* next = A.acc + (size_t)clear * 2 * C.Bp + b;
+      next[0] = 0ull;
+      next[C.Bp] = 0ull;
+    }
+    tile_arrive(bar);
+    target += (uint32_t)S;
+    // constants of the first variables, while the other blocks arrive
+    int4 rec = load_slot(first), rec1 = load_slot(first + n_warps),
+         rec2 = load_slot(first + 2 * n_warps);
+    const int2 win0 = load_inc(rec.y, rec.z);
+    int2 win1 = load_inc(rec1.y, rec1.z);
+    if (!tile_wait(bar, target, A.err, &s_go)) return;
+    // ---- best-keep
+    const int64_t csum = (int64_t)__ldcg(acc_cost);
+    const bool imp = csum < s_best[tid];
+    if (imp) s_best[tid] = csum;
+    s_imp[tid] = imp ? 1 : 0;
+    if (last && rank == 0) {
+      C.cost[b] = csum;
+      C.fe[b] = (float)((double)(long long)__ldcg(acc_fe) / A.fe_scale);
+      C.best[b] = s_best[tid];
+      C.improved[b] = imp ? 1 : 0;
+    }
+    // ---- visible update
+    uint64_t xold = 0;
+    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+    auto load_state = [&](int i, uint64_t& x, float4& a, float4& c) {
+      const size_t o = (size_t)i * C.Bp + b0;
+      x = __ldcg(reinterpret_cast<const unsigned long long*>(C.xt + o));
+      a = __ldcg(reinterpret_cast<const float4*>(C.nu + o));
+      c = __ldcg(reinterpret_cast<const float4*>(C.nu + o) + 1);
+    };
+    if (first < F.n) {
+      copy_rows(win0, min(rec.z, 32), 0);
+      load_state(rec.x, xold, n0, n1);
+    }
+    __syncthreads();  // s_imp
+    const uint64_t flags = *reinterpret_cast<const uint64_t*>(&s_imp[lane * 8]);
+    int vb = 0;
+    for (int slot = first; slot < F.n; slot += n_warps, vb ^= 1) {
+      const bool more = slot + n_warps < F.n;
+      uint64_t x1 = 0;
+      float4 m0 = n0, m1 = n1;
+      __syncwarp();  // the other buffer's readers are done
+      if (more) {
+        copy_rows(win1, min(rec1.z, 32), vb ^ 1);
+        load_state(rec1.x, x1, m0, m1);
+      }
+      win1 = load_inc(rec2.y, rec2.z);
+      const int4 rec3 = load_slot(slot + 3 * n_warps);
+      if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
+      const int cnt = rec.z;
+      int z[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) z[q] = 0;
+      for (int j = 0; j < cnt; j += 32) {
+        if (j > 0) {  // a further window of a variable in more than 32 clauses
+          const int2 w = load_inc(rec.y + j, cnt - j);
+          __syncwarp();
+          copy_rows(w, min(cnt - j, 32), vb);
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          __syncwarp();
+        }
+        const int cw = min(cnt - j, 32);
+        uint32_t acc[4] = {0u, 0u, 0u, 0u};
+        const uint32_t* hr = rows + vb * (kRowBuf / 4) + lane;
+        if (!two) {
+#pragma unroll 1
+          for (int k = 0; k < cw; k += 4) {
+            const uint4 of = *reinterpret_cast<const uint4*>(&s_off[warp][vb][k]);
+            uint32_t h[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) h[u] = hr[(k + u) * 32];
+            nib_add(lds128(tab + of.x), h[0], acc);
+            nib_add(lds128(tab + of.y), h[1], acc);
+            nib_add(lds128(tab + of.z), h[2], acc);
+            nib_add(lds128(tab + of.w), h[3], acc);
+          }
+        } else {
+          uint32_t mk[4];
+          nib_masks(split, mk);
+          const uint32_t tab1 = split < 8 ? tab + (uint32_t)T.ptab_stride : tab;
+#pragma unroll 1
+          for (int k = 0; k < cw; ++k) {
+            const uint32_t of = s_off[warp][vb][k];
+            nib_add2(lds128(tab + of), lds128(tab1 + of), hr[k * 32], mk, acc);
+          }
+        }
+        nib_flush(acc, cw * T.ptab_bias, z);
+      }
+      nib_tail(T, C, pva, A.keep, t, 0, rec.x, g8, (size_t)rec.x * C.Bp + b0, xold, flags, n0, n1,
+               z);
+      rec = rec1;
+      rec1 = rec2;
+      rec2 = rec3;
+      xold = x1;
+      n0 = m0;
+      n1 = m1;
+    }
+    if (last) break;
+    tile_arrive(bar);
+    target += (uint32_t)S;
+    if (!tile_wait(bar, target, A.err, &s_go)) return;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Persistent round: `rounds` Gibbs rounds in one cooperative launch. Every
+// block walks the virtual blocks of the gather (chain tile fastest, as the
+// gather's grid), meets the other blocks at a grid barrier, walks the
+// virtual blocks of the visible update (the visible launch's order), and
+// meets them again before the next round. The blocks are the same as the
+// two-launch round's, so states, costs, draws and free energies are the
+// same bit for bit. Clauses of at most 3 literals on single-temperature
+// octets, byte hidden patterns, tables in shared memory (the k_gather3 and
+// k_visible<true, uint8_t, 4> case); the host checks this.
+// ---------------------------------------------------------------------------
 // Grid barrier of a cooperative launch (every block resident): bar[0] counts
 // arrivals over the launch (zeroed before it), bar[1] is set when some block
 // gave up waiting. A wait gives up after about 2 s, records kErrGridBarrier
@@ -1636,6 +1915,56 @@ cudaError_t launch_visible(const DevFormula& F, const DevTables& T, const DevCha
   if (use_sm) return visible_variant<true, uint16_t>(grid, sm, st, F, T, C, alpha, tdev, t_rel, batch);
   if (!wide) return visible_variant<false, uint8_t>(grid, 0, st, F, T, C, alpha, tdev, t_rel, batch);
   return visible_variant<false, uint16_t>(grid, 0, st, F, T, C, alpha, tdev, t_rel, batch);
+}
+
+namespace {
+using RoundsFn = void (*)(DevFormula, DevTables, DevChains, RoundsArgs);
+RoundsFn rounds_kernel(const DevTables& T, bool cost16) {
+  if (T.plain3) return cost16 ? k_rounds<true, true> : k_rounds<true, false>;
+  return cost16 ? k_rounds<false, true> : k_rounds<false, false>;
+}
+int rounds_smem_bytes(const DevTables& T) {
+  return 256 + align16(T.rec3_words * 4) + nib_smem_bytes(T) + 16 + 8 * 2 * kRowBuf;
+}
+}  // namespace
+
+// resident blocks of k_rounds on this device (0 when it cannot run)
+int rounds_slots(const DevTables& T) {
+  if (!T.rec3 || !T.ptab || nib_smem_bytes(T) > kNibSmemLimit) return 0;
+  int slots = 1 << 30;
+  for (int v = 0; v < 2; ++v) {
+    auto kern = rounds_kernel(T, v != 0);
+    const int smem = rounds_smem_bytes(T);
+    int nb = 0;
+    if (allow_dynamic_smem(kern, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 256, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    slots = std::min(slots, nb * sm_count());
+  }
+  return slots;
+}
+
+cudaError_t launch_rounds(const DevFormula& F, const DevTables& T, const DevChains& C,
+                          RoundsArgs A, bool cost16, float alpha, cudaStream_t st) {
+  auto kern = rounds_kernel(T, cost16);
+  const int smem = rounds_smem_bytes(T);
+  const cudaError_t e = allow_dynamic_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  volatile float one = 1.0f;
+  A.keep = one - alpha;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(C.Bp / kChainTile * A.S));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, F, T, C, A);
 }
 
 bool persistent_round_supported(const DevTables& T, const DevChains& C, const DevFormula& F,
