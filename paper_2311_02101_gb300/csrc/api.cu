@@ -156,6 +156,11 @@ struct maxsat_ctx {
   int64_t* ev_part = nullptr;
   int32_t* ev_tickets = nullptr;
   int ev_Bp = 0;
+  // packed-bit evaluation (eval_bits.cu)
+  DevAllocs bits_mem;
+  BitsFormula bits;
+  uint32_t* d_bits = nullptr;  // packed assignments, grown on demand
+  size_t bits_words = 0;
   std::vector<int64_t> h_w;  // clause weights (host copy)
   // parallel tempering: Metropolis thresholds and per-round scratch
   DevAllocs pt_mem;
@@ -621,6 +626,32 @@ int upload(maxsat_ctx* ctx, DevAllocs& A, std::vector<T> h, const T** out) {
   *out = d;
   return MAXSAT_OK;
 }
+
+// Collects host arrays for one device block and one copy (a copy of its own per
+// array costs a create about 10 us each). Every array starts 256-byte aligned
+// and is padded with zeros to a multiple of 16 bytes; the pointers are set by
+// commit.
+class UploadArena {
+ public:
+  template <class T>
+  void add(const std::vector<T>& h, const T** out) {
+    const size_t at = buf_.size(), bytes = std::max<size_t>(h.size() * sizeof(T), sizeof(T));
+    buf_.resize(at + (bytes + 255) / 256 * 256, 0);
+    if (!h.empty()) std::memcpy(buf_.data() + at, h.data(), h.size() * sizeof(T));
+    outs_.emplace_back(at, reinterpret_cast<const void**>(out));
+  }
+  int commit(maxsat_ctx* ctx, DevAllocs& A) {
+    uint8_t* d = nullptr;
+    CK(ctx, A.alloc(&d, buf_.size()));
+    CK(ctx, cudaMemcpy(d, buf_.data(), buf_.size(), cudaMemcpyHostToDevice));
+    for (auto& o : outs_) *o.second = d + o.first;
+    return MAXSAT_OK;
+  }
+
+ private:
+  std::vector<uint8_t> buf_;
+  std::vector<std::pair<size_t, const void**>> outs_;
+};
 
 }  // namespace
 
@@ -1207,15 +1238,8 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   T.gq_len = (int32_t)ctx->tabs.gq.size();
   T.pv_len = (int32_t)ctx->tabs.pv.size();
   ctx->wide_h = ctx->tabs.max_nh > 8;
-#define UP(vec, dst)                                          \
-  do {                                                        \
-    int rc_ = upload(ctx, A, vec, &(dst));                    \
-    if (rc_ != MAXSAT_OK) {                                   \
-      std::string e_ = ctx->err;                              \
-      delete ctx;                                             \
-      return fail(nullptr, rc_, e_);                          \
-    }                                                         \
-  } while (0)
+  UploadArena arena;
+#define UP(vec, dst) arena.add(vec, &(dst))
   UP(cl_off, F.cl_off);
   UP(lit_var, F.lit_var);
   UP(cl_grp, F.cl_grp);
@@ -1355,6 +1379,28 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     UP(rec3, T.rec3);
     T.rec3_words = (int32_t)rec3.size();
   }
+  {
+    // the packed evaluation reads the clause lists as they are; a batch gets a
+    // list of runs of at most 2048 clauses of one formula (fewer than 65536 runs)
+    BitsFormula& E = ctx->bits;
+    E.m = (int32_t)m;
+    for (int k = 0; k < n_inst; ++k) E.n = std::max(E.n, var_base[k + 1] - var_base[k]);
+    for (int64_t c = 0; c < m && !E.wide; ++c)
+      if (cl_w[c] >= ((int64_t)1 << 26)) E.wide = 1;  // 32 of them below 2^31
+    if (n_inst > 1) {
+      const int64_t run = std::max<int64_t>(2048, (m / 32768 + 32) / 32 * 32);
+      std::vector<int4> items;
+      std::vector<int2> vars;
+      for (int k = 0; k < n_inst; ++k) {
+        vars.push_back(make_int2(var_base[k], var_base[k + 1] - var_base[k]));
+        for (int64_t c = cl_base[k]; c < cl_base[k + 1]; c += run)
+          items.push_back(make_int4((int)c, (int)std::min<int64_t>(cl_base[k + 1], c + run), k, 0));
+      }
+      E.n_items = (int32_t)items.size();
+      UP(items, E.items);
+      UP(vars, E.inst_vars);
+    }
+  }
   F.n_inst = n_inst;
   F.var_inst = nullptr;
   if (n_inst > 1) {
@@ -1374,15 +1420,17 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     UP(gq2, T.gq);
   }
   UP(ctx->tabs.pv, T.pv);
-#define UP2(vec, dst)                                         \
-  do {                                                        \
-    int rc_ = upload(ctx, A, vec, &(dst));                    \
-    if (rc_ != MAXSAT_OK) {                                   \
-      std::string e_ = ctx->err;                              \
-      delete ctx;                                             \
-      return fail(nullptr, rc_, e_);                          \
-    }                                                         \
-  } while (0)
+  {
+    const int rca = arena.commit(ctx, A);
+    if (rca != MAXSAT_OK) {
+      std::string e_ = ctx->err;
+      delete ctx;
+      return fail(nullptr, rca, e_);
+    }
+  }
+  ctx->bits.off = F.cl_off;
+  ctx->bits.lits = F.lit_var;
+  ctx->bits.w = F.cl_w;
   {
     cudaError_t e = A.alloc(&ctx->d_t, 1);
     if (e == cudaSuccess) e = A.alloc(&ctx->d_err, 1);
@@ -1725,11 +1773,40 @@ static int max_formula_vars(const maxsat_ctx* ctx) {
   return mx;
 }
 
+// costs are computed on packed assignments (eval_bits.cu)
+static bool bits_eval(const maxsat_ctx* ctx) { return max_formula_vars(ctx) <= kBitsMaxVars; }
+
+static int bits_stride(const maxsat_ctx* ctx) { return (ctx->n + 3) / 4 * 4; }
+
+// packed assignments of B assignments (grown on demand)
+static int ensure_bits_scratch(maxsat_ctx* ctx, int B) {
+  const size_t need = (size_t)((B + 31) / 32) * bits_stride(ctx);
+  if (need <= ctx->bits_words) return MAXSAT_OK;
+  ctx->bits_mem.release();
+  ctx->bits_words = 0;
+  CK(ctx, ctx->bits_mem.alloc(&ctx->d_bits, need));
+  ctx->bits_words = need;
+  return MAXSAT_OK;
+}
+
 int maxsat_eval(maxsat_ctx* ctx, const uint8_t* assign_dev, int32_t B, int64_t* cost_dev) {
   NvtxRange range("maxsat_eval");
   if (!ctx) return MAXSAT_EINVAL;
   if (B < 0 || (B > 0 && (!assign_dev || !cost_dev))) return fail(ctx, MAXSAT_EINVAL, "bad eval arguments");
   if (B == 0) return MAXSAT_OK;
+  // MAXSAT_PATH_DENSE asks for the tensor-core products by name; everywhere
+  // else the packed form runs where it applies
+  if (ctx->prm.path != MAXSAT_PATH_DENSE && bits_eval(ctx)) {
+    const int rc = ensure_bits_scratch(ctx, B);
+    if (rc != MAXSAT_OK) return rc;
+    const int stride = bits_stride(ctx);
+    TIMED(ctx, ctx->stream, "pack_bits",
+          launch_pack_bits(assign_dev, B, ctx->n, stride, ctx->d_bits, cost_dev,
+                           (size_t)ctx->n_inst * B, ctx->stream));
+    TIMED(ctx, ctx->stream, "bits_cost",
+          launch_bits_cost(ctx->bits, ctx->d_bits, stride, B, cost_dev, ctx->stream));
+    return MAXSAT_OK;
+  }
   if (ctx->dense_built) {
     const int Bp = (B + 255) / 256 * 256;
     if (Bp > ctx->dev_Bp) {
@@ -2163,11 +2240,20 @@ static int merge_on_device(maxsat_ctx* ctx, int B) {
   const int n = ctx->n, Bp = ctx->C.Bp, Bp2 = ctx->upg_Bp;
   CK(ctx, cudaMemcpy2DAsync(ctx->d_upg_cand, Bp2, ctx->C.xt, Bp, B, n, cudaMemcpyDeviceToDevice,
                             ctx->stream));
-  const int rc = ensure_eval_scratch(ctx, Bp2);
-  if (rc != MAXSAT_OK) return rc;
-  CK(ctx, launch_gather(kEval, ctx->F, ctx->T, ctx->C, ctx->d_upg_cand, 2 * B, Bp2, ctx->ev_plan,
-                        nullptr, 0, ctx->ev_part, nullptr, ctx->ev_tickets, ctx->d_upg_cost,
-                        ctx->wide_h, ctx->stream));
+  if (bits_eval(ctx)) {
+    const int rc = ensure_bits_scratch(ctx, 2 * B);
+    if (rc != MAXSAT_OK) return rc;
+    const int stride = bits_stride(ctx);
+    CK(ctx, cudaMemsetAsync(ctx->d_upg_cost, 0, 8 * (size_t)ctx->n_inst * 2 * B, ctx->stream));
+    CK(ctx, launch_pack_rows(ctx->d_upg_cand, Bp2, 2 * B, n, stride, ctx->d_bits, ctx->stream));
+    CK(ctx, launch_bits_cost(ctx->bits, ctx->d_bits, stride, 2 * B, ctx->d_upg_cost, ctx->stream));
+  } else {
+    const int rc = ensure_eval_scratch(ctx, Bp2);
+    if (rc != MAXSAT_OK) return rc;
+    CK(ctx, launch_gather(kEval, ctx->F, ctx->T, ctx->C, ctx->d_upg_cand, 2 * B, Bp2,
+                          ctx->ev_plan, nullptr, 0, ctx->ev_part, nullptr, ctx->ev_tickets,
+                          ctx->d_upg_cost, ctx->wide_h, ctx->stream));
+  }
   CK(ctx, launch_up_merge(ctx->d_upg_cost, ctx->n_inst, B, ctx->d_upg_rank, ctx->d_upg_perm,
                           ctx->d_upg_cand, Bp2, ctx->C.xt, ctx->C.nu, ctx->d_upg_nus, Bp, n,
                           ctx->F.var_inst, ctx->stream));

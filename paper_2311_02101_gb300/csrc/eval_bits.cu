@@ -1,0 +1,324 @@
+// Exact cost evaluation on assignments packed to one bit per variable.
+//
+// The weighted unsatisfied cost (Sec. 1) needs, for every clause and
+// assignment, one bit: whether no literal is true. Packed 32 assignments to a
+// word, a clause of K literals is K word loads and ORs for 32 assignments,
+// where the byte gather (k_gather<kEval>) takes K 8-byte loads for 8 of them
+// and the FP8 product a column of a 128 x 256 tile. What is left to do is the
+// weighted sum, and reading the assignments once (B n bytes).
+//   k_pack_bits  assignments (B x n bytes) -> X[word][variable], 32
+//                assignments per word; zeroes the costs. One warp = 32
+//                assignments x 128 variables: rows read 128 bytes at a time,
+//                8 rows folded into the bytes of one register by shifts, a
+//                4 x 4 byte transpose, one 16-byte store per lane.
+//   k_pack_rows  the same from variable-major bytes (n x Bp, 0 / 1).
+//   k_bits_cost  one block = one word of assignments x a run of clauses. The
+//                word's row of X (4 bytes per variable) is staged in shared
+//                memory; a warp takes 32 consecutive clauses, one per lane, so
+//                each lane ends with its clause's unsatisfied bits of 32
+//                assignments. A 32 x 32 bit transpose gives each lane one
+//                assignment's 32 clause bits, and eight look-ups of subset
+//                sums of four weights (built by the warp for these 32
+//                clauses) add their weights. Integers throughout: exact in
+//                any order.
+// The clause lists are read as they are (a warp's 32 lists are neighbours, so
+// their lines stay in the L1 while the lanes walk them): a first layout with
+// the clauses sorted by length and 32 literals side by side ran no faster and
+// cost 2.5 ms of host work before the first evaluation of 100000 clauses.
+// Bound by shared-memory look-ups (a literal's 32 random words over 32 banks
+// take about 3.5 passes) and the transpose's shuffles.
+#include <algorithm>
+#include <cstdint>
+
+#include "internal.h"
+#include "dense_common.cuh"
+
+namespace rbmsat {
+
+namespace {
+
+__device__ __forceinline__ void dependents_may_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_predecessor() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// 4 bytes from p, any alignment; [lo, hi) is the readable range
+__device__ __forceinline__ uint32_t load4(const uint8_t* p, const uint8_t* lo, const uint8_t* hi) {
+  const uint8_t* a = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)3);
+  if (a >= lo && a + 8 <= hi) {
+    const uint32_t w0 = __ldg(reinterpret_cast<const uint32_t*>(a));
+    const uint32_t w1 = __ldg(reinterpret_cast<const uint32_t*>(a) + 1);
+    return __funnelshift_r(w0, w1, 8u * (uint32_t)(p - a));
+  }
+  uint32_t v = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (p + k < hi) v |= (uint32_t)__ldg(p + k) << (8 * k);
+  return v;
+}
+
+// A: the base and n are multiples of 4 (every row segment is an aligned word)
+template <bool A>
+__global__ void __launch_bounds__(256) k_pack_bits(const uint8_t* __restrict__ assign, int B,
+                                                   int n, int W, int nstride,
+                                                   uint32_t* __restrict__ X,
+                                                   int64_t* __restrict__ cost, size_t n_cost) {
+  dependents_may_start();
+  // X and the costs may still be read or added into by the launch before
+  wait_for_predecessor();
+  const size_t threads = (size_t)gridDim.x * blockDim.x;
+  const size_t self = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (size_t k = self; k < n_cost; k += threads) cost[k] = 0;
+  const int lane = threadIdx.x & 31;
+  const int groups = (n + 127) / 128;  // of 128 variables
+  const size_t tasks = (size_t)groups * W, warps = threads / 32;
+  const uint8_t* end = assign + (size_t)B * n;
+  for (size_t task = self / 32; task < tasks; task += warps) {
+    const int w = (int)(task / groups), i = (int)(task % groups) * 128 + lane * 4;
+    const int rows = min(32, B - w * 32);
+    const uint8_t* p = assign + (size_t)w * 32 * n + i;
+    uint32_t a[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      uint32_t v[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        v[r] = 0u;
+        if (i < n && g * 8 + r < rows) {
+          const uint8_t* q = p + (size_t)(g * 8 + r) * n;
+          v[r] = A ? __ldg(reinterpret_cast<const uint32_t*>(q)) : load4(q, assign, end);
+        }
+      }
+      // bit r of byte k: row r's byte k is nonzero
+      uint32_t acc = 0u;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const uint32_t nz = ((v[r] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | v[r];
+        acc = ((acc >> 1) & 0x7F7F7F7Fu) | (nz & 0x80808080u);
+      }
+      a[g] = acc;
+    }
+    // byte k of a[0..3] -> the word of variable i + k
+    const uint32_t t0 = __byte_perm(a[0], a[1], 0x5140u), t1 = __byte_perm(a[2], a[3], 0x5140u);
+    const uint32_t t2 = __byte_perm(a[0], a[1], 0x7362u), t3 = __byte_perm(a[2], a[3], 0x7362u);
+    if (i < nstride)  // variables n .. nstride - 1 are padding, never read
+      *reinterpret_cast<uint4*>(X + (size_t)w * nstride + i) =
+          make_uint4(__byte_perm(t0, t1, 0x5410u), __byte_perm(t0, t1, 0x7632u),
+                     __byte_perm(t2, t3, 0x5410u), __byte_perm(t2, t3, 0x7632u));
+  }
+}
+
+// the four 0 / 1 bytes of v as 4 bits (byte k -> bit k)
+__device__ __forceinline__ uint32_t bytes_to_bits(uint32_t v) {
+  return (v * 0x10204080u) >> 28;
+}
+
+__global__ void __launch_bounds__(256) k_pack_rows(const uint8_t* __restrict__ xt, int Bp, int n,
+                                                   int W, int nstride, uint32_t* __restrict__ X) {
+  const int lane = threadIdx.x & 31;
+  const int i = (int)blockIdx.x * 32 + lane;
+  for (int w = (int)(blockIdx.y * 8 + (threadIdx.x >> 5)); w < W; w += (int)gridDim.y * 8) {
+    if (i >= n) continue;
+    const uint4* q = reinterpret_cast<const uint4*>(xt + (size_t)i * Bp + (size_t)w * 32);
+    const uint4 a = __ldg(q), b = __ldg(q + 1);
+    X[(size_t)w * nstride + i] =
+        bytes_to_bits(a.x) | bytes_to_bits(a.y) << 4 | bytes_to_bits(a.z) << 8 |
+        bytes_to_bits(a.w) << 12 | bytes_to_bits(b.x) << 16 | bytes_to_bits(b.y) << 20 |
+        bytes_to_bits(b.z) << 24 | bytes_to_bits(b.w) << 28;
+  }
+}
+
+// Subset sums of the warp's 32 weights (w: this lane's) in groups of four:
+// lut[16 g + s] = sum of weights 4 g + k over the bits k of s.
+template <typename V>
+__device__ __forceinline__ void build_subset_sums(V* lut, V w, int lane) {
+  const int g = lane >> 2;
+  const V w0 = __shfl_sync(0xFFFFFFFFu, w, 4 * g), w1 = __shfl_sync(0xFFFFFFFFu, w, 4 * g + 1);
+  const V w2 = __shfl_sync(0xFFFFFFFFu, w, 4 * g + 2), w3 = __shfl_sync(0xFFFFFFFFu, w, 4 * g + 3);
+  const V hi = ((lane & 1) ? w2 : V(0)) + ((lane & 2) ? w3 : V(0));
+  V* o = lut + 4 * lane;  // entries 16 g + 4 (lane % 4) + 0 .. 3
+  o[0] = hi;
+  o[1] = hi + w0;
+  o[2] = hi + w1;
+  o[3] = hi + w0 + w1;
+}
+
+// sum of the weights of the 32 clauses whose bit is set
+template <typename V>
+__device__ __forceinline__ V weigh(const V* lut, uint32_t bits) {
+  V s = 0;
+#pragma unroll
+  for (int g = 0; g < 8; ++g) s += lut[16 * g + ((bits >> (4 * g)) & 15u)];
+  return s;
+}
+
+// V: int32_t when every 32 consecutive clauses weigh less than 2^31, else
+// int64_t. RAW: a caller's DIMACS arrays, not checked before.
+template <typename V, bool RAW>
+__global__ void __launch_bounds__(256) k_bits_cost(BitsFormula F, RawFormula R,
+                                                   const uint32_t* __restrict__ X, int nstride,
+                                                   int B, unsigned long long* __restrict__ out) {
+  extern __shared__ __align__(16) uint32_t s_row[];
+  __shared__ V s_lut[8][128];
+  __shared__ long long s_sum[8][32];
+  dependents_may_start();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int word = (int)blockIdx.x;
+  // this block's clauses c_begin .. c_end - 1, and its formula's variables
+  int c_begin, c_end, inst = 0, v0 = 0, nv;
+  if (RAW || !F.items) {
+    const int m = RAW ? R.m : F.m, runs = (m + 31) / 32;
+    c_begin = 32 * (int)((long long)runs * blockIdx.y / gridDim.y);
+    c_end = min(m, 32 * (int)((long long)runs * (blockIdx.y + 1) / gridDim.y));
+    nv = RAW ? R.n : F.n;
+  } else {
+    const int4 it = __ldg(F.items + blockIdx.y);
+    c_begin = it.x;
+    c_end = it.y;
+    inst = it.z;
+    const int2 vs = __ldg(F.inst_vars + inst);
+    v0 = vs.x;
+    nv = vs.y;
+  }
+  wait_for_predecessor();
+  const uint32_t* row = X + (size_t)word * nstride + v0;
+  if ((v0 & 3) == 0) {
+    for (int k = threadIdx.x * 4; k < nv; k += 1024)
+      *reinterpret_cast<uint4*>(s_row + k) = __ldg(reinterpret_cast<const uint4*>(row + k));
+  } else {
+    for (int k = threadIdx.x; k < nv; k += 256) s_row[k] = __ldg(row + k);
+  }
+  __syncthreads();
+  V* lut = s_lut[warp];
+  long long sum = 0;
+  for (int c0 = c_begin + 32 * warp; c0 < c_end; c0 += 256) {
+    const int c = c0 + lane;
+    uint32_t sat = 0;
+    V w = 0;
+    if (c < c_end) {
+      if constexpr (RAW) {
+        w = R.w ? (V)__ldg(R.w + c) : V(1);
+        const int64_t o0 = min(max(__ldg(R.off + c), (int64_t)0), R.n_lits);
+        const int64_t o1 = min(max(__ldg(R.off + c + 1), o0), R.n_lits);
+        for (int64_t j = o0; j < o1; ++j) {
+          const int32_t l = __ldg(R.lits + j);
+          // |INT32_MIN| does not fit an int: such a literal is out of range
+          const int64_t v = (l > 0 ? (int64_t)l : -(int64_t)l) - 1;
+          if (l == 0 || v < 0 || v >= nv) continue;
+          sat |= s_row[v] ^ (uint32_t)(l >> 31);
+        }
+      } else {
+        w = (V)__ldg(F.w + c);
+        const int o0 = __ldg(F.off + c), o1 = __ldg(F.off + c + 1);
+        for (int j = o0; j < o1; j += 4) {
+          int32_t l[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) l[k] = j + k < o1 ? __ldg(F.lits + j + k) : 0;
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (j + k < o1) sat |= s_row[(l[k] & 0x7FFFFFFF) - v0] ^ (uint32_t)(l[k] >> 31);
+        }
+      }
+    }
+    __syncwarp();  // the previous 32 clauses' sums are read
+    build_subset_sums<V>(lut, w, lane);
+    const uint32_t bits = tc::transpose32(~sat, lane);  // lane = assignment
+    __syncwarp();
+    sum += (long long)weigh<V>(lut, bits);
+  }
+  s_sum[warp][lane] = sum;
+  __syncthreads();
+  if (warp == 0) {
+    long long c = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) c += s_sum[k][lane];
+    const int b = word * 32 + lane;
+    if (b < B && c != 0) atomicAdd(out + (size_t)inst * B + b, (unsigned long long)c);
+  }
+}
+
+template <typename... P, typename... Q>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, int smem, cudaStream_t st, Q... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+int sms() {
+  static int count = 0;
+  if (!count) {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+      v = 1;
+    count = v;
+  }
+  return count;
+}
+
+int row_bytes(int nv) { return 4 * ((nv + 3) / 4 * 4); }
+
+// blocks per word so that about three fall on every SM, each warp with at
+// least two runs of 32 clauses
+int cost_chunks(int W, int m) {
+  const int want = std::max(1, (3 * sms() + W - 1) / W);
+  return std::max(1, std::min(want, (m + 511) / 512));
+}
+
+template <typename V, bool RAW>
+cudaError_t cost_launch(const BitsFormula& F, const RawFormula& R, const uint32_t* X, int nstride,
+                        int B, int nv, int chunks, int64_t* cost, cudaStream_t st) {
+  auto kern = k_bits_cost<V, RAW>;
+  const int smem = row_bytes(nv);
+  const cudaError_t e = allow_dynamic_smem(kern, smem);
+  if (e != cudaSuccess) return e;
+  return launch_after(kern, dim3((unsigned)((B + 31) / 32), (unsigned)chunks), smem, st, F, R, X,
+                      nstride, B, reinterpret_cast<unsigned long long*>(cost));
+}
+
+}  // namespace
+
+cudaError_t launch_pack_bits(const uint8_t* assign, int B, int n, int nstride, uint32_t* X,
+                             int64_t* cost, size_t n_cost, cudaStream_t st) {
+  const int W = (B + 31) / 32;
+  const size_t tasks = (size_t)((n + 127) / 128) * W;
+  const unsigned grid = (unsigned)std::min<size_t>((tasks + 7) / 8, (size_t)8 * sms());
+  const bool aligned = ((reinterpret_cast<uintptr_t>(assign) | (uintptr_t)n) & 3u) == 0;
+  return launch_after(aligned ? k_pack_bits<true> : k_pack_bits<false>, dim3(grid), 0, st, assign,
+                      B, n, W, nstride, X, cost, n_cost);
+}
+
+cudaError_t launch_pack_rows(const uint8_t* xt, int Bp, int B, int n, int nstride, uint32_t* X,
+                             cudaStream_t st) {
+  const int W = (B + 31) / 32;
+  const dim3 grid((unsigned)((n + 31) / 32), (unsigned)std::min((W + 7) / 8, 65535));
+  k_pack_rows<<<grid, 256, 0, st>>>(xt, Bp, n, W, nstride, X);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_bits_cost(const BitsFormula& F, const uint32_t* X, int nstride, int B,
+                             int64_t* cost, cudaStream_t st) {
+  if (F.m == 0) return cudaSuccess;
+  const int chunks = F.items ? F.n_items : cost_chunks((B + 31) / 32, F.m);
+  return F.wide ? cost_launch<int64_t, false>(F, RawFormula{}, X, nstride, B, F.n, chunks, cost, st)
+                : cost_launch<int32_t, false>(F, RawFormula{}, X, nstride, B, F.n, chunks, cost, st);
+}
+
+cudaError_t launch_bits_cost_raw(const RawFormula& R, const uint32_t* X, int nstride, int B,
+                                 int64_t* cost, cudaStream_t st) {
+  if (R.m == 0) return cudaSuccess;
+  return cost_launch<int64_t, true>(BitsFormula{}, R, X, nstride, B, R.n,
+                                    cost_chunks((B + 31) / 32, R.m), cost, st);
+}
+
+}  // namespace rbmsat

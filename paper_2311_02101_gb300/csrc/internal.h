@@ -188,6 +188,38 @@ void up_prepare(int32_t n, int64_t m, const int64_t* off, const int32_t* lits, U
 void up_chains(const UpFormula& F, int32_t B, const uint8_t* x, const float* nu, uint8_t* out,
                int threads);
 
+// eval_bits.cu: exact costs on assignments packed to bits (X[word][variable],
+// 32 assignments per word, rows of nstride words, a multiple of 4)
+struct BitsFormula {
+  int32_t n = 0, m = 0;  // variables of the largest formula; clauses of all
+  int32_t n_items = 0, wide = 0;  // wide: 32 consecutive clauses may weigh 2^31 or more
+  const int32_t* off = nullptr;   // as DevFormula: literal offsets, literals, weights
+  const int32_t* lits = nullptr;
+  const int64_t* w = nullptr;
+  const int4* items = nullptr;    // batches: {first clause, end clause, formula, 0}; NULL: one formula
+  const int2* inst_vars = nullptr;  // per formula: {first variable, variables}
+};
+struct RawFormula {  // a caller's DIMACS arrays (maxsat_eval_noalloc)
+  int32_t m = 0, n = 0;
+  int64_t n_lits = 0;
+  const int64_t* off = nullptr;
+  const int32_t* lits = nullptr;
+  const int64_t* w = nullptr;
+};
+// largest formula whose row (4 bytes per variable) is staged in shared memory
+constexpr int kBitsMaxVars = 50000;
+// X from B x n bytes; zeroes n_cost costs
+cudaError_t launch_pack_bits(const uint8_t* assign, int B, int n, int nstride, uint32_t* X,
+                             int64_t* cost, size_t n_cost, cudaStream_t st);
+// X from the first B columns of n x Bp 0 / 1 bytes (Bp a multiple of 32)
+cudaError_t launch_pack_rows(const uint8_t* xt, int Bp, int B, int n, int nstride, uint32_t* X,
+                             cudaStream_t st);
+// adds the costs of B assignments to cost (n_inst x B, zeroed)
+cudaError_t launch_bits_cost(const BitsFormula& F, const uint32_t* X, int nstride, int B,
+                             int64_t* cost, cudaStream_t st);
+cudaError_t launch_bits_cost_raw(const RawFormula& R, const uint32_t* X, int nstride, int B,
+                                 int64_t* cost, cudaStream_t st);
+
 // up_gpu.cu: unit propagation and the B-of-2B merge on the GPU (sparse path)
 struct UpDev {
   int32_t n, m;            // all formulas of the context

@@ -168,6 +168,26 @@ extern "C" int maxsat_eval_noalloc(int32_t n, int64_t m, int64_t n_lits,
   uint8_t* xt = scratch;
   int64_t* part = reinterpret_cast<int64_t*>(scratch + xt_bytes);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  if (n <= kBitsMaxVars) {
+    // assignments packed to bits (eval_bits.cu): two launches; the packed words
+    // take an eighth of the scratch that the byte form needs
+    uint32_t* X = reinterpret_cast<uint32_t*>(scratch);
+    const int stride = (n + 3) / 4 * 4;
+    cudaError_t e = launch_pack_bits(assign_dev, B, n, stride, X, cost_dev, (size_t)B, st);
+    if (e != cudaSuccess)
+      return noalloc_fail(MAXSAT_ECUDA, std::string("pack launch: ") + cudaGetErrorString(e));
+    RawFormula R;
+    R.m = (int32_t)m;
+    R.n = n;
+    R.n_lits = n_lits;
+    R.off = off_dev;
+    R.lits = lits_dev;
+    R.w = w_dev;
+    e = launch_bits_cost_raw(R, X, stride, B, cost_dev, st);
+    if (e != cudaSuccess)
+      return noalloc_fail(MAXSAT_ECUDA, std::string("cost launch: ") + cudaGetErrorString(e));
+    return MAXSAT_OK;
+  }
   // every launch is checked before the next one is issued, so a failed
   // transpose never lets the gather and the reduce write costs from stale
   // scratch
