@@ -161,6 +161,10 @@ struct maxsat_ctx {
   BitsFormula bits;
   uint32_t* d_bits = nullptr;  // packed assignments, grown on demand
   size_t bits_words = 0;
+  // chain-major staging of the state copies (state_io.cu), grown on demand
+  DevAllocs stage_mem;
+  uint8_t* d_stage = nullptr;
+  size_t stage_bytes = 0;
   std::vector<int64_t> h_w;  // clause weights (host copy)
   // parallel tempering: Metropolis thresholds and per-round scratch
   DevAllocs pt_mem;
@@ -654,6 +658,55 @@ class UploadArena {
 };
 
 }  // namespace
+
+static int ensure_stage(maxsat_ctx* ctx, size_t bytes) {
+  if (bytes <= ctx->stage_bytes) return MAXSAT_OK;
+  ctx->stage_mem.release();
+  ctx->stage_bytes = 0;
+  CK(ctx, ctx->stage_mem.alloc(&ctx->d_stage, bytes));
+  ctx->stage_bytes = bytes;
+  return MAXSAT_OK;
+}
+
+// Chains per pass of a state copy: the staging buffer holds at most 64 MB.
+static int stage_chains(const maxsat_ctx* ctx, size_t elem, int B) {
+  const size_t row = (size_t)ctx->n * elem;
+  return (int)std::max<size_t>(1, std::min<size_t>((size_t)B, (size_t(64) << 20) / row));
+}
+
+// Chain-major host rows (B x n) from / into a variable-major device array;
+// ordered on the context's stream (the host side of a pageable copy is done
+// when the call returns or, at the latest, after a synchronisation).
+template <class V>
+static int state_to_host(maxsat_ctx* ctx, const V* src, V* dst) {
+  const int B = ctx->C.B, n = ctx->n, per = stage_chains(ctx, sizeof(V), B);
+  const int rc = ensure_stage(ctx, (size_t)per * n * sizeof(V));
+  if (rc != MAXSAT_OK) return rc;
+  V* buf = reinterpret_cast<V*>(ctx->d_stage);
+  for (int b = 0; b < B; b += per) {
+    const int cnt = std::min(per, B - b);
+    CK(ctx, launch_state_out(src, ctx->C.Bp, n, b, cnt, buf, ctx->stream));
+    CK(ctx, cudaMemcpyAsync(dst + (size_t)b * n, buf, (size_t)cnt * n * sizeof(V),
+                            cudaMemcpyDeviceToHost, ctx->stream));
+  }
+  return MAXSAT_OK;
+}
+
+template <class V>
+static int state_from_host(maxsat_ctx* ctx, V* dst, const V* src) {
+  const int B = ctx->C.B, n = ctx->n, per = stage_chains(ctx, sizeof(V), B);
+  const int rc = ensure_stage(ctx, (size_t)per * n * sizeof(V));
+  if (rc != MAXSAT_OK) return rc;
+  V* buf = reinterpret_cast<V*>(ctx->d_stage);
+  for (int b = 0; b < B; b += per) {
+    const int cnt = std::min(per, B - b);
+    CK(ctx, cudaMemcpyAsync(buf, src + (size_t)b * n, (size_t)cnt * n * sizeof(V),
+                            cudaMemcpyHostToDevice, ctx->stream));
+    CK(ctx, launch_state_in(buf, ctx->C.Bp, n, b, cnt, dst, ctx->stream));
+  }
+  CK(ctx, cudaStreamSynchronize(ctx->stream));
+  return MAXSAT_OK;
+}
 
 int build_dense(maxsat_ctx* ctx, int32_t n, int64_t m, const int64_t* off, const int32_t* lits,
                 const int64_t* weights, const std::vector<int32_t>& var_off,
@@ -1886,30 +1939,36 @@ int maxsat_solve_timed(maxsat_ctx* ctx, int32_t B, double seconds, int64_t max_s
 
 static int copy_best(maxsat_ctx* ctx, int32_t B, uint8_t* best_assign, int64_t* best_cost) {
   // per formula: its lowest best cost, ties to the lowest chain
-  const int K = ctx->n_inst, Bp = ctx->C.Bp;
-  std::vector<int64_t> best((size_t)K * B);
-  CK(ctx, cudaMemcpy2DAsync(best.data(), sizeof(int64_t) * B, ctx->C.best, sizeof(int64_t) * Bp,
-                            sizeof(int64_t) * B, K, cudaMemcpyDeviceToHost, ctx->stream));
-  CK(ctx, cudaStreamSynchronize(ctx->stream));
-  for (int k = 0; k < K; ++k) {
-    const int64_t* bk = best.data() + (size_t)k * B;
-    int bstar = 0;
-    for (int b = 1; b < B; ++b)
-      if (bk[b] < bk[bstar]) bstar = b;
-    if (best_cost) best_cost[k] = bk[bstar];
-    if (best_assign) {
-      const int v0 = ctx->inst_var_base[k], nk = ctx->inst_var_base[k + 1] - v0;
-      if (ctx->dense)
-        CK(ctx, cudaMemcpyAsync(best_assign, ctx->dbest_x + (size_t)bstar * ctx->n_pad, ctx->n,
-                                cudaMemcpyDeviceToHost, ctx->stream));
-      else
-        CK(ctx, cudaMemcpy2DAsync(best_assign + v0, 1, ctx->C.best_xt + (size_t)v0 * Bp + bstar, Bp,
-                                  1, nk, cudaMemcpyDeviceToHost, ctx->stream));
-    }
+  const int K = ctx->n_inst;
+  if (!ctx->dense) {
+    // found and gathered on the device: one copy of the costs, one of the bytes
+    const size_t cost_bytes = 8 * (size_t)K, chain_bytes = (4 * (size_t)K + 15) / 16 * 16;
+    int rc = ensure_stage(ctx, cost_bytes + chain_bytes + (size_t)ctx->n);
+    if (rc != MAXSAT_OK) return rc;
+    int64_t* cost = reinterpret_cast<int64_t*>(ctx->d_stage);
+    int32_t* chain = reinterpret_cast<int32_t*>(ctx->d_stage + cost_bytes);
+    uint8_t* assign = ctx->d_stage + cost_bytes + chain_bytes;
+    CK(ctx, launch_best(ctx->F, ctx->C, cost, chain, best_assign ? assign : nullptr, ctx->stream));
+    if (best_cost)
+      CK(ctx, cudaMemcpyAsync(best_cost, cost, cost_bytes, cudaMemcpyDeviceToHost, ctx->stream));
+    if (best_assign)
+      CK(ctx, cudaMemcpyAsync(best_assign, assign, ctx->n, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(ctx, cudaStreamSynchronize(ctx->stream));
+    if (ctx->persist_ran) return check_device_error(ctx);
+    return MAXSAT_OK;
   }
-  if (best_assign) CK(ctx, cudaStreamSynchronize(ctx->stream));
-  if (ctx->dense || ctx->persist_ran) return check_device_error(ctx);
-  return MAXSAT_OK;
+  std::vector<int64_t> best((size_t)B);
+  CK(ctx, cudaMemcpyAsync(best.data(), ctx->C.best, 8 * (size_t)B, cudaMemcpyDeviceToHost,
+                          ctx->stream));
+  CK(ctx, cudaStreamSynchronize(ctx->stream));
+  const int bstar = (int)(std::min_element(best.begin(), best.end()) - best.begin());
+  if (best_cost) *best_cost = best[bstar];
+  if (best_assign) {
+    CK(ctx, cudaMemcpyAsync(best_assign, ctx->dbest_x + (size_t)bstar * ctx->n_pad, ctx->n,
+                            cudaMemcpyDeviceToHost, ctx->stream));
+    CK(ctx, cudaStreamSynchronize(ctx->stream));
+  }
+  return check_device_error(ctx);
 }
 
 int maxsat_get_state(maxsat_ctx* ctx, uint8_t* x, float* nu, int64_t* best_cost,
@@ -1947,20 +2006,10 @@ int maxsat_get_state(maxsat_ctx* ctx, uint8_t* x, float* nu, int64_t* best_cost,
     if (t) *t = ctx->t;
     return check_device_error(ctx);
   }
-  auto fetch_T = [&](const void* dsrc, size_t elem, void* dst) -> int {
-    std::vector<uint8_t> h(nB * elem);
-    CK(ctx, cudaMemcpyAsync(h.data(), dsrc, nB * elem, cudaMemcpyDeviceToHost, ctx->stream));
-    CK(ctx, cudaStreamSynchronize(ctx->stream));
-    uint8_t* d = static_cast<uint8_t*>(dst);
-    for (int b = 0; b < B; ++b)
-      for (int i = 0; i < n; ++i)
-        std::memcpy(d + ((size_t)b * n + i) * elem, h.data() + ((size_t)i * Bp + b) * elem, elem);
-    return MAXSAT_OK;
-  };
   int rc;
-  if (x && (rc = fetch_T(ctx->C.xt, 1, x)) != MAXSAT_OK) return rc;
-  if (nu && (rc = fetch_T(ctx->C.nu, 4, nu)) != MAXSAT_OK) return rc;
-  if (best_x && (rc = fetch_T(ctx->C.best_xt, 1, best_x)) != MAXSAT_OK) return rc;
+  if (x && (rc = state_to_host(ctx, ctx->C.xt, x)) != MAXSAT_OK) return rc;
+  if (nu && (rc = state_to_host(ctx, ctx->C.nu, nu)) != MAXSAT_OK) return rc;
+  if (best_x && (rc = state_to_host(ctx, ctx->C.best_xt, best_x)) != MAXSAT_OK) return rc;
   // per-formula rows of B chains (Bp apart on the device)
   const int K = ctx->n_inst;
   if (best_cost)
@@ -2017,22 +2066,9 @@ int maxsat_set_state(maxsat_ctx* ctx, int32_t B, uint64_t seed, const uint8_t* x
     ctx->d_t_synced = false;
     return MAXSAT_OK;
   }
-  auto put_T = [&](void* ddst, size_t elem, const void* src) -> int {
-    std::vector<uint8_t> h(nB * elem);
-    CK(ctx, cudaMemcpy(h.data(), ddst, nB * elem, cudaMemcpyDeviceToHost));
-    const uint8_t* s = static_cast<const uint8_t*>(src);
-    for (int b = 0; b < B; ++b)
-      for (int i = 0; i < n; ++i)
-        std::memcpy(h.data() + ((size_t)i * Bp + b) * elem, s + ((size_t)b * n + i) * elem, elem);
-    if (elem == 1)
-      for (int b = 0; b < B; ++b)
-        for (int i = 0; i < n; ++i) h[(size_t)i * Bp + b] = h[(size_t)i * Bp + b] != 0;
-    CK(ctx, cudaMemcpy(ddst, h.data(), nB * elem, cudaMemcpyHostToDevice));
-    return MAXSAT_OK;
-  };
-  if ((rc = put_T(ctx->C.xt, 1, x)) != MAXSAT_OK) return rc;
-  if ((rc = put_T(ctx->C.nu, 4, nu)) != MAXSAT_OK) return rc;
-  if ((rc = put_T(ctx->C.best_xt, 1, best_x)) != MAXSAT_OK) return rc;
+  if ((rc = state_from_host(ctx, ctx->C.xt, x)) != MAXSAT_OK) return rc;
+  if ((rc = state_from_host(ctx, ctx->C.nu, nu)) != MAXSAT_OK) return rc;
+  if ((rc = state_from_host(ctx, ctx->C.best_xt, best_x)) != MAXSAT_OK) return rc;
   CK(ctx, cudaMemcpy2D(ctx->C.best, 8 * (size_t)Bp, best_cost, 8 * (size_t)B, 8 * (size_t)B,
                        ctx->n_inst, cudaMemcpyHostToDevice));
   ctx->t = t;
@@ -2064,19 +2100,8 @@ static int put_states(maxsat_ctx* ctx, const uint8_t* x, const float* nu) {
     CK(ctx, cudaMemcpy(ctx->dnu, hn.data(), 4 * hn.size(), cudaMemcpyHostToDevice));
     return MAXSAT_OK;
   }
-  const size_t nB = (size_t)n * Bp;
-  std::vector<uint8_t> hx(nB);
-  std::vector<float> hn(nB);
-  CK(ctx, cudaMemcpy(hx.data(), ctx->C.xt, nB, cudaMemcpyDeviceToHost));
-  CK(ctx, cudaMemcpy(hn.data(), ctx->C.nu, 4 * nB, cudaMemcpyDeviceToHost));
-  for (int b = 0; b < B; ++b)
-    for (int i = 0; i < n; ++i) {
-      hx[(size_t)i * Bp + b] = x[(size_t)b * n + i] ? 1 : 0;
-      hn[(size_t)i * Bp + b] = nu[(size_t)b * n + i];
-    }
-  CK(ctx, cudaMemcpy(ctx->C.xt, hx.data(), nB, cudaMemcpyHostToDevice));
-  CK(ctx, cudaMemcpy(ctx->C.nu, hn.data(), 4 * nB, cudaMemcpyHostToDevice));
-  return MAXSAT_OK;
+  const int rc = state_from_host(ctx, ctx->C.xt, x);
+  return rc != MAXSAT_OK ? rc : state_from_host(ctx, ctx->C.nu, nu);
 }
 
 static int ensure_merge_buffers(maxsat_ctx* ctx);

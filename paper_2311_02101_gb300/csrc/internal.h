@@ -220,6 +220,21 @@ cudaError_t launch_bits_cost(const BitsFormula& F, const uint32_t* X, int nstrid
 cudaError_t launch_bits_cost_raw(const RawFormula& R, const uint32_t* X, int nstride, int B,
                                  int64_t* cost, cudaStream_t st);
 
+// state_io.cu: columns b_begin .. b_begin + b_count - 1 of a variable-major array
+// (n x Bp) to chain-major rows (b_count x n) and back (bytes come back as 0 / 1)
+cudaError_t launch_state_out(const uint8_t* src, int Bp, int n, int b_begin, int b_count,
+                             uint8_t* dst, cudaStream_t st);
+cudaError_t launch_state_out(const float* src, int Bp, int n, int b_begin, int b_count, float* dst,
+                             cudaStream_t st);
+cudaError_t launch_state_in(const uint8_t* src, int Bp, int n, int b_begin, int b_count,
+                            uint8_t* dst, cudaStream_t st);
+cudaError_t launch_state_in(const float* src, int Bp, int n, int b_begin, int b_count, float* dst,
+                            cudaStream_t st);
+// per formula its lowest best cost and that chain, and (assign not NULL) the
+// chain's best assignment
+cudaError_t launch_best(const DevFormula& F, const DevChains& C, int64_t* cost, int32_t* chain,
+                        uint8_t* assign, cudaStream_t st);
+
 // up_gpu.cu: unit propagation and the B-of-2B merge on the GPU (sparse path)
 struct UpDev {
   int32_t n, m;            // all formulas of the context
