@@ -2416,8 +2416,8 @@ struct maxsat_mp {
   float* hc[kMpMaxLayers + 1] = {};
   float* mc[kMpMaxLayers] = {};
   float* av[kMpMaxLayers] = {};
-  float *dz = nullptr, *dhv = nullptr, *dhv2 = nullptr, *dav = nullptr, *dhc = nullptr,
-        *dhc2 = nullptr, *dmc = nullptr, *part = nullptr;
+  float *dz = nullptr, *dhv = nullptr, *dav = nullptr, *dhc = nullptr, *dmc = nullptr,
+        *part = nullptr;
   double* loss_part = nullptr;
   std::string err;
 };
@@ -2492,20 +2492,21 @@ int mp_reserve(maxsat_mp* mp, int n, int m) {
   }
   MPCK(mp, A.alloc(&mp->dz, (size_t)std::max(n, 1)));
   MPCK(mp, A.alloc(&mp->dhv, nH));
-  MPCK(mp, A.alloc(&mp->dhv2, nH));
   MPCK(mp, A.alloc(&mp->dav, nH));
   MPCK(mp, A.alloc(&mp->dhc, mH));
-  MPCK(mp, A.alloc(&mp->dhc2, mH));
   MPCK(mp, A.alloc(&mp->dmc, mH));
-  const size_t rows = (size_t)std::max(n, m);
-  MPCK(mp, A.alloc(&mp->part, ((rows + 255) / 256) * (kMpHidden * 2 * kMpHidden + kMpHidden)));
-  MPCK(mp, A.alloc(&mp->loss_part, (size_t)std::max(n, 1) / 8 + 1));
+  // block partials of every layer and side, the projections and the read-out
+  const size_t per_layer = (size_t)(mp_bwd_blocks(n) + mp_bwd_blocks(m)) * mp_part_floats();
+  const size_t embed = (size_t)(mp_embed_bwd_var_blocks(n) + mp_embed_bwd_clause_blocks(m)) * 3 * kMpHidden;
+  MPCK(mp, A.alloc(&mp->part, L * per_layer + embed + (size_t)mp_out_blocks(n) * (kMpHidden + 1) + 4));
+  MPCK(mp, A.alloc(&mp->loss_part, (size_t)mp_out_blocks(n)));
   mp->cap_n = n;
   mp->cap_m = m;
   return MAXSAT_OK;
 }
 
-// forward pass over the formula of ctx; with labels, dz and the loss partials
+// forward pass over the formula of ctx; with labels, dz, the loss partials and
+// the read-out's gradient partials (out_part)
 int mp_forward(maxsat_mp* mp, maxsat_ctx* ctx, const uint8_t* y, float* prob) {
   const DevFormula& F = ctx->F;
   const int n = F.n, m = F.m, L = mp->lay.L;
@@ -2513,19 +2514,16 @@ int mp_forward(maxsat_mp* mp, maxsat_ctx* ctx, const uint8_t* y, float* prob) {
   int rc = mp_reserve(mp, n, m);
   if (rc != MAXSAT_OK) return rc;
   const MpLayout& Y = mp->lay;
-  MPT(mp, ctx, "mp_features", mp_launch_features(F, mp->f, mp->g, mp->inv_len, mp->inv_deg, st));
-  MPT(mp, ctx, "mp_proj", mp_launch_proj(mp->f, n, mp->Pb + Y.Wf, mp->hv[0], st));
-  MPT(mp, ctx, "mp_proj", mp_launch_proj(mp->g, m, mp->Pb + Y.Wg, mp->hc[0], st));
+  MPT(mp, ctx, "mp_embed", mp_launch_embed(F, mp->Pb + Y.Wf, mp->Pb + Y.Wg, mp->f, mp->g, mp->inv_len,
+                                           mp->inv_deg, mp->hv[0], mp->hc[0], st));
   for (int l = 0; l < L; ++l) {
-    MPT(mp, ctx, "mp_clause_agg", mp_launch_clause_agg(F, mp->hv[l], mp->inv_len, nullptr, mp->mc[l], false, st));
-    MPT(mp, ctx, "mp_dense_fwd", mp_launch_dense_fwd(mp->mc[l], mp->hc[l], m, mp->Pb + Y.Wc[l], mp->P + Y.bc[l],
-                                 mp->hc[l + 1], st));
-    MPT(mp, ctx, "mp_var_agg", mp_launch_var_agg(F, mp->hc[l + 1], nullptr, mp->inv_deg, mp->av[l], false, st));
-    MPT(mp, ctx, "mp_dense_fwd", mp_launch_dense_fwd(mp->av[l], mp->hv[l], n, mp->Pb + Y.Wv[l], mp->P + Y.bv[l],
-                                 mp->hv[l + 1], st));
+    MPT(mp, ctx, "mp_dense_fwd", mp_launch_fwd(F, true, mp->hv[l], mp->inv_len, mp->hc[l], mp->Pb + Y.Wc[l],
+                                 mp->P + Y.bc[l], y ? mp->mc[l] : nullptr, mp->hc[l + 1], st));
+    MPT(mp, ctx, "mp_dense_fwd", mp_launch_fwd(F, false, mp->hc[l + 1], mp->inv_deg, mp->hv[l], mp->Pb + Y.Wv[l],
+                                 mp->P + Y.bv[l], y ? mp->av[l] : nullptr, mp->hv[l + 1], st));
   }
   MPT(mp, ctx, "mp_out", mp_launch_out(mp->hv[L], n, mp->P + Y.wo, mp->P + Y.bo, y, prob, y ? mp->dz : nullptr,
-                         y ? mp->loss_part : nullptr, st));
+                         y ? mp->loss_part : nullptr, y ? mp->part : nullptr, st));
   return MAXSAT_OK;
 }
 }  // namespace
@@ -2611,33 +2609,43 @@ int maxsat_mp_gradient(maxsat_mp* mp, maxsat_ctx* ctx, const uint8_t* labels_dev
   const MpLayout& Y = mp->lay;
   cudaStream_t st = ctx->stream;
   float* G = mp->G;
-  MPT(mp, ctx, "mp_out_bwd", mp_launch_out_bwd(mp->hv[L], mp->dz, n, mp->P + Y.wo, mp->dhv, mp->part, G + Y.wo, st));
-  bool carry = false;  // dhc holds the gradient of h_c^l from clause layer l + 1
+  // every partial gradient keeps its place until the one launch that sums them
+  MpSums S;
+  float* part = mp->part;
+  auto sum_later = [&](int nb, int stride, int count, float* dst) {
+    S.set[S.sets++] = MpSums::Set{part, dst, nb, stride, count};
+    part += ((size_t)nb * stride + 3) / 4 * 4;  // every set starts 16-byte aligned
+  };
+  sum_later(mp_out_blocks(n), kMpHidden + 1, kMpHidden + 1, G + Y.wo);  // wo, then bo
+  const int nbv = mp_bwd_blocks(n), nbc = mp_bwd_blocks(m), width = mp_part_floats();
   for (int l = L - 1; l >= 0; --l) {
-    // variable layer l: h_v^{l+1} = relu(Wv_l [a_v ; h_v^l] + bv_l)
-    MPT(mp, ctx, "mp_dense_bwd_x", mp_launch_dense_bwd_x(mp->dhv, mp->hv[l + 1], n,
-                                 mp->Pb + Y.Wv[l], mp->dav, mp->dhv2, st));
-    MPT(mp, ctx, "mp_dense_wgrad", mp_launch_dense_wgrad(mp->dhv, mp->hv[l + 1], mp->av[l],
-                                 mp->hv[l], n, mp->part, G + Y.Wv[l], st));
-    MPT(mp, ctx, "mp_dense_wsum", mp_launch_dense_wsum(mp->part, n, G + Y.Wv[l], st));
-    // a_v = (1 / deg_v) sum s h_c^{l+1}: gradient of h_c^{l+1}
-    MPT(mp, ctx, "mp_clause_agg", mp_launch_clause_agg(F, mp->dav, nullptr, mp->inv_deg, mp->dhc, carry, st));
-    // clause layer l: h_c^{l+1} = relu(Wc_l [m_c ; h_c^l] + bc_l)
-    MPT(mp, ctx, "mp_dense_bwd_x", mp_launch_dense_bwd_x(mp->dhc, mp->hc[l + 1], m,
-                                 mp->Pb + Y.Wc[l], mp->dmc, mp->dhc2, st));
-    MPT(mp, ctx, "mp_dense_wgrad", mp_launch_dense_wgrad(mp->dhc, mp->hc[l + 1], mp->mc[l],
-                                 mp->hc[l], m, mp->part, G + Y.Wc[l], st));
-    MPT(mp, ctx, "mp_dense_wsum", mp_launch_dense_wsum(mp->part, m, G + Y.Wc[l], st));
-    // m_c = (1 / len_c) sum s h_v^l: gradient of h_v^l
-    MPT(mp, ctx, "mp_var_agg", mp_launch_var_agg(F, mp->dmc, mp->inv_len, nullptr, mp->dhv2, true, st));
-    std::swap(mp->dhv, mp->dhv2);
-    std::swap(mp->dhc, mp->dhc2);
-    carry = true;
+    const bool top = l == L - 1;
+    // variable layer l: h_v^{l+1} = relu(Wv_l [a_v ; h_v^l] + bv_l); its gradient
+    // comes from the read-out at the top, else from layer l + 1: the own rows'
+    // (dhv) and, through m_c = (1 / len_c) sum s h_v, the clauses' (dmc)
+    MPT(mp, ctx, "mp_dense_bwd", mp_launch_bwd(F, false, mp->dmc, mp->inv_len, mp->dhv, top ? mp->dz : nullptr,
+                                 mp->P + Y.wo, mp->hv[l + 1], mp->av[l], mp->hv[l], mp->Pb + Y.Wv[l],
+                                 mp->dav, mp->dhv, part, st));
+    sum_later(nbv, width, width, G + Y.Wv[l]);
+    // clause layer l: h_c^{l+1} = relu(Wc_l [m_c ; h_c^l] + bc_l), its gradient
+    // through a_v = (1 / deg_v) sum s h_c^{l+1} and, below the top, from layer l + 1
+    if (m > 0) {
+      MPT(mp, ctx, "mp_dense_bwd", mp_launch_bwd(F, true, mp->dav, mp->inv_deg, top ? nullptr : mp->dhc, nullptr,
+                                   nullptr, mp->hc[l + 1], mp->mc[l], mp->hc[l], mp->Pb + Y.Wc[l],
+                                   mp->dmc, mp->dhc, part, st));
+      sum_later(nbc, width, width, G + Y.Wc[l]);
+    } else {
+      MPCK(mp, cudaMemsetAsync(G + Y.Wc[l], 0, sizeof(float) * width, st));
+    }
   }
-  MPT(mp, ctx, "mp_proj_bwd", mp_launch_proj_bwd(mp->dhv, mp->hv[0], mp->f, n, mp->part, G + Y.Wf, st));
-  MPT(mp, ctx, "mp_proj_bwd", mp_launch_proj_bwd(mp->dhc, mp->hc[0], mp->g, m, mp->part, G + Y.Wg, st));
+  const int ev = mp_embed_bwd_var_blocks(n), ec = mp_embed_bwd_clause_blocks(m);
+  MPT(mp, ctx, "mp_embed_bwd", mp_launch_embed_bwd(F, mp->dmc, mp->inv_len, mp->dhv, mp->hv[0], mp->f, mp->dhc,
+                               mp->hc[0], mp->g, part, st));
+  sum_later(ev, 3 * kMpHidden, 3 * kMpHidden, G + Y.Wf);
+  sum_later(ec, 3 * kMpHidden, 3 * kMpHidden, G + Y.Wg);
+  MPT(mp, ctx, "mp_sum", mp_launch_sums(S, st));
   if (loss) {
-    const int nb = (n + 7) / 8;
+    const int nb = mp_out_blocks(n);
     std::vector<double> lp((size_t)nb);
     MPCK(mp, cudaMemcpyAsync(lp.data(), mp->loss_part, 8 * (size_t)nb, cudaMemcpyDeviceToHost, st));
     MPCK(mp, cudaStreamSynchronize(st));

@@ -279,30 +279,48 @@ int mp_layout(int L, MpLayout* out);
 }  // namespace rbmsat
 #include <cuda_bf16.h>
 namespace rbmsat {
-cudaError_t mp_launch_features(const DevFormula& F, float* f, float* g, float* inv_len,
-                               float* inv_deg, cudaStream_t st);
-cudaError_t mp_launch_proj(const float* in, int rows, const __nv_bfloat16* W, float* out,
-                           cudaStream_t st);
-cudaError_t mp_launch_clause_agg(const DevFormula& F, const float* h, const float* cscale,
-                                 const float* vscale, float* out, bool acc, cudaStream_t st);
-cudaError_t mp_launch_var_agg(const DevFormula& F, const float* h, const float* cscale,
-                              const float* vscale, float* out, bool acc, cudaStream_t st);
-cudaError_t mp_launch_dense_fwd(const float* A, const float* Bm, int rows, const __nv_bfloat16* W,
-                                const float* b, float* out, cudaStream_t st);
-// gW receives 64 x 128 weight gradients followed by the 64 bias gradients
-cudaError_t mp_launch_dense_bwd_x(const float* dout, const float* out, int rows,
-                                  const __nv_bfloat16* W, float* dA, float* dB, cudaStream_t st);
-cudaError_t mp_launch_dense_wgrad(const float* dout, const float* out, const float* A,
-                                  const float* Bm, int rows, float* part, float* gW,
-                                  cudaStream_t st);
-cudaError_t mp_launch_dense_wsum(const float* part, int rows, float* gW, cudaStream_t st);
-cudaError_t mp_launch_proj_bwd(const float* dout, const float* out, const float* in, int rows,
-                               float* part, float* gW, cudaStream_t st);
-cudaError_t mp_launch_out(const float* h, int n, const float* wo, const float* bo,
-                          const uint8_t* y, float* prob, float* dz, double* loss_part,
+// features f, g (3 per row), 1 / degree and 1 / length, and both projections
+cudaError_t mp_launch_embed(const DevFormula& F, const __nv_bfloat16* Wf, const __nv_bfloat16* Wg,
+                            float* f, float* g, float* inv_len, float* inv_deg, float* hv,
+                            float* hc, cudaStream_t st);
+// out[r] = relu(W [agg ; self[r]] + b) over the clauses or variables, agg =
+// out_scale[r] * signed sum of src; agg_out (may be NULL) keeps agg
+cudaError_t mp_launch_fwd(const DevFormula& F, bool clauses, const float* src,
+                          const float* out_scale, const float* self, const __nv_bfloat16* W,
+                          const float* b, float* agg_out, float* out, cudaStream_t st);
+// the layer's gradient: rows' gradient = carry + signed sum of in_scale src, or
+// dz wo at the top; writes dA, dB (carry and dB may be one array) and
+// mp_bwd_blocks(rows) partials of mp_part_floats() floats (64 x 128 weights, 64 biases)
+cudaError_t mp_launch_bwd(const DevFormula& F, bool clauses, const float* src,
+                          const float* in_scale, const float* carry, const float* dz,
+                          const float* wo, const float* out, const float* agg, const float* self,
+                          const __nv_bfloat16* W, float* dA, float* dB, float* part,
                           cudaStream_t st);
-cudaError_t mp_launch_out_bwd(const float* h, const float* dz, int n, const float* wo, float* dh,
-                              float* part, float* g_wo, cudaStream_t st);
+// partials of 3 x 64 floats: the variables' blocks, then the clauses'
+cudaError_t mp_launch_embed_bwd(const DevFormula& F, const float* src, const float* in_scale,
+                                const float* carry_v, const float* hv, const float* f,
+                                const float* carry_c, const float* hc, const float* g, float* part,
+                                cudaStream_t st);
+// read-out; with labels mp_out_blocks(n) loss partials and partials of 65 floats
+cudaError_t mp_launch_out(const float* h, int n, const float* wo, const float* bo,
+                          const uint8_t* y, float* prob, float* dz, double* loss_part, float* part,
+                          cudaStream_t st);
+int mp_bwd_blocks(int rows);
+int mp_out_blocks(int n);
+int mp_embed_bwd_var_blocks(int n);
+int mp_embed_bwd_clause_blocks(int m);
+int mp_part_floats();
+// sums of block partials, every set in one launch
+struct MpSums {
+  struct Set {
+    const float* part;
+    float* dst;
+    int blocks, stride, count;
+  };
+  int sets = 0;
+  Set set[2 * kMpMaxLayers + 3];
+};
+cudaError_t mp_launch_sums(const MpSums& S, cudaStream_t st);
 cudaError_t mp_launch_adam(float* P, const float* G, float* M, float* V, int count, float lr,
                            float b1, float b2, float eps, int step, __nv_bfloat16* Pb,
                            cudaStream_t st);

@@ -13,12 +13,23 @@
 //
 // Weight matrices are used in BF16 (rounded from FP32 master weights after
 // every Adam step); activations, biases and all sums are FP32. Every kernel is
-// hand-written: the signed-mean aggregations walk the same clause and
-// variable incidence lists as the Gibbs round (one warp per clause or
-// variable, two features per lane), the 64 x 128 dense layers run on the
-// tensor cores (mma.sync BF16, activations as three BF16 terms), and weight
-// gradients are reduced in two deterministic stages (per-block partials,
-// then a fixed-order sum). No atomics.
+// hand-written. A step of the network is one launch per layer and side:
+//   k_mp_embed   input features and both projections (h_v^0, h_c^0)
+//   k_mp_fwd     64 rows at a time: the signed means of the other side's rows
+//                (gathered along the clause or variable incidence lists the
+//                Gibbs round walks), then relu(W [mean ; own] + b) on the
+//                tensor cores
+//   k_mp_out     read-out, loss, and its gradient
+//   k_mp_bwd     64 rows at a time: the rows' gradient (gathered signed sums of
+//                the other side's gradient plus the gradient of their own row),
+//                masked by relu, stays on the chip and feeds both the input
+//                gradient and the weight gradient
+//   k_mp_embed_bwd, k_mp_sum  the projections' gradients; all partial sums
+// What bounds a step is moving the rows (64 floats, 256 bytes) through HBM:
+// the means, the layers' inputs and the masked gradients are formed in shared
+// memory as the tensor cores' operands instead of passing through memory as
+// FP32 arrays between launches. Weight gradients are summed in a fixed order
+// (per block in registers over its rows, then over blocks); no atomics.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -35,113 +46,87 @@ namespace rbmsat {
 namespace {
 
 constexpr int kH = 64;
-constexpr int kRowsW = 256;    // rows per block of the projections' weight-gradient partials
-constexpr int kRowsTc = 256;   // rows per block of the dense layers' weight-gradient partials
-
 __device__ __forceinline__ float relu(float x) { return x > 0.f ? x : 0.f; }
 
-// ---------------------------------------------------------------- features
-__global__ void k_mp_var_features(DevFormula F, float* f, float* inv_deg) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= F.n) return;
-  const int j0 = F.var_off[v], j1 = F.var_off[v + 1];
-  int pos = 0;
-  for (int j = j0; j < j1; ++j) pos += F.var_inc[j].y >= 0 ? 1 : 0;
-  const int deg = j1 - j0;
-  f[3 * v + 0] = deg > 0 ? (float)pos / (float)deg - 0.5f : 0.f;
-  f[3 * v + 1] = log1pf((float)deg) * 0.25f;
-  f[3 * v + 2] = 1.f;
-  inv_deg[v] = deg > 0 ? 1.f / (float)deg : 0.f;
-}
+constexpr int kTile = 64;      // rows per tile of the layer kernels
+constexpr int kLdD = kH + 8;   // BF16 elements per row of a 64-column operand tile
+constexpr int kLdX = 2 * kH + 8;  // and of a 128-column one (both: 16-byte rows, ldmatrix
+                                  // without bank conflicts)
+constexpr int kWCount = kH * 2 * kH;   // weights of a layer
+constexpr int kPart = kWCount + kH;    // a block's weight and bias gradient
 
-__global__ void k_mp_clause_features(DevFormula F, float* g, float* inv_len) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= F.m) return;
-  const int len = F.cl_off[c + 1] - F.cl_off[c];
-  g[3 * c + 0] = logf((float)F.cl_w[c]) * 0.125f;
-  g[3 * c + 1] = (float)len * 0.25f;
-  g[3 * c + 2] = 1.f;
-  inv_len[c] = len > 0 ? 1.f / (float)len : 0.f;
-}
+// ------------------------------------------------------- features, projections
+// relu(W x) of three inputs for output columns 2 lane, 2 lane + 1
+struct Proj3 {
+  float w[6];
+  __device__ __forceinline__ void load(const __nv_bfloat16* W, int lane) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) w[k] = __bfloat162float(W[6 * lane + k]);
+  }
+  __device__ __forceinline__ float2 apply(float x0, float x1, float x2) const {
+    float a = w[0] * x0, b = w[3] * x0;
+    a = fmaf(w[1], x1, a);
+    b = fmaf(w[4], x1, b);
+    a = fmaf(w[2], x2, a);
+    b = fmaf(w[5], x2, b);
+    return make_float2(relu(a), relu(b));
+  }
+};
 
-// out[r][j] = relu(sum_k W[j][k] in[r][k]), K = 3
-__global__ void k_mp_proj(const float* in, int rows, const __nv_bfloat16* W, float* out) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)rows * kH) return;
-  const int r = (int)(e / kH), j = (int)(e % kH);
-  const float* x = in + 3 * (size_t)r;
-  float acc = __bfloat162float(W[3 * j]) * x[0];
-  acc = fmaf(__bfloat162float(W[3 * j + 1]), x[1], acc);
-  acc = fmaf(__bfloat162float(W[3 * j + 2]), x[2], acc);
-  out[e] = relu(acc);
-}
-
-// ------------------------------------------------------------- aggregation
-// Per clause c (one warp, two features per lane):
-//   out[c] (+)= cscale[c] * sum_{(v, s) in c} s * vscale[v] * h[v]
-// (scales NULL = 1).
-__global__ void k_mp_clause_agg(DevFormula F, const float* h, const float* cscale,
-                                const float* vscale, float* out, int accumulate) {
-  const int c = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (c >= F.m) return;
-  float2 acc = make_float2(0.f, 0.f);
-  for (int j = F.cl_off[c]; j < F.cl_off[c + 1]; ++j) {
-    const int32_t lv = __ldg(F.lit_var + j);
-    const int v = lv & 0x7FFFFFFF;
-    float s = lv < 0 ? -1.f : 1.f;
-    if (vscale) s *= __ldg(vscale + v);
-    const float2 x = __ldg(reinterpret_cast<const float2*>(h + (size_t)v * kH) + lane);
-    acc.x = fmaf(s, x.x, acc.x);
-    acc.y = fmaf(s, x.y, acc.y);
+// One warp = 32 rows: each lane computes one row's features, then the warp
+// writes the 32 rows' projections one after another (256 bytes each). Blocks
+// below nbv take variables, the others clauses.
+__global__ void __launch_bounds__(256) k_mp_embed(DevFormula F, const __nv_bfloat16* Wf,
+                                                  const __nv_bfloat16* Wg, int nbv, float* f,
+                                                  float* g, float* inv_len, float* inv_deg,
+                                                  float* hv, float* hc) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool var = (int)blockIdx.x < nbv;
+  const int rows = var ? F.n : F.m;
+  const int r0 = (((int)blockIdx.x - (var ? 0 : nbv)) * 8 + warp) * 32;
+  if (r0 >= rows) return;
+  Proj3 P;
+  P.load(var ? Wf : Wg, lane);
+  const int r = r0 + lane;
+  float x0 = 0.f, x1 = 0.f;
+  if (r < rows) {
+    if (var) {
+      const int j0 = F.var_off[r], j1 = F.var_off[r + 1];
+      int pos = 0;
+      for (int j = j0; j < j1; ++j) pos += F.var_inc[j].y >= 0 ? 1 : 0;
+      const int deg = j1 - j0;
+      x0 = deg > 0 ? (float)pos / (float)deg - 0.5f : 0.f;
+      x1 = log1pf((float)deg) * 0.25f;
+      inv_deg[r] = deg > 0 ? 1.f / (float)deg : 0.f;
+    } else {
+      const int len = F.cl_off[r + 1] - F.cl_off[r];
+      x0 = logf((float)F.cl_w[r]) * 0.125f;
+      x1 = (float)len * 0.25f;
+      inv_len[r] = len > 0 ? 1.f / (float)len : 0.f;
+    }
+    float* o = (var ? f : g) + 3 * (size_t)r;
+    o[0] = x0;
+    o[1] = x1;
+    o[2] = 1.f;
   }
-  const float cs = cscale ? cscale[c] : 1.f;
-  float2* o = reinterpret_cast<float2*>(out + (size_t)c * kH) + lane;
-  float2 r = make_float2(cs * acc.x, cs * acc.y);
-  if (accumulate) {
-    const float2 p = *o;
-    r.x += p.x;
-    r.y += p.y;
+  float* out = var ? hv : hc;
+  const int cnt = min(32, rows - r0);
+  for (int k = 0; k < cnt; ++k) {
+    const float a = __shfl_sync(0xFFFFFFFFu, x0, k), b = __shfl_sync(0xFFFFFFFFu, x1, k);
+    reinterpret_cast<float2*>(out + (size_t)(r0 + k) * kH)[lane] = P.apply(a, b, 1.f);
   }
-  *o = r;
-}
-
-// Per variable v (one warp): out[v] (+)= vscale[v] * sum_{(c, s) : v in c}
-// s * cscale[c] * h[c].
-__global__ void k_mp_var_agg(DevFormula F, const float* h, const float* cscale,
-                             const float* vscale, float* out, int accumulate) {
-  const int v = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (v >= F.n) return;
-  float2 acc = make_float2(0.f, 0.f);
-  for (int j = F.var_off[v]; j < F.var_off[v + 1]; ++j) {
-    const int4 inc = __ldg(F.var_inc + j);
-    float s = inc.y < 0 ? -1.f : 1.f;
-    if (cscale) s *= __ldg(cscale + inc.x);
-    const float2 x = __ldg(reinterpret_cast<const float2*>(h + (size_t)inc.x * kH) + lane);
-    acc.x = fmaf(s, x.x, acc.x);
-    acc.y = fmaf(s, x.y, acc.y);
-  }
-  const float vs = vscale ? vscale[v] : 1.f;
-  float2* o = reinterpret_cast<float2*>(out + (size_t)v * kH) + lane;
-  float2 r = make_float2(vs * acc.x, vs * acc.y);
-  if (accumulate) {
-    const float2 p = *o;
-    r.x += p.x;
-    r.y += p.y;
-  }
-  *o = r;
 }
 
 // ------------------------------------------------------------ dense layers
-// The three 64 x 128 contractions of a dense layer (forward, input gradient,
-// weight gradient) run on the tensor cores: mma.sync m16n8k16 with BF16
-// operands and FP32 accumulation. The weights are BF16 already; an FP32
-// activation or gradient v enters as three BF16 terms hi + mid + lo (hi =
-// bf16(v), mid = bf16(v - hi), lo = bf16(v - hi - mid)), so that products
-// with BF16 weights sum to FP32 accuracy; the weight gradient, a product of
-// two FP32 operands, keeps the three leading cross terms (hi x hi, hi x mid,
-// mid x hi).
+// The three 64 x 128 contractions of a layer (forward, input gradient, weight
+// gradient) run on the tensor cores: mma.sync m16n8k16 with BF16 operands and
+// FP32 accumulation. The weights are BF16 already; an FP32 activation or
+// gradient v enters as three BF16 terms hi + mid + lo (hi = bf16(v), mid =
+// bf16(v - hi), lo = bf16(v - hi - mid)), so that products with BF16 weights
+// sum to FP32 accuracy; the weight gradient, a product of two FP32 operands,
+// keeps the three leading cross terms (hi x hi, hi x mid, mid x hi). The terms
+// are written to shared memory once per value and read as fragments by
+// ldmatrix.
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
                                          uint32_t b1) {
@@ -152,353 +137,464 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+template <bool TRANS>
+__device__ __forceinline__ void ldm4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  if constexpr (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a));
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // .x (low half) = lo
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// the three BF16 terms of a pair of FP32 values, packed as BF16 pairs
-__device__ __forceinline__ void split3(float x0, float x1, uint32_t& t0, uint32_t& t1,
-                                       uint32_t& t2) {
-  const float h0 = __bfloat162float(__float2bfloat16_rn(x0));
-  const float h1 = __bfloat162float(__float2bfloat16_rn(x1));
-  const float r0 = x0 - h0, r1 = x1 - h1;  // exact
-  const float m0 = __bfloat162float(__float2bfloat16_rn(r0));
-  const float m1 = __bfloat162float(__float2bfloat16_rn(r1));
-  t0 = pack_bf16(h0, h1);
-  t1 = pack_bf16(m0, m1);
-  t2 = pack_bf16(r0 - m0, r1 - m1);
+// the leading BF16 term of a pair; the pair becomes its remainder (exact)
+__device__ __forceinline__ uint32_t take_term(float& x0, float& x1) {
+  const uint32_t t = pack_bf16(x0, x1);
+  x0 -= __uint_as_float(t << 16);
+  x1 -= __uint_as_float(t & 0xFFFF0000u);
+  return t;
 }
 
-__device__ __forceinline__ float2 ld2(const float* base, int rows, int r, int k) {
-  return r < rows ? *reinterpret_cast<const float2*>(base + (size_t)r * kH + k)
-                  : make_float2(0.f, 0.f);
-}
-
-// out[r] = relu(W [A[r] ; B[r]] + b), W 64 x 128 (BF16): one warp = 16 rows
-// x 64 outputs, 8 warps per block.
-__global__ void __launch_bounds__(256) k_mp_dense_fwd(const float* A, const float* Bm, int rows,
-                                                      const __nv_bfloat16* W, const float* b,
-                                                      float* out) {
-  __shared__ uint32_t Ws[kH][kH + 4];  // W as BF16 pairs along k: Ws[j][k / 2]
-  const uint32_t* W2 = reinterpret_cast<const uint32_t*>(W);
-  for (int e = threadIdx.x; e < kH * kH; e += 256) Ws[e / kH][e % kH] = W2[e];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int r0 = (blockIdx.x * 8 + warp) * 16;
-  if (r0 >= rows) return;
-  const int ra = r0 + g, rb = r0 + g + 8;
-  float acc[8][4];
+// the first TERMS BF16 terms of four values into tiles `tile` elements apart
+template <int TERMS>
+__device__ __forceinline__ void store_terms(__nv_bfloat16* dst, int tile, float4 v) {
 #pragma unroll
-  for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
-#pragma unroll 1
-  for (int s = 0; s < 8; ++s) {  // k-steps of 16: [A ; B]
-    const float* src = s < 4 ? A : Bm;
-    const int kc = (s & 3) * 16 + 2 * t;
-    const float2 x0 = ld2(src, rows, ra, kc), x1 = ld2(src, rows, rb, kc);
-    const float2 x2 = ld2(src, rows, ra, kc + 8), x3 = ld2(src, rows, rb, kc + 8);
-    uint32_t ah[4], am[4], al[4];
-    split3(x0.x, x0.y, ah[0], am[0], al[0]);
-    split3(x1.x, x1.y, ah[1], am[1], al[1]);
-    split3(x2.x, x2.y, ah[2], am[2], al[2]);
-    split3(x3.x, x3.y, ah[3], am[3], al[3]);
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int j = nt * 8 + g;
-      const uint32_t b0 = Ws[j][8 * s + t], b1 = Ws[j][8 * s + 4 + t];
-      mma_bf16(acc[nt], ah, b0, b1);
-      mma_bf16(acc[nt], am, b0, b1);
-      mma_bf16(acc[nt], al, b0, b1);
-    }
-  }
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt) {
-    const int j = nt * 8 + 2 * t;
-    const float b0 = b[j], b1 = b[j + 1];
-    if (ra < rows)
-      *reinterpret_cast<float2*>(out + (size_t)ra * kH + j) =
-          make_float2(relu(acc[nt][0] + b0), relu(acc[nt][1] + b1));
-    if (rb < rows)
-      *reinterpret_cast<float2*>(out + (size_t)rb * kH + j) =
-          make_float2(relu(acc[nt][2] + b0), relu(acc[nt][3] + b1));
+  for (int k = 0; k < TERMS; ++k) {
+    uint2 w;
+    w.x = take_term(v.x, v.y);
+    w.y = take_term(v.z, v.w);
+    *reinterpret_cast<uint2*>(dst + (size_t)k * tile) = w;
   }
 }
 
-__device__ __forceinline__ float2 ld_delta(const float* dout, const float* out, int rows, int r,
-                                           int j) {
-  if (r >= rows) return make_float2(0.f, 0.f);
-  const float2 d = *reinterpret_cast<const float2*>(dout + (size_t)r * kH + j);
-  const float2 o = *reinterpret_cast<const float2*>(out + (size_t)r * kH + j);
-  return make_float2(o.x > 0.f ? d.x : 0.f, o.y > 0.f ? d.y : 0.f);
-}
-
-// dX = (dout * [out > 0]) W: dA[r] = its first 64 columns, dB[r] the last
-// 64 (written). One warp = 16 rows x 128 columns.
-__global__ void __launch_bounds__(256) k_mp_dense_bwd_x(const float* dout, const float* out,
-                                                        int rows, const __nv_bfloat16* W,
-                                                        float* dA, float* dB) {
-  __shared__ uint32_t WT[2 * kH][kH / 2 + 4];  // W^T as BF16 pairs along j: WT[k][j / 2]
-  for (int e = threadIdx.x; e < 2 * kH * (kH / 2); e += 256) {
-    const int k = e / (kH / 2), jp = e % (kH / 2);
-    const __nv_bfloat16 lo = W[(2 * jp) * 2 * kH + k], hi = W[(2 * jp + 1) * 2 * kH + k];
-    WT[k][jp] = (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int r0 = (blockIdx.x * 8 + warp) * 16;
-  if (r0 >= rows) return;
-  const int ra = r0 + g, rb = r0 + g + 8;
-  float acc[16][4];
+// Row r's signed sum over its clause's literals (CL) or its variable's
+// occurrences: sum s * scale[other] * src[other] (scale NULL = 1), in list
+// order, columns 4 c .. 4 c + 3 of the 16 lanes that share the row.
+template <bool CL>
+__device__ __forceinline__ float4 gather_row(const DevFormula& F, const float* src,
+                                             const float* scale, int r, int c) {
+  const int j0 = CL ? __ldg(F.cl_off + r) : __ldg(F.var_off + r);
+  const int j1 = CL ? __ldg(F.cl_off + r + 1) : __ldg(F.var_off + r + 1);
+  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int j = j0; j < j1; j += 4) {
+    int o[4];
+    float s[4];
+    float4 x[4];
 #pragma unroll
-  for (int nt = 0; nt < 16; ++nt)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
-#pragma unroll 1
-  for (int s = 0; s < 4; ++s) {  // k-steps of 16 over the 64 outputs j
-    const int jc = s * 16 + 2 * t;
-    const float2 d0 = ld_delta(dout, out, rows, ra, jc), d1 = ld_delta(dout, out, rows, rb, jc);
-    const float2 d2 = ld_delta(dout, out, rows, ra, jc + 8);
-    const float2 d3 = ld_delta(dout, out, rows, rb, jc + 8);
-    uint32_t ah[4], am[4], al[4];
-    split3(d0.x, d0.y, ah[0], am[0], al[0]);
-    split3(d1.x, d1.y, ah[1], am[1], al[1]);
-    split3(d2.x, d2.y, ah[2], am[2], al[2]);
-    split3(d3.x, d3.y, ah[3], am[3], al[3]);
-#pragma unroll
-    for (int nt = 0; nt < 16; ++nt) {
-      const int k = nt * 8 + g;
-      const uint32_t b0 = WT[k][8 * s + t], b1 = WT[k][8 * s + 4 + t];
-      mma_bf16(acc[nt], ah, b0, b1);
-      mma_bf16(acc[nt], am, b0, b1);
-      mma_bf16(acc[nt], al, b0, b1);
-    }
-  }
-#pragma unroll
-  for (int nt = 0; nt < 16; ++nt) {
-    float* dst = nt < 8 ? dA : dB;
-    const int k = (nt & 7) * 8 + 2 * t;
-    if (ra < rows)
-      *reinterpret_cast<float2*>(dst + (size_t)ra * kH + k) = make_float2(acc[nt][0], acc[nt][1]);
-    if (rb < rows)
-      *reinterpret_cast<float2*>(dst + (size_t)rb * kH + k) = make_float2(acc[nt][2], acc[nt][3]);
-  }
-}
-
-// Per-block partial weight gradients of a 64 x 128 dense layer over kRowsTc
-// rows: part[blk] = [sum_r delta[r][j] x[r][k] (64 x 128) ; sum_r delta[r][j]
-// (64)], delta = dout * [out > 0], x = [A ; B]. Rows pass through shared
-// memory 32 at a time as BF16 terms, transposed so that a fragment's row pair
-// is one 32-bit word; warp w owns outputs j of tile w % 4 and columns k of
-// half w / 4. Each output's bias sum is split over the four threads that
-// stage it and combined in a fixed order.
-__global__ void __launch_bounds__(256) k_mp_wgrad_tc(const float* dout, const float* out,
-                                                     const float* A, const float* Bm, int rows,
-                                                     float* part) {
-  constexpr int R = 32;              // rows per pass
-  __shared__ uint32_t dT[2][kH][R / 2 + 4];       // hi, mid terms of delta: [j][row pair]
-  __shared__ uint32_t xT[2][2 * kH][R / 2 + 4];   // hi, mid terms of x: [k][row pair]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int mi = warp & 3, nh = warp >> 2;
-  float acc[8][4];
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
-  float accb = 0.f;
-  const int rbase = blockIdx.x * kRowsTc;
-  for (int c0 = rbase; c0 < rbase + kRowsTc && c0 < rows; c0 += R) {
-    __syncthreads();
-    // thread t always stages output j = t % 64 (row pairs t / 64, + 4, ...)
-    // and keeps its share of the bias sum
-    for (int e = threadIdx.x; e < (R / 2) * kH; e += 256) {
-      const int rp = e / kH, j = e % kH, r = c0 + 2 * rp;
-      float v0 = 0.f, v1 = 0.f;
-      if (r < rows && out[(size_t)r * kH + j] > 0.f) v0 = dout[(size_t)r * kH + j];
-      if (r + 1 < rows && out[(size_t)(r + 1) * kH + j] > 0.f) v1 = dout[(size_t)(r + 1) * kH + j];
-      accb += v0;
-      accb += v1;
-      uint32_t th, tm, tl;
-      split3(v0, v1, th, tm, tl);
-      dT[0][j][rp] = th;
-      dT[1][j][rp] = tm;
-    }
-    for (int e = threadIdx.x; e < (R / 2) * 2 * kH; e += 256) {
-      const int rp = e / (2 * kH), k = e % (2 * kH), r = c0 + 2 * rp;
-      const float* src = k < kH ? A : Bm;
-      const int kk = k < kH ? k : k - kH;
-      const float v0 = r < rows ? src[(size_t)r * kH + kk] : 0.f;
-      const float v1 = r + 1 < rows ? src[(size_t)(r + 1) * kH + kk] : 0.f;
-      uint32_t th, tm, tl;
-      split3(v0, v1, th, tm, tl);
-      xT[0][k][rp] = th;
-      xT[1][k][rp] = tm;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int ks = 0; ks < R / 16; ++ks) {
-      const int j = mi * 16 + g;
-      uint32_t a[2][4];
-#pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        a[p][0] = dT[p][j][8 * ks + t];
-        a[p][1] = dT[p][j + 8][8 * ks + t];
-        a[p][2] = dT[p][j][8 * ks + 4 + t];
-        a[p][3] = dT[p][j + 8][8 * ks + 4 + t];
+    for (int u = 0; u < 4; ++u) {
+      o[u] = -1;
+      if (j + u < j1) {
+        if constexpr (CL) {
+          const int32_t lv = __ldg(F.lit_var + j + u);
+          o[u] = lv & 0x7FFFFFFF;
+          s[u] = lv < 0 ? -1.f : 1.f;
+        } else {
+          const int2 inc = __ldg(reinterpret_cast<const int2*>(F.var_inc + j + u));
+          o[u] = inc.x;
+          s[u] = inc.y < 0 ? -1.f : 1.f;
+        }
       }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (o[u] >= 0) {
+        if (scale) s[u] *= __ldg(scale + o[u]);
+        x[u] = __ldg(reinterpret_cast<const float4*>(src + (size_t)o[u] * kH) + c);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (o[u] >= 0) {
+        acc.x = fmaf(s[u], x[u].x, acc.x);
+        acc.y = fmaf(s[u], x[u].y, acc.y);
+        acc.z = fmaf(s[u], x[u].z, acc.z);
+        acc.w = fmaf(s[u], x[u].w, acc.w);
+      }
+  }
+  return acc;
+}
+
+__device__ __forceinline__ float4 row4(const float* p, size_t r, int c) {
+  return *(reinterpret_cast<const float4*>(p + r * kH) + c);
+}
+
+// the layer's BF16 weights (64 x 128) as rows of kLdX
+__device__ __forceinline__ void stage_weights(__nv_bfloat16* Ws, const __nv_bfloat16* W) {
+  // W is 4-byte aligned only (parameter offsets)
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(W);
+  for (int e = threadIdx.x; e < kH * kH; e += 256)
+    *reinterpret_cast<uint32_t*>(Ws + (e >> 6) * kLdX + 2 * (e & 63)) = src[e];
+}
+
+constexpr int kFwdSmem = (3 * kTile + kH) * kLdX * 2;
+
+// out[r] = relu(W [agg ; self[r]] + b), agg = out_scale[r] * signed sum of src;
+// agg also goes to agg_out when given (the backward pass reads it). Resident
+// blocks of 8 warps walk tiles of 64 rows: 16 lanes gather a row (16 bytes
+// each), the three BF16 terms of [agg ; self] are the A operand; a warp
+// multiplies 16 rows x 32 outputs.
+template <bool CL>
+__global__ void __launch_bounds__(256, 3) k_mp_fwd(DevFormula F, const float* src,
+                                                   const float* out_scale, const float* self,
+                                                   int rows, const __nv_bfloat16* W,
+                                                   const float* b, float* agg_out, float* out) {
+  extern __shared__ __align__(16) __nv_bfloat16 sm[];
+  __nv_bfloat16* xs = sm;                         // [3][kTile][kLdX]
+  __nv_bfloat16* Ws = sm + 3 * kTile * kLdX;      // [kH][kLdX]
+  stage_weights(Ws, W);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rt = (warp & 3) * 16, ch = (warp >> 2) * 32, g = lane >> 2, t = lane & 3;
+  const int hr = tid >> 4, c = tid & 15;  // 16 lanes per row, 16 rows at a time
+  const int tiles = (rows + kTile - 1) / kTile;
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int r0 = tile * kTile;
+    __syncthreads();  // weights staged; the previous tile's fragments are read
+    float4 own[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      own[k] = r0 + hr + 16 * k < rows ? row4(self, r0 + hr + 16 * k, c)
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int lr = hr + 16 * k, r = r0 + lr;
+      store_terms<3>(xs + lr * kLdX + kH + 4 * c, kTile * kLdX, own[k]);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < rows) {
+        v = gather_row<CL>(F, src, nullptr, r, c);
+        const float sc = __ldg(out_scale + r);
+        v = make_float4(sc * v.x, sc * v.y, sc * v.z, sc * v.w);
+        if (agg_out) *(reinterpret_cast<float4*>(agg_out + (size_t)r * kH) + c) = v;
+      }
+      store_terms<3>(xs + lr * kLdX + 4 * c, kTile * kLdX, v);
+    }
+    __syncthreads();
+    float acc[4][4];
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+      uint32_t bw[2][4];
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+        ldm4<false>(bw[p], Ws + (ch + p * 16 + (lane & 7) + ((lane >> 4) << 3)) * kLdX + ks * 16 +
+                               ((lane >> 3) & 1) * 8);
+#pragma unroll
+      for (int term = 0; term < 3; ++term) {
+        uint32_t a[4];
+        ldm4<false>(a, xs + (term * kTile + rt + (lane & 15)) * kLdX + ks * 16 + (lane >> 4) * 8);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          mma_bf16(acc[2 * p], a, bw[p][0], bw[p][1]);
+          mma_bf16(acc[2 * p + 1], a, bw[p][2], bw[p][3]);
+        }
+      }
+    }
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+      const int j = ch + nt * 8 + 2 * t, ra = r0 + rt + g, rb = ra + 8;
+      const float b0 = __ldg(b + j), b1 = __ldg(b + j + 1);
+      if (ra < rows)
+        *reinterpret_cast<float2*>(out + (size_t)ra * kH + j) =
+            make_float2(relu(acc[nt][0] + b0), relu(acc[nt][1] + b1));
+      if (rb < rows)
+        *reinterpret_cast<float2*>(out + (size_t)rb * kH + j) =
+            make_float2(relu(acc[nt][2] + b0), relu(acc[nt][3] + b1));
+    }
+  }
+}
+
+constexpr int kBwdSmem = (3 * kTile * kLdD + (2 * kTile + kH) * kLdX) * 2;
+
+// Gradient of a layer for tiles of 64 rows. The gradient of row r of the
+// layer's output is carry[r] + sum s * in_scale[other] * src[other] (either
+// may be absent), or dz[r] wo at the top; delta is that where out > 0. Then
+// dA / dB = the two halves of delta W, and part[block] = this block's sums of
+// delta^T [agg ; self] (64 x 128) and delta (64). carry and dB may be the same
+// array (a tile's rows are read before they are written).
+template <bool CL>
+__global__ void __launch_bounds__(256, 2)
+    k_mp_bwd(DevFormula F, const float* src, const float* in_scale, const float* carry,
+             const float* dz, const float* wo, const float* out, const float* agg,
+             const float* self, int rows, const __nv_bfloat16* W, float* dA, float* dB,
+             float* part) {
+  extern __shared__ __align__(16) __nv_bfloat16 sm[];
+  __nv_bfloat16* ds = sm;                            // [3][kTile][kLdD]
+  __nv_bfloat16* xs = ds + 3 * kTile * kLdD;         // [2][kTile][kLdX]
+  __nv_bfloat16* Ws = xs + 2 * kTile * kLdX;         // [kH][kLdX]
+  stage_weights(Ws, W);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int q4 = warp & 3, half = warp >> 2;
+  const int hr = tid >> 4, c = tid & 15;
+  const int tiles = (rows + kTile - 1) / kTile;
+  float wacc[8][4];
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) wacc[nt][q] = 0.f;
+  float4 bacc = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    const int r0 = tile * kTile;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int lr = hr + 16 * k, r = r0 + lr;
+      float4 d = zero, xa = zero, xb = zero;
+      if (r < rows) {
+        xa = row4(agg, r, c);
+        xb = row4(self, r, c);
+        const float4 o = row4(out, r, c);
+        if (dz) {
+          const float z = __ldg(dz + r);
+          d = make_float4(z * __ldg(wo + 4 * c), z * __ldg(wo + 4 * c + 1),
+                          z * __ldg(wo + 4 * c + 2), z * __ldg(wo + 4 * c + 3));
+        } else {
+          d = gather_row<CL>(F, src, in_scale, r, c);
+          if (carry) {
+            const float4 e = row4(carry, r, c);
+            d = make_float4(d.x + e.x, d.y + e.y, d.z + e.z, d.w + e.w);
+          }
+        }
+        d = make_float4(o.x > 0.f ? d.x : 0.f, o.y > 0.f ? d.y : 0.f, o.z > 0.f ? d.z : 0.f,
+                        o.w > 0.f ? d.w : 0.f);
+        bacc = make_float4(bacc.x + d.x, bacc.y + d.y, bacc.z + d.z, bacc.w + d.w);
+      }
+      store_terms<3>(ds + lr * kLdD + 4 * c, kTile * kLdD, d);
+      store_terms<2>(xs + lr * kLdX + 4 * c, kTile * kLdX, xa);
+      store_terms<2>(xs + lr * kLdX + kH + 4 * c, kTile * kLdX, xb);
+    }
+    __syncthreads();
+    {  // input gradient: 16 rows x the 64 columns of one half
+      float acc[8][4];
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        uint32_t a[3][4];
+#pragma unroll
+        for (int term = 0; term < 3; ++term)
+          ldm4<false>(a[term], ds + (term * kTile + q4 * 16 + (lane & 15)) * kLdD + ks * 16 +
+                                   (lane >> 4) * 8);
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          uint32_t bw[4];
+          ldm4<true>(bw, Ws + (ks * 16 + (lane & 15)) * kLdX + half * kH + p * 16 + (lane >> 4) * 8);
+#pragma unroll
+          for (int term = 0; term < 3; ++term) {
+            mma_bf16(acc[2 * p], a[term], bw[0], bw[1]);
+            mma_bf16(acc[2 * p + 1], a[term], bw[2], bw[3]);
+          }
+        }
+      }
+      float* dst = half ? dB : dA;
+      const int ra = r0 + q4 * 16 + g, rb = ra + 8;
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
-        const int k = nh * 64 + nt * 8 + g;
-        const uint32_t bh0 = xT[0][k][8 * ks + t], bh1 = xT[0][k][8 * ks + 4 + t];
-        const uint32_t bm0 = xT[1][k][8 * ks + t], bm1 = xT[1][k][8 * ks + 4 + t];
-        mma_bf16(acc[nt], a[0], bh0, bh1);
-        mma_bf16(acc[nt], a[0], bm0, bm1);
-        mma_bf16(acc[nt], a[1], bh0, bh1);
+        const int k = nt * 8 + 2 * t;
+        if (ra < rows)
+          *reinterpret_cast<float2*>(dst + (size_t)ra * kH + k) = make_float2(acc[nt][0], acc[nt][1]);
+        if (rb < rows)
+          *reinterpret_cast<float2*>(dst + (size_t)rb * kH + k) = make_float2(acc[nt][2], acc[nt][3]);
+      }
+    }
+    // weight gradient: outputs 16 q4 .. + 15, inputs of one half, over the rows
+#pragma unroll
+    for (int ks = 0; ks < kTile / 16; ++ks) {
+      uint32_t ah[4], am[4];
+      const __nv_bfloat16* ap =
+          ds + (ks * 16 + (lane & 7) + ((lane >> 4) << 3)) * kLdD + q4 * 16 + ((lane >> 3) & 1) * 8;
+      ldm4<true>(ah, ap);
+      ldm4<true>(am, ap + kTile * kLdD);
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        uint32_t bh[4], bm[4];
+        const __nv_bfloat16* bp =
+            xs + (ks * 16 + (lane & 15)) * kLdX + half * kH + p * 16 + (lane >> 4) * 8;
+        ldm4<true>(bh, bp);
+        ldm4<true>(bm, bp + kTile * kLdX);
+        mma_bf16(wacc[2 * p], ah, bh[0], bh[1]);
+        mma_bf16(wacc[2 * p], ah, bm[0], bm[1]);
+        mma_bf16(wacc[2 * p], am, bh[0], bh[1]);
+        mma_bf16(wacc[2 * p + 1], ah, bh[2], bh[3]);
+        mma_bf16(wacc[2 * p + 1], ah, bm[2], bm[3]);
+        mma_bf16(wacc[2 * p + 1], am, bh[2], bh[3]);
       }
     }
   }
-  float* p = part + (size_t)blockIdx.x * (kH * 2 * kH + kH);
+  float* pt = part + (size_t)blockIdx.x * kPart;
 #pragma unroll
   for (int nt = 0; nt < 8; ++nt) {
-    const int j = mi * 16 + g, k = nh * 64 + nt * 8 + 2 * t;
-    p[j * 2 * kH + k] = acc[nt][0];
-    p[j * 2 * kH + k + 1] = acc[nt][1];
-    p[(j + 8) * 2 * kH + k] = acc[nt][2];
-    p[(j + 8) * 2 * kH + k + 1] = acc[nt][3];
+    const int j = q4 * 16 + g, k = half * kH + nt * 8 + 2 * t;
+    *reinterpret_cast<float2*>(pt + j * 2 * kH + k) = make_float2(wacc[nt][0], wacc[nt][1]);
+    *reinterpret_cast<float2*>(pt + (j + 8) * 2 * kH + k) = make_float2(wacc[nt][2], wacc[nt][3]);
   }
-  // the four threads of output j combine their bias shares in a fixed order
+  // bias: the 16 row slots' sums, in order
   __syncthreads();
-  float* sb = reinterpret_cast<float*>(&dT[0][0][0]);
-  sb[threadIdx.x] = accb;
+  float* sb = reinterpret_cast<float*>(sm);  // [16][kH]
+  *reinterpret_cast<float4*>(sb + hr * kH + 4 * c) = bacc;
   __syncthreads();
-  if (threadIdx.x < kH)
-    p[kH * 2 * kH + threadIdx.x] = ((sb[threadIdx.x] + sb[threadIdx.x + kH]) +
-                                    sb[threadIdx.x + 2 * kH]) + sb[threadIdx.x + 3 * kH];
+  if (tid < kH) {
+    float v = 0.f;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) v += sb[k * kH + tid];
+    pt[kWCount + tid] = v;
+  }
 }
 
-// Per-block partial weight gradients of a dense layer over kRowsW rows:
-// part[blk] = [sum_r delta[r][j] x[r][k] (64 x K) ; sum_r delta[r][j] (64)],
-// delta = dout * [out > 0], x = [A ; B] (K = 128) or A alone (K = 3).
-template <int K>
-__global__ void __launch_bounds__(256) k_mp_wgrad_parts(const float* dout, const float* out,
-                                                        const float* A, const float* Bm, int rows,
-                                                        float* part) {
-  constexpr int E = kH * K;
-  constexpr int PER = (E + 255) / 256;
-  __shared__ float d[16][kH];
-  __shared__ float x[16][K];
-  float acc[PER];
+// ------------------------------------------------- gradient of the projections
+// Per block: sum_r delta[r][j] x[r][k] (64 x 3), delta = (carry[r] + signed sum
+// of src) where h0 > 0. Blocks below nbv take variables (with the sum), the
+// others clauses (carry only). A warp takes rows strided over its side's warps.
+__global__ void __launch_bounds__(256) k_mp_embed_bwd(DevFormula F, int nbv, const float* src,
+                                                      const float* in_scale, const float* carry_v,
+                                                      const float* hv, const float* f,
+                                                      const float* carry_c, const float* hc,
+                                                      const float* g, float* part) {
+  __shared__ float s[8][3 * kH];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool var = (int)blockIdx.x < nbv;
+  const int rows = var ? F.n : F.m;
+  const int blocks = var ? nbv : (int)gridDim.x - nbv;
+  const int first = ((int)blockIdx.x - (var ? 0 : nbv)) * 8 + warp, step = blocks * 8;
+  float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  auto add = [&](float2 d, float2 h, const float* x) {
+    const float d0 = h.x > 0.f ? d.x : 0.f, d1 = h.y > 0.f ? d.y : 0.f;
 #pragma unroll
-  for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-  float accb = 0.f;
-  const int rbase = blockIdx.x * kRowsW;
-  for (int r0 = rbase; r0 < rbase + kRowsW; r0 += 16) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < 16 * kH; e += 256) {
-      const int rr = e / kH, j = e % kH, r = r0 + rr;
-      d[rr][j] = r < rows && out[(size_t)r * kH + j] > 0.f ? dout[(size_t)r * kH + j] : 0.f;
+    for (int k = 0; k < 3; ++k) {
+      const float xk = __ldg(x + k);
+      acc[k] = fmaf(d0, xk, acc[k]);
+      acc[3 + k] = fmaf(d1, xk, acc[3 + k]);
     }
-    for (int e = threadIdx.x; e < 16 * K; e += 256) {
-      const int rr = e / K, k = e % K, r = r0 + rr;
-      float v = 0.f;
-      if (r < rows) {
-        if (K == 2 * kH) v = k < kH ? A[(size_t)r * kH + k] : Bm[(size_t)r * kH + k - kH];
-        else v = A[(size_t)r * K + k];
+  };
+  if (var) {
+    for (int r = first; r < rows; r += step) {
+      float2 a = make_float2(0.f, 0.f);
+      const int j0 = __ldg(F.var_off + r), j1 = __ldg(F.var_off + r + 1);
+#pragma unroll 4
+      for (int j = j0; j < j1; ++j) {
+        const int2 inc = __ldg(reinterpret_cast<const int2*>(F.var_inc + j));
+        const float sc = (inc.y < 0 ? -1.f : 1.f) * __ldg(in_scale + inc.x);
+        const float2 x = __ldg(reinterpret_cast<const float2*>(src + (size_t)inc.x * kH) + lane);
+        a.x = fmaf(sc, x.x, a.x);
+        a.y = fmaf(sc, x.y, a.y);
       }
-      x[rr][k] = v;
+      const float2 e = reinterpret_cast<const float2*>(carry_v + (size_t)r * kH)[lane];
+      add(make_float2(a.x + e.x, a.y + e.y), reinterpret_cast<const float2*>(hv + (size_t)r * kH)[lane],
+          f + 3 * (size_t)r);
     }
-    __syncthreads();
-    for (int rr = 0; rr < 16; ++rr) {
+  } else {
+    for (int r = first; r < rows; r += 4 * step) {
+      float2 d[4], h[4];
 #pragma unroll
-      for (int i = 0; i < PER; ++i) {
-        const int e = threadIdx.x + 256 * i;
-        if (e < E) acc[i] = fmaf(d[rr][e / K], x[rr][e % K], acc[i]);
-      }
-      if (threadIdx.x < kH) accb += d[rr][threadIdx.x];
+      for (int u = 0; u < 4; ++u)
+        if (r + u * step < rows) {
+          d[u] = reinterpret_cast<const float2*>(carry_c + (size_t)(r + u * step) * kH)[lane];
+          h[u] = reinterpret_cast<const float2*>(hc + (size_t)(r + u * step) * kH)[lane];
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (r + u * step < rows) add(d[u], h[u], g + 3 * (size_t)(r + u * step));
     }
   }
-  float* p = part + (size_t)blockIdx.x * (E + kH);
 #pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const int e = threadIdx.x + 256 * i;
-    if (e < E) p[e] = acc[i];
+  for (int k = 0; k < 6; ++k) s[warp][6 * lane + k] = acc[k];
+  __syncthreads();
+  if (threadIdx.x < 3 * kH) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += s[w][threadIdx.x];
+    part[(size_t)blockIdx.x * 3 * kH + threadIdx.x] = v;
   }
-  if (threadIdx.x < kH) p[E + threadIdx.x] = accb;
 }
 
-// grad[e] = sum over blocks of part[blk][e], e < count; rows of part are
-// `stride` apart. One warp per entry: lane l sums blocks l, l + 32, ... in
-// order, then a fixed shuffle tree (the same order on every run).
-__global__ void k_mp_sum_parts(const float* part, int nblk, int stride, int count, float* grad) {
-  const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (e >= count) return;
-  float s = 0.f;
-  for (int b = lane; b < nblk; b += 32) s += part[(size_t)b * stride + e];
+// dst[e] = sum over blocks b of part[b stride + e], e < count, for every set
+// (blockIdx.y). A block takes 32 entries: warp w sums blocks w, w + 8, ... in
+// order (32 consecutive entries per load), then the eight sums in order.
+__global__ void __launch_bounds__(256) k_mp_sum(MpSums S) {
+  __shared__ float s[8][32];
+  const MpSums::Set set = S.set[blockIdx.y];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int e = (int)blockIdx.x * 32 + lane;
+  if ((int)blockIdx.x * 32 >= set.count) return;
+  float v = 0.f;
+  if (e < set.count) {
+#pragma unroll 8
+    for (int b = warp; b < set.blocks; b += 8) v += set.part[(size_t)b * set.stride + e];
+  }
+  s[warp][lane] = v;
+  __syncthreads();
+  if (warp == 0 && e < set.count) {
+    float t = 0.f;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-  if (lane == 0) grad[e] = s;
-}
-
-cudaError_t launch_sum_parts(const float* part, int nblk, int stride, int count, float* grad,
-                             cudaStream_t st) {
-  k_mp_sum_parts<<<(count + 7) / 8, 256, 0, st>>>(part, nblk, stride, count, grad);
-  return cudaGetLastError();
+    for (int w = 0; w < 8; ++w) t += s[w][lane];
+    set.dst[e] = t;
+  }
 }
 
 // ---------------------------------------------------------------- read-out
-// z = wo . h + bo, p = sigmoid(z); with labels: dz = (p - y) / n and the loss
-// terms softplus(z) - y z (per-block partial sums, 8 rows per block).
-__global__ void k_mp_out(const float* h, int n, const float* wo, const float* bo,
-                         const uint8_t* y, float* prob, float* dz, double* loss_part) {
+// z = wo . h + bo, p = sigmoid(z); with labels: dz = (p - y) / n, per block the
+// loss terms softplus(z) - y z and the sums of dz h (64) and dz. One warp = one
+// row, two columns per lane.
+__global__ void __launch_bounds__(256) k_mp_out(const float* h, int n, const float* wo,
+                                                const float* bo, const uint8_t* y, float* prob,
+                                                float* dz, double* loss_part, float* part) {
   __shared__ double lp[8];
+  __shared__ float sg[8][kH + 1];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * 8 + w;
+  const float2 o = make_float2(__ldg(wo + 2 * lane), __ldg(wo + 2 * lane + 1));
+  const float b = __ldg(bo);
   double term = 0.0;
-  if (r < n) {
+  float2 gw = make_float2(0.f, 0.f);
+  float gb = 0.f;
+  for (int r = (int)blockIdx.x * 8 + w; r < n; r += (int)gridDim.x * 8) {
     const float2 x = reinterpret_cast<const float2*>(h + (size_t)r * kH)[lane];
-    const float2 o = reinterpret_cast<const float2*>(wo)[lane];
     float acc = fmaf(x.x, o.x, x.y * o.y);
     for (int s = 16; s > 0; s >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, s);
-    const float z = acc + bo[0];
+    const float z = acc + b;
     const float p = 1.f / (1.f + expf(-z));
-    if (lane == 0) {
-      if (prob) prob[r] = p;
-      if (y) {
-        const float yy = y[r] ? 1.f : 0.f;
-        dz[r] = (p - yy) / (float)n;
-        term = (double)(z > 0.f ? z + log1pf(expf(-z)) : log1pf(expf(z))) - (double)(yy * z);
+    if (prob && lane == 0) prob[r] = p;
+    if (y) {
+      const float yy = y[r] ? 1.f : 0.f;
+      const float d = (p - yy) / (float)n;
+      gw.x = fmaf(d, x.x, gw.x);
+      gw.y = fmaf(d, x.y, gw.y);
+      gb += d;
+      if (lane == 0) {
+        dz[r] = d;
+        term += (double)(z > 0.f ? z + log1pf(expf(-z)) : log1pf(expf(z))) - (double)(yy * z);
       }
     }
   }
-  if (lane == 0) lp[w] = term;
-  __syncthreads();
-  if (threadIdx.x == 0 && loss_part) {
-    double s = 0.0;
-    for (int i = 0; i < 8; ++i) s += lp[i];
-    loss_part[blockIdx.x] = s;
+  if (!y) return;
+  if (lane == 0) {
+    lp[w] = term;
+    sg[w][kH] = gb;
   }
-}
-
-// dh[r][k] = dz[r] wo[k]; per-block partials of [sum_r dz[r] h[r][k] (64) ; sum_r dz[r]]
-__global__ void k_mp_out_bwd(const float* h, const float* dz, int n, const float* wo, float* dh,
-                             float* part) {
-  __shared__ float sh[kH + 1];
-  const int k = threadIdx.x;  // 64 threads
-  float acc = 0.f, accb = 0.f;
-  const int r0 = blockIdx.x * kRowsW;
-  for (int r = r0; r < min(r0 + kRowsW, n); ++r) {
-    const float d = dz[r];
-    dh[(size_t)r * kH + k] = d * wo[k];
-    acc = fmaf(d, h[(size_t)r * kH + k], acc);
-    accb += d;
-  }
-  sh[k] = acc;
-  if (k == 0) sh[kH] = accb;
+  sg[w][2 * lane] = gw.x;
+  sg[w][2 * lane + 1] = gw.y;
   __syncthreads();
-  float* p = part + (size_t)blockIdx.x * (kH + 1);
-  p[k] = sh[k];
-  if (k == 0) p[kH] = sh[kH];
+  if (threadIdx.x <= kH) {
+    float v = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v += sg[k][threadIdx.x];
+    part[(size_t)blockIdx.x * (kH + 1) + threadIdx.x] = v;
+  }
+  if (threadIdx.x == 0) {
+    double v = 0.0;
+    for (int k = 0; k < 8; ++k) v += lp[k];
+    loss_part[blockIdx.x] = v;
+  }
 }
 
 // --------------------------------------------------------------- optimiser
@@ -582,83 +678,84 @@ int mp_layout(int L, MpLayout* out) {
 
 namespace {
 inline int blocks(long long count, int per) { return (int)((count + per - 1) / per); }
+
+int mp_sms() {
+  static int count = 0;
+  if (!count) {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v < 1)
+      v = 1;
+    count = v;
+  }
+  return count;
+}
 }  // namespace
 
-cudaError_t mp_launch_features(const DevFormula& F, float* f, float* g, float* inv_len,
-                               float* inv_deg, cudaStream_t st) {
-  if (F.n > 0) k_mp_var_features<<<blocks(F.n, 256), 256, 0, st>>>(F, f, inv_deg);
-  if (F.m > 0) k_mp_clause_features<<<blocks(F.m, 256), 256, 0, st>>>(F, g, inv_len);
+int mp_bwd_blocks(int rows) { return std::max(1, std::min(blocks(rows, kTile), 2 * mp_sms())); }
+int mp_out_blocks(int n) { return std::max(1, std::min(blocks(n, 8), 2 * mp_sms())); }
+int mp_embed_bwd_var_blocks(int n) { return std::max(1, std::min(blocks(n, 32), mp_sms())); }
+int mp_embed_bwd_clause_blocks(int m) { return std::max(1, std::min(blocks(m, 64), 3 * mp_sms())); }
+int mp_part_floats() { return kPart; }
+
+cudaError_t mp_launch_embed(const DevFormula& F, const __nv_bfloat16* Wf, const __nv_bfloat16* Wg,
+                            float* f, float* g, float* inv_len, float* inv_deg, float* hv,
+                            float* hc, cudaStream_t st) {
+  const int nbv = blocks(F.n, 256), nbc = blocks(F.m, 256);
+  k_mp_embed<<<nbv + nbc, 256, 0, st>>>(F, Wf, Wg, nbv, f, g, inv_len, inv_deg, hv, hc);
   return cudaGetLastError();
 }
 
-cudaError_t mp_launch_proj(const float* in, int rows, const __nv_bfloat16* W, float* out,
-                           cudaStream_t st) {
-  if (rows > 0) k_mp_proj<<<blocks((long long)rows * kH, 256), 256, 0, st>>>(in, rows, W, out);
-  return cudaGetLastError();
-}
-
-cudaError_t mp_launch_clause_agg(const DevFormula& F, const float* h, const float* cscale,
-                                 const float* vscale, float* out, bool acc, cudaStream_t st) {
-  if (F.m > 0)
-    k_mp_clause_agg<<<blocks(F.m, 8), 256, 0, st>>>(F, h, cscale, vscale, out, acc ? 1 : 0);
-  return cudaGetLastError();
-}
-
-cudaError_t mp_launch_var_agg(const DevFormula& F, const float* h, const float* cscale,
-                              const float* vscale, float* out, bool acc, cudaStream_t st) {
-  if (F.n > 0)
-    k_mp_var_agg<<<blocks(F.n, 8), 256, 0, st>>>(F, h, cscale, vscale, out, acc ? 1 : 0);
-  return cudaGetLastError();
-}
-
-cudaError_t mp_launch_dense_fwd(const float* A, const float* Bm, int rows, const __nv_bfloat16* W,
-                                const float* b, float* out, cudaStream_t st) {
-  if (rows > 0) k_mp_dense_fwd<<<blocks(rows, 128), 256, 0, st>>>(A, Bm, rows, W, b, out);
-  return cudaGetLastError();
-}
-
-cudaError_t mp_launch_dense_bwd_x(const float* dout, const float* out, int rows,
-                                  const __nv_bfloat16* W, float* dA, float* dB, cudaStream_t st) {
-  if (rows > 0) k_mp_dense_bwd_x<<<blocks(rows, 128), 256, 0, st>>>(dout, out, rows, W, dA, dB);
-  return cudaGetLastError();
-}
-
-cudaError_t mp_launch_dense_wgrad(const float* dout, const float* out, const float* A,
-                                  const float* Bm, int rows, float* part, float* gW,
-                                  cudaStream_t st) {
-  if (rows <= 0) return cudaMemsetAsync(gW, 0, sizeof(float) * (kH * 2 * kH + kH), st);
-  k_mp_wgrad_tc<<<blocks(rows, kRowsTc), 256, 0, st>>>(dout, out, A, Bm, rows, part);
-  return cudaGetLastError();
-}
-
-// sums the weight-gradient partials of mp_launch_dense_wgrad over `rows` rows
-cudaError_t mp_launch_dense_wsum(const float* part, int rows, float* gW, cudaStream_t st) {
+cudaError_t mp_launch_fwd(const DevFormula& F, bool clauses, const float* src,
+                          const float* out_scale, const float* self, const __nv_bfloat16* W,
+                          const float* b, float* agg_out, float* out, cudaStream_t st) {
+  const int rows = clauses ? F.m : F.n;
   if (rows <= 0) return cudaSuccess;
-  const int width = kH * 2 * kH + kH;
-  return launch_sum_parts(part, blocks(rows, kRowsTc), width, width, gW, st);
+  auto kern = clauses ? k_mp_fwd<true> : k_mp_fwd<false>;
+  const cudaError_t e = allow_dynamic_smem(kern, kFwdSmem);
+  if (e != cudaSuccess) return e;
+  const int grid = std::min(blocks(rows, kTile), 3 * mp_sms());
+  kern<<<grid, 256, kFwdSmem, st>>>(F, src, out_scale, self, rows, W, b, agg_out, out);
+  return cudaGetLastError();
 }
 
-cudaError_t mp_launch_proj_bwd(const float* dout, const float* out, const float* in, int rows,
-                               float* part, float* gW, cudaStream_t st) {
-  if (rows <= 0) return cudaMemsetAsync(gW, 0, sizeof(float) * kH * 3, st);
-  const int nb = blocks(rows, kRowsW);
-  k_mp_wgrad_parts<3><<<nb, 256, 0, st>>>(dout, out, in, nullptr, rows, part);
-  // the projection has no bias: only the first 64 x 3 entries of each part
-  return launch_sum_parts(part, nb, kH * 3 + kH, kH * 3, gW, st);
+cudaError_t mp_launch_bwd(const DevFormula& F, bool clauses, const float* src,
+                          const float* in_scale, const float* carry, const float* dz,
+                          const float* wo, const float* out, const float* agg, const float* self,
+                          const __nv_bfloat16* W, float* dA, float* dB, float* part,
+                          cudaStream_t st) {
+  const int rows = clauses ? F.m : F.n;
+  auto kern = clauses ? k_mp_bwd<true> : k_mp_bwd<false>;
+  const cudaError_t e = allow_dynamic_smem(kern, kBwdSmem);
+  if (e != cudaSuccess) return e;
+  kern<<<mp_bwd_blocks(rows), 256, kBwdSmem, st>>>(F, src, in_scale, carry, dz, wo, out, agg, self,
+                                                   rows, W, dA, dB, part);
+  return cudaGetLastError();
+}
+
+cudaError_t mp_launch_embed_bwd(const DevFormula& F, const float* src, const float* in_scale,
+                                const float* carry_v, const float* hv, const float* f,
+                                const float* carry_c, const float* hc, const float* g, float* part,
+                                cudaStream_t st) {
+  const int nbv = mp_embed_bwd_var_blocks(F.n), nbc = mp_embed_bwd_clause_blocks(F.m);
+  k_mp_embed_bwd<<<nbv + nbc, 256, 0, st>>>(F, nbv, src, in_scale, carry_v, hv, f, carry_c, hc, g,
+                                            part);
+  return cudaGetLastError();
+}
+
+cudaError_t mp_launch_sums(const MpSums& S, cudaStream_t st) {
+  int most = 0;
+  for (int k = 0; k < S.sets; ++k) most = std::max(most, S.set[k].count);
+  k_mp_sum<<<dim3(blocks(most, 32), S.sets), 256, 0, st>>>(S);
+  return cudaGetLastError();
 }
 
 cudaError_t mp_launch_out(const float* h, int n, const float* wo, const float* bo,
-                          const uint8_t* y, float* prob, float* dz, double* loss_part,
+                          const uint8_t* y, float* prob, float* dz, double* loss_part, float* part,
                           cudaStream_t st) {
-  if (n > 0) k_mp_out<<<blocks(n, 8), 256, 0, st>>>(h, n, wo, bo, y, prob, dz, loss_part);
+  if (n > 0)
+    k_mp_out<<<mp_out_blocks(n), 256, 0, st>>>(h, n, wo, bo, y, prob, dz, loss_part, part);
   return cudaGetLastError();
-}
-
-cudaError_t mp_launch_out_bwd(const float* h, const float* dz, int n, const float* wo, float* dh,
-                              float* part, float* g_wo, cudaStream_t st) {
-  const int nb = blocks(n, kRowsW);
-  k_mp_out_bwd<<<nb, kH, 0, st>>>(h, dz, n, wo, dh, part);
-  return launch_sum_parts(part, nb, kH + 1, kH + 1, g_wo, st);  // wo then bo
 }
 
 cudaError_t mp_launch_adam(float* P, const float* G, float* M, float* V, int count, float lr,
