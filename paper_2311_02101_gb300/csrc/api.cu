@@ -602,7 +602,8 @@ int alloc_chains(maxsat_ctx* ctx, int32_t B) {
   CK(ctx, A.alloc(&C.fe_part, (size_t)nblk * Bp));
   CK(ctx, A.alloc(&C.tickets, (size_t)ctx->n_inst * (Bp / kChainTile)));
   uint8_t* H = nullptr;
-  CK(ctx, A.alloc(&H, (size_t)ctx->m * Bp * (ctx->wide_h ? 2 : 1)));
+  CK(ctx, A.alloc(&H, std::max((size_t)ctx->m * Bp * (ctx->wide_h ? 2 : 1),
+                               (size_t)ctx->F.h_rows * (Bp / 2))));
   C.H = H;
   return plan_rounds(ctx, A, Bp);
 }
@@ -740,7 +741,11 @@ void set_ensemble(maxsat_ctx* ctx, int32_t g8_off, int32_t B_total) {
   ctx->C.g8_off = g8_off;
   ctx->C.B_total = B_total;
   ctx->C.inv_B_total = 1.0f / (float)B_total;
-  ctx->C.nib = !ctx->dense && !ctx->wide_h && nib_patterns_supported(ctx->T, B_total) ? 1 : 0;
+  // (k_gather_nib keeps a block's costs in 32 bits)
+  ctx->C.nib = !ctx->dense && nib_patterns_supported(ctx->T, B_total) &&
+                       (ctx->T.one_chunk || ctx->C.cost32)
+                   ? 1
+                   : 0;
 }
 
 // Measured path choice (MAXSAT_PATH_AUTO): times a few Gibbs rounds of B
@@ -1319,29 +1324,61 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     F.var_slot = nullptr;
     T.ptab = nullptr;
     T.pva = nullptr;
-    if (T.one_chunk && ctx->tabs.gq_absmax <= kNibMaxContribution) {
-      const HostTables& H = ctx->tabs;
-      // rows {low bytes, high bytes} of contribution + bias per temperature,
-      // group, position and sign; row 0 of each temperature is zero
-      T.ptab_bias = H.gq_absmax;
-      T.ptab_stride = 16 * (1 + 6 * T.n_groups);
-      std::vector<uint32_t> rows((size_t)T.n_temps * T.ptab_stride / 4, 0u);
-      auto row_of = [](int g, int k, bool neg) { return 16 * (1 + (g * 3 + k) * 2 + (neg ? 1 : 0)); };
-      for (int e = 0; e < T.n_temps; ++e)
-        for (int g = 0; g < T.n_groups; ++g) {
-          const GroupMeta& gm = H.meta[g];
-          for (int k = 0; k < gm.len && k < 3; ++k)
-            for (int neg = 0; neg < 2; ++neg) {
-              uint8_t* row = reinterpret_cast<uint8_t*>(rows.data()) +
-                             (size_t)e * T.ptab_stride + row_of(g, k, neg != 0);
-              for (int hp = 0; hp < (1 << gm.nh); ++hp) {
-                const int v = H.gq[(size_t)gm.gq_off + ((size_t)e << gm.nh) * gm.len + hp * gm.len + k];
-                const int biased = (neg ? -v : v) + T.ptab_bias;
-                row[hp] = (uint8_t)(biased & 0xFF);
-                row[8 + hp] = (uint8_t)(biased >> 8);
+    F.cln = nullptr;
+    F.h_rows = (int32_t)m;
+    T.recn = nullptr;
+    T.recn_smem = 0;
+    const HostTables& H = ctx->tabs;
+    // chunks of three hidden units per group; contributions of a chunk's 8
+    // patterns (a hidden unit's own are the table entries of its single bit)
+    const int G = T.n_groups, E = T.n_temps;
+    std::vector<int32_t> chunks(G), row0(G);
+    int32_t n_rows = 1;
+    for (int g = 0; g < G; ++g) {
+      chunks[g] = (H.meta[g].nh + 2) / 3;
+      row0[g] = n_rows;
+      n_rows += chunks[g] * H.meta[g].len * 2;
+    }
+    auto contribution = [&](int g, int e, int j, int k, int hp) {
+      const GroupMeta& gm = H.meta[g];
+      int v = 0;
+      for (int b = 0; b < 3; ++b)
+        if (((hp >> b) & 1) && 3 * j + b < gm.nh)
+          v += H.gq[(size_t)gm.gq_off + (((size_t)e << gm.nh) + ((size_t)1 << (3 * j + b))) * gm.len + k];
+      return v;
+    };
+    int most = 0;
+    for (int g = 0; g < G; ++g)
+      for (int e = 0; e < E; ++e)
+        for (int j = 0; j < chunks[g]; ++j)
+          for (int k = 0; k < H.meta[g].len; ++k)
+            for (int hp = 1; hp < 8; ++hp) most = std::max(most, std::abs(contribution(g, e, j, k, hp)));
+    int64_t pseudo = 0, pattern_rows = 0;
+    for (int64_t c = 0; c < m; ++c)
+      if (cl_grp[c] >= 0) {
+        pseudo += (off[c + 1] - off[c]) * chunks[cl_grp[c]];
+        pattern_rows += chunks[cl_grp[c]];
+      }
+    if (most <= kNibMaxContribution && (int64_t)ctx->max_degree * H.gq_absmax < ((int64_t)1 << 30) &&
+        (int64_t)E * n_rows * 16 <= kNibMaxRowBytes && pseudo <= INT32_MAX / 2 &&
+        pattern_rows <= INT32_MAX / 2) {
+      T.ptab_bias = most;
+      T.ptab_stride = 16 * n_rows;
+      std::vector<uint32_t> rows((size_t)E * n_rows * 4, 0u);
+      for (int e = 0; e < E; ++e)
+        for (int g = 0; g < G; ++g)
+          for (int j = 0; j < chunks[g]; ++j)
+            for (int k = 0; k < H.meta[g].len; ++k)
+              for (int neg = 0; neg < 2; ++neg) {
+                uint8_t* row = reinterpret_cast<uint8_t*>(rows.data()) +
+                               16 * ((size_t)e * n_rows + row0[g] + (j * H.meta[g].len + k) * 2 + neg);
+                for (int hp = 0; hp < 8; ++hp) {
+                  const int v = contribution(g, e, j, k, hp);
+                  const int biased = (neg ? -v : v) + most;
+                  row[hp] = (uint8_t)(biased & 0xFF);
+                  row[8 + hp] = (uint8_t)(biased >> 8);
+                }
               }
-            }
-        }
       UP(rows, T.ptab);
       // nu's increment as the kernels round it: fl(alpha fl(P (65536 - P)) 2^-32)
       std::vector<uint2> pva(H.pv.size());
@@ -1355,24 +1392,82 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
         pva[q] = make_uint2(P, bits);
       }
       UP(pva, T.pva);
-      std::vector<int2> inc8(nnz);
+      // first pattern row of each clause, incidences with every chunk per variable
+      std::vector<int32_t> hrow;
+      std::vector<int32_t> inc_off;
+      if (!T.one_chunk) {
+        hrow.resize(m);
+        inc_off.assign(n + 1, 0);
+        int32_t next = 0;
+        for (int64_t c = 0; c < m; ++c) {
+          hrow[c] = next;
+          if (cl_grp[c] < 0) continue;
+          next += chunks[cl_grp[c]];
+          for (int64_t j = off[c]; j < off[c + 1]; ++j)
+            inc_off[lits[j] > 0 ? lits[j] : -lits[j]] += chunks[cl_grp[c]];
+        }
+        F.h_rows = next;
+        for (int i = 0; i < n; ++i) inc_off[i + 1] += inc_off[i];
+      }
+      const std::vector<int32_t>& ioff = T.one_chunk ? var_off : inc_off;
+      std::vector<int2> inc8((size_t)pseudo);
       {
-        std::vector<int32_t> fill(var_off.begin(), var_off.end() - 1);
-        for (int64_t c = 0; c < m; ++c)
-          for (int64_t j = off[c]; j < off[c + 1]; ++j) {
-            const int32_t l = lits[j];
-            inc8[fill[(l > 0 ? l : -l) - 1]++] =
-                make_int2((int32_t)c, row_of(cl_grp[c], (int)(j - off[c]), l < 0));
+        std::vector<int32_t> fill(ioff.begin(), ioff.end() - 1);
+        for (int64_t c = 0; c < m; ++c) {
+          const int g = cl_grp[c], len = (int)(off[c + 1] - off[c]);
+          for (int k = 0; k < len; ++k) {
+            const int32_t l = lits[off[c] + k];
+            int32_t& at = fill[(l > 0 ? l : -l) - 1];
+            for (int j = 0; j < chunks[g]; ++j)
+              inc8[at++] = make_int2(T.one_chunk ? (int32_t)c : hrow[c] + j,
+                                     16 * (row0[g] + (j * len + k) * 2 + (l < 0 ? 1 : 0)));
           }
+        }
       }
       UP(inc8, F.var_inc8);
       std::vector<int4> slots(n);
       for (int k = 0; k < n_inst; ++k)
         for (int s = var_base[k]; s < var_base[k + 1]; ++s) {
           const int i = order[s];
-          slots[s] = make_int4(i, var_off[i], var_off[i + 1] - var_off[i], k);
+          slots[s] = make_int4(i, ioff[i], ioff[i + 1] - ioff[i], k);
         }
       UP(slots, F.var_slot);
+      if (!T.one_chunk) {
+        // chunk records, the groups in order of size so that those with few
+        // patterns (most clauses of random lengths) form the staged prefix
+        std::vector<int32_t> by_size(G);
+        std::iota(by_size.begin(), by_size.end(), 0);
+        auto words = [&](int g) { return ((int64_t)E * chunks[g]) << H.meta[g].len; };
+        std::stable_sort(by_size.begin(), by_size.end(), [&](int a, int b) { return words(a) < words(b); });
+        std::vector<int32_t> rec_at(G);
+        std::vector<uint4> recn;
+        for (int g : by_size) {
+          const GroupMeta& gm = H.meta[g];
+          rec_at[g] = (int32_t)recn.size();
+          for (int e = 0; e < E; ++e)
+            for (int p = 0; p < (1 << gm.len); ++p) {
+              const uint32_t* r = H.rec.data() + gm.rec_off + (((size_t)e << gm.len) + p) * gm.stride;
+              auto unit = [&](int h) { return h < gm.nh ? r[1 + h] : 0u; };
+              for (int j = 0; j < chunks[g]; ++j)
+                recn.push_back(make_uint4(j == 0 ? r[0] : 0u, unit(3 * j), unit(3 * j + 1), unit(3 * j + 2)));
+            }
+          if ((int64_t)recn.size() * 16 <= kRecnSmemBytes) T.recn_smem = (int32_t)recn.size();
+        }
+        std::vector<int4> cln(m);
+        for (int64_t c = 0; c < m; ++c) {
+          const int g = cl_grp[c];
+          if (g < 0) {
+            cln[c] = make_int4(0, 0, 0, 0);
+            continue;
+          }
+          const GroupMeta& gm = H.meta[g];
+          cln[c] = make_int4(cl_off[c], rec_at[g], hrow[c],
+                             gm.len | (chunks[g] << 4) | (gm.nh << 8) | (gm.sat ? 1 << 13 : 0) |
+                                 (rec_at[g] < T.recn_smem ? 1 << 14 : 0));
+        }
+        UP(recn, T.recn);
+        UP(cln, F.cln);
+      }
     }
   }
   F.cl4 = nullptr;

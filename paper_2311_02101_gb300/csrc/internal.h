@@ -21,6 +21,9 @@ enum : uint32_t { kPhaseInit = 1, kPhaseHidden = 2, kPhaseVisible = 3, kPhaseSwa
 
 constexpr int kChainTile = 256;   // chains per block of the sparse kernels
 constexpr int kNibMaxContribution = 1023;  // largest |2^Q G| of the nibble update's rows
+constexpr int kNibMaxRowBytes = 88 * 1024;  // those rows (all temperatures) in shared memory
+constexpr int kRecnSmemBytes = 92 * 1024;   // staged chunk records of k_gather_nib: two
+                                            // blocks per SM
 constexpr int kClauseBlock = 64;  // clauses per block of the sparse gather
 
 // ---------------------------------------------------------------------------
@@ -59,11 +62,19 @@ struct DevFormula {
                            // hidden probability of the group is 65536, bit k of `negated` set when literal k is
                            // negated, when every clause has at most 3
                            // literals (one-chunk tables); else NULL
-  // one-chunk tables only (else NULL): the incidences of a variable as
-  // {clause, byte offset of its row in a temperature's block of ptab}, and per
-  // position of var_order {variable, first incidence, incidences, instance}
+  // 4-bit hidden patterns (else NULL): every three hidden units of a clause are
+  // a chunk with a pattern row of its own (h_rows rows). Per variable its
+  // incidences with every chunk as {pattern row, byte offset of its
+  // contributions in a temperature's block of ptab}; per position of var_order
+  // {variable, first incidence, incidences, instance}
   const int2* var_inc8;
   const int4* var_slot;
+  int32_t h_rows;
+  // formulas with clauses of more than 3 hidden units: m clause records {first
+  // literal, record offset in recn (16-byte words, temperature 0), first
+  // pattern row, length | chunks << 4 | hidden units << 8 | saturated << 13 |
+  // in shared memory << 14}; else NULL
+  const int4* cln;
   const int32_t* var_order;  // n: the visible update's order: variables by
                              // degree, highest first (ties to the lower index),
                              // within windows of 512 variables of one formula
@@ -99,10 +110,16 @@ struct DevTables {
   const int16_t* gq;   // 2 gq_len entries: 2^Q G, then -2^Q G (a negated
                        // literal's incidence reads the second half)
   const uint32_t* pv;
-  // one-chunk tables only (else NULL): per temperature a block of ptab_stride
-  // bytes of 16-byte rows, row 0 zero, then one per (group, position, sign):
-  // the low bytes of contribution + ptab_bias for the 8 hidden patterns, then
-  // their high bytes
+  // chunk records of k_gather_nib (else NULL): per (group, temperature, truth
+  // pattern, chunk) {free energy in chunk 0, else 0; three thresholds as in
+  // rec}, the groups in order of size; the first recn_smem records are staged
+  // in shared memory
+  const uint4* recn;
+  int32_t recn_smem;
+  // 4-bit patterns (else NULL): per temperature a block of ptab_stride bytes of
+  // 16-byte rows, row 0 zero, then one per (group, chunk, position, sign): the
+  // low bytes of contribution + ptab_bias for the chunk's 8 hidden patterns,
+  // then their high bytes
   const uint32_t* ptab;
   int32_t ptab_stride, ptab_bias;
   const uint2* pva;  // pv_len: {P, float bits of fl(alpha fl(P (65536 - P)) 2^-32)}
@@ -150,7 +167,7 @@ struct DevChains {
   int64_t* cost_part; // [clause block][Bp]
   float* fe_part;     // [clause block][Bp]
   void* H;            // m x Bp hidden patterns (uint8_t, or uint16_t when L > 8;
-                      // nib: m x Bp / 8 words)
+                      // nib: h_rows x Bp / 8 words)
   int32_t* tickets;   // Bp / kChainTile arrival counters of the gather blocks
 };
 

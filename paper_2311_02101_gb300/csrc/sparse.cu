@@ -652,6 +652,75 @@ __device__ __forceinline__ void gather3_clauses(const DevFormula& F, const DevCh
   }
 }
 
+// The end of a step gather block (chain tile bx of gx, clause block by): its 8
+// warps' costs and free energies per chain go to the block's partial sums; the
+// block that arrives last among its instance's blocks for this tile of 256
+// chains reduces them in block order and keeps improvements (as k_gather).
+template <bool PERSIST>
+__device__ __forceinline__ void gather_finish(const DevChains& C, const GatherPlan& P, int inst,
+                                              int bx, int by, int gx, const int32_t (&cost)[8],
+                                              const float (&fe)[8], int64_t* cost_part,
+                                              float* fe_part, int32_t* tickets) {
+  __shared__ int32_t s_cost[8][256];
+  __shared__ float s_fe[8][256];
+  __shared__ int s_last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, Bp = C.Bp;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    s_cost[warp][lane * 8 + q] = cost[q];
+    s_fe[warp][lane * 8 + q] = fe[q];
+  }
+  __syncthreads();
+  int64_t tc = 0;
+  float tf = 0.f;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    tc += s_cost[w][tid];
+    tf += s_fe[w][tid];
+  }
+  const size_t out = (size_t)by * Bp + (size_t)bx * 256 + tid;
+  cost_part[out] = tc;
+  fe_part[out] = tf;
+  __threadfence();
+  __syncthreads();
+  const int k0 = __ldg(P.inst_blk + inst), k1 = __ldg(P.inst_blk + inst + 1);
+  int32_t* ticket = tickets + inst * gx + bx;
+  if (tid == 0) s_last = atomicAdd(ticket, 1) == k1 - k0 - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const int b = bx * 256 + tid;
+  int64_t csum = 0;
+  float fsum = 0.f;
+  // eight blocks' partials in flight at a time (the sums stay in block order)
+  int k = k0;
+  for (; k + 8 <= k1; k += 8) {
+    int64_t cp[8];
+    float fp[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      cp[u] = __ldcg(cost_part + (size_t)(k + u) * Bp + b);
+      fp[u] = __ldcg(fe_part + (size_t)(k + u) * Bp + b);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      csum += cp[u];
+      fsum += fp[u];
+    }
+  }
+  for (; k < k1; ++k) {
+    csum += __ldcg(cost_part + (size_t)k * Bp + b);
+    fsum += __ldcg(fe_part + (size_t)k * Bp + b);
+  }
+  const size_t ib = (size_t)inst * Bp + b;
+  C.cost[ib] = csum;
+  C.fe[ib] = fsum;
+  const bool imp = csum < (PERSIST ? __ldcg(C.best + ib) : C.best[ib]);
+  if (imp) C.best[ib] = csum;
+  C.improved[ib] = imp ? 1 : 0;
+  if (tid == 0) *ticket = 0;
+}
+
 // One block of the gather: chain tile bx of gx, clause block by of gy.
 // PERSIST: a block of the persistent round (k_round_persistent), which has
 // staged the record blocks already, orders its phases by grid barriers
@@ -671,9 +740,6 @@ __device__ __forceinline__ void gather3_block(const DevFormula& F, const DevTabl
 #define G3_GY (PERSIST ? vgy : gridDim.y)
   if constexpr (!PERSIST) pdl_release();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int64_t s_cost[8][256];
-  __shared__ float s_fe[8][256];
-  __shared__ int s_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g8 = G3_BX * 32 + lane, b0 = g8 * 8;
   const int Bp = C.Bp;
@@ -716,46 +782,8 @@ __device__ __forceinline__ void gather3_block(const DevFormula& F, const DevTabl
   // per-block partial sums; the block that arrives last among its instance's
   // blocks for this tile of 256 chains reduces them in block order and keeps
   // improvements (as k_gather)
-  int32_t* my_cost32 = reinterpret_cast<int32_t*>(&s_cost[0][0]) + warp * 256 + lane * 8;
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    my_cost32[q] = cost[q];
-    s_fe[warp][lane * 8 + q] = fe[q];
-  }
-  __syncthreads();
-  const int tid = threadIdx.x;
-  int64_t tc = 0;
-  float tf = 0.f;
-#pragma unroll
-  for (int w = 0; w < 8; ++w) {
-    tc += reinterpret_cast<const int32_t*>(&s_cost[0][0])[w * 256 + tid];
-    tf += s_fe[w][tid];
-  }
-  const size_t out = (size_t)G3_BY * Bp + (size_t)G3_BX * 256 + tid;
-  cost_part[out] = tc;
-  fe_part[out] = tf;
-  __threadfence();
-  __syncthreads();
-  const int k0 = __ldg(P.inst_blk + inst), k1 = __ldg(P.inst_blk + inst + 1);
-  int32_t* ticket = tickets + inst * G3_GX + G3_BX;
-  if (tid == 0) s_last = atomicAdd(ticket, 1) == k1 - k0 - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const int b = G3_BX * 256 + tid;
-  int64_t csum = 0;
-  float fsum = 0.f;
-  for (int k = k0; k < k1; ++k) {
-    csum += __ldcg(cost_part + (size_t)k * Bp + b);
-    fsum += __ldcg(fe_part + (size_t)k * Bp + b);
-  }
-  const size_t ib = (size_t)inst * Bp + b;
-  C.cost[ib] = csum;
-  C.fe[ib] = fsum;
-  const bool imp = csum < (PERSIST ? __ldcg(C.best + ib) : C.best[ib]);
-  if (imp) C.best[ib] = csum;
-  C.improved[ib] = imp ? 1 : 0;
-  if (tid == 0) *ticket = 0;
+  gather_finish<PERSIST>(C, P, inst, (int)G3_BX, (int)G3_BY, (int)G3_GX, cost, fe, cost_part,
+                         fe_part, tickets);
 #undef G3_BX
 #undef G3_BY
 #undef G3_GX
@@ -769,6 +797,232 @@ __global__ void __launch_bounds__(256, 2) k_gather3(DevFormula F, DevTables T, D
                                                     float* fe_part, int32_t* tickets) {
   gather3_block<PLAIN3, COST16, false, NIB>(F, T, C, P, tdev, t_rel, cost_part, fe_part, tickets,
                                        blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
+}
+
+// ---------------------------------------------------------------------------
+// Step gather for formulas with clauses of any length and 4-bit hidden patterns
+// (C.nib): a clause RBM with L hidden units is taken as ceil(L / 3) chunks of
+// three units, each with its own pattern word of 4 bits per chain, so that
+// k_visible_nib adds its contributions chunk by chunk (they are linear in the
+// hidden units). The record of a truth pattern is one 16-byte word per chunk:
+// {clause free energy in chunk 0, else 0; thresholds of the chunk's units}.
+// Results are those of k_gather<kStep>, bit for bit.
+//
+// What bounded k_gather here (lengths 2..12, n = 20000, m = 100000, 1024 chains:
+// 424 us a launch): 275 M warp instructions at 56 % issue, 13 M of them spills,
+// a full Philox block per unit, and tables too large for shared memory as a
+// whole (every look-up through the L1). Now the clause's share of Philox rounds
+// 0..2 is computed once, three units' blocks run interleaved, the groups with
+// few patterns (most clauses) keep their records in shared memory (the host
+// orders the groups by size; the first T.recn_smem words are staged), costs
+// stay in registers, and the next clause's record, literals and states are
+// loaded while the current one is sampled.
+// ---------------------------------------------------------------------------
+struct ChunkAddr {
+  uint32_t off[8];  // byte address (shared memory) or byte offset (global) per chain
+};
+
+template <bool SAT, bool SMEM, int Q>
+__device__ __forceinline__ void chunk_chain(const uint32_t off, const char* base,
+                                            const uint4 (&R)[3], float& fe, uint32_t& hw) {
+  const uint4 r = SMEM ? lds128(off) : __ldg(reinterpret_cast<const uint4*>(base + off));
+  fe += __uint_as_float(r.x);
+  unit_draw<SAT, true, Q, 0>(R, r.y, hw);
+  unit_draw<SAT, true, Q, 1>(R, r.z, hw);
+  unit_draw<SAT, true, Q, 2>(R, r.w, hw);
+}
+
+template <bool SAT, bool SMEM>
+__device__ __forceinline__ uint32_t chunk_draws(const ChunkAddr& A, uint32_t add, const char* base,
+                                                const uint4 (&R)[3], float (&fe)[8]) {
+  uint32_t hw = 0;
+  chunk_chain<SAT, SMEM, 0>(A.off[0] + add, base, R, fe[0], hw);
+  chunk_chain<SAT, SMEM, 1>(A.off[1] + add, base, R, fe[1], hw);
+  chunk_chain<SAT, SMEM, 2>(A.off[2] + add, base, R, fe[2], hw);
+  chunk_chain<SAT, SMEM, 3>(A.off[3] + add, base, R, fe[3], hw);
+  chunk_chain<SAT, SMEM, 4>(A.off[4] + add, base, R, fe[4], hw);
+  chunk_chain<SAT, SMEM, 5>(A.off[5] + add, base, R, fe[5], hw);
+  chunk_chain<SAT, SMEM, 6>(A.off[6] + add, base, R, fe[6], hw);
+  chunk_chain<SAT, SMEM, 7>(A.off[7] + add, base, R, fe[7], hw);
+  return hw;
+}
+
+__global__ void __launch_bounds__(256, 2) k_gather_nib(DevFormula F, DevTables T, DevChains C,
+                                                       GatherPlan P, const uint32_t* tdev,
+                                                       uint32_t t_rel, int64_t* cost_part,
+                                                       float* fe_part, int32_t* tickets) {
+  pdl_release();
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g8 = blockIdx.x * 32 + lane, b0 = g8 * 8, Bp = C.Bp;
+  const int4 bd = __ldg(P.blk + blockIdx.y);
+  const int inst = bd.x, c_begin = bd.y, c_end = bd.z, cl_base = bd.w;
+  stage(smem, T.recn, T.recn_smem * 16);
+  __syncthreads();
+  const uint32_t tab = (uint32_t)__cvta_generic_to_shared(smem);
+  const char* gtab = reinterpret_cast<const char*>(T.recn);
+  // temperature of the octet's chains: e0, from chain `split` on the next one
+  const int E = T.n_temps, gb0 = C.g8_off * 8 + b0;
+  const int e0 = temp_of(gb0, E, C.B_total, C.inv_B_total);
+  int split = 8;
+  if (e0 != temp_of(gb0 + 7, E, C.B_total, C.inv_B_total))
+    split = (int)(((long long)(e0 + 1) * C.B_total + E - 1) / E) - gb0;
+  int32_t cost[8];
+  float fe[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    cost[q] = 0;
+    fe[q] = 0.f;
+  }
+  // records of the first three clauses of this warp, literals of the first two
+  auto load_rec = [&](int c) { return c < c_end ? __ldg(F.cln + c) : make_int4(0, 0, 0, 0); };
+  auto load_lits = [&](const int4& r, int32_t (&l)[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) l[k] = k < (r.w & 15) ? __ldg(F.lit_var + r.x + k) : 0;
+  };
+  const uint8_t* xtb = C.xt + b0;
+  auto state_of = [&](int32_t l) {
+    return __ldg(reinterpret_cast<const uint2*>(xtb + (size_t)(l & 0x7FFFFFFF) * Bp));
+  };
+  auto load_states = [&](const int4& r, const int32_t (&l)[4], uint2 (&x)[4]) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[k] = make_uint2(0u, 0u);
+      if (k < (r.w & 15)) {
+        const uint32_t flip = l[k] < 0 ? 0x01010101u : 0u;
+        x[k] = state_of(l[k]);
+        x[k].x ^= flip;
+        x[k].y ^= flip;
+      }
+    }
+  };
+  int4 rec = load_rec(c_begin + warp), rec1 = load_rec(c_begin + warp + 8);
+  int32_t lits[4], lits1[4];
+  load_lits(rec, lits);
+  load_lits(rec1, lits1);
+  pdl_wait();  // chain state from here on
+  const uint32_t t = step_index(tdev, t_rel);
+  uint2 x[4];
+  load_states(rec, lits, x);
+
+  const RoundKeys& K = C.keys;
+  const uint32_t octet = (uint32_t)(g8 + C.g8_off);
+  const uint32_t phase = kPhaseHidden | ((uint32_t)inst << 8);
+  const uint64_t pt = (uint64_t)kPhiloxM1 * t;
+  const uint32_t u1 = (uint32_t)(pt >> 32) ^ K.k0[0], u2 = (uint32_t)pt;
+  uint32_t* H = static_cast<uint32_t*>(C.H) + g8;
+  const size_t hstride = (size_t)(Bp / 8);
+
+  for (int c = c_begin + warp; c < c_end; c += 8) {
+    const int4 rec2 = load_rec(c + 16);
+    const int32_t wc = (int32_t)__ldg(F.cl_w + c);
+    const int len = rec.w & 15, chunks = (rec.w >> 4) & 15, nh = (rec.w >> 8) & 31;
+    // byte q of lo0|lo1: bits 0..7 of chain q's truth pattern; of hi0|hi1: bits 8..15
+    uint32_t lo0 = x[0].x | (x[1].x << 1) | (x[2].x << 2) | (x[3].x << 3);
+    uint32_t lo1 = x[0].y | (x[1].y << 1) | (x[2].y << 2) | (x[3].y << 3);
+    uint32_t hi0 = 0, hi1 = 0;
+    for (int k = 4; k < len; k += 4) {
+      int32_t l[4];
+      uint2 y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) l[u] = k + u < len ? __ldg(F.lit_var + rec.x + k + u) : 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        y[u] = make_uint2(0u, 0u);
+        if (k + u < len) {
+          const uint32_t flip = l[u] < 0 ? 0x01010101u : 0u;
+          y[u] = state_of(l[u]);
+          y[u].x ^= flip;
+          y[u].y ^= flip;
+        }
+      }
+      const uint32_t a = y[0].x | (y[1].x << 1) | (y[2].x << 2) | (y[3].x << 3);
+      const uint32_t b = y[0].y | (y[1].y << 1) | (y[2].y << 2) | (y[3].y << 3);
+      if (k == 4) {
+        lo0 |= a << 4;
+        lo1 |= b << 4;
+      } else {
+        hi0 |= a << (k - 8);
+        hi1 |= b << (k - 8);
+      }
+    }
+    // the next clause's states and the one after its literals
+    load_states(rec1, lits1, x);
+    load_lits(rec2, lits1);
+    // chains without a true literal add the weight
+    const uint32_t any0 = lo0 | hi0, any1 = lo1 | hi1;
+    const uint32_t un0 = ~(((any0 & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | any0) & 0x80808080u;
+    const uint32_t un1 = ~(((any1 & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | any1) & 0x80808080u;
+    if (un0 | un1) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        cost[q] += ((un0 >> (8 * q + 7)) & 1u) ? wc : 0;
+        cost[q + 4] += ((un1 >> (8 * q + 7)) & 1u) ? wc : 0;
+      }
+    }
+    if (len > 0) {
+      const bool sat = (rec.w >> 13) & 1, in_smem = (rec.w >> 14) & 1;
+      const uint32_t rstride = 16u * (uint32_t)chunks, estride = rstride << len;
+      const uint32_t base = (in_smem ? tab : 0u) + 16u * (uint32_t)rec.y + (uint32_t)e0 * estride;
+      ChunkAddr A;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t p0 = __byte_perm(lo0, hi0, ((4u + q) << 4) | q) & 0xFFFFu;
+        const uint32_t p1 = __byte_perm(lo1, hi1, ((4u + q) << 4) | q) & 0xFFFFu;
+        A.off[q] = base + p0 * rstride;
+        A.off[q + 4] = base + p1 * rstride;
+      }
+      if (split < 8) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q)
+          if (q >= split) A.off[q] += estride;
+      }
+      // Philox rounds 0..2: the clause's share
+      const uint32_t cl = (uint32_t)(c - cl_base);
+      const uint64_t p0 = (uint64_t)kPhiloxM0 * cl;
+      const uint32_t c1 = (uint32_t)(p0 >> 32) ^ phase ^ K.k1[0];
+      const uint32_t c2 = (uint32_t)p0;
+      const uint64_t p1 = (uint64_t)kPhiloxM1 * c1;
+      const uint32_t c3 = (uint32_t)(p1 >> 32) ^ u2 ^ K.k0[1];
+      const uint32_t c4 = (uint32_t)p1;
+      const uint64_t p2 = (uint64_t)kPhiloxM0 * c3;
+      const uint32_t c5 = (uint32_t)(p2 >> 32) ^ K.k1[2];
+      const uint32_t c6 = (uint32_t)p2;
+      auto unit_block = [&](int unit) {
+        const uint64_t px = (uint64_t)kPhiloxM0 * ((octet | ((uint32_t)unit << 24)) ^ u1);
+        const uint64_t pz =
+            (uint64_t)kPhiloxM1 * ((uint32_t)(px >> 32) ^ K.k1[1] ^ c2);
+        return philox_rounds<3>(make_uint4((uint32_t)(pz >> 32) ^ c4 ^ K.k0[2], (uint32_t)pz,
+                                           c5 ^ (uint32_t)px, c6),
+                                K);
+      };
+      uint32_t* Hc = H + (size_t)rec.z * hstride;
+      for (int j = 0; j < chunks; ++j, Hc += hstride) {
+        uint4 R[3];
+        if (3 * j + 3 <= nh) {
+#pragma unroll
+          for (int h = 0; h < 3; ++h) R[h] = unit_block(3 * j + h);
+        } else {  // one or two units left; absent ones have threshold 0
+          R[0] = unit_block(3 * j);
+          R[1] = 3 * j + 1 < nh ? unit_block(3 * j + 1) : make_uint4(0u, 0u, 0u, 0u);
+          R[2] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        const uint32_t add = 16u * (uint32_t)j;
+        uint32_t hw;
+        if (in_smem)
+          hw = sat ? chunk_draws<true, true>(A, add, gtab, R, fe)
+                   : chunk_draws<false, true>(A, add, gtab, R, fe);
+        else
+          hw = sat ? chunk_draws<true, false>(A, add, gtab, R, fe)
+                   : chunk_draws<false, false>(A, add, gtab, R, fe);
+        *Hc = hw;
+      }
+    }
+    rec = rec1;
+    rec1 = rec2;
+  }
+  gather_finish<false>(C, P, inst, (int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x, cost, fe,
+                       cost_part, fe_part, tickets);
 }
 
 // CG: the improved flags come from the L2 (a persistent launch: another
@@ -958,8 +1212,9 @@ __global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4) k_visible(DevFormula 
 }
 
 // ---------------------------------------------------------------------------
-// Visible update on nibble patterns (C.nib): formulas whose clause groups all
-// have at most 3 hidden units. The results are those of k_visible, bit for bit.
+// Visible update on nibble patterns (C.nib): every three hidden units of a
+// clause are one row of 4-bit fields (formulas of clauses of at most 3 literals
+// have one row per clause). The results are those of k_visible, bit for bit.
 //
 // The sum over a variable's incidences is what the update does most of: at
 // weighted 3-SAT n = 1000, m = 6000 and 4096 chains, 18000 incidences x 4096
@@ -1614,7 +1869,7 @@ int visible_smem_bytes(const DevTables& T) {
 }
 
 constexpr int kSmemLimit = 160 * 1024;
-constexpr int kNibSmemLimit = 48 * 1024;
+constexpr int kNibSmemLimit = 96 * 1024;
 int l2_bytes();
 constexpr int kMaxGridY = 65535;
 
@@ -1705,11 +1960,22 @@ int gather_occupancy(int smem) {
   return nb > 0 ? nb : 1;
 }
 
+int gather_nib_smem_bytes(const DevTables& T) { return T.recn_smem * 16; }
+
 template <int MODE>
 cudaError_t gather_mode(dim3 grid, cudaStream_t st, bool wide, const DevFormula& F,
                         const DevTables& T, const DevChains& C, const uint8_t* xt, int B, int Bp,
                         const GatherPlan& P, const uint32_t* tdev, uint32_t t_rel,
                         int64_t* cost_part, float* fe_part, int32_t* tickets, int64_t* eval_out) {
+  if constexpr (MODE == kStep) {
+    if (C.nib && !T.one_chunk) {
+      const int smn = gather_nib_smem_bytes(T);
+      const cudaError_t e = allow_dynamic_smem(k_gather_nib, smn);
+      if (e != cudaSuccess) return e;
+      return launch_pdl(k_gather_nib, grid, smn, st, F, T, C, P, tdev, t_rel, cost_part, fe_part,
+                        tickets);
+    }
+  }
   const int sm = gather_smem_bytes(T);
   const bool use_sm = MODE != kEval && sm <= kSmemLimit;
   if (use_sm && !wide)
@@ -1791,8 +2057,12 @@ cudaError_t visible_nib(const DevFormula& F, const DevTables& T, const DevChains
   const cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const long long items = (long long)F.n * (C.Bp / kChainTile);
-  const long long grid = std::min<long long>((items + 7) / 8, (batch >= 8 ? 3LL : 4LL) * sm_count());
-  const int tm = (double)F.m * C.Bp * 0.5 > 0.5 * (double)l2_bytes() ? 1 : 0;
+  int per_sm = 1;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem) != cudaSuccess ||
+      per_sm < 1)
+    per_sm = 1;
+  const long long grid = std::min<long long>((items + 7) / 8, (long long)per_sm * sm_count());
+  const int tm = (double)F.h_rows * C.Bp * 0.5 > 0.5 * (double)l2_bytes() ? 1 : 0;
   // 1 - alpha as the device's one rounding gives it
   volatile float one = 1.0f;
   const float keep = one - alpha;
@@ -1801,12 +2071,12 @@ cudaError_t visible_nib(const DevFormula& F, const DevTables& T, const DevChains
 
 }  // namespace
 
-// Nibble patterns: every group has at most 3 hidden units, the contribution
-// rows were built (|2^Q G| <= 1023, so a window of 32 incidences fits 16 bits)
-// and leave room for 4 blocks per SM, and no octet of chains spans more than
+// Nibble patterns: the contribution rows were built (every chunk's |2^Q G| <=
+// 1023, so a window of 32 incidences fits 16 bits) and fit shared memory with
+// two blocks per SM, and no octet of chains spans more than
 // two temperatures (temperature blocks of at least 8 chains).
 bool nib_patterns_supported(const DevTables& T, int B_total) {
-  return T.one_chunk && T.ptab && nib_smem_bytes(T) <= kNibSmemLimit &&
+  return (T.one_chunk || T.recn) && T.ptab && nib_smem_bytes(T) <= kNibSmemLimit &&
          (T.n_temps == 1 || B_total / T.n_temps >= 8);
 }
 
@@ -1851,6 +2121,14 @@ int gather_clause_block(int m, int tiles, int slots) {
 // resident blocks per SM of the step gather that will run (the one-chunk
 // variant when every record is one chunk)
 int gather_blocks_per_sm(const DevTables& T, bool wide) {
+  if (!T.one_chunk && T.recn) {
+    const int smn = gather_nib_smem_bytes(T);
+    int nb = 0;
+    if (allow_dynamic_smem(k_gather_nib, smn) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_gather_nib, 256, smn) != cudaSuccess)
+      return 1;
+    return nb > 0 ? nb : 1;
+  }
   const int sm = gather_smem_bytes(T);
   const bool use_sm = sm <= kSmemLimit;
   const bool one = T.one_chunk && !wide;
@@ -1906,7 +2184,7 @@ cudaError_t launch_gather(GatherMode mode, const DevFormula& F, const DevTables&
 cudaError_t launch_visible(const DevFormula& F, const DevTables& T, const DevChains& C,
                            float alpha, const uint32_t* tdev, uint32_t t_rel, bool wide,
                            cudaStream_t st, int batch) {
-  if (C.nib && !wide) return visible_nib(F, T, C, alpha, tdev, t_rel, batch, st);
+  if (C.nib) return visible_nib(F, T, C, alpha, tdev, t_rel, batch, st);
   dim3 grid(C.Bp / kChainTile, (F.n + 7) / 8);
   const int sm = visible_smem_bytes(T);
   const bool use_sm = sm <= kSmemLimit;

@@ -1,8 +1,8 @@
-"""Rounds on formulas of at most 3 literals per clause, where their kernels
-change form: variables in more than 32 clauses (several incidence windows),
-octets of chains across two temperatures, temperature blocks too small or
-contributions too large for 4-bit patterns, several chain tiles, formulas
-smaller than a block. Every case against the oracle, bit for bit (the free
+"""Rounds where their kernels change form: variables in more than 32 clauses
+(several incidence windows), octets of chains across two temperatures,
+temperature blocks too small, contributions or weights too large for 4-bit
+patterns, several chain tiles, formulas smaller than a block, clauses whose
+hidden units fill one to four chunks of three. Every case against the oracle, bit for bit (the free
 energy within the 1e-3 bar of the other parity tests)."""
 import os
 
@@ -31,21 +31,23 @@ def ms():
 _tables = {}
 
 
-def table_for(temps, Q):
-    if (temps, Q) not in _tables:
-        table = oracle.make_table([1, 2, 3], FSTARS[:temps], n_buckets=2, Q=Q, iters=1500)
+def table_for(temps, Q, longest):
+    key = temps, Q, longest
+    if key not in _tables:
+        table = oracle.make_table(list(range(1, longest + 1)), FSTARS[:temps], n_buckets=2, Q=Q,
+                                  iters=1500 if longest <= 3 else 100)
         for s in table.sets:
             s["W"] = 6.0 * np.asarray(s["W"])  # on the grid, sized as converged fits are
-        _tables[temps, Q] = table
-    return _tables[temps, Q]
+        _tables[key] = table
+    return _tables[key]
 
 
-def short_clauses(n, m, seed):
-    """m clauses of 0..3 literals, repeated and opposite literals included."""
+def short_clauses(n, m, seed, longest=3, wmax=9):
+    """m clauses of 0..longest literals, repeated and opposite literals included."""
     rng = np.random.default_rng(seed)
     cl = [list(rng.integers(1, n + 1, size=k) * (1 - 2 * rng.integers(0, 2, size=k)))
-          for k in rng.integers(0, 4, size=m)]
-    return oracle.Instance.from_clauses(n, cl, list(rng.integers(1, 9, size=m)))
+          for k in rng.integers(0, longest + 1, size=m)]
+    return oracle.Instance.from_clauses(n, cl, [int(w) for w in rng.integers(1, wmax, size=m)])
 
 
 CASES = {
@@ -60,6 +62,11 @@ CASES = {
     "tiles": (lambda: oracle.Instance(*workloads.random_ksat(70, 333, 3, 7, 30000)), 1300, 2, 4),
     "more-variables-than-clauses": (lambda: oracle.Instance(*workloads.random_ksat(900, 20, 3, 8)),
                                     256, 2, 4),
+    "lengths-0-9": (lambda: short_clauses(60, 300, 9, 9), 520, 3, 4),
+    "lengths-thin-temperatures": (lambda: short_clauses(60, 200, 10, 9), 44, 6, 4),
+    "lengths-wide-contributions": (lambda: short_clauses(60, 200, 11, 9), 256, 2, 8),
+    "lengths-heavy": (lambda: short_clauses(60, 200, 12, 9, 2 ** 33), 256, 2, 4),
+    "lengths-high-degree": (lambda: short_clauses(12, 500, 13, 9), 300, 2, 4),
 }
 
 
@@ -69,7 +76,8 @@ def test_rounds_match_oracle(ms, case, profiled):
     """`profiled` keeps the two-launch round (events around every launch)."""
     import torch
     make, B, temps, Q = CASES[case]
-    inst, table, alpha, seed = make(), table_for(temps, Q), 0.05, 21
+    inst, alpha, seed = make(), 0.05, 21
+    table = table_for(temps, Q, 9 if case.startswith("lengths") else 3)
     p = ms.maxsat_default_params(sets=table.sets, n_temps=temps, n_buckets=2, alpha=alpha,
                                  quant_bits=Q, path=ms.MAXSAT_PATH_SPARSE, steps_per_graph=4)
     ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, torch.cuda.Stream())
