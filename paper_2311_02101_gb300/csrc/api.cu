@@ -250,7 +250,10 @@ struct maxsat_ctx {
   // not used), its buffers, and what the next launch starts from
   RoundsArgs rounds;
   bool rounds_cost16 = false;
+  LocalFormula local;             // lists of the local rounds (local.cu; NULL: too large)
+  LocalPlan local_shape;          // for the current chains (threads 0: not used)
   int rounds_slot_count = -1;     // resident blocks of k_rounds (-1: not queried)
+  int rounds_per_sm = 0;
   bool persist_ran = false;       // some maxsat_step ran persistent launches (read d_err)
   // dense scatter-add (GEMM2): block-diagonal variable x incidence matrix
   int tiles_v = 0, kmax = 0;
@@ -500,9 +503,16 @@ void split_weights(const maxsat_ctx* ctx, int nb, int64_t* wmax, int64_t* wmax8)
 int plan_rounds(maxsat_ctx* ctx, DevAllocs& A, int Bp) {
   RoundsArgs& R = ctx->rounds;
   R = RoundsArgs{};
+  ctx->local_shape = ctx->local.cl ? local_plan(ctx->F, ctx->T, Bp) : LocalPlan{};
   if (ctx->n_inst != 1 || ctx->wide_h || !ctx->F.cl4) return MAXSAT_OK;
-  if (ctx->rounds_slot_count < 0) ctx->rounds_slot_count = rounds_slots(ctx->T);
-  const int slots = ctx->rounds_slot_count, tiles = Bp / kChainTile;
+  if (ctx->rounds_slot_count < 0) ctx->rounds_slot_count = rounds_slots(ctx->T, &ctx->rounds_per_sm);
+  int slots = ctx->rounds_slot_count;
+  const int tiles = Bp / kChainTile;
+  // three blocks per SM from 12 clauses per warp on; below that fewer blocks
+  // meet sooner at their barriers (n = 1000, m = 6000, 1024 chains: 6.6 clauses
+  // per warp 21.5 us a round, 9.9 on two blocks per SM 19.9)
+  if (ctx->rounds_per_sm >= 3 && (double)ctx->m * tiles < 12.0 * 8.0 * slots)
+    slots = slots / ctx->rounds_per_sm * 2;
   const int most = slots / tiles;
   if (most < 2) return MAXSAT_OK;
   const int S = std::min(most, std::max(1, ctx->plan.n_blk));
@@ -545,6 +555,7 @@ int alloc_chains(maxsat_ctx* ctx, int32_t B) {
   ctx->chain_mem.release();
   ctx->have_chains = false;
   ctx->rounds = RoundsArgs{};
+  ctx->local_shape = LocalPlan{};
   const int Bp = (B + kChainTile - 1) / kChainTile * kChainTile;
   const size_t nB = (size_t)ctx->n * Bp;
   if (ctx->gather_slots == 0) {
@@ -897,7 +908,8 @@ int tune_blocks(maxsat_ctx* ctx, int32_t B) {
   }
   ctx->cb_force = best;
   std::map<int, float> vis_of;  // visible batch -> fastest ms per round
-  for (int pass = 0; pass < 2 && rc == MAXSAT_OK && !vis_fixed; ++pass)
+  // (4-bit patterns are copied a window at a time, whatever the batch)
+  for (int pass = 0; pass < 2 && rc == MAXSAT_OK && !vis_fixed && !ctx->C.nib; ++pass)
     for (int vb : {2, 4, 8}) {
       ctx->vis_batch = vb;
       float ms = 0.f;
@@ -1432,6 +1444,36 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
           slots[s] = make_int4(i, ioff[i], ioff[i + 1] - ioff[i], k);
         }
       UP(slots, F.var_slot);
+      // lists of the local rounds: 16-bit indices, all weights together below
+      // 2^31 - 1, and (28 bytes a clause, 52 a variable) within an SM
+      int64_t weight = 0;
+      for (int64_t c = 0; c < m; ++c) weight += cl_w[c];
+      if (T.one_chunk && n_inst == 1 && n_rows <= 65535 && 28 * m + 52 * (int64_t)n <= 220 * 1024 &&
+          weight < (int64_t)INT32_MAX) {
+        std::vector<uint2> lcl(m);
+        std::vector<uint32_t> linc((size_t)nnz);
+        bool fits = m <= 65535 && n <= 65535 && G <= 1023;
+        for (int64_t c = 0; c < m && fits; ++c) {
+          const int len = (int)(off[c + 1] - off[c]);
+          if (len > 3) fits = false;
+          uint32_t v[3] = {0, 0, 0}, neg = 0;
+          for (int k = 0; k < len && fits; ++k) {
+            const int32_t l = lits[off[c] + k];
+            v[k] = (uint32_t)((l > 0 ? l : -l) - 1);
+            neg |= (l < 0 ? 1u : 0u) << k;
+          }
+          const uint32_t info =
+              len > 0 ? ((uint32_t)cl_grp[c] << 6) | (H.meta[cl_grp[c]].sat ? 32u : 0u) | (neg << 2) | (uint32_t)len
+                      : 0u;
+          lcl[c] = make_uint2(v[0] | (v[1] << 16), v[2] | (info << 16));
+        }
+        for (int64_t j = 0; j < nnz && fits; ++j)
+          linc[j] = (uint32_t)inc8[j].x | ((uint32_t)(inc8[j].y / 16) << 16);
+        if (fits) {
+          UP(lcl, ctx->local.cl);
+          UP(linc, ctx->local.inc);
+        }
+      }
       if (!T.one_chunk) {
         // chunk records, the groups in order of size so that those with few
         // patterns (most clauses of random lengths) form the staged prefix
@@ -1707,6 +1749,16 @@ static bool stream_capturing(cudaStream_t st) {
 // rounds per launch of the resident rounds
 static constexpr int64_t kMaxResidentRounds = 1000;
 
+// rounds of a call from which the local rounds pay for loading the formula into
+// every block
+static constexpr int64_t kMinLocalRounds = 8;
+
+// maxsat_step runs local rounds (local.cu)
+static bool local_rounds_active(const maxsat_ctx* ctx) {
+  return ctx->have_chains && !ctx->dense && ctx->local_shape.threads > 0 && ctx->C.nib &&
+         !ctx->profiling && !stream_capturing(ctx->stream);
+}
+
 // maxsat_step runs resident rounds (k_rounds): planned for these chains, no
 // per-kernel profiling, no GPU unit propagation pending (it runs beside the
 // rounds on a side stream, and a cooperative launch would wait for its SMs)
@@ -1777,6 +1829,17 @@ int maxsat_step(maxsat_ctx* ctx, int64_t steps) {
   if (!ctx->have_chains) return fail(ctx, MAXSAT_ESTATE, "maxsat_step before maxsat_reset");
   if (steps < 0) return fail(ctx, MAXSAT_EINVAL, "steps must be >= 0");
   if ((uint64_t)ctx->t + (uint64_t)steps > 0xFFFFFFFFull) return fail(ctx, MAXSAT_EINVAL, "round index would exceed 2^32");
+  if (steps >= kMinLocalRounds && local_rounds_active(ctx)) {
+    while (steps > 0) {
+      const int r = (int)std::min<int64_t>(steps, kMaxResidentRounds);
+      CK(ctx, launch_rounds_local(ctx->F, ctx->T, ctx->C, ctx->local, ctx->local_shape, ctx->t, r,
+                                  (float)ctx->prm.alpha, ctx->stream));
+      ctx->t += (uint32_t)r;
+      ctx->d_t_synced = false;
+      steps -= r;
+    }
+    return MAXSAT_OK;
+  }
   if (resident_rounds_active(ctx)) {
     while (steps > 0) {
       RoundsArgs& R = ctx->rounds;

@@ -21,7 +21,7 @@ enum : uint32_t { kPhaseInit = 1, kPhaseHidden = 2, kPhaseVisible = 3, kPhaseSwa
 
 constexpr int kChainTile = 256;   // chains per block of the sparse kernels
 constexpr int kNibMaxContribution = 1023;  // largest |2^Q G| of the nibble update's rows
-constexpr int kNibMaxRowBytes = 88 * 1024;  // those rows (all temperatures) in shared memory
+constexpr int kNibMaxRowBytes = 72 * 1024;  // those rows (all temperatures) in shared memory
 constexpr int kRecnSmemBytes = 92 * 1024;   // staged chunk records of k_gather_nib: two
                                             // blocks per SM
 constexpr int kClauseBlock = 64;  // clauses per block of the sparse gather
@@ -412,9 +412,25 @@ struct RoundsArgs {
   double fe_scale = 1.0;  // a power of two: block free energies as 64-bit fixed point
   float keep = 0.f;       // 1 - alpha (set by the launch)
 };
-int rounds_slots(const DevTables& T);
+int rounds_slots(const DevTables& T, int* per_sm);
 cudaError_t launch_rounds(const DevFormula& F, const DevTables& T, const DevChains& C,
                           RoundsArgs A, bool cost16, float alpha, cudaStream_t st);
+// Local rounds (local.cu): all rounds of eight chains in one block, for formulas
+// of at most 3 literals per clause that fit shared memory. cl: per clause
+// {variables 0 and 1, variable 2 | info << 16}, 16 bits each, info = group << 6 |
+// saturated << 5 | negated << 2 | length (absent literals: variable 0); inc: the
+// incidences of var_off as clause | contribution row of ptab << 16.
+struct LocalFormula {
+  const uint2* cl = nullptr;
+  const uint32_t* inc = nullptr;
+};
+struct LocalPlan {
+  int threads = 0, tpv = 1;  // threads per block (0: not used), per variable
+};
+LocalPlan local_plan(const DevFormula& F, const DevTables& T, int Bp);
+cudaError_t launch_rounds_local(const DevFormula& F, const DevTables& T, const DevChains& C,
+                                const LocalFormula& L, const LocalPlan& P, uint32_t t0, int rounds,
+                                float alpha, cudaStream_t st);
 // the persistent round (one cooperative launch of `rounds` Gibbs rounds,
 // grid barriers between the phases) covers this context's sparse round:
 // clauses of at most 3 literals, single-temperature octets, byte patterns

@@ -33,6 +33,7 @@
 
 #include "internal.h"
 #include "philox.cuh"
+#include "round_ops.cuh"
 
 namespace rbmsat {
 
@@ -416,26 +417,6 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
 //    measured faster than 3 or 4 blocks with spills, and than two clauses per
 //    loop trip).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
-  uint32_t v;
-  asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
-}
-
-__device__ __forceinline__ uint4 lds128(uint32_t addr) {
-  uint4 v;
-  asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-  return v;
-}
-
-// acc |= BIT when x < w (unsigned): one compare and one predicated OR
-template <uint32_t BIT>
-__device__ __forceinline__ void or_if_below(uint32_t& acc, uint32_t x, uint32_t w) {
-  asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-      : "+r"(acc)
-      : "r"(x), "r"(w), "n"(BIT));
-}
-
 // Asks the L2 to fetch `bytes` (a multiple of 16) from a 16-byte aligned
 // global address (a bulk prefetch: no data returns to the thread).
 __device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
@@ -462,43 +443,6 @@ __device__ __forceinline__ void load_clause_state(const uint8_t* xtb, int Bp, co
   xa = len > 0 ? ld_state<CG>(reinterpret_cast<const uint2*>(xtb + (size_t)r.x * Bp)) : make_uint2(0u, 0u);
   xb = len > 1 ? ld_state<CG>(reinterpret_cast<const uint2*>(xtb + (size_t)r.y * Bp)) : make_uint2(0u, 0u);
   xc = len > 2 ? ld_state<CG>(reinterpret_cast<const uint2*>(xtb + (size_t)r.z * Bp)) : make_uint2(0u, 0u);
-}
-
-// Unit H's draw for chain Q of the octet against threshold word w: bit
-// 4 Q + H of hw (NIB), else bit 8 (Q & 3) + H.
-template <bool SAT, bool NIB, int Q, int H>
-__device__ __forceinline__ void unit_draw(const uint4 (&R)[3], uint32_t w, uint32_t& hw) {
-  const uint32_t word = word_of(R[H], Q >> 1);
-  const uint32_t x = (Q & 1) ? (SAT ? (word & 0xFFFF0000u) : word) : (word << 16);
-  or_if_below<(1u << ((NIB ? 4 * Q : 8 * (Q & 3)) + H))>(hw, x, w);
-}
-
-// Chain Q of the octet: its record (free energy, thresholds of units 0..2)
-// and its three draws.
-template <bool SAT, bool NIB, int Q>
-__device__ __forceinline__ void chain_draws(uint32_t addr_bytes, uint32_t rb, const uint4 (&R)[3],
-                                            float& fe, uint32_t& hw) {
-  const uint4 r = lds128(__byte_perm(addr_bytes, rb, 0x7650u | (Q & 3)));
-  fe += __uint_as_float(r.x);
-  unit_draw<SAT, NIB, Q, 0>(R, r.y, hw);
-  unit_draw<SAT, NIB, Q, 1>(R, r.z, hw);
-  unit_draw<SAT, NIB, Q, 2>(R, r.w, hw);
-}
-
-// The octet's hidden pattern: with NIB all 8 chains in h_lo, 4 bits each;
-// else chains 0..3 in the bytes of h_lo and 4..7 in those of h_hi.
-template <bool SAT, bool NIB>
-__device__ __forceinline__ void octet_draws(uint32_t a_lo, uint32_t a_hi, uint32_t rb,
-                                            const uint4 (&R)[3], float (&fe)[8], uint32_t& h_lo,
-                                            uint32_t& h_hi) {
-  chain_draws<SAT, NIB, 0>(a_lo, rb, R, fe[0], h_lo);
-  chain_draws<SAT, NIB, 1>(a_lo, rb, R, fe[1], h_lo);
-  chain_draws<SAT, NIB, 2>(a_lo, rb, R, fe[2], h_lo);
-  chain_draws<SAT, NIB, 3>(a_lo, rb, R, fe[3], h_lo);
-  chain_draws<SAT, NIB, 4>(a_hi, rb, R, fe[4], NIB ? h_lo : h_hi);
-  chain_draws<SAT, NIB, 5>(a_hi, rb, R, fe[5], NIB ? h_lo : h_hi);
-  chain_draws<SAT, NIB, 6>(a_hi, rb, R, fe[6], NIB ? h_lo : h_hi);
-  chain_draws<SAT, NIB, 7>(a_hi, rb, R, fe[7], NIB ? h_lo : h_hi);
 }
 
 // Where a thread's 8 chains read their records: the block of group 0 at the
@@ -544,18 +488,7 @@ __device__ __forceinline__ void gather3_clauses(const DevFormula& F, const DevCh
   const RoundKeys& K = C.keys;
   const uint32_t octet = (uint32_t)(g8 + C.g8_off);
   const uint32_t phase = kPhaseHidden | ((uint32_t)inst << 8);
-  // round 0, word z = t: common to every unit and clause
-  const uint64_t pt = (uint64_t)kPhiloxM1 * t;
-  const uint32_t u1 = (uint32_t)(pt >> 32) ^ K.k0[0];
-  const uint32_t u2 = (uint32_t)pt;
-  // round 1, word x = round 0's (octet | h << 24) ^ u1: per thread and unit
-  uint32_t th[3], sh[3];
-#pragma unroll
-  for (int h = 0; h < 3; ++h) {
-    const uint64_t p = (uint64_t)kPhiloxM0 * ((octet | ((uint32_t)h << 24)) ^ u1);
-    th[h] = (uint32_t)(p >> 32) ^ K.k1[1];
-    sh[h] = (uint32_t)p;
-  }
+  const HiddenThread Q = hidden_thread(octet, t, K);
   const uint8_t* xtb = C.xt + b0;
   uint8_t* hb = static_cast<uint8_t*>(C.H) + (NIB ? b0 / 2 : b0);
   const int hstride = NIB ? Bp / 2 : Bp;
@@ -614,24 +547,8 @@ __device__ __forceinline__ void gather3_clauses(const DevFormula& F, const DevCh
 
     const uint32_t rb = G.tab_e + grp * G.gstride;
     const bool sat = !PLAIN3 && ((cinfo >> 5) & 1u) != 0;
-    // Philox rounds 0..2: the clause's share, then each unit's
-    const uint32_t cl = (uint32_t)(c - cl_base);
-    const uint64_t p0 = (uint64_t)kPhiloxM0 * cl;
-    const uint32_t c1 = (uint32_t)(p0 >> 32) ^ phase ^ K.k1[0];
-    const uint32_t c2 = (uint32_t)p0;
-    const uint64_t p1 = (uint64_t)kPhiloxM1 * c1;
-    const uint32_t c3 = (uint32_t)(p1 >> 32) ^ u2 ^ K.k0[1];
-    const uint32_t c4 = (uint32_t)p1;
-    const uint64_t p2 = (uint64_t)kPhiloxM0 * c3;
-    const uint32_t c5 = (uint32_t)(p2 >> 32) ^ K.k1[2];
-    const uint32_t c6 = (uint32_t)p2;
     uint4 R[3];
-#pragma unroll
-    for (int h = 0; h < 3; ++h) {
-      const uint64_t pz = (uint64_t)kPhiloxM1 * (th[h] ^ c2);
-      R[h] = philox_rounds<3>(
-          make_uint4((uint32_t)(pz >> 32) ^ c4 ^ K.k0[2], (uint32_t)pz, c5 ^ sh[h], c6), K);
-    }
+    hidden_blocks3(Q, (uint32_t)(c - cl_base), phase, K, R);
     uint32_t h_lo = 0, h_hi = 0;
     if (!sat)
       octet_draws<false, NIB>((lo << 4) | G.up_lo, (hi << 4) | G.up_hi, rb, R, fe, h_lo, h_hi);
@@ -791,7 +708,7 @@ __device__ __forceinline__ void gather3_block(const DevFormula& F, const DevTabl
 }
 
 template <bool PLAIN3, bool COST16, bool NIB>
-__global__ void __launch_bounds__(256, 2) k_gather3(DevFormula F, DevTables T, DevChains C,
+__global__ void __launch_bounds__(256, 3) k_gather3(DevFormula F, DevTables T, DevChains C,
                                                     GatherPlan P, const uint32_t* tdev,
                                                     uint32_t t_rel, int64_t* cost_part,
                                                     float* fe_part, int32_t* tickets) {
@@ -977,24 +894,10 @@ __global__ void __launch_bounds__(256, 2) k_gather_nib(DevFormula F, DevTables T
         for (int q = 1; q < 8; ++q)
           if (q >= split) A.off[q] += estride;
       }
-      // Philox rounds 0..2: the clause's share
-      const uint32_t cl = (uint32_t)(c - cl_base);
-      const uint64_t p0 = (uint64_t)kPhiloxM0 * cl;
-      const uint32_t c1 = (uint32_t)(p0 >> 32) ^ phase ^ K.k1[0];
-      const uint32_t c2 = (uint32_t)p0;
-      const uint64_t p1 = (uint64_t)kPhiloxM1 * c1;
-      const uint32_t c3 = (uint32_t)(p1 >> 32) ^ u2 ^ K.k0[1];
-      const uint32_t c4 = (uint32_t)p1;
-      const uint64_t p2 = (uint64_t)kPhiloxM0 * c3;
-      const uint32_t c5 = (uint32_t)(p2 >> 32) ^ K.k1[2];
-      const uint32_t c6 = (uint32_t)p2;
+      const HiddenClause hc = hidden_clause(u2, (uint32_t)(c - cl_base), phase, K);
       auto unit_block = [&](int unit) {
         const uint64_t px = (uint64_t)kPhiloxM0 * ((octet | ((uint32_t)unit << 24)) ^ u1);
-        const uint64_t pz =
-            (uint64_t)kPhiloxM1 * ((uint32_t)(px >> 32) ^ K.k1[1] ^ c2);
-        return philox_rounds<3>(make_uint4((uint32_t)(pz >> 32) ^ c4 ^ K.k0[2], (uint32_t)pz,
-                                           c5 ^ (uint32_t)px, c6),
-                                K);
+        return hidden_unit(hc, (uint32_t)(px >> 32) ^ K.k1[1], (uint32_t)px, K);
       };
       uint32_t* Hc = H + (size_t)rec.z * hstride;
       for (int j = 0; j < chunks; ++j, Hc += hstride) {
@@ -1232,9 +1135,13 @@ __global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4) k_visible(DevFormula 
 // incidences stays below 2^16 (the host takes this kernel only for
 // |2^Q G| <= 1023), then the sums move to 32 bits.
 //
-// The blocks are resident (4 per SM) and each warp walks variables: the tables
-// are staged once per block instead of once per 8 variables, and the next
-// variable's record and incidences are loaded while the current one is summed.
+// The blocks are resident and each warp walks variables: the tables are staged
+// once per block instead of once per 8 variables, and the pattern rows of the
+// next variable are copied into shared memory (cp.async, 16 bytes: four rows of
+// the tile per warp instruction) while the current one is summed. Loads of the
+// patterns into registers, 4 or 8 at a time, left the kernel waiting on the L2
+// (long scoreboard 11.7 of 18 cycles per issue, 27 us a launch at n = 1000, m =
+// 6000, 4096 chains; 200 us at mixed lengths, n = 20000, m = 100000, 1024 chains).
 // ---------------------------------------------------------------------------
 struct VisPos {  // position in the walk over (chain tile, variable slot)
   int fast, slow;
@@ -1248,66 +1155,6 @@ __device__ __forceinline__ VisPos vis_next(VisPos p, int dfast, int dslow, int n
     ++p.slow;
   }
   return p;
-}
-
-// the contributions of four chains (selector s, low 16 bits) as pairs
-__device__ __forceinline__ void nib_pairs(const uint4& tb, uint32_t s, uint32_t& p01,
-                                          uint32_t& p23) {
-  const uint32_t lo = __byte_perm(tb.x, tb.y, s), hi = __byte_perm(tb.z, tb.w, s);
-  p01 = __byte_perm(lo, hi, 0x5140u);
-  p23 = __byte_perm(lo, hi, 0x7362u);
-}
-
-// adds the contributions of the octet's 8 chains (pattern word h)
-__device__ __forceinline__ void nib_add(const uint4& tb, uint32_t h, uint32_t (&acc)[4]) {
-  uint32_t a, b;
-  nib_pairs(tb, h, a, b);
-  acc[0] += a;
-  acc[1] += b;
-  nib_pairs(tb, h >> 16, a, b);
-  acc[2] += a;
-  acc[3] += b;
-}
-
-// as nib_add for an octet across two temperatures: table ta, and tb for the
-// chains of mask mk (one 16-bit half per chain)
-__device__ __forceinline__ void nib_add2(const uint4& ta, const uint4& tb, uint32_t h,
-                                         const uint32_t (&mk)[4], uint32_t (&acc)[4]) {
-#pragma unroll
-  for (int w = 0; w < 4; w += 2) {
-    uint32_t a, b, a1, b1;
-    nib_pairs(ta, w ? h >> 16 : h, a, b);
-    nib_pairs(tb, w ? h >> 16 : h, a1, b1);
-    acc[w] += (a & ~mk[w]) | (a1 & mk[w]);
-    acc[w + 1] += (b & ~mk[w + 1]) | (b1 & mk[w + 1]);
-  }
-}
-
-// the masks of the chains from `split` on
-__device__ __forceinline__ void nib_masks(int split, uint32_t (&mk)[4]) {
-#pragma unroll
-  for (int w = 0; w < 4; ++w)
-    mk[w] = (2 * w >= split ? 0x0000FFFFu : 0u) | (2 * w + 1 >= split ? 0xFFFF0000u : 0u);
-}
-
-// the octet's temperatures: tab at the first chain's; returns the first chain
-// of the next temperature (8: none; octets have at most two)
-__device__ __forceinline__ int nib_split(const DevTables& T, const DevChains& C, int b0,
-                                         uint32_t tab0, uint32_t& tab) {
-  const int gb0 = C.g8_off * 8 + b0;
-  const int e0 = temp_of(gb0, T.n_temps, C.B_total, C.inv_B_total);
-  tab = tab0 + (uint32_t)(e0 * T.ptab_stride);
-  if (e0 == temp_of(gb0 + 7, T.n_temps, C.B_total, C.inv_B_total)) return 8;
-  return (int)(((long long)(e0 + 1) * C.B_total + T.n_temps - 1) / T.n_temps) - gb0;
-}
-
-// moves a window's sums (with cw biases) to 32 bits
-__device__ __forceinline__ void nib_flush(const uint32_t (&acc)[4], int bias, int (&z)[8]) {
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    z[2 * w] += (int)(acc[w] & 0xFFFFu) - bias;
-    z[2 * w + 1] += (int)(acc[w] >> 16) - bias;
-  }
 }
 
 // The end of a visible update, as visible_tail: best-so-far of the chains
@@ -1346,24 +1193,28 @@ __host__ __device__ __forceinline__ int nib_rows_bytes(const DevTables& T) {
   return T.n_temps * T.ptab_stride;
 }
 
-template <int BATCH>
-__global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4)
+// W: incidences per window (a multiple of 4); a warp has two buffers of W rows
+template <int W, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS)
     k_visible_nib(DevFormula F, DevTables T, DevChains C, float keep, const uint32_t* tdev,
                   uint32_t t_rel, int tile_major) {
-  static_assert(32 % BATCH == 0, "incidence windows hold whole batches");
+  static_assert(W % 4 == 0 && W <= 32, "windows are whole groups of four rows");
+  constexpr int kBuf = W * 128;
   pdl_release();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int2 s_inc[8][32];  // per warp: a window of its variable's incidences
+  __shared__ __align__(16) uint32_t s_off[8][2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rows = nib_rows_bytes(T);
-  stage(smem, T.ptab, rows);
-  stage(smem + rows, T.pva, align16(T.pv_len * 8));
+  const int pva_at = nib_rows_bytes(T), buf_at = pva_at + align16(T.pv_len * 8);
+  stage(smem, T.ptab, pva_at);
+  stage(smem + pva_at, T.pva, align16(T.pv_len * 8));
   __syncthreads();
   const uint32_t tab0 = (uint32_t)__cvta_generic_to_shared(smem);
-  const uint2* pva = reinterpret_cast<const uint2*>(smem + rows);
+  const uint2* pva = reinterpret_cast<const uint2*>(smem + pva_at);
+  const uint32_t rows_s = tab0 + (uint32_t)(buf_at + warp * 2 * kBuf);
+  const uint32_t off_s = (uint32_t)__cvta_generic_to_shared(&s_off[warp][0][0]);
   const int tiles = C.Bp / kChainTile;
   // tile_major: every variable of one chain tile before the next tile (its
-  // patterns, m x 128 bytes, then stay in the L2)
+  // patterns, 128 bytes a row, then stay in the L2)
   const int nfast = tile_major ? F.n : tiles, nslow = tile_major ? tiles : F.n;
   const int stride = (int)gridDim.x * 8;
   const int dslow = stride / nfast, dfast = stride - dslow * nfast;
@@ -1373,92 +1224,118 @@ __global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4)
     p.slow = first / nfast;
     p.fast = first - p.slow * nfast;
   }
-  auto slot_of = [&](const VisPos& q) { return tile_major ? q.fast : q.slow; };
   auto load_slot = [&](const VisPos& q) {
-    return q.slow < nslow ? __ldg(F.var_slot + slot_of(q)) : make_int4(0, 0, 0, 0);
+    return q.slow < nslow ? __ldg(F.var_slot + (tile_major ? q.fast : q.slow))
+                          : make_int4(0, 0, 0, 0);
   };
-  // a window of up to 32 incidences; the padding reads clause 0 and the zero row
+  auto tile_of = [&](const VisPos& q) { return tile_major ? q.slow : q.fast; };
+  // up to W incidences; the padding reads the zero row
   auto load_inc = [&](int j0, int cnt) {
-    return lane < cnt ? __ldg(F.var_inc8 + j0 + lane) : make_int2(0, 0);
+    return lane < min(cnt, W) ? __ldg(F.var_inc8 + j0 + lane) : make_int2(0, 0);
   };
-  int4 rec = load_slot(p);
-  VisPos p1 = vis_next(p, dfast, dslow, nfast);
-  int4 rec1 = load_slot(p1);
-  int2 win = load_inc(rec.y, rec.z);
+  const size_t hstride = (size_t)(C.Bp / 8);
+  const uint32_t* H = static_cast<const uint32_t*>(C.H) + (lane & 7) * 4;
+  auto copy = [&](const int2& w, int cnt, int tile, int buf) {
+    nib_copy_rows(w, min(cnt, W), H + tile * 32, hstride, rows_s + (uint32_t)(buf * kBuf),
+                  s_off[warp][buf], lane);
+  };
+  uint64_t xold = 0, imp = 0;
+  int local = 0;  // the variable's index within its formula
+  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+  auto load_state = [&](const int4& r, int tile, uint64_t& x, uint64_t& im, int& lo, float4& a,
+                        float4& c) {
+    const size_t o = (size_t)r.x * C.Bp + tile * kChainTile + lane * 8;
+    im = *reinterpret_cast<const unsigned long long*>(C.improved + (size_t)r.w * C.Bp +
+                                                      tile * kChainTile + lane * 8);
+    lo = F.var_inst ? __ldg(F.var_inst + r.x).y : r.x;
+    x = *reinterpret_cast<const uint64_t*>(C.xt + o);
+    a = reinterpret_cast<const float4*>(C.nu + o)[0];
+    c = reinterpret_cast<const float4*>(C.nu + o)[1];
+  };
+  // The walk goes window by window (a variable with cnt incidences has
+  // max(1, ceil(cnt / W)) windows): A is summed, B's rows are on their way, C's
+  // incidences are in registers, and the record of the variable after C's is
+  // loaded.
+  struct Window {
+    int4 rec;  // .z < 0: none
+    int tile, j;
+  };
+  VisPos pn = p;  // the variable after the last window's
+  int4 recn = load_slot(pn);
+  auto start = [&]() {  // the first window of the variable at pn
+    Window w;
+    w.rec = recn;
+    w.tile = tile_of(pn);
+    w.j = 0;
+    if (pn.slow >= nslow) w.rec.z = -1;  // past the end
+    pn = vis_next(pn, dfast, dslow, nfast);
+    recn = load_slot(pn);
+    return w;
+  };
+  auto after = [&](const Window& w) {
+    if (w.j + W < w.rec.z) {
+      Window v = w;
+      v.j += W;
+      return v;
+    }
+    return start();
+  };
+  auto win_of = [&](const Window& w) { return load_inc(w.rec.y + w.j, w.rec.z - w.j); };
+  Window A = start();
+  const int2 winA = win_of(A);
+  Window Bw = after(A);
+  int2 winB = win_of(Bw);
   pdl_wait();  // chain state from here on
   const uint32_t t = step_index(tdev, t_rel);
-  int last_tile = -1, split = 8;
+  int last_tile = -1, split = 8, vb = 0;
   uint32_t tab = tab0;
   bool two = false;
-  const size_t hstride = (size_t)(C.Bp / 8);
-
-  while (p.slow < nslow) {
-    const int tile = tile_major ? p.slow : p.fast;
-    const int g8 = tile * 32 + lane, b0 = g8 * 8;
-    __syncwarp();
-    s_inc[warp][lane] = win;
-    __syncwarp();
-    // this item's state and the next item's incidences go out first
-    const int i = rec.x, cnt = rec.z;
-    const size_t o = (size_t)i * C.Bp + b0;
-    const uint64_t xold = *reinterpret_cast<const uint64_t*>(C.xt + o);
-    const float4 n0 = reinterpret_cast<const float4*>(C.nu + o)[0];
-    const float4 n1 = reinterpret_cast<const float4*>(C.nu + o)[1];
-    const int local = F.var_inst ? __ldg(F.var_inst + i).y : i;
-    const VisPos p2 = vis_next(p1, dfast, dslow, nfast);
-    const int4 rec2 = load_slot(p2);
-    win = load_inc(rec1.y, rec1.z);
-    if (tile != last_tile) {
-      last_tile = tile;
-      split = nib_split(T, C, b0, tab0, tab);
+  if (A.rec.z >= 0) {
+    copy(winA, A.rec.z, A.tile, 0);
+    load_state(A.rec, A.tile, xold, imp, local, n0, n1);
+  }
+  int z[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) z[q] = 0;
+  while (A.rec.z >= 0) {
+    uint64_t x1 = 0, imp1 = 0;
+    int local1 = 0;
+    float4 m0 = n0, m1 = n1;
+    __syncwarp();  // the other buffer's readers are done
+    if (Bw.rec.z >= 0) {
+      copy(winB, Bw.rec.z - Bw.j, Bw.tile, vb ^ 1);
+      if (Bw.j == 0) load_state(Bw.rec, Bw.tile, x1, imp1, local1, m0, m1);
+    }
+    const Window Cw = after(Bw);
+    winB = win_of(Cw);
+    const int g8 = A.tile * 32 + lane;
+    if (A.tile != last_tile) {
+      last_tile = A.tile;
+      split = nib_split(T, C, g8 * 8, tab0, tab);
       two = __any_sync(0xFFFFFFFFu, split < 8);
     }
-    const uint32_t* H = static_cast<const uint32_t*>(C.H) + g8;
-    int z[8];
+    if (Bw.rec.z >= 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    const int cw = min(A.rec.z - A.j, W);
+    uint32_t acc[4] = {0u, 0u, 0u, 0u};
+    nib_sum_rows(tab, split < 8 ? tab + (uint32_t)T.ptab_stride : tab, two, split,
+                 off_s + (uint32_t)vb * 128u, rows_s + (uint32_t)(vb * kBuf + lane * 4), cw, acc);
+    nib_flush(acc, cw * T.ptab_bias, z);
+    if (A.j + W >= A.rec.z) {  // the variable's last window
+      nib_tail(T, C, pva, keep, t, A.rec.w, local, g8, (size_t)A.rec.x * C.Bp + g8 * 8, xold, imp,
+               n0, n1, z);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) z[q] = 0;
-    for (int j = 0; j < cnt; j += 32) {
-      if (j > 0) {
-        const int2 w = load_inc(rec.y + j, cnt - j);
-        __syncwarp();
-        s_inc[warp][lane] = w;
-        __syncwarp();
-      }
-      const int cw = min(cnt - j, 32);
-      uint32_t acc[4] = {0u, 0u, 0u, 0u};
-      if (!two) {
-#pragma unroll 1
-        for (int k = 0; k < cw; k += BATCH) {
-          uint32_t h[BATCH];
-#pragma unroll
-          for (int u = 0; u < BATCH; ++u) h[u] = __ldg(H + (size_t)s_inc[warp][k + u].x * hstride);
-#pragma unroll
-          for (int u = 0; u < BATCH; ++u) {
-            nib_add(lds128(tab + (uint32_t)s_inc[warp][k + u].y), h[u], acc);
-          }
-        }
-      } else {
-        // some octet of the warp lies across two temperatures: both tables,
-        // the upper one for the chains from `split` on
-        uint32_t mk[4];
-        nib_masks(split, mk);
-        const uint32_t tab1 = split < 8 ? tab + (uint32_t)T.ptab_stride : tab;
-#pragma unroll 1
-        for (int k = 0; k < cw; ++k) {
-          const int2 inc = s_inc[warp][k];
-          nib_add2(lds128(tab + (uint32_t)inc.y), lds128(tab1 + (uint32_t)inc.y),
-                   __ldg(H + (size_t)inc.x * hstride), mk, acc);
-        }
-      }
-      nib_flush(acc, cw * T.ptab_bias, z);
+      for (int q = 0; q < 8; ++q) z[q] = 0;
+      xold = x1;
+      imp = imp1;
+      local = local1;
+      n0 = m0;
+      n1 = m1;
     }
-    const uint64_t imp = *reinterpret_cast<const unsigned long long*>(
-        C.improved + (size_t)rec.w * C.Bp + b0);
-    nib_tail(T, C, pva, keep, t, rec.w, local, g8, o, xold, imp, n0, n1, z);
-    p = p1;
-    p1 = p2;
-    rec = rec1;
-    rec1 = rec2;
+    A = Bw;
+    Bw = Cw;
+    vb ^= 1;
   }
 }
 
@@ -1506,6 +1383,12 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
   return v;
 }
 
+__device__ __forceinline__ uint32_t ld_relaxed_gpu(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // Barrier of a tile's blocks in two halves. bar counts arrivals and is never
 // cleared; target is the count at which every block of this phase has arrived.
 __device__ __forceinline__ void tile_arrive(uint32_t* bar) {
@@ -1516,12 +1399,14 @@ __device__ __forceinline__ void tile_arrive(uint32_t* bar) {
   }
 }
 
+// (polls with relaxed loads, one fence at the end: an acquire per poll would
+// drop the SM's L1 under the block that is still computing)
 __device__ __forceinline__ bool tile_wait(const uint32_t* bar, uint32_t target, int* err,
                                           int* s_go) {
   if (threadIdx.x == 0) {
     int go = 1;
     const long long t0 = clock64();
-    while ((int32_t)(ld_acquire_gpu(bar) - target) < 0) {
+    while ((int32_t)(ld_relaxed_gpu(bar) - target) < 0) {
       if (clock64() - t0 > kBarrierWaitCycles) {
         atomicCAS(err, 0, kErrGridBarrier);
         go = 0;
@@ -1535,15 +1420,13 @@ __device__ __forceinline__ bool tile_wait(const uint32_t* bar, uint32_t target, 
   return *s_go != 0;
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-
-// bytes of pattern rows per warp: two buffers of 32 rows of 128 bytes
-constexpr int kRowBuf = 32 * 128;
+// incidences per window, and the bytes of its pattern rows (two buffers per
+// warp): 28 rows leave room for three blocks per SM
+constexpr int kRowWin = 28;
+constexpr int kRowBuf = kRowWin * 128;
 
 template <bool PLAIN3, bool COST16>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 3)
     k_rounds(DevFormula F, DevTables T, DevChains C, RoundsArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int64_t s_best[256];
@@ -1568,8 +1451,8 @@ __global__ void __launch_bounds__(256, 2)
   const uint2* pva = reinterpret_cast<const uint2*>(smem + pva_at);
   int32_t* s_cost = reinterpret_cast<int32_t*>(smem + buf_at);       // [8][256]
   float* s_fe = reinterpret_cast<float*>(smem + buf_at) + 8 * 256;   // [8][256]
-  const uint32_t* rows = reinterpret_cast<const uint32_t*>(smem + buf_at) + warp * (2 * kRowBuf / 4);
   const uint32_t rows_s = s0 + (uint32_t)(buf_at + warp * 2 * kRowBuf);
+  const uint32_t off_s = (uint32_t)__cvta_generic_to_shared(&s_off[warp][0][0]);
   s_best[tid] = C.best[b];
   const G3Tables G = gather3_tables(T, C, rec_tab, b0);
   uint32_t tab;
@@ -1591,22 +1474,12 @@ __global__ void __launch_bounds__(256, 2)
   auto load_slot = [&](int slot) {
     return slot < F.n ? __ldg(F.var_slot + slot) : make_int4(0, 0, 0, 0);
   };
-  // up to 32 incidences; the padding reads the zero row
+  // up to kRowWin incidences; the padding reads the zero row
   auto load_inc = [&](int j0, int cnt) {
-    return lane < cnt ? __ldg(F.var_inc8 + j0 + lane) : make_int2(0, 0);
+    return lane < min(cnt, kRowWin) ? __ldg(F.var_inc8 + j0 + lane) : make_int2(0, 0);
   };
-  // copies the pattern rows of a window into buffer `buf`: lane / 8 picks one
-  // of four rows, lane % 8 its 16 bytes
   auto copy_rows = [&](const int2& win, int cnt, int buf) {
-    s_off[warp][buf][lane] = (uint32_t)win.y;
-    for (int u = 0; u < cnt; u += 4) {
-      const int row = u + (lane >> 3);
-      const int c = __shfl_sync(0xFFFFFFFFu, win.x, row & 31);
-      if (row < cnt)
-        cp_async16(rows_s + (uint32_t)(buf * kRowBuf + row * 128 + (lane & 7) * 16),
-                   H + (size_t)c * hstride);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+    nib_copy_rows(win, cnt, H, hstride, rows_s + (uint32_t)(buf * kRowBuf), s_off[warp][buf], lane);
   };
   __syncthreads();
 
@@ -1675,7 +1548,7 @@ __global__ void __launch_bounds__(256, 2)
       c = __ldcg(reinterpret_cast<const float4*>(C.nu + o) + 1);
     };
     if (first < F.n) {
-      copy_rows(win0, min(rec.z, 32), 0);
+      copy_rows(win0, min(rec.z, kRowWin), 0);
       load_state(rec.x, xold, n0, n1);
     }
     __syncthreads();  // s_imp
@@ -1687,7 +1560,7 @@ __global__ void __launch_bounds__(256, 2)
       float4 m0 = n0, m1 = n1;
       __syncwarp();  // the other buffer's readers are done
       if (more) {
-        copy_rows(win1, min(rec1.z, 32), vb ^ 1);
+        copy_rows(win1, min(rec1.z, kRowWin), vb ^ 1);
         load_state(rec1.x, x1, m0, m1);
       }
       win1 = load_inc(rec2.y, rec2.z);
@@ -1699,39 +1572,19 @@ __global__ void __launch_bounds__(256, 2)
       int z[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) z[q] = 0;
-      for (int j = 0; j < cnt; j += 32) {
-        if (j > 0) {  // a further window of a variable in more than 32 clauses
+      for (int j = 0; j < cnt; j += kRowWin) {
+        if (j > 0) {  // a further window
           const int2 w = load_inc(rec.y + j, cnt - j);
           __syncwarp();
-          copy_rows(w, min(cnt - j, 32), vb);
+          copy_rows(w, min(cnt - j, kRowWin), vb);
           asm volatile("cp.async.wait_group 0;" ::: "memory");
           __syncwarp();
         }
-        const int cw = min(cnt - j, 32);
+        const int cw = min(cnt - j, kRowWin);
         uint32_t acc[4] = {0u, 0u, 0u, 0u};
-        const uint32_t* hr = rows + vb * (kRowBuf / 4) + lane;
-        if (!two) {
-#pragma unroll 1
-          for (int k = 0; k < cw; k += 4) {
-            const uint4 of = *reinterpret_cast<const uint4*>(&s_off[warp][vb][k]);
-            uint32_t h[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) h[u] = hr[(k + u) * 32];
-            nib_add(lds128(tab + of.x), h[0], acc);
-            nib_add(lds128(tab + of.y), h[1], acc);
-            nib_add(lds128(tab + of.z), h[2], acc);
-            nib_add(lds128(tab + of.w), h[3], acc);
-          }
-        } else {
-          uint32_t mk[4];
-          nib_masks(split, mk);
-          const uint32_t tab1 = split < 8 ? tab + (uint32_t)T.ptab_stride : tab;
-#pragma unroll 1
-          for (int k = 0; k < cw; ++k) {
-            const uint32_t of = s_off[warp][vb][k];
-            nib_add2(lds128(tab + of), lds128(tab1 + of), hr[k * 32], mk, acc);
-          }
-        }
+        nib_sum_rows(tab, split < 8 ? tab + (uint32_t)T.ptab_stride : tab, two, split,
+                     off_s + (uint32_t)vb * 128u, rows_s + (uint32_t)(vb * kRowBuf + lane * 4), cw,
+                     acc);
         nib_flush(acc, cw * T.ptab_bias, z);
       }
       nib_tail(T, C, pva, A.keep, t, 0, rec.x, g8, (size_t)rec.x * C.Bp + b0, xold, flags, n0, n1,
@@ -1869,7 +1722,7 @@ int visible_smem_bytes(const DevTables& T) {
 }
 
 constexpr int kSmemLimit = 160 * 1024;
-constexpr int kNibSmemLimit = 96 * 1024;
+constexpr int kNibSmemLimit = 76 * 1024;  // with windows of 16 rows two blocks fit an SM
 int l2_bytes();
 constexpr int kMaxGridY = 65535;
 
@@ -2050,23 +1903,30 @@ int sm_count() {
 
 int nib_smem_bytes(const DevTables& T) { return nib_rows_bytes(T) + align16(T.pv_len * 8); }
 
-cudaError_t visible_nib(const DevFormula& F, const DevTables& T, const DevChains& C, float alpha,
-                        const uint32_t* tdev, uint32_t t_rel, int batch, cudaStream_t st) {
-  auto kern = batch >= 8 ? k_visible_nib<8> : batch <= 2 ? k_visible_nib<2> : k_visible_nib<4>;
-  const int smem = nib_smem_bytes(T);
+template <int W, int BLOCKS>
+cudaError_t visible_nib_window(const DevFormula& F, const DevTables& T, const DevChains& C,
+                               float keep, const uint32_t* tdev, uint32_t t_rel, cudaStream_t st) {
+  auto kern = k_visible_nib<W, BLOCKS>;
+  const int smem = nib_smem_bytes(T) + 8 * 2 * W * 128;
   const cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
   const long long items = (long long)F.n * (C.Bp / kChainTile);
-  int per_sm = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem) != cudaSuccess ||
-      per_sm < 1)
-    per_sm = 1;
-  const long long grid = std::min<long long>((items + 7) / 8, (long long)per_sm * sm_count());
+  const long long grid = std::min<long long>((items + 7) / 8, (long long)BLOCKS * sm_count());
   const int tm = (double)F.h_rows * C.Bp * 0.5 > 0.5 * (double)l2_bytes() ? 1 : 0;
+  return launch_pdl(kern, dim3((unsigned)grid), smem, st, F, T, C, keep, tdev, t_rel, tm);
+}
+
+cudaError_t visible_nib(const DevFormula& F, const DevTables& T, const DevChains& C, float alpha,
+                        const uint32_t* tdev, uint32_t t_rel, cudaStream_t st) {
   // 1 - alpha as the device's one rounding gives it
   volatile float one = 1.0f;
   const float keep = one - alpha;
-  return launch_pdl(kern, dim3((unsigned)grid), smem, st, F, T, C, keep, tdev, t_rel, tm);
+  // as many blocks per SM as the tables leave room for, then the wider window
+  const int tables = nib_smem_bytes(T) + 3 * 1024;  // with the static part
+  auto fits = [&](int blocks, int W) { return blocks * (tables + 2048 * W) <= 227 * 1024; };
+  if (fits(3, 28)) return visible_nib_window<28, 3>(F, T, C, keep, tdev, t_rel, st);
+  if (fits(2, 28)) return visible_nib_window<28, 2>(F, T, C, keep, tdev, t_rel, st);
+  return visible_nib_window<16, 2>(F, T, C, keep, tdev, t_rel, st);
 }
 
 }  // namespace
@@ -2184,7 +2044,7 @@ cudaError_t launch_gather(GatherMode mode, const DevFormula& F, const DevTables&
 cudaError_t launch_visible(const DevFormula& F, const DevTables& T, const DevChains& C,
                            float alpha, const uint32_t* tdev, uint32_t t_rel, bool wide,
                            cudaStream_t st, int batch) {
-  if (C.nib) return visible_nib(F, T, C, alpha, tdev, t_rel, batch, st);
+  if (C.nib) return visible_nib(F, T, C, alpha, tdev, t_rel, st);
   dim3 grid(C.Bp / kChainTile, (F.n + 7) / 8);
   const int sm = visible_smem_bytes(T);
   const bool use_sm = sm <= kSmemLimit;
@@ -2207,7 +2067,8 @@ int rounds_smem_bytes(const DevTables& T) {
 }  // namespace
 
 // resident blocks of k_rounds on this device (0 when it cannot run)
-int rounds_slots(const DevTables& T) {
+int rounds_slots(const DevTables& T, int* per_sm) {
+  *per_sm = 0;
   if (!T.rec3 || !T.ptab || nib_smem_bytes(T) > kNibSmemLimit) return 0;
   int slots = 1 << 30;
   for (int v = 0; v < 2; ++v) {
@@ -2221,6 +2082,7 @@ int rounds_slots(const DevTables& T) {
     }
     slots = std::min(slots, nb * sm_count());
   }
+  *per_sm = slots / sm_count();
   return slots;
 }
 
