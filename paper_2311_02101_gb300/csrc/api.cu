@@ -2675,9 +2675,9 @@ int mp_forward(maxsat_mp* mp, maxsat_ctx* ctx, const uint8_t* y, float* prob) {
   MPT(mp, ctx, "mp_embed", mp_launch_embed(F, mp->Pb + Y.Wf, mp->Pb + Y.Wg, mp->f, mp->g, mp->inv_len,
                                            mp->inv_deg, mp->hv[0], mp->hc[0], st));
   for (int l = 0; l < L; ++l) {
-    MPT(mp, ctx, "mp_dense_fwd", mp_launch_fwd(F, true, mp->hv[l], mp->inv_len, mp->hc[l], mp->Pb + Y.Wc[l],
+    MPT(mp, ctx, "mp_dense_fwd_clauses", mp_launch_fwd(F, true, mp->hv[l], mp->inv_len, mp->hc[l], mp->Pb + Y.Wc[l],
                                  mp->P + Y.bc[l], y ? mp->mc[l] : nullptr, mp->hc[l + 1], st));
-    MPT(mp, ctx, "mp_dense_fwd", mp_launch_fwd(F, false, mp->hc[l + 1], mp->inv_deg, mp->hv[l], mp->Pb + Y.Wv[l],
+    MPT(mp, ctx, "mp_dense_fwd_vars", mp_launch_fwd(F, false, mp->hc[l + 1], mp->inv_deg, mp->hv[l], mp->Pb + Y.Wv[l],
                                  mp->P + Y.bv[l], y ? mp->av[l] : nullptr, mp->hv[l + 1], st));
   }
   MPT(mp, ctx, "mp_out", mp_launch_out(mp->hv[L], n, mp->P + Y.wo, mp->P + Y.bo, y, prob, y ? mp->dz : nullptr,
@@ -2781,14 +2781,14 @@ int maxsat_mp_gradient(maxsat_mp* mp, maxsat_ctx* ctx, const uint8_t* labels_dev
     // variable layer l: h_v^{l+1} = relu(Wv_l [a_v ; h_v^l] + bv_l); its gradient
     // comes from the read-out at the top, else from layer l + 1: the own rows'
     // (dhv) and, through m_c = (1 / len_c) sum s h_v, the clauses' (dmc)
-    MPT(mp, ctx, "mp_dense_bwd", mp_launch_bwd(F, false, mp->dmc, mp->inv_len, mp->dhv, top ? mp->dz : nullptr,
+    MPT(mp, ctx, "mp_dense_bwd_vars", mp_launch_bwd(F, false, mp->dmc, mp->inv_len, mp->dhv, top ? mp->dz : nullptr,
                                  mp->P + Y.wo, mp->hv[l + 1], mp->av[l], mp->hv[l], mp->Pb + Y.Wv[l],
                                  mp->dav, mp->dhv, part, st));
     sum_later(nbv, width, width, G + Y.Wv[l]);
     // clause layer l: h_c^{l+1} = relu(Wc_l [m_c ; h_c^l] + bc_l), its gradient
     // through a_v = (1 / deg_v) sum s h_c^{l+1} and, below the top, from layer l + 1
     if (m > 0) {
-      MPT(mp, ctx, "mp_dense_bwd", mp_launch_bwd(F, true, mp->dav, mp->inv_deg, top ? nullptr : mp->dhc, nullptr,
+      MPT(mp, ctx, "mp_dense_bwd_clauses", mp_launch_bwd(F, true, mp->dav, mp->inv_deg, top ? nullptr : mp->dhc, nullptr,
                                    nullptr, mp->hc[l + 1], mp->mc[l], mp->hc[l], mp->Pb + Y.Wc[l],
                                    mp->dmc, mp->dhc, part, st));
       sum_later(nbc, width, width, G + Y.Wc[l]);

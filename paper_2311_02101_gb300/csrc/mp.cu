@@ -175,54 +175,103 @@ __device__ __forceinline__ void store_terms(__nv_bfloat16* dst, int tile, float4
   }
 }
 
-// Row r's signed sum over its clause's literals (CL) or its variable's
-// occurrences: sum s * scale[other] * src[other] (scale NULL = 1), in list
-// order, columns 4 c .. 4 c + 3 of the 16 lanes that share the row.
+// A row's list: its clause's literals (CL) or its variable's occurrences. The 16
+// lanes that share the row hold its first 16 entries, one each: the other side's
+// index, bit 31 when negated.
+struct RowList {
+  int j0, cnt;
+  int32_t entry;
+};
+
 template <bool CL>
-__device__ __forceinline__ float4 gather_row(const DevFormula& F, const float* src,
-                                             const float* scale, int r, int c) {
-  const int j0 = CL ? __ldg(F.cl_off + r) : __ldg(F.var_off + r);
-  const int j1 = CL ? __ldg(F.cl_off + r + 1) : __ldg(F.var_off + r + 1);
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int j = j0; j < j1; j += 4) {
-    int o[4];
-    float s[4];
-    float4 x[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      o[u] = -1;
-      if (j + u < j1) {
-        if constexpr (CL) {
-          const int32_t lv = __ldg(F.lit_var + j + u);
-          o[u] = lv & 0x7FFFFFFF;
-          s[u] = lv < 0 ? -1.f : 1.f;
-        } else {
-          const int2 inc = __ldg(reinterpret_cast<const int2*>(F.var_inc + j + u));
-          o[u] = inc.x;
-          s[u] = inc.y < 0 ? -1.f : 1.f;
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (o[u] >= 0) {
-        if (scale) s[u] *= __ldg(scale + o[u]);
-        x[u] = __ldg(reinterpret_cast<const float4*>(src + (size_t)o[u] * kH) + c);
-      }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (o[u] >= 0) {
-        acc.x = fmaf(s[u], x[u].x, acc.x);
-        acc.y = fmaf(s[u], x[u].y, acc.y);
-        acc.z = fmaf(s[u], x[u].z, acc.z);
-        acc.w = fmaf(s[u], x[u].w, acc.w);
-      }
+__device__ __forceinline__ int32_t list_entry(const DevFormula& F, int j) {
+  if constexpr (CL) {
+    return __ldg(F.lit_var + j);
+  } else {
+    const int2 inc = __ldg(reinterpret_cast<const int2*>(F.var_inc + j));
+    return inc.x | (inc.y & (int32_t)0x80000000);
   }
-  return acc;
 }
 
-__device__ __forceinline__ float4 row4(const float* p, size_t r, int c) {
-  return *(reinterpret_cast<const float4*>(p + r * kH) + c);
+// where the lists of the thread's four rows (16 apart from r0) begin and end
+struct RowRanges {
+  int j0[4], j1[4];
+};
+
+template <bool CL>
+__device__ __forceinline__ RowRanges row_ranges(const DevFormula& F, int r0, int rows) {
+  RowRanges R;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int r = r0 + 16 * k;
+    const bool in = r < rows;
+    R.j0[k] = in ? __ldg((CL ? F.cl_off : F.var_off) + r) : 0;
+    R.j1[k] = in ? __ldg((CL ? F.cl_off : F.var_off) + r + 1) : 0;
+  }
+  return R;
+}
+
+template <bool CL>
+__device__ __forceinline__ void row_lists(const DevFormula& F, const RowRanges& R, int c,
+                                          RowList (&L)[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    L[k].j0 = R.j0[k];
+    L[k].cnt = R.j1[k] - R.j0[k];
+    L[k].entry = c < L[k].cnt ? list_entry<CL>(F, R.j0[k] + c) : 0;
+  }
+}
+
+// The signed sums of two rows (16 lanes each, columns 4 c .. 4 c + 3): sum s *
+// scale[other] * src[other] in list order (scale NULL = 1). Four entries of both
+// rows are loaded together.
+template <bool CL>
+__device__ __forceinline__ void gather_pair(const DevFormula& F, const float* src,
+                                            const float* scale, const RowList& L0,
+                                            const RowList& L1, int c, float4 (&acc)[2]) {
+  const unsigned mask = 0xFFFFu << (threadIdx.x & 16);
+  acc[0] = acc[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int most = max(L0.cnt, L1.cnt);
+  int32_t e0 = L0.entry, e1 = L1.entry;
+  for (int base = 0; base < most; base += 16) {
+    if (base > 0) {
+      e0 = base + c < L0.cnt ? list_entry<CL>(F, L0.j0 + base + c) : 0;
+      e1 = base + c < L1.cnt ? list_entry<CL>(F, L1.j0 + base + c) : 0;
+    }
+    const int lim = min(16, most - base);
+    for (int u = 0; u < lim; u += 4) {
+      float s[2][4];
+      float4 x[2][4];
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          const int32_t e = __shfl_sync(mask, q ? e1 : e0, u + v, 16);
+          s[q][v] = 0.f;
+          x[q][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (base + u + v < (q ? L1.cnt : L0.cnt)) {
+            const int o = e & 0x7FFFFFFF;
+            s[q][v] = e < 0 ? -1.f : 1.f;
+            if (scale) s[q][v] *= __ldg(scale + o);
+            x[q][v] = __ldg(reinterpret_cast<const float4*>(src + (size_t)o * kH) + c);
+          }
+        }
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+          acc[q].x = fmaf(s[q][v], x[q][v].x, acc[q].x);
+          acc[q].y = fmaf(s[q][v], x[q][v].y, acc[q].y);
+          acc[q].z = fmaf(s[q][v], x[q][v].z, acc[q].z);
+          acc[q].w = fmaf(s[q][v], x[q][v].w, acc[q].w);
+        }
+    }
+  }
+}
+
+__device__ __forceinline__ float4 row4(const float* p, int r, bool in, int c) {
+  return in ? *(reinterpret_cast<const float4*>(p + (size_t)r * kH) + c)
+            : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // the layer's BF16 weights (64 x 128) as rows of kLdX
@@ -233,81 +282,96 @@ __device__ __forceinline__ void stage_weights(__nv_bfloat16* Ws, const __nv_bflo
     *reinterpret_cast<uint32_t*>(Ws + (e >> 6) * kLdX + 2 * (e & 63)) = src[e];
 }
 
+// The layer kernels walk tiles of 64 rows with resident blocks of 8 warps. A
+// tile's rows hang on a chain of three loads (where the lists begin, their
+// entries, the rows those name): the first two are made one and two tiles ahead,
+// in registers, so that only the rows themselves are waited for. (16 warps of
+// which half fetched and half multiplied were slower: 480 us a clause layer's
+// backward pass at 280000 clauses, against 290 with the chain in turn on 16
+// warps that do both.)
 constexpr int kFwdSmem = (3 * kTile + kH) * kLdX * 2;
 
 // out[r] = relu(W [agg ; self[r]] + b), agg = out_scale[r] * signed sum of src;
-// agg also goes to agg_out when given (the backward pass reads it). Resident
-// blocks of 8 warps walk tiles of 64 rows: 16 lanes gather a row (16 bytes
-// each), the three BF16 terms of [agg ; self] are the A operand; a warp
-// multiplies 16 rows x 32 outputs.
+// agg also goes to agg_out when given (the backward pass reads it). The three
+// BF16 terms of [agg ; self] are the A operand; a warp multiplies 16 rows x 32
+// outputs.
 template <bool CL>
 __global__ void __launch_bounds__(256, 3) k_mp_fwd(DevFormula F, const float* src,
                                                    const float* out_scale, const float* self,
                                                    int rows, const __nv_bfloat16* W,
                                                    const float* b, float* agg_out, float* out) {
   extern __shared__ __align__(16) __nv_bfloat16 sm[];
-  __nv_bfloat16* xs = sm;                         // [3][kTile][kLdX]
-  __nv_bfloat16* Ws = sm + 3 * kTile * kLdX;      // [kH][kLdX]
+  __nv_bfloat16* xs = sm;                     // [3][kTile][kLdX]
+  __nv_bfloat16* Ws = sm + 3 * kTile * kLdX;  // [kH][kLdX]
   stage_weights(Ws, W);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int rt = (warp & 3) * 16, ch = (warp >> 2) * 32, g = lane >> 2, t = lane & 3;
   const int hr = tid >> 4, c = tid & 15;  // 16 lanes per row, 16 rows at a time
-  const int tiles = (rows + kTile - 1) / kTile;
-  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const int r0 = tile * kTile;
+  const int tiles = (rows + kTile - 1) / kTile, step = (int)gridDim.x;
+  RowList lists[4];
+  row_lists<CL>(F, row_ranges<CL>(F, (int)blockIdx.x * kTile + hr, rows), c, lists);
+  RowRanges next = row_ranges<CL>(F, ((int)blockIdx.x + step) * kTile + hr, rows);
+  for (int tile = blockIdx.x; tile < tiles; tile += step) {
     __syncthreads();  // weights staged; the previous tile's fragments are read
-    float4 own[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      own[k] = r0 + hr + 16 * k < rows ? row4(self, r0 + hr + 16 * k, c)
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = 0; k < 4; k += 2) {
+      float4 own[2], v[2];
+      float sc[2];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int lr = hr + 16 * k, r = r0 + lr;
-      store_terms<3>(xs + lr * kLdX + kH + 4 * c, kTile * kLdX, own[k]);
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (r < rows) {
-        v = gather_row<CL>(F, src, nullptr, r, c);
-        const float sc = __ldg(out_scale + r);
-        v = make_float4(sc * v.x, sc * v.y, sc * v.z, sc * v.w);
-        if (agg_out) *(reinterpret_cast<float4*>(agg_out + (size_t)r * kH) + c) = v;
+      for (int q = 0; q < 2; ++q) {
+        const int r = tile * kTile + hr + 16 * (k + q);
+        own[q] = row4(self, r, r < rows, c);
+        sc[q] = r < rows ? __ldg(out_scale + r) : 0.f;
       }
-      store_terms<3>(xs + lr * kLdX + 4 * c, kTile * kLdX, v);
+      gather_pair<CL>(F, src, nullptr, lists[k], lists[k + 1], c, v);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int lr = hr + 16 * (k + q), r = tile * kTile + lr;
+        __nv_bfloat16* row = xs + lr * kLdX + 4 * c;
+        v[q] = make_float4(sc[q] * v[q].x, sc[q] * v[q].y, sc[q] * v[q].z, sc[q] * v[q].w);
+        if (agg_out && r < rows) *(reinterpret_cast<float4*>(agg_out + (size_t)r * kH) + c) = v[q];
+        store_terms<3>(row, kTile * kLdX, v[q]);
+        store_terms<3>(row + kH, kTile * kLdX, own[q]);
+      }
     }
+    row_lists<CL>(F, next, c, lists);
+    next = row_ranges<CL>(F, (tile + 2 * step) * kTile + hr, rows);
     __syncthreads();
-    float acc[4][4];
+    {
+      const int rt = (warp & 3) * 16, ch = (warp >> 2) * 32, g = lane >> 2, t = lane & 3;
+      float acc[4][4];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+      for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
+        for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      uint32_t bw[2][4];
+      for (int ks = 0; ks < 8; ++ks) {
+        uint32_t bw[2][4];
 #pragma unroll
-      for (int p = 0; p < 2; ++p)
-        ldm4<false>(bw[p], Ws + (ch + p * 16 + (lane & 7) + ((lane >> 4) << 3)) * kLdX + ks * 16 +
-                               ((lane >> 3) & 1) * 8);
+        for (int p = 0; p < 2; ++p)
+          ldm4<false>(bw[p], Ws + (ch + p * 16 + (lane & 7) + ((lane >> 4) << 3)) * kLdX + ks * 16 +
+                                 ((lane >> 3) & 1) * 8);
 #pragma unroll
-      for (int term = 0; term < 3; ++term) {
-        uint32_t a[4];
-        ldm4<false>(a, xs + (term * kTile + rt + (lane & 15)) * kLdX + ks * 16 + (lane >> 4) * 8);
+        for (int term = 0; term < 3; ++term) {
+          uint32_t a[4];
+          ldm4<false>(a, xs + (term * kTile + rt + (lane & 15)) * kLdX + ks * 16 + (lane >> 4) * 8);
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          mma_bf16(acc[2 * p], a, bw[p][0], bw[p][1]);
-          mma_bf16(acc[2 * p + 1], a, bw[p][2], bw[p][3]);
+          for (int p = 0; p < 2; ++p) {
+            mma_bf16(acc[2 * p], a, bw[p][0], bw[p][1]);
+            mma_bf16(acc[2 * p + 1], a, bw[p][2], bw[p][3]);
+          }
         }
       }
-    }
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-      const int j = ch + nt * 8 + 2 * t, ra = r0 + rt + g, rb = ra + 8;
-      const float b0 = __ldg(b + j), b1 = __ldg(b + j + 1);
-      if (ra < rows)
-        *reinterpret_cast<float2*>(out + (size_t)ra * kH + j) =
-            make_float2(relu(acc[nt][0] + b0), relu(acc[nt][1] + b1));
-      if (rb < rows)
-        *reinterpret_cast<float2*>(out + (size_t)rb * kH + j) =
-            make_float2(relu(acc[nt][2] + b0), relu(acc[nt][3] + b1));
+      for (int nt = 0; nt < 4; ++nt) {
+        const int j = ch + nt * 8 + 2 * t, ra = tile * kTile + rt + g, rb = ra + 8;
+        const float b0 = __ldg(b + j), b1 = __ldg(b + j + 1);
+        if (ra < rows)
+          *reinterpret_cast<float2*>(out + (size_t)ra * kH + j) =
+              make_float2(relu(acc[nt][0] + b0), relu(acc[nt][1] + b1));
+        if (rb < rows)
+          *reinterpret_cast<float2*>(out + (size_t)rb * kH + j) =
+              make_float2(relu(acc[nt][2] + b0), relu(acc[nt][3] + b1));
+      }
     }
   }
 }
@@ -315,11 +379,11 @@ __global__ void __launch_bounds__(256, 3) k_mp_fwd(DevFormula F, const float* sr
 constexpr int kBwdSmem = (3 * kTile * kLdD + (2 * kTile + kH) * kLdX) * 2;
 
 // Gradient of a layer for tiles of 64 rows. The gradient of row r of the
-// layer's output is carry[r] + sum s * in_scale[other] * src[other] (either
-// may be absent), or dz[r] wo at the top; delta is that where out > 0. Then
-// dA / dB = the two halves of delta W, and part[block] = this block's sums of
-// delta^T [agg ; self] (64 x 128) and delta (64). carry and dB may be the same
-// array (a tile's rows are read before they are written).
+// layer's output is carry[r] + sum s * in_scale[other] * src[other] (carry may
+// be absent), or dz[r] wo at the top; delta is that where out > 0. Then dA / dB
+// = the two halves of delta W, and part[block] = this block's sums of delta^T
+// [agg ; self] (64 x 128) and delta (64). carry and dB may be the same array (a
+// tile's rows are read before they are written, and only by their block).
 template <bool CL>
 __global__ void __launch_bounds__(256, 2)
     k_mp_bwd(DevFormula F, const float* src, const float* in_scale, const float* carry,
@@ -327,108 +391,135 @@ __global__ void __launch_bounds__(256, 2)
              const float* self, int rows, const __nv_bfloat16* W, float* dA, float* dB,
              float* part) {
   extern __shared__ __align__(16) __nv_bfloat16 sm[];
-  __nv_bfloat16* ds = sm;                            // [3][kTile][kLdD]
-  __nv_bfloat16* xs = ds + 3 * kTile * kLdD;         // [2][kTile][kLdX]
-  __nv_bfloat16* Ws = xs + 2 * kTile * kLdX;         // [kH][kLdX]
+  __nv_bfloat16* ds = sm;                     // [3][kTile][kLdD]
+  __nv_bfloat16* xs = ds + 3 * kTile * kLdD;  // [2][kTile][kLdX]
+  __nv_bfloat16* Ws = xs + 2 * kTile * kLdX;  // [kH][kLdX]
   stage_weights(Ws, W);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int q4 = warp & 3, half = warp >> 2;
   const int hr = tid >> 4, c = tid & 15;
-  const int tiles = (rows + kTile - 1) / kTile;
+  const int tiles = (rows + kTile - 1) / kTile, step = (int)gridDim.x;
   float wacc[8][4];
 #pragma unroll
   for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
     for (int q = 0; q < 4; ++q) wacc[nt][q] = 0.f;
   float4 bacc = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-    const int r0 = tile * kTile;
+  RowList lists[4];
+  RowRanges next{};
+  if (!dz) {
+    row_lists<CL>(F, row_ranges<CL>(F, (int)blockIdx.x * kTile + hr, rows), c, lists);
+    next = row_ranges<CL>(F, ((int)blockIdx.x + step) * kTile + hr, rows);
+  }
+  for (int tile = blockIdx.x; tile < tiles; tile += step) {
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int lr = hr + 16 * k, r = r0 + lr;
-      float4 d = zero, xa = zero, xb = zero;
-      if (r < rows) {
-        xa = row4(agg, r, c);
-        xb = row4(self, r, c);
-        const float4 o = row4(out, r, c);
-        if (dz) {
-          const float z = __ldg(dz + r);
-          d = make_float4(z * __ldg(wo + 4 * c), z * __ldg(wo + 4 * c + 1),
-                          z * __ldg(wo + 4 * c + 2), z * __ldg(wo + 4 * c + 3));
-        } else {
-          d = gather_row<CL>(F, src, in_scale, r, c);
-          if (carry) {
-            const float4 e = row4(carry, r, c);
-            d = make_float4(d.x + e.x, d.y + e.y, d.z + e.z, d.w + e.w);
-          }
-        }
-        d = make_float4(o.x > 0.f ? d.x : 0.f, o.y > 0.f ? d.y : 0.f, o.z > 0.f ? d.z : 0.f,
-                        o.w > 0.f ? d.w : 0.f);
-        bacc = make_float4(bacc.x + d.x, bacc.y + d.y, bacc.z + d.z, bacc.w + d.w);
+    for (int k = 0; k < 4; k += 2) {
+      float4 e[2], d[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int r = tile * kTile + hr + 16 * (k + q);
+        e[q] = row4(carry, r, r < rows && carry != nullptr && dz == nullptr, c);
       }
-      store_terms<3>(ds + lr * kLdD + 4 * c, kTile * kLdD, d);
-      store_terms<2>(xs + lr * kLdX + 4 * c, kTile * kLdX, xa);
-      store_terms<2>(xs + lr * kLdX + kH + 4 * c, kTile * kLdX, xb);
+      if (dz) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int r = tile * kTile + hr + 16 * (k + q);
+          const float z = r < rows ? __ldg(dz + r) : 0.f;
+          d[q] = make_float4(z * __ldg(wo + 4 * c), z * __ldg(wo + 4 * c + 1),
+                             z * __ldg(wo + 4 * c + 2), z * __ldg(wo + 4 * c + 3));
+        }
+      } else {
+        gather_pair<CL>(F, src, in_scale, lists[k], lists[k + 1], c, d);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+          d[q] = make_float4(d[q].x + e[q].x, d[q].y + e[q].y, d[q].z + e[q].z, d[q].w + e[q].w);
+      }
+      float4 xa[2], xb[2], o[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int r = tile * kTile + hr + 16 * (k + q);
+        xa[q] = row4(agg, r, r < rows, c);
+        xb[q] = row4(self, r, r < rows, c);
+        o[q] = row4(out, r, r < rows, c);
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int lr = hr + 16 * (k + q);
+        d[q] = make_float4(o[q].x > 0.f ? d[q].x : 0.f, o[q].y > 0.f ? d[q].y : 0.f,
+                           o[q].z > 0.f ? d[q].z : 0.f, o[q].w > 0.f ? d[q].w : 0.f);
+        bacc = make_float4(bacc.x + d[q].x, bacc.y + d[q].y, bacc.z + d[q].z, bacc.w + d[q].w);
+        store_terms<3>(ds + lr * kLdD + 4 * c, kTile * kLdD, d[q]);
+        store_terms<2>(xs + lr * kLdX + 4 * c, kTile * kLdX, xa[q]);
+        store_terms<2>(xs + lr * kLdX + kH + 4 * c, kTile * kLdX, xb[q]);
+      }
+    }
+    if (!dz) {
+      row_lists<CL>(F, next, c, lists);
+      next = row_ranges<CL>(F, (tile + 2 * step) * kTile + hr, rows);
     }
     __syncthreads();
-    {  // input gradient: 16 rows x the 64 columns of one half
-      float acc[8][4];
+    {
+      {  // input gradient: 16 rows x the 64 columns of one half
+        float acc[8][4];
 #pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
+        for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
+          for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        uint32_t a[3][4];
+        for (int ks = 0; ks < 4; ++ks) {
+          uint32_t a[3][4];
 #pragma unroll
-        for (int term = 0; term < 3; ++term)
-          ldm4<false>(a[term], ds + (term * kTile + q4 * 16 + (lane & 15)) * kLdD + ks * 16 +
-                                   (lane >> 4) * 8);
+          for (int term = 0; term < 3; ++term)
+            ldm4<false>(a[term], ds + (term * kTile + q4 * 16 + (lane & 15)) * kLdD + ks * 16 +
+                                     (lane >> 4) * 8);
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            uint32_t bw[4];
+            ldm4<true>(bw,
+                       Ws + (ks * 16 + (lane & 15)) * kLdX + half * kH + p * 16 + (lane >> 4) * 8);
+#pragma unroll
+            for (int term = 0; term < 3; ++term) {
+              mma_bf16(acc[2 * p], a[term], bw[0], bw[1]);
+              mma_bf16(acc[2 * p + 1], a[term], bw[2], bw[3]);
+            }
+          }
+        }
+        float* dst = half ? dB : dA;
+        const int ra = tile * kTile + q4 * 16 + g, rb = ra + 8;
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+          const int k = nt * 8 + 2 * t;
+          if (ra < rows)
+            *reinterpret_cast<float2*>(dst + (size_t)ra * kH + k) =
+                make_float2(acc[nt][0], acc[nt][1]);
+          if (rb < rows)
+            *reinterpret_cast<float2*>(dst + (size_t)rb * kH + k) =
+                make_float2(acc[nt][2], acc[nt][3]);
+        }
+      }
+      // weight gradient: outputs 16 q4 .. + 15, inputs of one half, over the rows
+#pragma unroll
+      for (int ks = 0; ks < kTile / 16; ++ks) {
+        uint32_t ah[4], am[4];
+        const __nv_bfloat16* ap = ds + (ks * 16 + (lane & 7) + ((lane >> 4) << 3)) * kLdD + q4 * 16 +
+                                  ((lane >> 3) & 1) * 8;
+        ldm4<true>(ah, ap);
+        ldm4<true>(am, ap + kTile * kLdD);
 #pragma unroll
         for (int p = 0; p < 4; ++p) {
-          uint32_t bw[4];
-          ldm4<true>(bw, Ws + (ks * 16 + (lane & 15)) * kLdX + half * kH + p * 16 + (lane >> 4) * 8);
-#pragma unroll
-          for (int term = 0; term < 3; ++term) {
-            mma_bf16(acc[2 * p], a[term], bw[0], bw[1]);
-            mma_bf16(acc[2 * p + 1], a[term], bw[2], bw[3]);
-          }
+          uint32_t bh[4], bm[4];
+          const __nv_bfloat16* bp =
+              xs + (ks * 16 + (lane & 15)) * kLdX + half * kH + p * 16 + (lane >> 4) * 8;
+          ldm4<true>(bh, bp);
+          ldm4<true>(bm, bp + kTile * kLdX);
+          mma_bf16(wacc[2 * p], ah, bh[0], bh[1]);
+          mma_bf16(wacc[2 * p], ah, bm[0], bm[1]);
+          mma_bf16(wacc[2 * p], am, bh[0], bh[1]);
+          mma_bf16(wacc[2 * p + 1], ah, bh[2], bh[3]);
+          mma_bf16(wacc[2 * p + 1], ah, bm[2], bm[3]);
+          mma_bf16(wacc[2 * p + 1], am, bh[2], bh[3]);
         }
-      }
-      float* dst = half ? dB : dA;
-      const int ra = r0 + q4 * 16 + g, rb = ra + 8;
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt) {
-        const int k = nt * 8 + 2 * t;
-        if (ra < rows)
-          *reinterpret_cast<float2*>(dst + (size_t)ra * kH + k) = make_float2(acc[nt][0], acc[nt][1]);
-        if (rb < rows)
-          *reinterpret_cast<float2*>(dst + (size_t)rb * kH + k) = make_float2(acc[nt][2], acc[nt][3]);
-      }
-    }
-    // weight gradient: outputs 16 q4 .. + 15, inputs of one half, over the rows
-#pragma unroll
-    for (int ks = 0; ks < kTile / 16; ++ks) {
-      uint32_t ah[4], am[4];
-      const __nv_bfloat16* ap =
-          ds + (ks * 16 + (lane & 7) + ((lane >> 4) << 3)) * kLdD + q4 * 16 + ((lane >> 3) & 1) * 8;
-      ldm4<true>(ah, ap);
-      ldm4<true>(am, ap + kTile * kLdD);
-#pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        uint32_t bh[4], bm[4];
-        const __nv_bfloat16* bp =
-            xs + (ks * 16 + (lane & 15)) * kLdX + half * kH + p * 16 + (lane >> 4) * 8;
-        ldm4<true>(bh, bp);
-        ldm4<true>(bm, bp + kTile * kLdX);
-        mma_bf16(wacc[2 * p], ah, bh[0], bh[1]);
-        mma_bf16(wacc[2 * p], ah, bm[0], bm[1]);
-        mma_bf16(wacc[2 * p], am, bh[0], bh[1]);
-        mma_bf16(wacc[2 * p + 1], ah, bh[2], bh[3]);
-        mma_bf16(wacc[2 * p + 1], ah, bm[2], bm[3]);
-        mma_bf16(wacc[2 * p + 1], am, bh[2], bh[3]);
       }
     }
   }
@@ -693,8 +784,9 @@ int mp_sms() {
 }  // namespace
 
 int mp_bwd_blocks(int rows) { return std::max(1, std::min(blocks(rows, kTile), 2 * mp_sms())); }
-int mp_out_blocks(int n) { return std::max(1, std::min(blocks(n, 8), 2 * mp_sms())); }
-int mp_embed_bwd_var_blocks(int n) { return std::max(1, std::min(blocks(n, 32), mp_sms())); }
+int mp_out_blocks(int n) { return std::max(1, std::min(blocks(n, 16), 8 * mp_sms())); }
+// about five variables a warp: each waits on its list, then on its rows
+int mp_embed_bwd_var_blocks(int n) { return std::max(1, std::min(blocks(n, 16), 8 * mp_sms())); }
 int mp_embed_bwd_clause_blocks(int m) { return std::max(1, std::min(blocks(m, 64), 3 * mp_sms())); }
 int mp_part_floats() { return kPart; }
 
