@@ -260,6 +260,9 @@ struct maxsat_ctx {
   bool g_bf16 = true;             // G operand BF16 (else FP16)
   int32_t* d_kstart = nullptr;    // tiles_v + 1
   int32_t* d_kblocks = nullptr;   // tiles_v
+  const int4* d_inc_nib = nullptr;  // 4-bit patterns: incidence records, contribution rows
+  const uint32_t* d_grow = nullptr;
+  int grow_stride = 0;              // 0: not built
   uint16_t* d_gq16 = nullptr;     // contribution table as BF16 / FP16 bits
   CUtensorMap tmA2{};
   // dense chain state
@@ -376,7 +379,7 @@ int launch_round(maxsat_ctx* ctx, cudaStream_t st, const uint32_t* tdev, uint32_
           launch_gemm2(ctx->tmA2, ctx->n, ctx->n_pad, C.B, C.Bp, ctx->tiles_v, ctx->d_kstart,
                        ctx->d_kblocks, ctx->F.var_inc, ctx->d_gq16, C.H, ctx->wide_h, ctx->dX, ctx->dnu,
                        ctx->dbest_x, ctx->e5m2, ctx->g_bf16, (float)ctx->prm.alpha, tdev, t_rel,
-                       ctx->d_err, ctx->T, C, st));
+                       ctx->d_err, ctx->d_inc_nib, ctx->d_grow, ctx->grow_stride, ctx->T, C, st));
     return MAXSAT_OK;
   }
   TIMED(ctx, st, "gather_hidden",
@@ -753,7 +756,11 @@ void set_ensemble(maxsat_ctx* ctx, int32_t g8_off, int32_t B_total) {
   ctx->C.B_total = B_total;
   ctx->C.inv_B_total = 1.0f / (float)B_total;
   // (k_gather_nib keeps a block's costs in 32 bits)
-  ctx->C.nib = !ctx->dense && nib_patterns_supported(ctx->T, B_total) &&
+  if (ctx->dense) {
+    ctx->C.nib = dense_nib_supported(ctx->T, ctx->grow_stride, B_total) ? 1 : 0;
+    return;
+  }
+  ctx->C.nib = nib_patterns_supported(ctx->T, B_total) &&
                        (ctx->T.one_chunk || ctx->C.cost32)
                    ? 1
                    : 0;
@@ -1041,6 +1048,36 @@ int build_dense(maxsat_ctx* ctx, int32_t n, int64_t m, const int64_t* off, const
       if (v < 0) bits |= 0x8000;
     }
     gq16[k] = bits;
+  }
+  if (ctx->T.one_chunk) {
+    // 4-bit patterns: rows of a group's contributions to a position, patterns
+    // past its hidden units zero
+    const int G = ctx->T.n_groups;
+    ctx->grow_stride = 16 * std::max(1, 3 * G);
+    std::vector<uint32_t> grow((size_t)ctx->T.n_temps * ctx->grow_stride / 4, 0u);
+    for (int e = 0; e < ctx->T.n_temps; ++e)
+      for (int g = 0; g < G; ++g) {
+        const GroupMeta& gm = ctx->tabs.meta[g];
+        for (int k = 0; k < gm.len && k < 3; ++k) {
+          uint8_t* row = reinterpret_cast<uint8_t*>(grow.data()) + (size_t)e * ctx->grow_stride +
+                         16 * (g * 3 + k);
+          for (int hp = 0; hp < (1 << gm.nh); ++hp) {
+            const uint16_t bits = gq16[(size_t)gm.gq_off + (((size_t)e << gm.nh) + hp) * gm.len + k];
+            row[hp] = (uint8_t)(bits & 0xFF);
+            row[8 + hp] = (uint8_t)(bits >> 8);
+          }
+        }
+      }
+    std::vector<int4> inc(var_inc.size());
+    for (size_t jj = 0; jj < inc.size(); ++jj) {
+      // the record's table offset is gq_off + position, plus gq_len if negated
+      const int o = (var_inc[jj].y & 0x7FFFFFFF) - (var_inc[jj].y < 0 ? (int)gq_len : 0);
+      int g = 0;
+      while (g + 1 < G && ctx->tabs.meta[g + 1].gq_off <= o) ++g;
+      inc[jj] = make_int4(var_inc[jj].x, 16 * (g * 3 + o - ctx->tabs.meta[g].gq_off), 0, 0);
+    }
+    UPD(inc, ctx->d_inc_nib);
+    UPD(grow, ctx->d_grow);
   }
   const uint16_t* dA2 = nullptr;
   const int32_t* dks = nullptr;

@@ -36,6 +36,7 @@
 #include "dense_common.cuh"
 #include "internal.h"
 #include "philox.cuh"
+#include "round_ops.cuh"
 #include "tc_ptx.cuh"
 
 namespace rbmsat {
@@ -60,6 +61,14 @@ __device__ __forceinline__ uint32_t step_index(const uint32_t* tdev, uint32_t t_
 }
 
 __host__ __device__ __forceinline__ int align16(int bytes) { return (bytes + 15) & ~15; }
+
+// Programmatic dependent launch between a round's three kernels: each sets up
+// (barriers, TMEM, tables) while its predecessor finishes, and waits for it
+// before it touches what the predecessor writes.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 __device__ __forceinline__ void stage16(void* dst, const void* src, int bytes, int tid, int nthr) {
   const int4* s = reinterpret_cast<const int4*>(src);
@@ -97,7 +106,12 @@ struct G1Args {
   int* err;
 };
 
-template <bool SAMPLE, bool SM, typename HT, bool ONE>
+// NIB (clauses of at most 3 literals, C.nib): the hidden patterns go out as one
+// word of 4-bit fields per clause and octet, and a thread, which has one clause
+// and eight octets of a tile, computes the clause's part of Philox rounds 0..2
+// once, takes its records by byte permutes from 256-byte blocks (T.rec3) and
+// writes its eight words as one 32-byte run.
+template <bool SAMPLE, bool SM, typename HT, bool ONE, bool NIB>
 __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
     k_gemm1_step(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const G1Args a, const DevTables T, const DevChains C) {
@@ -116,7 +130,10 @@ __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
   // clause-RBM tables: staged in shared memory when small
   const GroupMeta* meta = T.meta;
   const uint32_t* rec = T.rec;
-  if (SM) {
+  const uint32_t rec3 = (tc::smem_u32(tabs) + 255u) & ~255u;  // NIB: record blocks
+  if constexpr (NIB) {
+    stage16(tabs + (rec3 - tc::smem_u32(tabs)), T.rec3, T.rec3_words * 4, threadIdx.x, blockDim.x);
+  } else if (SM) {
     const int mb = align16(T.n_groups * (int)sizeof(GroupMeta));
     stage16(tabs, T.meta, mb, threadIdx.x, blockDim.x);
     stage16(tabs + mb, T.rec, align16(T.rec_len * 4), threadIdx.x, blockDim.x);
@@ -144,6 +161,8 @@ __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = S.tmem_slot;
+  pdl_wait();
+  pdl_release();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -212,13 +231,30 @@ __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
       const float unsat_d = -(float)bias;
       const bool same_w = __ldg(a.grp_same + tm * 4 + quarter) != 0;
       GroupMeta gm{};
-      if (grp >= 0) gm = meta[grp];
+      if (!NIB && grp >= 0) gm = meta[grp];
+      HiddenClause hc{};
+      uint32_t u1 = 0, rb0 = 0;
+      bool sat = false;
+      uint32_t words[NIB ? kCols / 8 : 1];
+      // temperature of the warp's columns when they share one
+      int e_tile = -1;
+      if constexpr (NIB) {
+        const uint64_t pt = (uint64_t)kPhiloxM1 * tround;
+        u1 = (uint32_t)(pt >> 32) ^ C.keys.k0[0];
+        hc = hidden_clause((uint32_t)pt, (uint32_t)c, kPhaseHidden, C.keys);
+        rb0 = rec3 + (uint32_t)(max(grp, 0) * E) * 256u;
+        sat = grp >= 0 && __ldg(&T.meta[grp].sat) != 0;
+        const int g0 = C.g8_off * 8 + tn * kBN + cgrp * kCols;
+        e_tile = temp_of(g0, E, C.B_total, C.inv_B_total);
+        if (e_tile != temp_of(g0 + kCols - 1, E, C.B_total, C.inv_B_total)) e_tile = -1;
+      }
       S.w[ew][lane] = w;
       __syncwarp();
       const bool ok = tc::mbar_wait(&S.tfull[buf], (uint32_t)(li >> 1) & 1u, a.err, 13, kWait);
       tc::fence_after_sync();
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) +
                              (uint32_t)(buf * kBN + cgrp * kCols);
+#pragma unroll(NIB ? 2 : 1)
       for (int j = 0; j < kCols / 32; ++j) {
         uint32_t r[32];
         tc::tmem_ld32(taddr + (uint32_t)(j * 32), r);
@@ -244,6 +280,55 @@ __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
         for (int sub = 0; sub < 4; ++sub) {
           const int b0 = tn * kBN + cgrp * kCols + j * 32 + sub * 8;
           const int gb0 = C.g8_off * 8 + b0;  // global chain index
+          if constexpr (NIB) {
+            int e0 = e_tile, split = 8;
+            if (e0 < 0) {
+              e0 = temp_of(gb0, E, C.B_total, C.inv_B_total);
+              if (e0 != temp_of(gb0 + 7, E, C.B_total, C.inv_B_total))
+                split = (int)(((long long)(e0 + 1) * C.B_total + E - 1) / E) - gb0;
+            }
+            const uint64_t up = split < 8 ? 0x8080808080808080ull << (8 * split) : 0ull;
+            // twice the truth pattern, D + bias, as the low byte of the float
+            // 2^23 + bias + D; the mask keeps record addresses in range even if
+            // the accumulator is invalid after a timed-out wait
+            const float mid = (float)bias + 8388608.0f;
+            uint32_t pb[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              pb[q] = __float_as_uint(__uint_as_float(r[sub * 8 + q]) + mid);
+            const uint32_t in = (uint32_t)bias * 0x02020202u;
+            const uint32_t lo = __byte_perm(__byte_perm(pb[0], pb[1], 0x0040u),
+                                            __byte_perm(pb[2], pb[3], 0x0040u), 0x5410u) & in;
+            const uint32_t hi = __byte_perm(__byte_perm(pb[4], pb[5], 0x0040u),
+                                            __byte_perm(pb[6], pb[7], 0x0040u), 0x5410u) & in;
+            float f[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f[q] = 0.f;
+            uint32_t hw = 0, unused = 0;
+            if (grp >= 0) {
+              const uint32_t octet = (uint32_t)(gb0 >> 3);
+              uint4 R[3];
+#pragma unroll
+              for (int h = 0; h < 3; ++h) {
+                const uint64_t px = (uint64_t)kPhiloxM0 * ((octet | ((uint32_t)h << 24)) ^ u1);
+                R[h] = hidden_unit(hc, (uint32_t)(px >> 32) ^ C.keys.k1[1], (uint32_t)px, C.keys);
+              }
+              const uint32_t rb = rb0 + (uint32_t)e0 * 256u;
+              if (!sat)
+                octet_draws<false, true>((lo << 3) | (uint32_t)up, (hi << 3) | (uint32_t)(up >> 32),
+                                         rb, R, f, hw, unused);
+              else
+                octet_draws<true, true>((lo << 3) | (uint32_t)up, (hi << 3) | (uint32_t)(up >> 32),
+                                        rb, R, f, hw, unused);
+            }
+            if (j == 0)
+              words[sub] = hw;
+            else
+              words[4 + sub] = hw;
+            const float fs = tc::column_sums8(f, lane);
+            if (lane < 8) S.fe[buf][ew * kCols + j * 32 + sub * 8 + lane] = fs;
+            continue;
+          }
           const int e0 = temp_of(gb0, E, C.B_total, C.inv_B_total);
           const bool e_uni = e0 == temp_of(gb0 + 7, E, C.B_total, C.inv_B_total);
           int row[8];
@@ -292,6 +377,15 @@ __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
           if (lane < 8) S.fe[buf][ew * kCols + j * 32 + sub * 8 + lane] = fs;
         }
       }
+      if constexpr (NIB) {
+        static_assert(kCols == 64, "a row's eight words are one 32-byte run");
+        if (grp >= 0) {
+          uint4* H = reinterpret_cast<uint4*>(static_cast<uint32_t*>(a.H) + (size_t)c * (a.Bp / 8) +
+                                              tn * (kBN / 8) + cgrp * (kCols / 8));
+          H[0] = make_uint4(words[0], words[1], words[2], words[3]);
+          H[1] = make_uint4(words[4], words[5], words[6], words[7]);
+        }
+      }
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&S.tempty[buf]);
@@ -323,6 +417,8 @@ __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
 __global__ void k_keep_dense(const int64_t* __restrict__ cost_part, const float* __restrict__ fe_part,
                              int tiles_m, DevChains C) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_release();
   if (b >= C.Bp) return;
   int64_t cs = 0;
   float fs = 0.f;
@@ -394,6 +490,8 @@ struct G2Args {
   uint8_t* X;              // Bp x n_pad FP8 states
   float* nu;               // Bp x n_pad
   uint8_t* best_x;         // Bp x n_pad (0 / 1)
+  const uint32_t* grow;    // C.nib: rows of 8 contributions (low bytes, high bytes)
+  int grow_stride;         // bytes of a temperature's rows
   uint8_t one, minus_one;  // FP8 encodings of +1 / -1
   bool bf16;               // G operand type (else FP16)
   float alpha;
@@ -456,6 +554,8 @@ __global__ void __launch_bounds__(64 + 32 * (kBld + kEpi2), 1)
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = S.tmem_slot;
+  pdl_wait();
+  pdl_release();
 
   // visible update (Eq. 3, nu of Sec. 4.4, best-keep copy) of 8 chains,
   // TMEM columns 8 c .. 8 c + 7 of accumulator buf, for the calling warp's
@@ -790,6 +890,391 @@ __global__ void __launch_bounds__(64 + 32 * (kBld + kEpi2), 1)
   }
 }
 
+// GEMM2 on 4-bit hidden patterns (C.nib: clauses of at most 3 literals), tiles of
+// BN chains (256, or 128 where that leaves fewer SMs idle). The builders' table
+// look-ups, one per incidence and chain, bounded k_gemm2 (57 us a launch at n =
+// 777, m = 4001, 2000 chains; its 56 tiles of 256 chains left two thirds of the
+// SMs idle): here one word selects four chains' contributions by byte permutes
+// from a row of 8, and a K-block's staged patterns take half the bytes.
+template <int BN>
+struct G2NibStage {
+  static constexpr int kA = kStage2A;
+  static constexpr int kH = kBK2 * BN / 2;  // staged hidden patterns [u][chain]
+  static constexpr int kInc = 1024;
+  static constexpr int kBytes = kA + kH + kInc;  // multiple of 1024
+  static constexpr int kStages = 4;
+  static constexpr int kAhead = kStages - 2;
+  static constexpr int kB = BN * kBK2 * 2;
+  static constexpr int kBOff = kStages * kBytes;
+  static constexpr int kTabOff = (kBOff + 2 * kB + (int)sizeof(G2Smem) + 127) / 128 * 128;
+  static_assert(kBytes % 1024 == 0 && kB % 1024 == 0, "swizzled tiles start at 1024 bytes");
+};
+
+template <int BN>
+__global__ void __launch_bounds__(64 + 32 * (kBld + kEpi2), 1)
+    k_gemm2_nib(const __grid_constant__ CUtensorMap tmA2, const G2Args a, const DevTables T,
+            const DevChains C) {
+  using St = G2NibStage<BN>;
+  constexpr int NS = St::kStages;
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  const uint32_t base = (tc::smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* ring = smem_raw + (base - tc::smem_u32(smem_raw));
+  G2Smem& S = *reinterpret_cast<G2Smem*>(ring + St::kBOff + 2 * St::kB);
+  // staged tables start on a 128-byte boundary (16-byte vector stores)
+  uint8_t* tabs = ring + St::kTabOff;
+  auto stA = [&](int s) { return ring + s * St::kBytes; };
+  auto stH = [&](int s) { return ring + s * St::kBytes + St::kA; };
+  auto stI = [&](int s) {
+    return reinterpret_cast<int4*>(ring + s * St::kBytes + St::kA + St::kH);
+  };
+  auto stB = [&](uint32_t g) { return ring + St::kBOff + (g & 1u) * St::kB; };  // G of K-block g
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int num_tiles = a.tiles_v * a.tiles_n;
+
+  // contribution rows, then visible entries
+  const int rows_bytes = T.n_temps * a.grow_stride;
+  stage16(tabs, a.grow, rows_bytes, threadIdx.x, blockDim.x);
+  stage16(tabs + rows_bytes, T.pva, align16(T.pv_len * 8), threadIdx.x, blockDim.x);
+  const uint2* pva = reinterpret_cast<const uint2*>(tabs + rows_bytes);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < NS; ++s) {
+      tc::mbar_init(&S.loaded[s], 1);
+      tc::mbar_init(&S.built[s], kBld);
+      tc::mbar_init(&S.hready[s], 32 * kBld);
+      tc::mbar_init(&S.empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&S.tfull[b], 1);
+      tc::mbar_init(&S.tempty[b], kEpi2);
+    }
+    tc::fence_mbar_init();
+    tc::prefetch_tmap(&tmA2);
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(&S.tmem_slot, 2 * BN);
+    tc::tmem_relinquish();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = S.tmem_slot;
+  pdl_wait();
+  pdl_release();
+
+  // visible update (Eq. 3, nu of Sec. 4.4, best-keep copy) of 8 chains,
+  // TMEM columns 8 c .. 8 c + 7 of accumulator buf, for the calling warp's
+  // TMEM lane quarter (32 variables) of tile (tv, tn): the accumulators and
+  // state loads first, then the draws and the stores
+  auto visible8 = [&](int tv, int tn, int buf, int c) {
+    const uint32_t tround = step_index(a.tdev, a.t_rel);
+    const float keep = __fsub_rn(1.0f, a.alpha);  // the sparse path's exact FP32 operation sequence
+    uint8_t* __restrict__ Xs = a.X;
+    float* __restrict__ nus = a.nu;
+    uint8_t* __restrict__ bxs = a.best_x;
+    const uint8_t* __restrict__ impv = C.improved;
+    const int quarter = warp & 3;
+    const int i = tv * kBM + quarter * 32 + lane;
+    const bool valid = i < a.n;
+    const int b0 = tn * BN + c * 8;
+    uint32_t r[8];
+    tc::tmem_ld8(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * BN + c * 8), r);
+    uint32_t xo[8];
+    float nv[8];
+    if (valid) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const size_t o = (size_t)(b0 + q) * a.n_pad + i;
+        xo[q] = Xs[o];
+        nv[q] = nus[o];
+      }
+    }
+    const uint2 imp = *reinterpret_cast<const uint2*>(impv + b0);  // 8 flag bytes
+    const uint4 R = philox4x32_10(
+        make_uint4((uint32_t)i, (uint32_t)(C.g8_off + (b0 >> 3)), tround, kPhaseVisible), C.keys);
+    tc::tmem_ld_wait();
+    if (!valid) return;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int z = __float2int_rn(__uint_as_float(r[q]));
+      const uint2 pv = pva[max(-T.qmax, min(T.qmax, z)) + T.qmax];
+      const size_t o = (size_t)(b0 + q) * a.n_pad + i;
+      if (((q < 4 ? imp.x : imp.y) >> (8 * (q & 3))) & 0xFFu) bxs[o] = xo[q] == a.one ? 1 : 0;
+      nus[o] = __fmaf_rn(keep, nv[q], __uint_as_float(pv.y));
+      Xs[o] = lane16(R, q) < pv.x ? a.one : a.minus_one;
+    }
+  };
+  constexpr int kShare = kEpi2 / 4 + kBld / 4;  // warps per lane quarter on a CTA's last tile
+
+  if (warp == 0) {
+    // producer warp: P^T tile by TMA and the K-block's incidence records by
+    // one bulk copy
+    uint32_t g = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      const int tv = tile / a.tiles_n;
+      const int k0 = __ldg(a.kstart + tv), k1 = __ldg(a.kstart + tv + 1);
+      const int nkb = __ldg(a.kblocks + tv);
+      for (int kb = 0; kb < nkb; ++kb, ++g) {
+        const int s = (int)(g % NS);
+        const uint32_t ph = (g / NS) & 1u;
+        if (lane == 0) {
+          ok = tc::mbar_wait(&S.empty[s], ph ^ 1u, a.err, 21, kWait);
+          if (ok) {
+            const int jj0 = k0 + kb * kBK2;
+            const int nvalid = max(0, min(kBK2, k1 - jj0));
+            tc::mbar_arrive_expect_tx(&S.loaded[s], (uint32_t)(St::kA + nvalid * 16));
+            tc::tma_load_2d(stA(s), &tmA2, &S.loaded[s], kb * kBK2, tv * kBM);
+            if (nvalid > 0)
+              tc::bulk_load(stI(s), a.var_inc + jj0, (uint32_t)(nvalid * 16), &S.loaded[s]);
+          }
+        }
+        ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+        if (!ok) break;
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      uint32_t g = 0;
+      bool ok = true;
+      int li = 0;
+      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++li) {
+        const int tv = tile / a.tiles_n;
+        const int nkb = __ldg(a.kblocks + tv);
+        const int buf = li & 1;
+        ok = tc::mbar_wait(&S.tempty[buf], ((uint32_t)(li >> 1) & 1u) ^ 1u, a.err, 24, kWait);
+        if (!ok) break;
+        tc::fence_after_sync();
+        const uint32_t d = tmem + (uint32_t)(buf * BN);
+        for (int kb = 0; kb < nkb; ++kb, ++g) {
+          const int s = (int)(g % NS);
+          const uint32_t ph = (g / NS) & 1u;
+          ok = tc::mbar_wait(&S.built[s], ph, a.err, 22, kWait);
+          if (!ok) break;
+          tc::fence_after_sync();
+          const uint32_t a0 = tc::smem_u32(stA(s)), b0 = tc::smem_u32(stB(g));
+#pragma unroll
+          for (int kk = 0; kk < kBK2 / 16; ++kk)
+            tc::mma<false>(d, tc::sw128_desc(a0 + kk * 32), tc::sw128_desc(b0 + kk * 32), a.idesc,
+                           (kb > 0 || kk > 0) ? 1u : 0u);
+          tc::commit(&S.empty[s]);
+        }
+        tc::commit(&S.tfull[buf]);
+      }
+    }
+    __syncwarp();
+  } else if (warp < 2 + kBld) {
+    // builders. Copy phase: 16 bytes (32 chains) of an incidence's pattern row
+    // per thread, cp.async into the stage kAhead K-blocks ahead. Build phase:
+    // thread = 4 consecutive chains x kIpt incidences: per incidence one word
+    // of the 4 patterns, which selects the chains' low and high bytes from the
+    // row of 8 contributions by two byte permutes; two incidences' bytes make
+    // the chains' words, and 2 kIpt bytes of the G tile (row = chain, 128-byte
+    // swizzle) are stored per chain.
+    const int bt = threadIdx.x - 64;  // 0 .. 511
+    auto issue_copies = [&](int s, int jk0, int jk1, int ttn) {
+      constexpr int kParts = BN / 32;  // 16-byte parts of a row
+      const int u = bt / kParts, part = bt % kParts;
+      if (u < kBK2 && jk0 + u < jk1) {
+        const uint32_t* src = static_cast<const uint32_t*>(a.H) +
+                              (size_t)stI(s)[u].x * (a.Bp / 8) + ttn * (BN / 8) + part * 4;
+        tc::cp_async16(stH(s) + u * (BN / 2) + part * 16, src);
+      }
+      tc::cp_async_arrive(&S.hready[s]);
+    };
+    // two cursors over (tile, K-block) in the producer's order: copies (cc,
+    // flat index gc) run kAhead K-blocks ahead of the build (cb, flat index g)
+    struct Cursor {
+      int tile, kb, tn, k0, k1, nkb;
+    };
+    auto enter_tile = [&](Cursor& c) {
+      if (c.tile < num_tiles) {
+        const int tv = c.tile / a.tiles_n;
+        c.tn = c.tile % a.tiles_n;
+        c.k0 = __ldg(a.kstart + tv);
+        c.k1 = __ldg(a.kstart + tv + 1);
+        c.nkb = __ldg(a.kblocks + tv);
+      }
+    };
+    auto advance = [&](Cursor& c) {
+      if (++c.kb >= c.nkb) {
+        c.tile += gridDim.x;
+        c.kb = 0;
+        enter_tile(c);
+      }
+    };
+    Cursor cb{(int)blockIdx.x, 0, 0, 0, 0, 0};
+    enter_tile(cb);
+    Cursor cc = cb;
+    uint32_t gc = 0, g = 0;
+    bool ok = true;
+    auto wait_records = [&]() {
+      ok = tc::mbar_wait(&S.loaded[gc % NS], (gc / NS) & 1u, a.err, 23, kWait);
+    };
+    auto copy_next = [&]() {
+      issue_copies((int)(gc % NS), cc.k0 + cc.kb * kBK2, cc.k1, cc.tn);
+      advance(cc);
+      ++gc;
+    };
+    for (int d = 0; d < St::kAhead && ok && cc.tile < num_tiles; ++d) {
+      wait_records();
+      if (ok) copy_next();
+    }
+    constexpr int kIpt = BN / 32;         // incidences per thread: 8 or 4
+    const int quad = bt & (BN / 4 - 1);   // chains 4 quad .. 4 quad + 3
+    const int chunk = bt / (BN / 4);      // incidences kIpt chunk .. + kIpt - 1
+    // slot r of a thread holds chain 4 quad + (r + quad / 2) % 4: the rotation
+    // spreads the store phases over the 16-byte bank groups
+    const int rot = (quad >> 1) & 3;
+    const uint32_t rows_s = tc::smem_u32(tabs);
+    while (ok && cb.tile < num_tiles) {
+      // the copies of K-block g + kAhead are issued after this build's proxy
+      // fence, so that the fence does not wait for them to land
+      const bool more = cc.tile < num_tiles;
+      if (more) {
+        wait_records();
+        if (!ok) break;
+      } else if (g >= 2) {
+        // no copies left to order it: wait for the MMA that last read this
+        // G buffer (K-block g - 2)
+        ok = tc::mbar_wait(&S.empty[(g - 2) % NS], ((g - 2) / NS) & 1u, a.err, 27, kWait);
+        if (!ok) break;
+      }
+      // build the current K-block once every builder's copies have landed
+      const int s = (int)(g % NS);
+      ok = tc::mbar_wait(&S.hready[s], (g / NS) & 1u, a.err, 26, kWait);
+      if (!ok) break;
+      {
+        const uint32_t inc_s = tc::smem_u32(stI(s)) + (uint32_t)(chunk * kIpt * 16);
+        const uint32_t hs = tc::smem_u32(stH(s)) + (uint32_t)(chunk * kIpt * (BN / 2) + quad * 2);
+        uint8_t* gt = stB(g);
+        // the quad's temperatures: e0, and e0 + 1 for the slots of mask `up`
+        const int gq0 = C.g8_off * 8 + cb.tn * BN + 4 * quad;
+        const int e0 = temp_of(gq0, T.n_temps, C.B_total, C.inv_B_total);
+        uint32_t up = 0;
+        if (e0 != temp_of(gq0 + 3, T.n_temps, C.B_total, C.inv_B_total)) {
+          const int split =
+              (int)(((long long)(e0 + 1) * C.B_total + T.n_temps - 1) / T.n_temps) - gq0;
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (((r + rot) & 3) >= split) up |= 0xFFu << (8 * r);
+        }
+        const uint32_t row_e = rows_s + (uint32_t)(e0 * a.grow_stride);
+        uint32_t pk[4][kIpt / 2];
+        const int jj0 = cb.k0 + cb.kb * kBK2, k1 = cb.k1;
+        // FULL: all 64 incidences of the K-block exist (every K-block but a
+        // tile's last), so that the loads of different incidences carry no
+        // branch between them and overlap
+        auto lookups = [&](auto full) {
+#pragma unroll
+          for (int p = 0; p < kIpt / 2; ++p) {
+            uint32_t lo[2] = {0u, 0u}, hi[2] = {0u, 0u};  // 0 = +0.0
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+              const int u = 2 * p + hf;
+              if (decltype(full)::value || jj0 + chunk * kIpt + u < k1) {
+                uint32_t off, h;
+                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(off) : "r"(inc_s + 16u * u + 4u));
+                asm volatile("{\n\t.reg .u16 t;\n\tld.shared.u16 t, [%1];\n\tcvt.u32.u16 %0, t;\n\t}"
+                             : "=r"(h)
+                             : "r"(hs + (uint32_t)(u * (BN / 2))));
+                const uint32_t sel = __funnelshift_r(h | (h << 16), 0u, 4u * (uint32_t)rot);
+                const uint4 tb = lds128(row_e + off);
+                lo[hf] = prmt(tb.x, tb.y, sel);
+                hi[hf] = prmt(tb.z, tb.w, sel);
+                if (up) {
+                  const uint4 t1 = lds128(row_e + (uint32_t)a.grow_stride + off);
+                  lo[hf] = (lo[hf] & ~up) | (prmt(t1.x, t1.y, sel) & up);
+                  hi[hf] = (hi[hf] & ~up) | (prmt(t1.z, t1.w, sel) & up);
+                }
+              }
+            }
+            const uint32_t a0 = __byte_perm(lo[0], hi[0], 0x5140u), a1 = __byte_perm(lo[0], hi[0], 0x7362u);
+            const uint32_t c0 = __byte_perm(lo[1], hi[1], 0x5140u), c1 = __byte_perm(lo[1], hi[1], 0x7362u);
+            pk[0][p] = __byte_perm(a0, c0, 0x5410u);
+            pk[1][p] = __byte_perm(a0, c0, 0x7632u);
+            pk[2][p] = __byte_perm(a1, c1, 0x5410u);
+            pk[3][p] = __byte_perm(a1, c1, 0x7632u);
+          }
+        };
+        if (jj0 + kBK2 <= k1)
+          lookups(std::true_type{});
+        else
+          lookups(std::false_type{});
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int chain = 4 * quad + ((r + rot) & 3);
+          if constexpr (kIpt == 8)
+            *reinterpret_cast<uint4*>(gt + chain * 128 + ((chunk ^ (chain & 7)) << 4)) =
+                make_uint4(pk[r][0], pk[r][1], pk[r][2], pk[r][3]);
+          else
+            *reinterpret_cast<uint2*>(gt + chain * 128 + (((chunk >> 1) ^ (chain & 7)) << 4) +
+                                      (chunk & 1) * 8) = make_uint2(pk[r][0], pk[r][1]);
+        }
+        tc::fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&S.built[s]);
+      }
+      if (more) copy_next();
+      ++g;
+      advance(cb);
+    }
+    // the visible update of the CTA's last tile, shared with the epilogue
+    // warps (worker kEpi2 / 4 + index among the quarter's builder warps)
+    if (ok && (int)blockIdx.x < num_tiles) {
+      const int nt = (num_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x;  // its local index
+      const int lt = (int)blockIdx.x + nt * (int)gridDim.x;
+      tc::mbar_wait(&S.tfull[nt & 1], (uint32_t)(nt >> 1) & 1u, a.err, 28, kWait);
+      tc::fence_after_sync();
+#pragma unroll 1
+      for (int c = kEpi2 / 4 + (warp - 2) / 4; c < BN / 8; c += kShare)
+        visible8(lt / a.tiles_n, lt % a.tiles_n, nt & 1, c);
+    }
+  } else {
+    // epilogue: row = variable. A tile's 32 groups of 8 chains go to the
+    // epilogue warps of each lane quarter; the CTA's last tile is shared with
+    // the builder warps, idle by then (kShare warps per quarter)
+    const int ew = warp - 2 - kBld;  // 0 .. kEpi2 - 1
+    const int cgrp = ew / 4;
+    int li = 0;
+    for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x, ++li) {
+      const int tv = tile / a.tiles_n, tn = tile % a.tiles_n;
+      const int buf = li & 1;
+      {
+        // the tile's state rows into L2 while its mainloop runs: thread =
+        // one chain, its 128 variables (one line of x, four of nu; n_pad is
+        // a multiple of 128)
+        for (int ch = ew * 32 + lane; ch < BN; ch += kEpi2 * 32) {
+          const size_t row = (size_t)(tn * BN + ch) * a.n_pad + (size_t)tv * kBM;
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(a.X + row));
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.nu + row + 32 * q));
+        }
+      }
+      tc::mbar_wait(&S.tfull[buf], (uint32_t)(li >> 1) & 1u, a.err, 25, kWait);
+      tc::fence_after_sync();
+      if (tile + (int)gridDim.x < num_tiles) {
+#pragma unroll 1
+        for (int c = cgrp; c < BN / 8; c += kEpi2 / 4) visible8(tv, tn, buf, c);
+      } else {
+#pragma unroll 1
+        for (int c = cgrp; c < BN / 8; c += kShare) visible8(tv, tn, buf, c);
+      }
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&S.tempty[buf]);
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    tc::fence_after_sync();
+    tc::tmem_dealloc(tmem, 2 * BN);
+  }
+}
+
 // ---------------------------------------------------------------- state
 __global__ void k_init_dense(DevChains C, uint8_t* X, float* nu, uint8_t* best_x, int n,
                              int n_pad, uint8_t one, uint8_t minus_one) {
@@ -824,28 +1309,41 @@ __global__ void k_keep_copy_dense(const DevChains C, const uint8_t* X, uint8_t* 
   }
 }
 
+template <typename... P, typename... Q>
+cudaError_t launch_pdl(void (*kern)(P...), int grid, int threads, int smem, cudaStream_t st,
+                       const Q&... args) {
+  const cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 template <bool SAMPLE, bool SM, typename HT>
 cudaError_t g1_variant(int grid, int smem, cudaStream_t st, const CUtensorMap& tmA,
                        const CUtensorMap& tmB, const G1Args& a, const DevTables& T,
                        const DevChains& C) {
   // one-chunk records (L <= 3 everywhere): the sampling has no chunk loop
-  auto kern = k_gemm1_step<SAMPLE, SM, HT, false>;
+  auto kern = k_gemm1_step<SAMPLE, SM, HT, false, false>;
   if constexpr (SAMPLE && sizeof(HT) == 1)
-    if (T.one_chunk) kern = k_gemm1_step<SAMPLE, SM, HT, true>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid, 64 + 32 * kEpi1, smem, st>>>(tmA, tmB, a, T, C);
-  return cudaGetLastError();
+    if (T.one_chunk) kern = k_gemm1_step<SAMPLE, SM, HT, true, false>;
+  return launch_pdl(kern, grid, 64 + 32 * kEpi1, smem, st, tmA, tmB, a, T, C);
 }
 
 template <bool SM, typename HT>
 cudaError_t g2_variant(int grid, int smem, cudaStream_t st, const CUtensorMap& tmA2,
                        const G2Args& a, const DevTables& T, const DevChains& C) {
   auto kern = k_gemm2<SM, HT>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  kern<<<grid, 64 + 32 * (kBld + kEpi2), smem, st>>>(tmA2, a, T, C);
-  return cudaGetLastError();
+  return launch_pdl(kern, grid, 64 + 32 * (kBld + kEpi2), smem, st, tmA2, a, T, C);
 }
 
 int sm_count() {
@@ -862,6 +1360,16 @@ int sm_count() {
 constexpr int kSmemMax = 227 * 1024;
 
 }  // namespace
+
+// whether the dense round takes 4-bit patterns: record blocks and contribution
+// rows fit beside the rings, octets of at most two temperatures
+bool dense_nib_supported(const DevTables& T, int grow_stride, int B_total) {
+  return T.one_chunk && T.rec3 && T.ptab && grow_stride > 0 &&
+         1024 + kTabOff1 + 256 + T.rec3_words * 4 <= kSmemMax &&
+         1024 + G2NibStage<256>::kTabOff + T.n_temps * grow_stride + align16(T.pv_len * 8) <=
+             kSmemMax &&
+         (T.n_temps == 1 || B_total / T.n_temps >= 8);
+}
 
 int dense_g1_table_bytes(const DevTables& T) {
   return align16(T.n_groups * (int)sizeof(GroupMeta)) + align16(T.rec_len * 4);
@@ -897,6 +1405,9 @@ cudaError_t launch_gemm1_step(bool sample, const CUtensorMap& tmA, const CUtenso
   const bool sm = base_smem + tb <= kSmemMax;
   const int smem = base_smem + (sm ? tb : 0);
   const int grid = std::min(sm_count(), a.tiles_m * a.tiles_n);
+  if (sample && C.nib)
+    return launch_pdl(k_gemm1_step<true, true, uint8_t, true, true>, grid, 64 + 32 * kEpi1,
+                      base_smem + 256 + T.rec3_words * 4, st, tmA, tmB, a, T, C);
   if (sample) {
     if (sm) return wide ? g1_variant<true, true, uint16_t>(grid, smem, st, tmA, tmB, a, T, C)
                         : g1_variant<true, true, uint8_t>(grid, smem, st, tmA, tmB, a, T, C);
@@ -909,8 +1420,7 @@ cudaError_t launch_gemm1_step(bool sample, const CUtensorMap& tmA, const CUtenso
 
 cudaError_t launch_keep_dense(const int64_t* cost_part, const float* fe_part, int tiles_m,
                               const DevChains& C, cudaStream_t st) {
-  k_keep_dense<<<(C.Bp + 63) / 64, 64, 0, st>>>(cost_part, fe_part, tiles_m, C);
-  return cudaGetLastError();
+  return launch_pdl(k_keep_dense, (C.Bp + 63) / 64, 64, 0, st, cost_part, fe_part, tiles_m, C);
 }
 
 cudaError_t launch_gemm2(const CUtensorMap& tmA2, int n, int n_pad, int B, int Bp, int tiles_v,
@@ -918,8 +1428,11 @@ cudaError_t launch_gemm2(const CUtensorMap& tmA2, int n, int n_pad, int B, int B
                          const uint16_t* gq16, const void* H, bool wide, uint8_t* X, float* nu,
                          uint8_t* best_x,
                          bool e5m2, bool bf16, float alpha, const uint32_t* tdev, uint32_t t_rel,
-                         int* err, const DevTables& T, const DevChains& C, cudaStream_t st) {
+                         int* err, const int4* inc_nib, const uint32_t* grow, int grow_stride,
+                         const DevTables& T, const DevChains& C, cudaStream_t st) {
   G2Args a;
+  a.grow = grow;
+  a.grow_stride = grow_stride;
   a.n = n;
   a.n_pad = n_pad;
   a.B = B;
@@ -943,6 +1456,21 @@ cudaError_t launch_gemm2(const CUtensorMap& tmA2, int n, int n_pad, int B, int B
   a.tdev = tdev;
   a.t_rel = t_rel;
   a.err = err;
+  if (C.nib) {
+    a.var_inc = inc_nib;
+    const int tbn = T.n_temps * grow_stride + align16(T.pv_len * 8);
+    const int threads = 64 + 32 * (kBld + kEpi2);
+    // tiles of 128 chains where they take less than twice the waves
+    const int t256 = tiles_v * (Bp / 256), sms = sm_count();
+    if ((t256 * 2 + sms - 1) / sms < 2 * ((t256 + sms - 1) / sms)) {
+      a.tiles_n = Bp / 128;
+      a.idesc = tc::instr_desc(kBM, 128, fmt, fmt);
+      return launch_pdl(k_gemm2_nib<128>, std::min(sms, 2 * t256), threads,
+                        1024 + G2NibStage<128>::kTabOff + tbn, st, tmA2, a, T, C);
+    }
+    return launch_pdl(k_gemm2_nib<256>, std::min(sms, t256), threads,
+                      1024 + G2NibStage<256>::kTabOff + tbn, st, tmA2, a, T, C);
+  }
   const int tb = align16(T.gq_len * 4) + align16(T.pv_len * 4);
   const int grid = std::min(sm_count(), a.tiles_v * a.tiles_n);
   if (wide) {

@@ -481,7 +481,13 @@ cudaError_t launch_gemm2(const CUtensorMap& tmA2, int n, int n_pad, int B, int B
                          const uint16_t* gq16, const void* H, bool wide, uint8_t* X, float* nu,
                          uint8_t* best_x,
                          bool e5m2, bool bf16, float alpha, const uint32_t* tdev, uint32_t t_rel,
-                         int* err, const DevTables& T, const DevChains& C, cudaStream_t st);
+                         int* err, const int4* inc_nib, const uint32_t* grow, int grow_stride,
+                         const DevTables& T, const DevChains& C, cudaStream_t st);
+// 4-bit patterns on the dense path (C.nib): inc_nib per incidence {clause, byte
+// offset of its row, 0, 0}, grow per temperature grow_stride bytes of 16-byte
+// rows (group, position): low, then high bytes of the contributions of the 8
+// patterns as BF16 / FP16
+bool dense_nib_supported(const DevTables& T, int grow_stride, int B_total);
 cudaError_t launch_init_dense(const DevChains& C, uint8_t* X, float* nu, uint8_t* best_x, int n,
                               int n_pad, bool e5m2, cudaStream_t st);
 cudaError_t launch_keep_copy_dense(const DevChains& C, const uint8_t* X, uint8_t* best_x, int n,
