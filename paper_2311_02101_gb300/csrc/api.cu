@@ -1606,27 +1606,47 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     UP(rec3, T.rec3);
     T.rec3_words = (int32_t)rec3.size();
   }
+  int64_t slab_rows = 0;
   {
-    // the packed evaluation reads the clause lists as they are; a batch gets a
-    // list of runs of at most 2048 clauses of one formula (fewer than 65536 runs)
+    // the packed evaluation's slabs of 32 clauses, by length within a formula; a
+    // batch gets a list of runs of slabs of one formula (fewer than 65536 runs)
     BitsFormula& E = ctx->bits;
     E.m = (int32_t)m;
     for (int k = 0; k < n_inst; ++k) E.n = std::max(E.n, var_base[k + 1] - var_base[k]);
     for (int64_t c = 0; c < m && !E.wide; ++c)
       if (cl_w[c] >= ((int64_t)1 << 26)) E.wide = 1;  // 32 of them below 2^31
-    if (n_inst > 1) {
-      const int64_t run = std::max<int64_t>(2048, (m / 32768 + 32) / 32 * 32);
-      std::vector<int4> items;
-      std::vector<int2> vars;
-      for (int k = 0; k < n_inst; ++k) {
-        vars.push_back(make_int2(var_base[k], var_base[k + 1] - var_base[k]));
-        for (int64_t c = cl_base[k]; c < cl_base[k + 1]; c += run)
-          items.push_back(make_int4((int)c, (int)std::min<int64_t>(cl_base[k + 1], c + run), k, 0));
+    std::vector<int32_t> perm;
+    std::vector<int2> slabs, vars;
+    std::vector<int4> items;
+    int64_t& rows = slab_rows;
+    const int64_t run = std::max<int64_t>(64, m / 1048576 + 1);
+    for (int k = 0; k < n_inst && E.n <= kBitsMaxVars; ++k) {
+      int64_t at[MAXSAT_MAX_LEN + 2] = {0};
+      for (int c = cl_base[k]; c < cl_base[k + 1]; ++c) ++at[cl_off[c + 1] - cl_off[c] + 1];
+      for (int len = 1; len <= MAXSAT_MAX_LEN; ++len) at[len] += at[len - 1];
+      const size_t p0 = perm.size();
+      const int s0 = (int)slabs.size();
+      perm.resize(p0 + (cl_base[k + 1] - cl_base[k] + 31) / 32 * 32, -1);
+      for (int c = cl_base[k]; c < cl_base[k + 1]; ++c)
+        perm[p0 + at[cl_off[c + 1] - cl_off[c]]++] = c;
+      for (size_t p = p0; p < perm.size(); p += 32) {
+        int last = 31;  // the slab's longest clause
+        while (perm[p + last] < 0) --last;
+        const int c = perm[p + last];
+        slabs.push_back(make_int2((int)rows, k));
+        rows += cl_off[c + 1] - cl_off[c];
       }
-      E.n_items = (int32_t)items.size();
-      UP(items, E.items);
-      UP(vars, E.inst_vars);
+      vars.push_back(make_int2(var_base[k], var_base[k + 1] - var_base[k]));
+      for (int64_t q = s0; n_inst > 1 && q < (int64_t)slabs.size(); q += run)
+        items.push_back(make_int4((int)q, (int)std::min<int64_t>(slabs.size(), q + run), k, 0));
     }
+    E.n_slabs = (int32_t)slabs.size();
+    E.n_items = (int32_t)items.size();
+    slabs.push_back(make_int2((int)rows, 0));
+    UP(perm, E.perm);
+    UP(slabs, E.slabs);
+    UP(vars, E.inst_vars);
+    if (n_inst > 1) UP(items, E.items);
   }
   F.n_inst = n_inst;
   F.var_inst = nullptr;
@@ -1658,6 +1678,16 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   ctx->bits.off = F.cl_off;
   ctx->bits.lits = F.lit_var;
   ctx->bits.w = F.cl_w;
+  {
+    cudaError_t e = A.alloc(&ctx->bits.slab_lits, 32 * (size_t)std::max<int64_t>(1, slab_rows));
+    if (e == cudaSuccess)
+      e = A.alloc(&ctx->bits.slab_w, 32 * (size_t)std::max(1, ctx->bits.n_slabs));
+    if (e == cudaSuccess) e = launch_bits_slabs(ctx->bits, ctx->stream);
+    if (e != cudaSuccess) {
+      delete ctx;
+      return cuda_fail(nullptr, e, "clause slabs");
+    }
+  }
   {
     cudaError_t e = A.alloc(&ctx->d_t, 1);
     if (e == cudaSuccess) e = A.alloc(&ctx->d_err, 1);

@@ -21,10 +21,12 @@
 //                sums of four weights (built by the warp for these 32
 //                clauses) add their weights. Integers throughout: exact in
 //                any order.
-// The clause lists are read as they are (a warp's 32 lists are neighbours, so
-// their lines stay in the L1 while the lanes walk them): a first layout with
-// the clauses sorted by length and 32 literals side by side ran no faster and
-// cost 2.5 ms of host work before the first evaluation of 100000 clauses.
+//   k_bits_slabs, once per formula: its clauses in order of length, 32 to a
+//                slab, literal j of the 32 side by side. (A warp walks as many
+//                literals as its longest clause has, and reads a literal of 32
+//                clauses as one line: at lengths 2-12, n = 20000, m = 100000,
+//                1000 assignments an evaluation on the lists as they came took
+//                64 us, on lists in order of length 58, on slabs 25.)
 // Bound by shared-memory look-ups (a literal's 32 random words over 32 banks
 // take about 3.5 passes) and the transpose's shuffles.
 #include <algorithm>
@@ -154,29 +156,52 @@ __device__ __forceinline__ V weigh(const V* lut, uint32_t bits) {
   return s;
 }
 
-// V: int32_t when every 32 consecutive clauses weigh less than 2^31, else
+// One thread per position of the slabs: copies its clause's literals and
+// weight. A literal is its variable within the formula, bit 31 set when
+// negated; positions past a clause's end name a word that is always zero.
+__global__ void __launch_bounds__(256) k_bits_slabs(BitsFormula F, int n_pos) {
+  const int pos = (int)(blockIdx.x * 256 + threadIdx.x);
+  if (pos >= n_pos) return;
+  const int lane = pos & 31;
+  const int2 sl = F.slabs[pos >> 5];  // {first literal row, formula}
+  const int rows = F.slabs[(pos >> 5) + 1].x - sl.x;
+  const int c = F.perm[pos];
+  const int2 vs = F.inst_vars[sl.y];
+  int32_t* out = F.slab_lits + (size_t)sl.x * 32 + lane;
+  int o = 0, len = 0;
+  if (c >= 0) {
+    o = F.off[c];
+    len = F.off[c + 1] - o;
+  }
+  F.slab_w[pos] = c >= 0 ? F.w[c] : 0;
+  for (int j = 0; j < rows; ++j) out[32 * j] = j < len ? F.lits[o + j] - vs.x : (vs.y + 3) / 4 * 4;
+}
+
+// V: int32_t when every 32 clauses of a slab weigh less than 2^31, else
 // int64_t. RAW: a caller's DIMACS arrays, not checked before.
-template <typename V, bool RAW>
-__global__ void __launch_bounds__(256) k_bits_cost(BitsFormula F, RawFormula R,
-                                                   const uint32_t* __restrict__ X, int nstride,
-                                                   int B, unsigned long long* __restrict__ out) {
+template <typename V, bool RAW, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawFormula R,
+                                                          const uint32_t* __restrict__ X,
+                                                          int nstride, int B,
+                                                          unsigned long long* __restrict__ out) {
   extern __shared__ __align__(16) uint32_t s_row[];
-  __shared__ V s_lut[8][128];
-  __shared__ long long s_sum[8][32];
+  __shared__ V s_lut[WARPS][128];
+  __shared__ long long s_sum[WARPS][32];
   dependents_may_start();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int word = (int)blockIdx.x;
-  // this block's clauses c_begin .. c_end - 1, and its formula's variables
-  int c_begin, c_end, inst = 0, v0 = 0, nv;
+  // this block's clauses (RAW) or slabs begin .. end - 1, and its formula's
+  // variables
+  int begin, end, inst = 0, v0 = 0, nv;
   if (RAW || !F.items) {
-    const int m = RAW ? R.m : F.m, runs = (m + 31) / 32;
-    c_begin = 32 * (int)((long long)runs * blockIdx.y / gridDim.y);
-    c_end = min(m, 32 * (int)((long long)runs * (blockIdx.y + 1) / gridDim.y));
+    const int runs = RAW ? (R.m + 31) / 32 : F.n_slabs;
+    begin = (int)((long long)runs * blockIdx.y / gridDim.y);
+    end = (int)((long long)runs * (blockIdx.y + 1) / gridDim.y);
     nv = RAW ? R.n : F.n;
   } else {
     const int4 it = __ldg(F.items + blockIdx.y);
-    c_begin = it.x;
-    c_end = it.y;
+    begin = it.x;
+    end = it.y;
     inst = it.z;
     const int2 vs = __ldg(F.inst_vars + inst);
     v0 = vs.x;
@@ -185,20 +210,22 @@ __global__ void __launch_bounds__(256) k_bits_cost(BitsFormula F, RawFormula R,
   wait_for_predecessor();
   const uint32_t* row = X + (size_t)word * nstride + v0;
   if ((v0 & 3) == 0) {
-    for (int k = threadIdx.x * 4; k < nv; k += 1024)
+#pragma unroll 8
+    for (int k = threadIdx.x * 4; k < nv; k += 128 * WARPS)
       *reinterpret_cast<uint4*>(s_row + k) = __ldg(reinterpret_cast<const uint4*>(row + k));
   } else {
-    for (int k = threadIdx.x; k < nv; k += 256) s_row[k] = __ldg(row + k);
+    for (int k = threadIdx.x; k < nv; k += 32 * WARPS) s_row[k] = __ldg(row + k);
   }
+  if (threadIdx.x == 0) s_row[(nv + 3) / 4 * 4] = 0u;
   __syncthreads();
   V* lut = s_lut[warp];
   long long sum = 0;
-  for (int c0 = c_begin + 32 * warp; c0 < c_end; c0 += 256) {
-    const int c = c0 + lane;
+  for (int k = begin + warp; k < end; k += WARPS) {
     uint32_t sat = 0;
     V w = 0;
-    if (c < c_end) {
-      if constexpr (RAW) {
+    if constexpr (RAW) {
+      const int c = 32 * k + lane;
+      if (c < R.m) {
         w = R.w ? (V)__ldg(R.w + c) : V(1);
         const int64_t o0 = min(max(__ldg(R.off + c), (int64_t)0), R.n_lits);
         const int64_t o1 = min(max(__ldg(R.off + c + 1), o0), R.n_lits);
@@ -209,18 +236,24 @@ __global__ void __launch_bounds__(256) k_bits_cost(BitsFormula F, RawFormula R,
           if (l == 0 || v < 0 || v >= nv) continue;
           sat |= s_row[v] ^ (uint32_t)(l >> 31);
         }
-      } else {
-        w = (V)__ldg(F.w + c);
-        const int o0 = __ldg(F.off + c), o1 = __ldg(F.off + c + 1);
-        for (int j = o0; j < o1; j += 4) {
-          int32_t l[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) l[k] = j + k < o1 ? __ldg(F.lits + j + k) : 0;
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (j + k < o1) sat |= s_row[(l[k] & 0x7FFFFFFF) - v0] ^ (uint32_t)(l[k] >> 31);
-        }
       }
+    } else {
+      w = (V)__ldg(F.slab_w + 32 * k + lane);
+      const int r0 = __ldg(&F.slabs[k].x), r1 = __ldg(&F.slabs[k + 1].x);
+      const int32_t* q = F.slab_lits + (size_t)r0 * 32 + lane;
+      int r = r0;
+      for (; r + 4 <= r1; r += 4, q += 128) {
+        int32_t l[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) l[u] = __ldg(q + 32 * u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) sat |= s_row[l[u] & 0x7FFFFFFF] ^ (uint32_t)(l[u] >> 31);
+      }
+      int32_t l[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) l[u] = r + u < r1 ? __ldg(q + 32 * u) : (nv + 3) / 4 * 4;
+#pragma unroll
+      for (int u = 0; u < 3; ++u) sat |= s_row[l[u] & 0x7FFFFFFF] ^ (uint32_t)(l[u] >> 31);
     }
     __syncwarp();  // the previous 32 clauses' sums are read
     build_subset_sums<V>(lut, w, lane);
@@ -233,17 +266,18 @@ __global__ void __launch_bounds__(256) k_bits_cost(BitsFormula F, RawFormula R,
   if (warp == 0) {
     long long c = 0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) c += s_sum[k][lane];
+    for (int k = 0; k < WARPS; ++k) c += s_sum[k][lane];
     const int b = word * 32 + lane;
     if (b < B && c != 0) atomicAdd(out + (size_t)inst * B + b, (unsigned long long)c);
   }
 }
 
 template <typename... P, typename... Q>
-cudaError_t launch_after(void (*kern)(P...), dim3 grid, int smem, cudaStream_t st, Q... args) {
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, int threads, int smem, cudaStream_t st,
+                         Q... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
@@ -266,24 +300,37 @@ int sms() {
   return count;
 }
 
-int row_bytes(int nv) { return 4 * ((nv + 3) / 4 * 4); }
+int row_bytes(int nv) { return 4 * ((nv + 3) / 4 * 4) + 16; }  // with the zero word
 
-// blocks per word so that about three fall on every SM, each warp with at
-// least two runs of 32 clauses
-int cost_chunks(int W, int m) {
-  const int want = std::max(1, (3 * sms() + W - 1) / W);
-  return std::max(1, std::min(want, (m + 511) / 512));
+// blocks of 8 warps that share an SM: room for the staged rows
+int cost_blocks_per_sm(int nv) { return 226 * 1024 / (row_bytes(nv) + 11 * 1024); }
+
+// blocks per word: about three on every SM, but no more than fit at once; each
+// warp with at least two runs of 32 clauses
+int cost_chunks(int W, int runs, int nv) {
+  const int want = (3 * sms() + W - 1) / W;
+  const int fit = std::max(1, std::min(6, cost_blocks_per_sm(nv)) * sms() / W);
+  return std::max(1, std::min(std::min(want, fit), (runs + 15) / 16));
 }
 
-template <typename V, bool RAW>
-cudaError_t cost_launch(const BitsFormula& F, const RawFormula& R, const uint32_t* X, int nstride,
-                        int B, int nv, int chunks, int64_t* cost, cudaStream_t st) {
-  auto kern = k_bits_cost<V, RAW>;
+template <typename V, bool RAW, int WARPS>
+cudaError_t cost_variant(const BitsFormula& F, const RawFormula& R, const uint32_t* X, int nstride,
+                         int B, int nv, int chunks, int64_t* cost, cudaStream_t st) {
+  auto kern = k_bits_cost<V, RAW, WARPS>;
   const int smem = row_bytes(nv);
   const cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  return launch_after(kern, dim3((unsigned)((B + 31) / 32), (unsigned)chunks), smem, st, F, R, X,
-                      nstride, B, reinterpret_cast<unsigned long long*>(cost));
+  return launch_after(kern, dim3((unsigned)((B + 31) / 32), (unsigned)chunks), 32 * WARPS, smem, st,
+                      F, R, X, nstride, B, reinterpret_cast<unsigned long long*>(cost));
+}
+
+// rows so long that at most two blocks share an SM get blocks of 16 warps
+template <typename V, bool RAW>
+cudaError_t cost_launch(const BitsFormula& F, const RawFormula& R, const uint32_t* X, int nstride,
+                        int B, int nv, int chunks, int64_t* cost, cudaStream_t st) {
+  return cost_blocks_per_sm(nv) <= 2
+             ? cost_variant<V, RAW, 16>(F, R, X, nstride, B, nv, chunks, cost, st)
+             : cost_variant<V, RAW, 8>(F, R, X, nstride, B, nv, chunks, cost, st);
 }
 
 }  // namespace
@@ -294,7 +341,7 @@ cudaError_t launch_pack_bits(const uint8_t* assign, int B, int n, int nstride, u
   const size_t tasks = (size_t)((n + 127) / 128) * W;
   const unsigned grid = (unsigned)std::min<size_t>((tasks + 7) / 8, (size_t)8 * sms());
   const bool aligned = ((reinterpret_cast<uintptr_t>(assign) | (uintptr_t)n) & 3u) == 0;
-  return launch_after(aligned ? k_pack_bits<true> : k_pack_bits<false>, dim3(grid), 0, st, assign,
+  return launch_after(aligned ? k_pack_bits<true> : k_pack_bits<false>, dim3(grid), 256, 0, st, assign,
                       B, n, W, nstride, X, cost, n_cost);
 }
 
@@ -306,10 +353,16 @@ cudaError_t launch_pack_rows(const uint8_t* xt, int Bp, int B, int n, int nstrid
   return cudaGetLastError();
 }
 
+cudaError_t launch_bits_slabs(const BitsFormula& F, cudaStream_t st) {
+  if (F.n_slabs == 0) return cudaSuccess;
+  k_bits_slabs<<<(unsigned)((F.n_slabs + 7) / 8), 256, 0, st>>>(F, 32 * F.n_slabs);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_bits_cost(const BitsFormula& F, const uint32_t* X, int nstride, int B,
                              int64_t* cost, cudaStream_t st) {
   if (F.m == 0) return cudaSuccess;
-  const int chunks = F.items ? F.n_items : cost_chunks((B + 31) / 32, F.m);
+  const int chunks = F.items ? F.n_items : cost_chunks((B + 31) / 32, F.n_slabs, F.n);
   return F.wide ? cost_launch<int64_t, false>(F, RawFormula{}, X, nstride, B, F.n, chunks, cost, st)
                 : cost_launch<int32_t, false>(F, RawFormula{}, X, nstride, B, F.n, chunks, cost, st);
 }
@@ -318,7 +371,7 @@ cudaError_t launch_bits_cost_raw(const RawFormula& R, const uint32_t* X, int nst
                                  int64_t* cost, cudaStream_t st) {
   if (R.m == 0) return cudaSuccess;
   return cost_launch<int64_t, true>(BitsFormula{}, R, X, nstride, B, R.n,
-                                    cost_chunks((B + 31) / 32, R.m), cost, st);
+                                    cost_chunks((B + 31) / 32, (R.m + 31) / 32, R.n), cost, st);
 }
 
 }  // namespace rbmsat

@@ -209,11 +209,18 @@ void up_chains(const UpFormula& F, int32_t B, const uint8_t* x, const float* nu,
 // 32 assignments per word, rows of nstride words, a multiple of 4)
 struct BitsFormula {
   int32_t n = 0, m = 0;  // variables of the largest formula; clauses of all
-  int32_t n_items = 0, wide = 0;  // wide: 32 consecutive clauses may weigh 2^31 or more
+  int32_t n_items = 0, wide = 0;  // wide: 32 clauses may weigh 2^31 or more
   const int32_t* off = nullptr;   // as DevFormula: literal offsets, literals, weights
   const int32_t* lits = nullptr;
   const int64_t* w = nullptr;
-  const int4* items = nullptr;    // batches: {first clause, end clause, formula, 0}; NULL: one formula
+  // slabs of 32 clauses of one formula in order of length, literal j of the 32
+  // side by side (rows of 32 literals), filled by launch_bits_slabs
+  int32_t n_slabs = 0;
+  const int32_t* perm = nullptr;  // [32 n_slabs]: clause at a position, or -1
+  const int2* slabs = nullptr;    // [n_slabs + 1]: {first literal row, formula}
+  int32_t* slab_lits = nullptr;
+  int64_t* slab_w = nullptr;      // [32 n_slabs]
+  const int4* items = nullptr;    // batches: {first slab, end slab, formula, 0}; NULL: one formula
   const int2* inst_vars = nullptr;  // per formula: {first variable, variables}
 };
 struct RawFormula {  // a caller's DIMACS arrays (maxsat_eval_noalloc)
@@ -231,6 +238,7 @@ cudaError_t launch_pack_bits(const uint8_t* assign, int B, int n, int nstride, u
 // X from the first B columns of n x Bp 0 / 1 bytes (Bp a multiple of 32)
 cudaError_t launch_pack_rows(const uint8_t* xt, int Bp, int B, int n, int nstride, uint32_t* X,
                              cudaStream_t st);
+cudaError_t launch_bits_slabs(const BitsFormula& F, cudaStream_t st);
 // adds the costs of B assignments to cost (n_inst x B, zeroed)
 cudaError_t launch_bits_cost(const BitsFormula& F, const uint32_t* X, int nstride, int B,
                              int64_t* cost, cudaStream_t st);

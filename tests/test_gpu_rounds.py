@@ -97,3 +97,30 @@ def test_rounds_match_oracle(ms, case, profiled):
     for k in ("cost", "best_cost", "best_x"):
         assert np.array_equal(g[k], getattr(st, k)), k
     np.testing.assert_allclose(g["free_energy"], st.free_energy, rtol=1e-3, atol=1e-6)
+
+
+@pytest.mark.parametrize("case", [c for c in CASES if not c.startswith("lengths")])
+def test_long_steps_match_oracle(ms, case):
+    """Steps of eight rounds and more: small formulas take all of a step's
+    rounds with one block per octet."""
+    import torch
+    make, B, temps, Q = CASES[case]
+    inst, alpha, seed = make(), 0.05, 22
+    table = table_for(temps, Q, 3)
+    p = ms.maxsat_default_params(sets=table.sets, n_temps=temps, n_buckets=2, alpha=alpha,
+                                 quant_bits=Q, path=ms.MAXSAT_PATH_SPARSE)
+    ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, torch.cuda.Stream())
+    ms.maxsat_reset(ctx, B, seed)
+    for steps in (8, 1, 11):
+        ms.maxsat_step(ctx, steps)
+    g = ms.maxsat_get_state(ctx)
+    ms.maxsat_destroy(ctx)
+    st = oracle.init_chains(inst.n, B, seed)
+    oracle.gibbs(inst, table, st, 20, seed, n_temps=temps, n_buckets=2, alpha=alpha,
+                 threads=os.cpu_count() or 4)
+    assert g["t"] == 20
+    assert np.array_equal(g["x"], st.x)
+    assert np.array_equal(g["nu"], st.nu32)
+    for k in ("cost", "best_cost", "best_x"):
+        assert np.array_equal(g[k], getattr(st, k)), k
+    np.testing.assert_allclose(g["free_energy"], st.free_energy, rtol=1e-3, atol=1e-6)
