@@ -66,6 +66,7 @@ CASES = {
     "lengths-thin-temperatures": (lambda: short_clauses(60, 200, 10, 9), 44, 6, 4),
     "lengths-wide-contributions": (lambda: short_clauses(60, 200, 11, 9), 256, 2, 8),
     "lengths-heavy": (lambda: short_clauses(60, 200, 12, 9, 2 ** 33), 256, 2, 4),
+    "lengths-0-12": (lambda: short_clauses(60, 300, 14, 12), 264, 2, 4),
     "lengths-high-degree": (lambda: short_clauses(12, 500, 13, 9), 300, 2, 4),
 }
 
@@ -77,7 +78,8 @@ def test_rounds_match_oracle(ms, case, profiled):
     import torch
     make, B, temps, Q = CASES[case]
     inst, alpha, seed = make(), 0.05, 21
-    table = table_for(temps, Q, 9 if case.startswith("lengths") else 3)
+    longest = 12 if case == "lengths-0-12" else 9 if case.startswith("lengths") else 3
+    table = table_for(temps, Q, longest)
     p = ms.maxsat_default_params(sets=table.sets, n_temps=temps, n_buckets=2, alpha=alpha,
                                  quant_bits=Q, path=ms.MAXSAT_PATH_SPARSE, steps_per_graph=4)
     ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, torch.cuda.Stream())
