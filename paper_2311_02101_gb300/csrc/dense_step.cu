@@ -35,6 +35,7 @@
 
 #include "dense_common.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 #include "philox.cuh"
 #include "round_ops.cuh"
 #include "tc_ptx.cuh"
@@ -61,14 +62,6 @@ __device__ __forceinline__ uint32_t step_index(const uint32_t* tdev, uint32_t t_
 }
 
 __host__ __device__ __forceinline__ int align16(int bytes) { return (bytes + 15) & ~15; }
-
-// Programmatic dependent launch between a round's three kernels: each sets up
-// (barriers, TMEM, tables) while its predecessor finishes, and waits for it
-// before it touches what the predecessor writes.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
 
 __device__ __forceinline__ void stage16(void* dst, const void* src, int bytes, int tid, int nthr) {
   const int4* s = reinterpret_cast<const int4*>(src);
@@ -1310,22 +1303,11 @@ __global__ void k_keep_copy_dense(const DevChains C, const uint8_t* X, uint8_t* 
 }
 
 template <typename... P, typename... Q>
-cudaError_t launch_pdl(void (*kern)(P...), int grid, int threads, int smem, cudaStream_t st,
-                       const Q&... args) {
+cudaError_t launch_step(void (*kern)(P...), int grid, int threads, int smem, cudaStream_t st,
+                        const Q&... args) {
   const cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
+  return e != cudaSuccess ? e : launch_pdl(kern, dim3((unsigned)grid), threads, smem, st, args...);
 }
 
 template <bool SAMPLE, bool SM, typename HT>
@@ -1336,14 +1318,14 @@ cudaError_t g1_variant(int grid, int smem, cudaStream_t st, const CUtensorMap& t
   auto kern = k_gemm1_step<SAMPLE, SM, HT, false, false>;
   if constexpr (SAMPLE && sizeof(HT) == 1)
     if (T.one_chunk) kern = k_gemm1_step<SAMPLE, SM, HT, true, false>;
-  return launch_pdl(kern, grid, 64 + 32 * kEpi1, smem, st, tmA, tmB, a, T, C);
+  return launch_step(kern, grid, 64 + 32 * kEpi1, smem, st, tmA, tmB, a, T, C);
 }
 
 template <bool SM, typename HT>
 cudaError_t g2_variant(int grid, int smem, cudaStream_t st, const CUtensorMap& tmA2,
                        const G2Args& a, const DevTables& T, const DevChains& C) {
   auto kern = k_gemm2<SM, HT>;
-  return launch_pdl(kern, grid, 64 + 32 * (kBld + kEpi2), smem, st, tmA2, a, T, C);
+  return launch_step(kern, grid, 64 + 32 * (kBld + kEpi2), smem, st, tmA2, a, T, C);
 }
 
 int sm_count() {
@@ -1406,7 +1388,7 @@ cudaError_t launch_gemm1_step(bool sample, const CUtensorMap& tmA, const CUtenso
   const int smem = base_smem + (sm ? tb : 0);
   const int grid = std::min(sm_count(), a.tiles_m * a.tiles_n);
   if (sample && C.nib)
-    return launch_pdl(k_gemm1_step<true, true, uint8_t, true, true>, grid, 64 + 32 * kEpi1,
+    return launch_step(k_gemm1_step<true, true, uint8_t, true, true>, grid, 64 + 32 * kEpi1,
                       base_smem + 256 + T.rec3_words * 4, st, tmA, tmB, a, T, C);
   if (sample) {
     if (sm) return wide ? g1_variant<true, true, uint16_t>(grid, smem, st, tmA, tmB, a, T, C)
@@ -1420,7 +1402,7 @@ cudaError_t launch_gemm1_step(bool sample, const CUtensorMap& tmA, const CUtenso
 
 cudaError_t launch_keep_dense(const int64_t* cost_part, const float* fe_part, int tiles_m,
                               const DevChains& C, cudaStream_t st) {
-  return launch_pdl(k_keep_dense, (C.Bp + 63) / 64, 64, 0, st, cost_part, fe_part, tiles_m, C);
+  return launch_step(k_keep_dense, (C.Bp + 63) / 64, 64, 0, st, cost_part, fe_part, tiles_m, C);
 }
 
 cudaError_t launch_gemm2(const CUtensorMap& tmA2, int n, int n_pad, int B, int Bp, int tiles_v,
@@ -1465,10 +1447,10 @@ cudaError_t launch_gemm2(const CUtensorMap& tmA2, int n, int n_pad, int B, int B
     if ((t256 * 2 + sms - 1) / sms < 2 * ((t256 + sms - 1) / sms)) {
       a.tiles_n = Bp / 128;
       a.idesc = tc::instr_desc(kBM, 128, fmt, fmt);
-      return launch_pdl(k_gemm2_nib<128>, std::min(sms, 2 * t256), threads,
+      return launch_step(k_gemm2_nib<128>, std::min(sms, 2 * t256), threads,
                         1024 + G2NibStage<128>::kTabOff + tbn, st, tmA2, a, T, C);
     }
-    return launch_pdl(k_gemm2_nib<256>, std::min(sms, t256), threads,
+    return launch_step(k_gemm2_nib<256>, std::min(sms, t256), threads,
                       1024 + G2NibStage<256>::kTabOff + tbn, st, tmA2, a, T, C);
   }
   const int tb = align16(T.gq_len * 4) + align16(T.pv_len * 4);

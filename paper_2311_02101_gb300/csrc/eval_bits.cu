@@ -34,17 +34,11 @@
 
 #include "internal.h"
 #include "dense_common.cuh"
+#include "pdl.cuh"
 
 namespace rbmsat {
 
 namespace {
-
-__device__ __forceinline__ void dependents_may_start() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void wait_for_predecessor() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
 
 // 4 bytes from p, any alignment; [lo, hi) is the readable range
 __device__ __forceinline__ uint32_t load4(const uint8_t* p, const uint8_t* lo, const uint8_t* hi) {
@@ -67,9 +61,9 @@ __global__ void __launch_bounds__(256) k_pack_bits(const uint8_t* __restrict__ a
                                                    int n, int W, int nstride,
                                                    uint32_t* __restrict__ X,
                                                    int64_t* __restrict__ cost, size_t n_cost) {
-  dependents_may_start();
+  pdl_release();
   // X and the costs may still be read or added into by the launch before
-  wait_for_predecessor();
+  pdl_wait();
   const size_t threads = (size_t)gridDim.x * blockDim.x;
   const size_t self = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (size_t k = self; k < n_cost; k += threads) cost[k] = 0;
@@ -187,7 +181,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawForm
   extern __shared__ __align__(16) uint32_t s_row[];
   __shared__ V s_lut[WARPS][128];
   __shared__ long long s_sum[WARPS][32];
-  dependents_may_start();
+  pdl_release();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int word = (int)blockIdx.x;
   // this block's clauses (RAW) or slabs begin .. end - 1, and its formula's
@@ -207,7 +201,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawForm
     v0 = vs.x;
     nv = vs.y;
   }
-  wait_for_predecessor();
+  pdl_wait();
   const uint32_t* row = X + (size_t)word * nstride + v0;
   if ((v0 & 3) == 0) {
 #pragma unroll 8
@@ -272,22 +266,6 @@ __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawForm
   }
 }
 
-template <typename... P, typename... Q>
-cudaError_t launch_after(void (*kern)(P...), dim3 grid, int threads, int smem, cudaStream_t st,
-                         Q... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 int sms() {
   static int count = 0;
   if (!count) {
@@ -320,7 +298,7 @@ cudaError_t cost_variant(const BitsFormula& F, const RawFormula& R, const uint32
   const int smem = row_bytes(nv);
   const cudaError_t e = allow_dynamic_smem(kern, smem);
   if (e != cudaSuccess) return e;
-  return launch_after(kern, dim3((unsigned)((B + 31) / 32), (unsigned)chunks), 32 * WARPS, smem, st,
+  return launch_pdl(kern, dim3((unsigned)((B + 31) / 32), (unsigned)chunks), 32 * WARPS, smem, st,
                       F, R, X, nstride, B, reinterpret_cast<unsigned long long*>(cost));
 }
 
@@ -341,7 +319,7 @@ cudaError_t launch_pack_bits(const uint8_t* assign, int B, int n, int nstride, u
   const size_t tasks = (size_t)((n + 127) / 128) * W;
   const unsigned grid = (unsigned)std::min<size_t>((tasks + 7) / 8, (size_t)8 * sms());
   const bool aligned = ((reinterpret_cast<uintptr_t>(assign) | (uintptr_t)n) & 3u) == 0;
-  return launch_after(aligned ? k_pack_bits<true> : k_pack_bits<false>, dim3(grid), 256, 0, st, assign,
+  return launch_pdl(aligned ? k_pack_bits<true> : k_pack_bits<false>, dim3(grid), 256, 0, st, assign,
                       B, n, W, nstride, X, cost, n_cost);
 }
 

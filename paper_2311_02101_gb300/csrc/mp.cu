@@ -39,6 +39,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pdl.cuh"
 #include "philox.cuh"
 
 namespace rbmsat {
@@ -80,6 +81,8 @@ __global__ void __launch_bounds__(256) k_mp_embed(DevFormula F, const __nv_bfloa
                                                   const __nv_bfloat16* Wg, int nbv, float* f,
                                                   float* g, float* inv_len, float* inv_deg,
                                                   float* hv, float* hc) {
+  pdl_wait();
+  pdl_release();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool var = (int)blockIdx.x < nbv;
   const int rows = var ? F.n : F.m;
@@ -310,6 +313,8 @@ __global__ void __launch_bounds__(256, 3) k_mp_fwd(DevFormula F, const float* sr
   RowList lists[4];
   row_lists<CL>(F, row_ranges<CL>(F, (int)blockIdx.x * kTile + hr, rows), c, lists);
   RowRanges next = row_ranges<CL>(F, ((int)blockIdx.x + step) * kTile + hr, rows);
+  pdl_wait();
+  pdl_release();
   for (int tile = blockIdx.x; tile < tiles; tile += step) {
     __syncthreads();  // weights staged; the previous tile's fragments are read
 #pragma unroll
@@ -411,6 +416,8 @@ __global__ void __launch_bounds__(256, 2)
     row_lists<CL>(F, row_ranges<CL>(F, (int)blockIdx.x * kTile + hr, rows), c, lists);
     next = row_ranges<CL>(F, ((int)blockIdx.x + step) * kTile + hr, rows);
   }
+  pdl_wait();
+  pdl_release();
   for (int tile = blockIdx.x; tile < tiles; tile += step) {
     __syncthreads();
 #pragma unroll
@@ -559,6 +566,8 @@ __global__ void __launch_bounds__(256) k_mp_embed_bwd(DevFormula F, int nbv, con
   const int blocks = var ? nbv : (int)gridDim.x - nbv;
   const int first = ((int)blockIdx.x - (var ? 0 : nbv)) * 8 + warp, step = blocks * 8;
   float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  pdl_wait();
+  pdl_release();
   auto add = [&](float2 d, float2 h, const float* x) {
     const float d0 = h.x > 0.f ? d.x : 0.f, d1 = h.y > 0.f ? d.y : 0.f;
 #pragma unroll
@@ -614,6 +623,8 @@ __global__ void __launch_bounds__(256) k_mp_embed_bwd(DevFormula F, int nbv, con
 // order (32 consecutive entries per load), then the eight sums in order.
 __global__ void __launch_bounds__(256) k_mp_sum(MpSums S) {
   __shared__ float s[8][32];
+  pdl_wait();
+  pdl_release();
   const MpSums::Set set = S.set[blockIdx.y];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int e = (int)blockIdx.x * 32 + lane;
@@ -645,6 +656,8 @@ __global__ void __launch_bounds__(256) k_mp_out(const float* h, int n, const flo
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float2 o = make_float2(__ldg(wo + 2 * lane), __ldg(wo + 2 * lane + 1));
   const float b = __ldg(bo);
+  pdl_wait();
+  pdl_release();
   double term = 0.0;
   float2 gw = make_float2(0.f, 0.f);
   float gb = 0.f;
@@ -794,8 +807,8 @@ cudaError_t mp_launch_embed(const DevFormula& F, const __nv_bfloat16* Wf, const 
                             float* f, float* g, float* inv_len, float* inv_deg, float* hv,
                             float* hc, cudaStream_t st) {
   const int nbv = blocks(F.n, 256), nbc = blocks(F.m, 256);
-  k_mp_embed<<<nbv + nbc, 256, 0, st>>>(F, Wf, Wg, nbv, f, g, inv_len, inv_deg, hv, hc);
-  return cudaGetLastError();
+  return launch_pdl(k_mp_embed, nbv + nbc, 256, 0, st, F, Wf, Wg, nbv, f, g, inv_len, inv_deg, hv,
+                    hc);
 }
 
 cudaError_t mp_launch_fwd(const DevFormula& F, bool clauses, const float* src,
@@ -807,8 +820,8 @@ cudaError_t mp_launch_fwd(const DevFormula& F, bool clauses, const float* src,
   const cudaError_t e = allow_dynamic_smem(kern, kFwdSmem);
   if (e != cudaSuccess) return e;
   const int grid = std::min(blocks(rows, kTile), 3 * mp_sms());
-  kern<<<grid, 256, kFwdSmem, st>>>(F, src, out_scale, self, rows, W, b, agg_out, out);
-  return cudaGetLastError();
+  return launch_pdl(kern, grid, 256, kFwdSmem, st, F, src, out_scale, self, rows, W, b, agg_out,
+                    out);
 }
 
 cudaError_t mp_launch_bwd(const DevFormula& F, bool clauses, const float* src,
@@ -820,9 +833,8 @@ cudaError_t mp_launch_bwd(const DevFormula& F, bool clauses, const float* src,
   auto kern = clauses ? k_mp_bwd<true> : k_mp_bwd<false>;
   const cudaError_t e = allow_dynamic_smem(kern, kBwdSmem);
   if (e != cudaSuccess) return e;
-  kern<<<mp_bwd_blocks(rows), 256, kBwdSmem, st>>>(F, src, in_scale, carry, dz, wo, out, agg, self,
-                                                   rows, W, dA, dB, part);
-  return cudaGetLastError();
+  return launch_pdl(kern, mp_bwd_blocks(rows), 256, kBwdSmem, st, F, src, in_scale, carry, dz, wo,
+                    out, agg, self, rows, W, dA, dB, part);
 }
 
 cudaError_t mp_launch_embed_bwd(const DevFormula& F, const float* src, const float* in_scale,
@@ -830,24 +842,22 @@ cudaError_t mp_launch_embed_bwd(const DevFormula& F, const float* src, const flo
                                 const float* carry_c, const float* hc, const float* g, float* part,
                                 cudaStream_t st) {
   const int nbv = mp_embed_bwd_var_blocks(F.n), nbc = mp_embed_bwd_clause_blocks(F.m);
-  k_mp_embed_bwd<<<nbv + nbc, 256, 0, st>>>(F, nbv, src, in_scale, carry_v, hv, f, carry_c, hc, g,
-                                            part);
-  return cudaGetLastError();
+  return launch_pdl(k_mp_embed_bwd, nbv + nbc, 256, 0, st, F, nbv, src, in_scale, carry_v, hv, f,
+                    carry_c, hc, g, part);
 }
 
 cudaError_t mp_launch_sums(const MpSums& S, cudaStream_t st) {
   int most = 0;
   for (int k = 0; k < S.sets; ++k) most = std::max(most, S.set[k].count);
-  k_mp_sum<<<dim3(blocks(most, 32), S.sets), 256, 0, st>>>(S);
-  return cudaGetLastError();
+  return launch_pdl(k_mp_sum, dim3(blocks(most, 32), S.sets), 256, 0, st, S);
 }
 
 cudaError_t mp_launch_out(const float* h, int n, const float* wo, const float* bo,
                           const uint8_t* y, float* prob, float* dz, double* loss_part, float* part,
                           cudaStream_t st) {
-  if (n > 0)
-    k_mp_out<<<mp_out_blocks(n), 256, 0, st>>>(h, n, wo, bo, y, prob, dz, loss_part, part);
-  return cudaGetLastError();
+  if (n <= 0) return cudaSuccess;
+  return launch_pdl(k_mp_out, mp_out_blocks(n), 256, 0, st, h, n, wo, bo, y, prob, dz, loss_part,
+                    part);
 }
 
 cudaError_t mp_launch_adam(float* P, const float* G, float* M, float* V, int count, float lr,

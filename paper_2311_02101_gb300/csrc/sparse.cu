@@ -32,6 +32,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "pdl.cuh"
 #include "philox.cuh"
 #include "round_ops.cuh"
 
@@ -52,16 +53,9 @@ __device__ __forceinline__ void stage(void* dst, const void* src, int bytes) {
 
 __host__ __device__ __forceinline__ int align16(int bytes) { return (bytes + 15) & ~15; }
 
-// Programmatic dependent launch between the rounds' kernels: a gather or
-// visible launch may start while its predecessor in the stream finishes. It
-// lets its own dependent start early (release), stages its constant tables,
-// and waits for the predecessor's completion and memory (griddepcontrol.wait)
-// before it reads or writes any chain state. Without a programmatic
-// predecessor both are no-ops.
-__device__ __forceinline__ void pdl_release() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Between the rounds' kernels a launch lets its own dependent start early
+// (pdl_release first), stages its constant tables, and waits before it reads or
+// writes any chain state. Without a programmatic predecessor both are no-ops.
 
 // (instance, index within it) of variable i
 __device__ __forceinline__ int2 var_instance(const DevFormula& F, int i) {
@@ -1726,23 +1720,6 @@ constexpr int kNibSmemLimit = 76 * 1024;  // with windows of 16 rows two blocks 
 int l2_bytes();
 constexpr int kMaxGridY = 65535;
 
-// a launch that may overlap its predecessor's tail (see pdl_wait)
-template <typename... Params, typename... Args>
-cudaError_t launch_pdl(void (*kern)(Params...), dim3 grid, int smem, cudaStream_t st,
-                       Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 // dynamic shared memory of k_gather3: the record blocks plus the slack that
 // moves them to a 256-byte boundary
 int gather3_smem_bytes(const DevTables& T) { return T.rec3_words * 4 + 256; }
@@ -1784,7 +1761,7 @@ cudaError_t gather_variant(dim3 grid, int smem, cudaStream_t st, const DevFormul
       auto kern = C.nib ? gather3_kernel<true>(T, C) : gather3_kernel<false>(T, C);
       const cudaError_t e = allow_dynamic_smem(kern, sm3);
       if (e != cudaSuccess) return e;
-      return launch_pdl(kern, grid, sm3, st, F, T, C, P, tdev, t_rel, cost_part, fe_part,
+      return launch_pdl(kern, grid, 256, sm3, st, F, T, C, P, tdev, t_rel, cost_part, fe_part,
                         tickets);
     }
   }
@@ -1797,7 +1774,7 @@ cudaError_t gather_variant(dim3 grid, int smem, cudaStream_t st, const DevFormul
     if (e != cudaSuccess) return e;
   }
   if constexpr (MODE == kStep)
-    return launch_pdl(kern, grid, smem, st, F, T, C, xt, B, Bp, P, tdev, t_rel, cost_part,
+    return launch_pdl(kern, grid, 256, smem, st, F, T, C, xt, B, Bp, P, tdev, t_rel, cost_part,
                       fe_part, tickets, eval_out);
   kern<<<grid, 256, smem, st>>>(F, T, C, xt, B, Bp, P, tdev, t_rel, cost_part, fe_part, tickets,
                                 eval_out);
@@ -1825,7 +1802,7 @@ cudaError_t gather_mode(dim3 grid, cudaStream_t st, bool wide, const DevFormula&
       const int smn = gather_nib_smem_bytes(T);
       const cudaError_t e = allow_dynamic_smem(k_gather_nib, smn);
       if (e != cudaSuccess) return e;
-      return launch_pdl(k_gather_nib, grid, smn, st, F, T, C, P, tdev, t_rel, cost_part, fe_part,
+      return launch_pdl(k_gather_nib, grid, 256, smn, st, F, T, C, P, tdev, t_rel, cost_part, fe_part,
                         tickets);
     }
   }
@@ -1862,14 +1839,14 @@ cudaError_t visible_variant(dim3 grid, int smem, cudaStream_t st, const DevFormu
     grid.x = (unsigned)groups;
     for (int t0 = 0; t0 < tiles; t0 += kMaxGridY) {
       grid.y = std::min(kMaxGridY, tiles - t0);
-      const cudaError_t e = launch_pdl(kern, grid, smem, st, F, T, C, alpha, tdev, t_rel, t0, tm);
+      const cudaError_t e = launch_pdl(kern, grid, 256, smem, st, F, T, C, alpha, tdev, t_rel, t0, tm);
       if (e != cudaSuccess) return e;
     }
   } else {
     // x = chain tiles, y = variable groups (launches of at most kMaxGridY groups)
     for (int vg0 = 0; vg0 < groups; vg0 += kMaxGridY) {
       grid.y = std::min(kMaxGridY, groups - vg0);
-      const cudaError_t e = launch_pdl(kern, grid, smem, st, F, T, C, alpha, tdev, t_rel, vg0, tm);
+      const cudaError_t e = launch_pdl(kern, grid, 256, smem, st, F, T, C, alpha, tdev, t_rel, vg0, tm);
       if (e != cudaSuccess) return e;
     }
   }
@@ -1913,7 +1890,7 @@ cudaError_t visible_nib_window(const DevFormula& F, const DevTables& T, const De
   const long long items = (long long)F.n * (C.Bp / kChainTile);
   const long long grid = std::min<long long>((items + 7) / 8, (long long)BLOCKS * sm_count());
   const int tm = (double)F.h_rows * C.Bp * 0.5 > 0.5 * (double)l2_bytes() ? 1 : 0;
-  return launch_pdl(kern, dim3((unsigned)grid), smem, st, F, T, C, keep, tdev, t_rel, tm);
+  return launch_pdl(kern, dim3((unsigned)grid), 256, smem, st, F, T, C, keep, tdev, t_rel, tm);
 }
 
 cudaError_t visible_nib(const DevFormula& F, const DevTables& T, const DevChains& C, float alpha,
