@@ -677,28 +677,47 @@ int upload(maxsat_ctx* ctx, DevAllocs& A, std::vector<T> h, const T** out) {
   return MAXSAT_OK;
 }
 
-// Collects host arrays for one device block and one copy (a copy of its own per
-// array costs a create about 10 us each). Every array starts 256-byte aligned
-// and is padded with zeros to a multiple of 16 bytes; the pointers are set by
-// commit.
+// Uploads of a create. Small arrays are collected for one device block and one
+// copy (a copy of its own per array costs a create about 10 us each); one of
+// 256 KB and more is copied at once, rather than a second time on the host.
+// Every array is padded with zeros to a multiple of 16 bytes; the collected ones
+// start 256-byte aligned, and commit sets their pointers.
 class UploadArena {
  public:
+  UploadArena(maxsat_ctx* ctx, DevAllocs& A) : ctx_(ctx), A_(A) {}
   template <class T>
   void add(const std::vector<T>& h, const T** out) {
     const size_t at = buf_.size(), bytes = std::max<size_t>(h.size() * sizeof(T), sizeof(T));
+    if (bytes >= 256 * 1024) {
+      if (rc_ == MAXSAT_OK) rc_ = copy(h.data(), bytes, out);
+      return;
+    }
     buf_.resize(at + (bytes + 255) / 256 * 256, 0);
     if (!h.empty()) std::memcpy(buf_.data() + at, h.data(), h.size() * sizeof(T));
     outs_.emplace_back(at, reinterpret_cast<const void**>(out));
   }
-  int commit(maxsat_ctx* ctx, DevAllocs& A) {
-    uint8_t* d = nullptr;
-    CK(ctx, A.alloc(&d, buf_.size()));
-    CK(ctx, cudaMemcpy(d, buf_.data(), buf_.size(), cudaMemcpyHostToDevice));
+  int commit() {
+    if (rc_ != MAXSAT_OK) return rc_;
+    const uint8_t* d = nullptr;
+    const int rc = copy(buf_.data(), buf_.size(), &d);
     for (auto& o : outs_) *o.second = d + o.first;
-    return MAXSAT_OK;
+    return rc;
   }
 
  private:
+  template <class T>
+  int copy(const void* h, size_t bytes, const T** out) {
+    const size_t padded = (bytes + 15) / 16 * 16;
+    uint8_t* d = nullptr;
+    CK(ctx_, A_.alloc(&d, padded));
+    CK(ctx_, cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice));
+    if (padded > bytes) CK(ctx_, cudaMemset(d + bytes, 0, padded - bytes));
+    *out = reinterpret_cast<const T*>(d);
+    return MAXSAT_OK;
+  }
+  maxsat_ctx* ctx_;
+  DevAllocs& A_;
+  int rc_ = MAXSAT_OK;
   std::vector<uint8_t> buf_;
   std::vector<std::pair<size_t, const void**>> outs_;
 };
@@ -1376,7 +1395,9 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   T.gq_len = (int32_t)ctx->tabs.gq.size();
   T.pv_len = (int32_t)ctx->tabs.pv.size();
   ctx->wide_h = ctx->tabs.max_nh > 8;
-  UploadArena arena;
+  UploadArena arena(ctx, A);
+  int64_t n_inc8 = -1;  // entries of var_inc8 (-1: not built)
+  const int4* inc_groups = nullptr;
 #define UP(vec, dst) arena.add(vec, &(dst))
   UP(cl_off, F.cl_off);
   UP(lit_var, F.lit_var);
@@ -1490,21 +1511,12 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
         for (int i = 0; i < n; ++i) inc_off[i + 1] += inc_off[i];
       }
       const std::vector<int32_t>& ioff = T.one_chunk ? var_off : inc_off;
-      std::vector<int2> inc8((size_t)pseudo);
-      {
-        std::vector<int32_t> fill(ioff.begin(), ioff.end() - 1);
-        for (int64_t c = 0; c < m; ++c) {
-          const int g = cl_grp[c], len = (int)(off[c + 1] - off[c]);
-          for (int k = 0; k < len; ++k) {
-            const int32_t l = lits[off[c] + k];
-            int32_t& at = fill[(l > 0 ? l : -l) - 1];
-            for (int j = 0; j < chunks[g]; ++j)
-              inc8[at++] = make_int2(T.one_chunk ? (int32_t)c : hrow[c] + j,
-                                     16 * (row0[g] + (j * len + k) * 2 + (l < 0 ? 1 : 0)));
-          }
-        }
-      }
-      UP(inc8, F.var_inc8);
+      // the lists are written on the device, from var_inc, once it is there
+      n_inc8 = pseudo;
+      std::vector<int4> groups(G);
+      for (int g = 0; g < G; ++g)
+        groups[g] = make_int4(row0[g], chunks[g], H.meta[g].len, H.meta[g].gq_off);
+      UP(groups, inc_groups);
       std::vector<int4> slots(n);
       for (int k = 0; k < n_inst; ++k)
         for (int s = var_base[k]; s < var_base[k + 1]; ++s) {
@@ -1536,7 +1548,10 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
           lcl[c] = make_uint2(v[0] | (v[1] << 16), v[2] | (info << 16));
         }
         for (int64_t j = 0; j < nnz && fits; ++j)
-          linc[j] = (uint32_t)inc8[j].x | ((uint32_t)(inc8[j].y / 16) << 16);
+          linc[j] = (uint32_t)var_inc[j].x |
+                    ((uint32_t)contribution_row(groups[cl_grp[var_inc[j].x]], (int)H.gq.size(),
+                                                var_inc[j].y, 0)
+                     << 16);
         if (fits) {
           UP(lcl, ctx->local.cl);
           UP(linc, ctx->local.inc);
@@ -1647,34 +1662,37 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     for (int64_t c = 0; c < m && !E.wide; ++c)
       if (cl_w[c] >= ((int64_t)1 << 26)) E.wide = 1;  // 32 of them below 2^31
     std::vector<int32_t> perm;
-    std::vector<int2> slabs, vars;
-    std::vector<int4> items;
+    std::vector<int4> slabs, items;
+    std::vector<int2> vars;
     int64_t& rows = slab_rows;
     const int64_t run = std::max<int64_t>(64, m / 1048576 + 1);
+    bool one_length = true;  // of every clause: they keep their order
+    for (int64_t c = 1; c < m && one_length; ++c)
+      one_length = cl_off[c + 1] - cl_off[c] == cl_off[1];
     for (int k = 0; k < n_inst && E.n <= kBitsMaxVars; ++k) {
-      int64_t at[MAXSAT_MAX_LEN + 2] = {0};
-      for (int c = cl_base[k]; c < cl_base[k + 1]; ++c) ++at[cl_off[c + 1] - cl_off[c] + 1];
-      for (int len = 1; len <= MAXSAT_MAX_LEN; ++len) at[len] += at[len - 1];
-      const size_t p0 = perm.size();
-      const int s0 = (int)slabs.size();
-      perm.resize(p0 + (cl_base[k + 1] - cl_base[k] + 31) / 32 * 32, -1);
-      for (int c = cl_base[k]; c < cl_base[k + 1]; ++c)
-        perm[p0 + at[cl_off[c + 1] - cl_off[c]]++] = c;
-      for (size_t p = p0; p < perm.size(); p += 32) {
-        int last = 31;  // the slab's longest clause
-        while (perm[p + last] < 0) --last;
-        const int c = perm[p + last];
-        slabs.push_back(make_int2((int)rows, k));
+      const int c0 = cl_base[k], mk = cl_base[k + 1] - c0;
+      const size_t p0 = perm.size(), s0 = slabs.size();
+      if (!one_length) {
+        int64_t at[MAXSAT_MAX_LEN + 2] = {0};
+        for (int c = c0; c < c0 + mk; ++c) ++at[cl_off[c + 1] - cl_off[c] + 1];
+        for (int len = 1; len <= MAXSAT_MAX_LEN; ++len) at[len] += at[len - 1];
+        perm.resize(p0 + (mk + 31) / 32 * 32, -1);
+        for (int c = c0; c < c0 + mk; ++c) perm[p0 + at[cl_off[c + 1] - cl_off[c]]++] = c;
+      }
+      for (int p = 0; p < mk; p += 32) {
+        const int cnt = std::min(32, mk - p);
+        const int c = one_length ? c0 : perm[p0 + p + cnt - 1];  // the slab's longest
+        slabs.push_back(make_int4((int)rows, k, c0 + p, cnt));
         rows += cl_off[c + 1] - cl_off[c];
       }
       vars.push_back(make_int2(var_base[k], var_base[k + 1] - var_base[k]));
-      for (int64_t q = s0; n_inst > 1 && q < (int64_t)slabs.size(); q += run)
+      for (size_t q = s0; n_inst > 1 && q < slabs.size(); q += run)
         items.push_back(make_int4((int)q, (int)std::min<int64_t>(slabs.size(), q + run), k, 0));
     }
     E.n_slabs = (int32_t)slabs.size();
     E.n_items = (int32_t)items.size();
-    slabs.push_back(make_int2((int)rows, 0));
-    UP(perm, E.perm);
+    slabs.push_back(make_int4((int)rows, 0, 0, 0));
+    if (!one_length) UP(perm, E.perm);
     UP(slabs, E.slabs);
     UP(vars, E.inst_vars);
     if (n_inst > 1) UP(items, E.items);
@@ -1699,12 +1717,24 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   }
   UP(ctx->tabs.pv, T.pv);
   {
-    const int rca = arena.commit(ctx, A);
+    const int rca = arena.commit();
     if (rca != MAXSAT_OK) {
       std::string e_ = ctx->err;
       delete ctx;
       return fail(nullptr, rca, e_);
     }
+  }
+  if (n_inc8 >= 0) {
+    int2* inc8 = nullptr;
+    cudaError_t e = A.alloc(&inc8, (size_t)std::max<int64_t>(1, n_inc8));
+    if (e == cudaSuccess)
+      e = launch_inc_rows(F, inc_groups, (int)ctx->tabs.gq.size(), T.one_chunk != 0, inc8,
+                          ctx->stream);
+    if (e != cudaSuccess) {
+      delete ctx;
+      return cuda_fail(nullptr, e, "incidence lists");
+    }
+    F.var_inc8 = inc8;
   }
   ctx->bits.off = F.cl_off;
   ctx->bits.lits = F.lit_var;
@@ -2233,7 +2263,6 @@ int maxsat_get_state(maxsat_ctx* ctx, uint8_t* x, float* nu, int64_t* best_cost,
   if (!ctx) return MAXSAT_EINVAL;
   if (!ctx->have_chains) return fail(ctx, MAXSAT_ESTATE, "no chains (call maxsat_reset)");
   const int B = ctx->C.B, Bp = ctx->C.Bp, n = ctx->n;
-  const size_t nB = (size_t)n * Bp;
   if (ctx->dense) {
     const int np = ctx->n_pad;
     uint8_t one;
@@ -2293,7 +2322,6 @@ int maxsat_set_state(maxsat_ctx* ctx, int32_t B, uint64_t seed, const uint8_t* x
   if (rc != MAXSAT_OK) return rc;
   CK(ctx, cudaStreamSynchronize(ctx->stream));
   const int Bp = ctx->C.Bp, n = ctx->n;
-  const size_t nB = (size_t)n * Bp;
   if (ctx->dense) {
     const int np = ctx->n_pad;
     uint8_t one, minus_one;

@@ -157,9 +157,9 @@ __global__ void __launch_bounds__(256) k_bits_slabs(BitsFormula F, int n_pos) {
   const int pos = (int)(blockIdx.x * 256 + threadIdx.x);
   if (pos >= n_pos) return;
   const int lane = pos & 31;
-  const int2 sl = F.slabs[pos >> 5];  // {first literal row, formula}
+  const int4 sl = F.slabs[pos >> 5];
   const int rows = F.slabs[(pos >> 5) + 1].x - sl.x;
-  const int c = F.perm[pos];
+  const int c = lane >= sl.w ? -1 : F.perm ? F.perm[pos] : sl.z + lane;
   const int2 vs = F.inst_vars[sl.y];
   int32_t* out = F.slab_lits + (size_t)sl.x * 32 + lane;
   int o = 0, len = 0;

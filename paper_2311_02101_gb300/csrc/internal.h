@@ -216,8 +216,9 @@ struct BitsFormula {
   // slabs of 32 clauses of one formula in order of length, literal j of the 32
   // side by side (rows of 32 literals), filled by launch_bits_slabs
   int32_t n_slabs = 0;
-  const int32_t* perm = nullptr;  // [32 n_slabs]: clause at a position, or -1
-  const int2* slabs = nullptr;    // [n_slabs + 1]: {first literal row, formula}
+  const int32_t* perm = nullptr;  // [32 n_slabs]: clause at a position (NULL: in order)
+  // [n_slabs + 1]: {first literal row, formula, first clause if in order, clauses}
+  const int4* slabs = nullptr;
   int32_t* slab_lits = nullptr;
   int64_t* slab_w = nullptr;      // [32 n_slabs]
   const int4* items = nullptr;    // batches: {first slab, end slab, formula, 0}; NULL: one formula
@@ -386,6 +387,17 @@ int gather_blocks_per_sm(const DevTables& T, bool wide_h);
 
 // sparse.cu launchers (all asynchronous on `st`)
 enum GatherMode { kStep = 0, kScore = 1, kEval = 2 };
+// Row (of 16 bytes) of the contributions that an incidence gets from chunk j of
+// its clause's hidden units: group {first row, chunks, length, gq_off}, y as in
+// var_inc (gq_off + position, plus gq_len and bit 31 if negated).
+__host__ __device__ inline int contribution_row(const int4& group, int gq_len, int32_t y, int j) {
+  const int neg = y < 0 ? 1 : 0;
+  const int k = (y & 0x7FFFFFFF) - (neg ? gq_len : 0) - group.w;
+  return group.x + (j * group.z + k) * 2 + neg;
+}
+// writes var_inc8 from var_inc
+cudaError_t launch_inc_rows(const DevFormula& F, const int4* groups, int gq_len, bool one_chunk,
+                            int2* inc8, cudaStream_t st);
 cudaError_t launch_init_sparse(const DevFormula& F, const DevChains& C, int n, cudaStream_t st);
 // kStep: cost, free energy, hidden draws, then (last block of each instance
 // and chain tile) best-keep; kScore: the same without draws; kEval: cost only,
