@@ -108,8 +108,9 @@ typedef struct {
                             passes with CUDA events, and keep the fastest.
                             Costs, states and draws do not depend on either;
                             the free energy's float summation order depends
-                            on the blocking. Default 0 (the wave-fitted size,
-                            batch 4) */
+                            on the blocking. Hidden patterns of 4 bits have
+                            no load batch to measure. Default 0 (the
+                            wave-fitted size, batch 4) */
   int32_t up_device;     /* 1: maxsat_up_begin / maxsat_up_end run unit
                             propagation and the merge on the GPU when the
                             chains are on the sparse path and one chain's
@@ -122,7 +123,9 @@ typedef struct {
   int32_t visible_batch; /* incidences per thread whose hidden-pattern loads
                             the sparse visible update keeps in flight: 2, 4
                             or 8, or 0 for 4 unless tune_blocks measures
-                            another. Same results for every value. Default 0 */
+                            another. Same results for every value; no effect
+                            where hidden patterns take 4 bits (that update
+                            copies whole windows ahead). Default 0 */
   int32_t persistent_round; /* 1: maxsat_step runs its sparse rounds as one
                             persistent cooperative launch per
                             max(1, steps_per_graph) rounds: every block
@@ -136,9 +139,13 @@ typedef struct {
                             without profiling and while no GPU unit
                             propagation is pending; otherwise the two-launch
                             round runs (maxsat_get_persistent_round tells).
-                            Same results bit for bit. Default 0 (two launches
-                            per round with programmatic dependent launch,
-                            replayed from CUDA graphs) */
+                            Same results bit for bit. Default 0: one formula
+                            of clauses of at most 3 literals with 4-bit hidden
+                            patterns runs many rounds per launch too (each
+                            tile of 256 chains with barriers of its own, or
+                            small formulas one block per 8 chains); the rest
+                            takes two launches per round with programmatic
+                            dependent launch, replayed from CUDA graphs */
 } maxsat_params;
 
 typedef struct maxsat_ctx maxsat_ctx;

@@ -435,9 +435,9 @@ int plan_blocks(const maxsat_ctx* ctx, int cb) {
 // Clauses per gather block for `tiles` chain tiles. A batch's formulas are split
 // one by one, so that the rule for one formula gives some blocks more than fit
 // at once (96 formulas, 500 blocks on 456 places: the 44 left over cost a launch
-// 23 % of its time, 348 us against 261). A batch takes the smallest size whose blocks fill one, two,
-// ... waves, whichever keeps the places busiest when a block's start costs as
-// much as 16 clauses.
+// 23 % of its time, 348 us against 261). A batch takes the smallest size whose
+// blocks fill one, two, ... waves, whichever keeps the places busiest when a
+// block's start costs as much as 16 clauses.
 int fitted_clause_block(const maxsat_ctx* ctx, int tiles) {
   const int slots = ctx->gather_slots;
   if (ctx->n_inst == 1 || ctx->m <= 0 || slots <= 0)
@@ -1729,7 +1729,7 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     cudaError_t e = A.alloc(&inc8, (size_t)std::max<int64_t>(1, n_inc8));
     if (e == cudaSuccess)
       e = launch_inc_rows(F, inc_groups, (int)ctx->tabs.gq.size(), T.one_chunk != 0, inc8,
-                          ctx->stream);
+                          nullptr);
     if (e != cudaSuccess) {
       delete ctx;
       return cuda_fail(nullptr, e, "incidence lists");
@@ -1743,7 +1743,10 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     cudaError_t e = A.alloc(&ctx->bits.slab_lits, 32 * (size_t)std::max<int64_t>(1, slab_rows));
     if (e == cudaSuccess)
       e = A.alloc(&ctx->bits.slab_w, 32 * (size_t)std::max(1, ctx->bits.n_slabs));
-    if (e == cudaSuccess) e = launch_bits_slabs(ctx->bits, ctx->stream);
+    if (e == cudaSuccess) e = launch_bits_slabs(ctx->bits, nullptr);
+    // like the copies above, finished when the context is handed out, whatever
+    // its stream is doing
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
       delete ctx;
       return cuda_fail(nullptr, e, "clause slabs");

@@ -10,12 +10,14 @@
 // MAXSAT_NOALLOC_SCRATCH_BYTES bytes that every GPU that loads the library
 // holds until the process exits.
 //
-// It is a variant of the sparse evaluation pipeline of sparse.cu (transpose
-// the assignments to variable-major, gather the literal truths of every clause
-// for 8 chains per thread, reduce the per-block weighted costs), reading the
-// DIMACS clause lists directly instead of the context's converted copy.
+// Up to kBitsMaxVars variables it packs the assignments to one bit per variable
+// into the scratch and scores them there (eval_bits.cu, reading the DIMACS lists
+// as they are). Larger formulas take a variant of the sparse evaluation pipeline
+// of sparse.cu (transpose the assignments to variable-major, gather the literal
+// truths of every clause for 8 chains per thread, reduce the per-block weighted
+// costs), again on the DIMACS lists.
 //
-// Scratch layout: [transposed assignments: n x Bp bytes][cost partials:
+// Scratch layout of the latter: [transposed assignments: n x Bp bytes][cost partials:
 // blocks x Bp int64], Bp = B rounded up to 256. Every call overwrites all of
 // the scratch it reads, so nothing has to start at zero; calls that overlap on
 // the GPU (on different streams, or from different host threads) share the

@@ -9,7 +9,9 @@
 //              variable-major state), forms each chain's truth pattern, adds
 //              the weight of unsatisfied clauses and the clause free energy
 //              (Eq. 1), draws the hidden units (Eq. 2 / Eq. 6) and stores the
-//              hidden pattern (one byte per clause and chain). The last block
+//              hidden pattern (one byte per clause and chain; 4 bits per chunk
+//              of three hidden units in k_gather3 and k_gather_nib, which run
+//              wherever nib_patterns_supported allows). The last block
 //              to finish a tile of 256 chains reduces the per-block costs in a
 //              fixed order and keeps improving states (Sec. 4.2).
 //   k_visible  one thread = one variable x 8 chains: pull-based scatter-sum
@@ -17,7 +19,11 @@
 //              selected by the clause's hidden pattern (Eq. 7; integer sums,
 //              no atomics, deterministic), draws the new visible states
 //              (Eq. 3), updates nu (Sec. 4.4) and copies improved states into
-//              the best-so-far before they are overwritten.
+//              the best-so-far before they are overwritten. k_visible_nib is
+//              the form for 4-bit patterns.
+//   k_rounds   both phases of many rounds in one launch (one formula of
+//              clauses of at most 3 literals); local.cu has the form for
+//              formulas that fit one block's shared memory.
 // State layout: x and nu are variable-major (n x Bp) so 8 consecutive chains of
 // one variable are one 8-byte (x) or 32-byte (nu) access. The small
 // probability tables are staged in shared memory when they fit.
@@ -407,9 +413,10 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
 //    the current one is sampled, and each block first asks the L2 for its
 //    slice of the chain tile's state rows and for its clause records and
 //    weights (bulk prefetches), so the loop rarely waits on DRAM after the
-//    previous round's writes. 2 blocks of 256 threads per SM (no spills;
-//    measured faster than 3 or 4 blocks with spills, and than two clauses per
-//    loop trip).
+//    previous round's writes. 3 blocks of 256 threads per SM at 80 registers
+//    (with 4-bit patterns; 47 us a launch at weighted 3-SAT n = 1000, m = 6000,
+//    4096 chains, 190 M warp instructions at 59 % issue for 686000 clauses and
+//    256 chains, the multiplier pipe of the Philox rounds 69 % busy).
 // ---------------------------------------------------------------------------
 // Asks the L2 to fetch `bytes` (a multiple of 16) from a 16-byte aligned
 // global address (a bulk prefetch: no data returns to the thread).
@@ -727,7 +734,12 @@ __global__ void __launch_bounds__(256, 3) k_gather3(DevFormula F, DevTables T, D
 // few patterns (most clauses) keep their records in shared memory (the host
 // orders the groups by size; the first T.recn_smem words are staged), costs
 // stay in registers, and the next clause's record, literals and states are
-// loaded while the current one is sampled.
+// loaded while the current one is sampled: 367 us, 232 M warp instructions at
+// 54 % issue. Slower or no faster: the next clause's states in rows of shared
+// memory by cp.async (543 us: the rows take the L1 that the long clauses'
+// records are read through), eight states ahead in registers (371 us), fewer
+// staged records (343 us a launch at 24 KB, but a round of both kernels 501 us
+// against 494, as the SM's shared memory is divided anew between them).
 // ---------------------------------------------------------------------------
 struct ChunkAddr {
   uint32_t off[8];  // byte address (shared memory) or byte offset (global) per chain
@@ -1135,7 +1147,9 @@ __global__ void __launch_bounds__(256, BATCH >= 8 ? 3 : 4) k_visible(DevFormula 
 // the tile per warp instruction) while the current one is summed. Loads of the
 // patterns into registers, 4 or 8 at a time, left the kernel waiting on the L2
 // (long scoreboard 11.7 of 18 cycles per issue, 27 us a launch at n = 1000, m =
-// 6000, 4096 chains; 200 us at mixed lengths, n = 20000, m = 100000, 1024 chains).
+// 6000, 4096 chains; 200 us at mixed lengths, n = 20000, m = 100000, 1024 chains;
+// now 142 us there, and 163 us for 96 formulas of 686000 clauses and 256 chains,
+// of which its 390 MB of DRAM traffic would take 57).
 // ---------------------------------------------------------------------------
 struct VisPos {  // position in the walk over (chain tile, variable slot)
   int fast, slow;
@@ -1340,8 +1354,8 @@ __global__ void __launch_bounds__(256, BLOCKS)
 // blocks (blocks tile, tile + tiles, ...) that runs the tile's rounds alone:
 // every block gathers its share of the clauses, the group meets at its own
 // barrier, every warp updates its share of the variables, the group meets
-// again. An SM holds two blocks, mostly of different tiles, so one computes
-// while the other waits. The states, costs and draws are those of the
+// again. An SM holds up to three blocks, mostly of different tiles, so others
+// compute while one waits. The states, costs and draws are those of the
 // two-launch round, bit for bit.
 //
 // What bounds the two-launch round is not its arithmetic alone (weighted 3-SAT
@@ -1350,7 +1364,8 @@ __global__ void __launch_bounds__(256, BLOCKS)
 // tables and its last wave (a round of 256 chains of the same formula, 1/16 of
 // the work, takes 24.9 us; of n = 50, m = 215, 10.5 us), and the gather's last
 // block adds the partial sums of all blocks one after another (300 of them at
-// 256 chains).
+// 256 chains). Resident: 56 us a round, of 116000 cycles 50000 in the gather,
+// 30000 in the update and 33000 waiting for the slowest block of the tile.
 //  - Costs: each block adds its weighted costs to the tile's accumulators in
 //    the L2 (int64, exact in any order) before the first barrier; after it
 //    every block reads them back and keeps its own copy of the tile's best
