@@ -531,8 +531,8 @@ void split_weights(const maxsat_ctx* ctx, int nb, int64_t* wmax, int64_t* wmax8)
 }
 
 // Sets up the resident rounds for the chains being allocated (Bp chains, the
-// gather's plan made): S blocks per chain tile, as many as the plan has when
-// they are all resident, else as many as are. S = 0 (two launches per round)
+// gather's plan made): S blocks per chain tile, as many as the plan has or as
+// are resident at most. S = 0 (two launches per round)
 // for a batch, for more chain tiles than half the resident blocks, or when
 // whole tiles would leave more than a sixth of them idle.
 int plan_rounds(maxsat_ctx* ctx, DevAllocs& A, int Bp) {
@@ -550,7 +550,11 @@ int plan_rounds(maxsat_ctx* ctx, DevAllocs& A, int Bp) {
     slots = slots / ctx->rounds_per_sm * 2;
   const int most = slots / tiles;
   if (most < 2) return MAXSAT_OK;
-  const int S = std::min(most, std::max(1, ctx->plan.n_blk));
+  // one block per SM for a tile, more where its warps still have 12 clauses each:
+  // n = 1200, m = 7200, 256 chains, one context / 16 on 16 streams: 152 blocks 11.7
+  // / 5.3 us a round and context, 304 blocks 12.6 / 8.2, 76 blocks 16.7 / 4.4
+  const int sms = ctx->rounds_slot_count / std::max(1, ctx->rounds_per_sm);
+  const int S = std::min({most, std::max(1, ctx->plan.n_blk), std::max(sms, ctx->m / 96)});
   if (S == most && tiles * most < slots - slots / 6) return MAXSAT_OK;
   int64_t w = 0, w8 = 0;
   split_weights(ctx, S, &w, &w8);
@@ -565,7 +569,8 @@ int plan_rounds(maxsat_ctx* ctx, DevAllocs& A, int Bp) {
   const double sum = std::max(1.0, 2.0 * fmax * std::max(ctx->m, 1));
   R.fe_scale = std::ldexp(1.0, std::min(40, 61 - (int)std::ceil(std::log2(sum))));
   ctx->rounds_cost16 = w8 < 65536;
-  CK(ctx, A.alloc(&R.bar, (size_t)tiles * kBarStride));
+  CK(ctx, A.alloc(&R.bar, (size_t)tiles * 2 * kBarStride));
+  CK(ctx, A.alloc(&R.best, (size_t)Bp));
   CK(ctx, A.alloc(&R.acc, (size_t)6 * Bp));
   R.err = ctx->d_err;
   R.S = S;
@@ -577,9 +582,10 @@ int clear_rounds(maxsat_ctx* ctx) {
   RoundsArgs& R = ctx->rounds;
   if (R.S == 0) return MAXSAT_OK;
   const int Bp = ctx->C.Bp;
-  CK(ctx, cudaMemsetAsync(R.bar, 0, 4 * (size_t)(Bp / kChainTile) * kBarStride, ctx->stream));
+  CK(ctx, cudaMemsetAsync(R.bar, 0, 4 * (size_t)(Bp / kChainTile) * 2 * kBarStride,
+                          ctx->stream));
   CK(ctx, cudaMemsetAsync(R.acc, 0, 8 * (size_t)6 * Bp, ctx->stream));
-  R.bar0 = 0;
+  R.done0 = R.ticket0 = 0;
   R.acc0 = 0;
   return MAXSAT_OK;
 }
@@ -1892,7 +1898,7 @@ static bool local_rounds_active(const maxsat_ctx* ctx) {
 
 // maxsat_step runs resident rounds (k_rounds): planned for these chains, no
 // per-kernel profiling, no GPU unit propagation pending (it runs beside the
-// rounds on a side stream, and a cooperative launch would wait for its SMs)
+// rounds on a side stream; blocks that wait would hold the SMs it could use)
 static bool resident_rounds_active(const maxsat_ctx* ctx) {
   return ctx->have_chains && !ctx->dense && ctx->rounds.S > 0 && ctx->C.nib && !ctx->profiling &&
          !(ctx->up_pending && ctx->up_on_gpu) && !stream_capturing(ctx->stream);
@@ -1979,7 +1985,9 @@ int maxsat_step(maxsat_ctx* ctx, int64_t steps) {
       CK(ctx, launch_rounds(ctx->F, ctx->T, ctx->C, R, ctx->rounds_cost16, (float)ctx->prm.alpha,
                             ctx->stream));
       ctx->persist_ran = true;
-      R.bar0 += (uint32_t)R.S * (2u * (uint32_t)R.rounds - 1u);
+      // every share finished; every block drew one ticket past the last
+      R.done0 += 2u * (uint32_t)R.rounds * (uint32_t)R.S;
+      R.ticket0 += (2u * (uint32_t)R.rounds + 1u) * (uint32_t)R.S;
       R.acc0 = (R.acc0 + R.rounds) % 3;
       ctx->t += (uint32_t)R.rounds;
       ctx->d_t_synced = false;

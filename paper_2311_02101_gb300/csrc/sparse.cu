@@ -1349,13 +1349,18 @@ __global__ void __launch_bounds__(256, BLOCKS)
 
 // ---------------------------------------------------------------------------
 // Resident rounds (one formula of clauses of at most 3 literals): many Gibbs
-// rounds in one cooperative launch, without a grid-wide barrier. Chains never
-// meet during a round, so each tile of 256 chains is given its own group of S
-// blocks (blocks tile, tile + tiles, ...) that runs the tile's rounds alone:
-// every block gathers its share of the clauses, the group meets at its own
-// barrier, every warp updates its share of the variables, the group meets
-// again. An SM holds up to three blocks, mostly of different tiles, so others
-// compute while one waits. The states, costs and draws are those of the
+// rounds in one launch, without a grid-wide barrier. Chains never meet during a
+// round, so each tile of 256 chains is given its own group of S blocks (blocks
+// tile, tile + tiles, ...) that runs the tile's rounds alone. A phase (a round's
+// gather, then its visible update) is S shares: a block gathers a share of the
+// clauses, or its warps update a share of the variables. An SM holds up to three
+// blocks, mostly of different tiles, so others compute while one waits. Blocks
+// draw shares from the tile's ticket counter in order, and a share waits until
+// all of the phase before are finished: the shares waited for are held by blocks
+// that run already, so the launch needs no block to be resident beside another
+// (a cooperative launch does, and two of those never overlap: 16 contexts of n =
+// 1200, m = 7200, 256 chains on 16 streams ran one after another, 12.1 us a round
+// and context against 5.3 with tickets and 7.0 as two launches). The states, costs and draws are those of the
 // two-launch round, bit for bit.
 //
 // What bounds the two-launch round is not its arithmetic alone (weighted 3-SAT
@@ -1364,12 +1369,12 @@ __global__ void __launch_bounds__(256, BLOCKS)
 // tables and its last wave (a round of 256 chains of the same formula, 1/16 of
 // the work, takes 24.9 us; of n = 50, m = 215, 10.5 us), and the gather's last
 // block adds the partial sums of all blocks one after another (300 of them at
-// 256 chains). Resident: 56 us a round, of 116000 cycles 50000 in the gather,
-// 30000 in the update and 33000 waiting for the slowest block of the tile.
+// 256 chains). Resident: 55 us a round, of 115000 cycles about 50000 in the
+// gather, 30000 in the update and the rest waiting for the tile's slowest block;
+// 256 chains 11.7 us.
 //  - Costs: each block adds its weighted costs to the tile's accumulators in
-//    the L2 (int64, exact in any order) before the first barrier; after it
-//    every block reads them back and keeps its own copy of the tile's best
-//    costs in shared memory. Three accumulator buffers take turns: round r
+//    the L2 (int64, exact in any order); in the next phase every share reads
+//    them back beside the best costs of the rounds before. Three accumulator buffers take turns: round r
 //    adds to buffer r, reads it after the barrier, and clears buffer r + 1
 //    (last read two barriers ago).
 //  - The free energy is accumulated over clauses in every round as the
@@ -1398,14 +1403,21 @@ __device__ __forceinline__ uint32_t ld_relaxed_gpu(const uint32_t* p) {
   return v;
 }
 
-// Barrier of a tile's blocks in two halves. bar counts arrivals and is never
-// cleared; target is the count at which every block of this phase has arrived.
-__device__ __forceinline__ void tile_arrive(uint32_t* bar) {
+// The end of a share, and the block's next ticket: done counts finished shares
+// and is never cleared; *s_seen receives the count with this one.
+// The block's next ticket is drawn only now: drawn at a share's start, two of
+// one phase can fall to one block and none to another, and that repeats.
+__device__ __forceinline__ uint32_t tile_next(uint32_t* done, uint32_t* tickets, int* s_seen,
+                                              uint32_t* s_ticket) {
   __syncthreads();
   if (threadIdx.x == 0) {
+    const uint32_t ticket = atomicAdd(tickets, 1u);
     __threadfence();
-    atomicAdd(bar, 1u);
+    *s_seen = (int)(atomicAdd(done, 1u) + 1u);
+    *s_ticket = ticket;
   }
+  __syncthreads();
+  return *s_ticket;
 }
 
 // (polls with relaxed loads, one fence at the end: an acquire per poll would
@@ -1438,13 +1450,13 @@ template <bool PLAIN3, bool COST16>
 __global__ void __launch_bounds__(256, 3)
     k_rounds(DevFormula F, DevTables T, DevChains C, RoundsArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int64_t s_best[256];
   __shared__ __align__(8) uint8_t s_imp[256];
   __shared__ __align__(16) uint32_t s_off[8][2][32];
   __shared__ int s_go;
+  __shared__ uint32_t s_ticket;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tiles = C.Bp / kChainTile;
-  const int tile = (int)blockIdx.x % tiles, rank = (int)blockIdx.x / tiles, S = A.S;
+  const int tile = (int)blockIdx.x % tiles, S = A.S;
   const int g8 = tile * 32 + lane, b0 = g8 * 8, b = tile * kChainTile + tid;
   // shared memory: record blocks (256-byte aligned), contribution rows,
   // visible entries, then the pattern rows (the gather's block sums share
@@ -1462,22 +1474,13 @@ __global__ void __launch_bounds__(256, 3)
   float* s_fe = reinterpret_cast<float*>(smem + buf_at) + 8 * 256;   // [8][256]
   const uint32_t rows_s = s0 + (uint32_t)(buf_at + warp * 2 * kRowBuf);
   const uint32_t off_s = (uint32_t)__cvta_generic_to_shared(&s_off[warp][0][0]);
-  s_best[tid] = C.best[b];
   const G3Tables G = gather3_tables(T, C, rec_tab, b0);
   uint32_t tab;
   const int split = nib_split(T, C, b0, s0 + (uint32_t)rows_at, tab);
   const bool two = __any_sync(0xFFFFFFFFu, split < 8);
-  // this block's clauses: whole groups of 8, as even as possible
-  int c_begin, c_end;
-  {
-    const int groups = (F.m + 7) / 8, per = groups / S, more = groups % S;
-    const int g0 = rank * per + min(rank, more);
-    c_begin = min(F.m, 8 * g0);
-    c_end = min(F.m, 8 * (g0 + per + (rank < more ? 1 : 0)));
-  }
-  uint32_t* bar = A.bar + tile * kBarStride;
-  uint32_t target = A.bar0;
-  const int n_warps = S * 8, first = rank * 8 + warp;
+  uint32_t* done = A.bar + (size_t)tile * 2 * kBarStride;  // finished shares of the tile
+  uint32_t* tickets = done + kBarStride;                   // shares handed out
+  const int n_warps = S * 8;
   const uint32_t* H = static_cast<const uint32_t*>(C.H) + tile * 32 + (lane & 7) * 4;
   const size_t hstride = (size_t)(C.Bp / 8);
   auto load_slot = [&](int slot) {
@@ -1490,126 +1493,145 @@ __global__ void __launch_bounds__(256, 3)
   auto copy_rows = [&](const int2& win, int cnt, int buf) {
     nib_copy_rows(win, cnt, H, hstride, rows_s + (uint32_t)(buf * kRowBuf), s_off[warp][buf], lane);
   };
+  if (tid == 0) {
+    s_ticket = atomicAdd(tickets, 1u) - A.ticket0;
+    s_go = (int)A.done0;
+  }
   __syncthreads();
 
-  for (int r = 0; r < A.rounds; ++r) {
+  const uint32_t items = 2u * (uint32_t)A.rounds * (uint32_t)S;
+  uint32_t cur = s_ticket;
+  while (cur < items) {
+    const uint32_t phase = cur / (uint32_t)S;
+    const int share = (int)(cur - phase * (uint32_t)S), r = (int)(phase >> 1);
+    const uint32_t target = A.done0 + phase * (uint32_t)S;
     const uint32_t t = A.t0 + (uint32_t)r;
     const bool last = r + 1 == A.rounds;
     const int buf = (A.acc0 + r) % 3, clear = (A.acc0 + r + 1) % 3;
     unsigned long long* acc_cost = A.acc + (size_t)buf * 2 * C.Bp + b;
     unsigned long long* acc_fe = acc_cost + C.Bp;
-    // ---- gather
-    int32_t cost[8];
-    float fe[8];
+    if ((phase & 1u) == 0) {
+      if (!tile_wait(done, target, A.err, &s_go)) return;
+      // this share's clauses: whole groups of 8, as even as possible
+      const int groups = (F.m + 7) / 8, per = groups / S, extra = groups % S;
+      const int first8 = share * per + min(share, extra);
+      const int c_begin = min(F.m, 8 * first8);
+      const int c_end = min(F.m, 8 * (first8 + per + (share < extra ? 1 : 0)));
+      // ---- gather
+      int32_t cost[8];
+      float fe[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      cost[q] = 0;
-      fe[q] = 0.f;
-    }
-    gather3_clauses<PLAIN3, COST16, true, true>(F, C, G, 0, c_begin, c_end, 0, t, g8, warp, cost,
-                                                fe);
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      s_cost[warp * 256 + lane * 8 + q] = cost[q];
-      s_fe[warp * 256 + lane * 8 + q] = fe[q];
-    }
-    __syncthreads();
-    int64_t tc = 0;
-    float tf = 0.f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) {
-      tc += s_cost[w * 256 + tid];
-      tf += s_fe[w * 256 + tid];
-    }
-    atomicAdd(acc_cost, (unsigned long long)tc);
-    if (last) atomicAdd(acc_fe, (unsigned long long)__double2ll_rn((double)tf * A.fe_scale));
-    if (rank == 0) {
-      unsigned long long* next = A.acc + (size_t)clear * 2 * C.Bp + b;
-      next[0] = 0ull;
-      next[C.Bp] = 0ull;
-    }
-    tile_arrive(bar);
-    target += (uint32_t)S;
-    // constants of the first variables, while the other blocks arrive
-    int4 rec = load_slot(first), rec1 = load_slot(first + n_warps),
-         rec2 = load_slot(first + 2 * n_warps);
-    const int2 win0 = load_inc(rec.y, rec.z);
-    int2 win1 = load_inc(rec1.y, rec1.z);
-    if (!tile_wait(bar, target, A.err, &s_go)) return;
-    // ---- best-keep
-    const int64_t csum = (int64_t)__ldcg(acc_cost);
-    const bool imp = csum < s_best[tid];
-    if (imp) s_best[tid] = csum;
-    s_imp[tid] = imp ? 1 : 0;
-    if (last && rank == 0) {
-      C.cost[b] = csum;
-      C.fe[b] = (float)((double)(long long)__ldcg(acc_fe) / A.fe_scale);
-      C.best[b] = s_best[tid];
-      C.improved[b] = imp ? 1 : 0;
-    }
-    // ---- visible update
-    uint64_t xold = 0;
-    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
-    auto load_state = [&](int i, uint64_t& x, float4& a, float4& c) {
-      const size_t o = (size_t)i * C.Bp + b0;
-      x = __ldcg(reinterpret_cast<const unsigned long long*>(C.xt + o));
-      a = __ldcg(reinterpret_cast<const float4*>(C.nu + o));
-      c = __ldcg(reinterpret_cast<const float4*>(C.nu + o) + 1);
-    };
-    if (first < F.n) {
-      copy_rows(win0, min(rec.z, kRowWin), 0);
-      load_state(rec.x, xold, n0, n1);
-    }
-    __syncthreads();  // s_imp
-    const uint64_t flags = *reinterpret_cast<const uint64_t*>(&s_imp[lane * 8]);
-    int vb = 0;
-    for (int slot = first; slot < F.n; slot += n_warps, vb ^= 1) {
-      const bool more = slot + n_warps < F.n;
-      uint64_t x1 = 0;
-      float4 m0 = n0, m1 = n1;
-      __syncwarp();  // the other buffer's readers are done
-      if (more) {
-        copy_rows(win1, min(rec1.z, kRowWin), vb ^ 1);
-        load_state(rec1.x, x1, m0, m1);
+      for (int q = 0; q < 8; ++q) {
+        cost[q] = 0;
+        fe[q] = 0.f;
       }
-      win1 = load_inc(rec2.y, rec2.z);
-      const int4 rec3 = load_slot(slot + 3 * n_warps);
-      if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
-      else asm volatile("cp.async.wait_group 0;" ::: "memory");
-      __syncwarp();
-      const int cnt = rec.z;
-      int z[8];
+      gather3_clauses<PLAIN3, COST16, true, true>(F, C, G, 0, c_begin, c_end, 0, t, g8, warp, cost,
+                                                  fe);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) z[q] = 0;
-      for (int j = 0; j < cnt; j += kRowWin) {
-        if (j > 0) {  // a further window
-          const int2 w = load_inc(rec.y + j, cnt - j);
-          __syncwarp();
-          copy_rows(w, min(cnt - j, kRowWin), vb);
-          asm volatile("cp.async.wait_group 0;" ::: "memory");
-          __syncwarp();
+      for (int q = 0; q < 8; ++q) {
+        s_cost[warp * 256 + lane * 8 + q] = cost[q];
+        s_fe[warp * 256 + lane * 8 + q] = fe[q];
+      }
+      __syncthreads();
+      int64_t tc = 0;
+      float tf = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        tc += s_cost[w * 256 + tid];
+        tf += s_fe[w * 256 + tid];
+      }
+      atomicAdd(acc_cost, (unsigned long long)tc);
+      if (last) atomicAdd(acc_fe, (unsigned long long)__double2ll_rn((double)tf * A.fe_scale));
+      if (share == 0) {
+        unsigned long long* zero = A.acc + (size_t)clear * 2 * C.Bp + b;
+        zero[0] = 0ull;
+        zero[C.Bp] = 0ull;
+      }
+    } else {
+      // constants of the first variables, while the other blocks arrive
+      const int first = share * 8 + warp;
+      int4 rec = load_slot(first), rec1 = load_slot(first + n_warps),
+           rec2 = load_slot(first + 2 * n_warps);
+      const int2 win0 = load_inc(rec.y, rec.z);
+      int2 win1 = load_inc(rec1.y, rec1.z);
+      if (!tile_wait(done, target, A.err, &s_go)) return;
+      // ---- best-keep: round r reads the best costs of before from one of two
+      // buffers (C.best first), one share writes the new ones to the other
+      const int64_t csum = (int64_t)__ldcg(acc_cost);
+      const int64_t best = __ldcg(((r & 1) ? A.best : C.best) + b);
+      const bool imp = csum < best;
+      s_imp[tid] = imp ? 1 : 0;
+      if (share == 0) ((r & 1) ? C.best : A.best)[b] = imp ? csum : best;
+      if (last && share == 0) {
+        C.cost[b] = csum;
+        C.fe[b] = (float)((double)(long long)__ldcg(acc_fe) / A.fe_scale);
+        C.improved[b] = imp ? 1 : 0;
+      }
+      // ---- visible update
+      uint64_t xold = 0;
+      float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+      auto load_state = [&](int i, uint64_t& x, float4& a, float4& c) {
+        const size_t o = (size_t)i * C.Bp + b0;
+        x = __ldcg(reinterpret_cast<const unsigned long long*>(C.xt + o));
+        a = __ldcg(reinterpret_cast<const float4*>(C.nu + o));
+        c = __ldcg(reinterpret_cast<const float4*>(C.nu + o) + 1);
+      };
+      if (first < F.n) {
+        copy_rows(win0, min(rec.z, kRowWin), 0);
+        load_state(rec.x, xold, n0, n1);
+      }
+      __syncthreads();  // s_imp
+      const uint64_t flags = *reinterpret_cast<const uint64_t*>(&s_imp[lane * 8]);
+      int vb = 0;
+      for (int slot = first; slot < F.n; slot += n_warps, vb ^= 1) {
+        const bool more = slot + n_warps < F.n;
+        uint64_t x1 = 0;
+        float4 m0 = n0, m1 = n1;
+        __syncwarp();  // the other buffer's readers are done
+        if (more) {
+          copy_rows(win1, min(rec1.z, kRowWin), vb ^ 1);
+          load_state(rec1.x, x1, m0, m1);
         }
-        const int cw = min(cnt - j, kRowWin);
-        uint32_t acc[4] = {0u, 0u, 0u, 0u};
-        nib_sum_rows(tab, split < 8 ? tab + (uint32_t)T.ptab_stride : tab, two, split,
-                     off_s + (uint32_t)vb * 128u, rows_s + (uint32_t)(vb * kRowBuf + lane * 4), cw,
-                     acc);
-        nib_flush(acc, cw * T.ptab_bias, z);
+        win1 = load_inc(rec2.y, rec2.z);
+        const int4 rec3 = load_slot(slot + 3 * n_warps);
+        if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+        const int cnt = rec.z;
+        int z[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) z[q] = 0;
+        for (int j = 0; j < cnt; j += kRowWin) {
+          if (j > 0) {  // a further window
+            const int2 w = load_inc(rec.y + j, cnt - j);
+            __syncwarp();
+            copy_rows(w, min(cnt - j, kRowWin), vb);
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncwarp();
+          }
+          const int cw = min(cnt - j, kRowWin);
+          uint32_t acc[4] = {0u, 0u, 0u, 0u};
+          nib_sum_rows(tab, split < 8 ? tab + (uint32_t)T.ptab_stride : tab, two, split,
+                       off_s + (uint32_t)vb * 128u, rows_s + (uint32_t)(vb * kRowBuf + lane * 4), cw,
+                       acc);
+          nib_flush(acc, cw * T.ptab_bias, z);
+        }
+        nib_tail(T, C, pva, A.keep, t, 0, rec.x, g8, (size_t)rec.x * C.Bp + b0, xold, flags, n0, n1,
+                 z);
+        rec = rec1;
+        rec1 = rec2;
+        rec2 = rec3;
+        xold = x1;
+        n0 = m0;
+        n1 = m1;
       }
-      nib_tail(T, C, pva, A.keep, t, 0, rec.x, g8, (size_t)rec.x * C.Bp + b0, xold, flags, n0, n1,
-               z);
-      rec = rec1;
-      rec1 = rec2;
-      rec2 = rec3;
-      xold = x1;
-      n0 = m0;
-      n1 = m1;
     }
-    if (last) break;
-    tile_arrive(bar);
-    target += (uint32_t)S;
-    if (!tile_wait(bar, target, A.err, &s_go)) return;
+    cur = tile_next(done, tickets, &s_go, &s_ticket) - A.ticket0;
   }
+  // an odd number of rounds leaves the best costs in the second buffer: the
+  // block that finished the tile's last share moves them
+  __threadfence();
+  if ((A.rounds & 1) && s_go == (int)(A.done0 + items)) C.best[b] = __ldcg(A.best + b);
 }
 
 // ---------------------------------------------------------------------------
@@ -2110,17 +2132,8 @@ cudaError_t launch_rounds(const DevFormula& F, const DevTables& T, const DevChai
   if (e != cudaSuccess) return e;
   volatile float one = 1.0f;
   A.keep = one - alpha;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(C.Bp / kChainTile * A.S));
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = (size_t)smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, F, T, C, A);
+  kern<<<(unsigned)(C.Bp / kChainTile * A.S), 256, smem, st>>>(F, T, C, A);
+  return cudaGetLastError();
 }
 
 bool persistent_round_supported(const DevTables& T, const DevChains& C, const DevFormula& F,

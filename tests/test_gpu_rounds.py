@@ -126,3 +126,31 @@ def test_long_steps_match_oracle(ms, case):
     for k in ("cost", "best_cost", "best_x"):
         assert np.array_equal(g[k], getattr(st, k)), k
     np.testing.assert_allclose(g["free_energy"], st.free_energy, rtol=1e-3, atol=1e-6)
+
+
+def test_contexts_side_by_side_match_oracle(ms):
+    """Rounds of several contexts on streams of their own, in flight together:
+    blocks of each run whatever shares of its rounds are open, however many of
+    them the device has room for."""
+    import torch
+    table, alpha, B = table_for(2, 4, 3), 0.05, 1300
+    p = ms.maxsat_default_params(sets=table.sets, n_temps=2, n_buckets=2, alpha=alpha,
+                                 quant_bits=4, path=ms.MAXSAT_PATH_SPARSE)
+    insts = [oracle.Instance(*workloads.random_ksat(60 + 25 * k, 300 + 110 * k, 3, 30 + k))
+             for k in range(4)]
+    ctxs = [ms.maxsat_create(i.n, i.off, i.lits, i.w, p, torch.cuda.Stream()) for i in insts]
+    for k, ctx in enumerate(ctxs):
+        ms.maxsat_reset(ctx, B, 40 + k)
+    for steps in (7, 6, 7):
+        for ctx in ctxs:
+            ms.maxsat_step(ctx, steps)
+    for k, (inst, ctx) in enumerate(zip(insts, ctxs)):
+        g = ms.maxsat_get_state(ctx)
+        ms.maxsat_destroy(ctx)
+        st = oracle.init_chains(inst.n, B, 40 + k)
+        oracle.gibbs(inst, table, st, 20, 40 + k, n_temps=2, n_buckets=2, alpha=alpha,
+                     threads=os.cpu_count() or 4)
+        assert np.array_equal(g["x"], st.x)
+        assert np.array_equal(g["nu"], st.nu32)
+        for name in ("cost", "best_cost", "best_x"):
+            assert np.array_equal(g[name], getattr(st, name)), name
