@@ -299,13 +299,13 @@ def kernel_roofline(kernel, n, m, nnz, B, off, lits, peaks, clock_mhz, sms, fp8=
 def algorithmic_bytes(kernel, n, m, nnz, B):
     """Compulsory bytes one launch moves (sparse path): the state it must read
     and write once, nothing re-read. Per clause and chain the hidden state is
-    one byte (up to 8 hidden units); per variable and chain the state is one
-    byte and nu four bytes."""
+    four bits (clauses of at most 3 literals); per variable and chain the state
+    is one byte and nu four bytes."""
     formula = 4 * (m + 1) + 4 * nnz + 4 * m + 8 * m
     if kernel == "gather_hidden":
-        return n * B + m * B + formula
+        return n * B + m * B // 2 + formula
     if kernel == "visible":
-        return m * B + 2 * n * B + 8 * n * B + 8 * nnz
+        return m * B // 2 + 2 * n * B + 8 * n * B + 8 * nnz
     if kernel == "best_keep":
         return 12 * B
     return None
@@ -412,8 +412,8 @@ def run_mine(args):
         ms_warm = float(t.item())
     steady = dict(value=m * B * args.steps * ws / (ms_warm / 1e3), unit=UNIT,
                   ms_per_step=ms_warm / args.steps,
-                  note=f"L2 not flushed: state carried round to round, CUDA graphs of "
-                       f"{params.steps_per_graph} rounds")
+                  note="L2 not flushed: state carried round to round, all rounds from one "
+                       "maxsat_step")
 
     # per-kernel device times over a third region of the same length, flushed
     # as the timed one (plain launches, CUDA events around every launch on the
@@ -521,15 +521,19 @@ def run_mine(args):
     pt = pt_probe(ms, torch, n, off, lits, w, B, stream, args) if not args.no_pt else None
     configs = config_probe(ms, torch, stream, args) if not args.no_configs else None
 
-    # the chains' state per round: hidden patterns (2 bytes when some clause
-    # has 8 literals or more), x and best x, nu, per-block partials
+    # the chains' state per round: hidden patterns (4 bits per three hidden units: half a
+    # byte up to 3 literals, about 2 bytes at mixed lengths), x and best x, nu, per-block
+    # partials
     Bp = (B + 255) // 256 * 256
-    hbytes = 2 if int(np.max(np.diff(off), initial=0)) >= 8 else 1
+    hbytes = 0.5 if int(np.max(np.diff(off), initial=0)) <= 3 else 2
     state_mb = (m * Bp * hbytes + n * Bp * 6 + 12 * Bp * (m // 100 + 1)) / 2**20
     S = params.steps_per_graph
     per_round = len([k for k in kt if k not in ("gather_score", "keep_copy", "gemm1_score")])
-    launches_timed = per_round * args.steps  # one plain-launch round per interval
     path = {1: "dense", 2: "sparse"}[ms.maxsat_get_path(ctx)]
+    # one round per interval: on the sparse path a formula of clauses of at most 3
+    # literals runs both phases in one launch (the profiled region takes them apart)
+    short = int(np.max(np.diff(off), initial=0)) <= 3
+    launches_timed = (1 if path == "sparse" and short else per_round) * args.steps
     line = dict(metric=METRIC, value=value, unit=UNIT, n_gpus=ws, steps=args.steps,
                 warmup=args.warmup, ms_per_step=ms_total / args.steps, higher_is_better=True,
                 scaling="weak", vs_baseline=None, dtype="fp8" if path == "dense" else "int32",
