@@ -2147,6 +2147,11 @@ int maxsat_eval(maxsat_ctx* ctx, const uint8_t* assign_dev, int32_t B, int64_t* 
   // MAXSAT_PATH_DENSE asks for the tensor-core products by name; everywhere
   // else the packed form runs where it applies
   if (ctx->prm.path != MAXSAT_PATH_DENSE && bits_eval(ctx)) {
+    if (ctx->n_inst == 1 && bits_one_launch(ctx->n, ctx->m)) {
+      TIMED(ctx, ctx->stream, "bits_cost",
+            launch_bits_eval(ctx->bits, assign_dev, B, cost_dev, ctx->stream));
+      return MAXSAT_OK;
+    }
     const int rc = ensure_bits_scratch(ctx, B);
     if (rc != MAXSAT_OK) return rc;
     const int stride = bits_stride(ctx);

@@ -55,7 +55,40 @@ __device__ __forceinline__ uint32_t load4(const uint8_t* p, const uint8_t* lo, c
   return v;
 }
 
-// A: the base and n are multiples of 4 (every row segment is an aligned word)
+// Variables i .. i + 3 of `rows` (at most 32) assignments of n bytes from row:
+// word k has bit r set when byte i + k of assignment r is nonzero. A: the base
+// and n are multiples of 4 (every row segment is an aligned word).
+template <bool A>
+__device__ __forceinline__ uint4 pack4(const uint8_t* row, int rows, int i, int n,
+                                       const uint8_t* lo, const uint8_t* hi) {
+  uint32_t a[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    uint32_t v[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      v[r] = 0u;
+      if (i < n && g * 8 + r < rows) {
+        const uint8_t* q = row + i + (size_t)(g * 8 + r) * n;
+        v[r] = A ? __ldg(reinterpret_cast<const uint32_t*>(q)) : load4(q, lo, hi);
+      }
+    }
+    // bit r of byte k: row r's byte k is nonzero
+    uint32_t acc = 0u;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const uint32_t nz = ((v[r] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | v[r];
+      acc = ((acc >> 1) & 0x7F7F7F7Fu) | (nz & 0x80808080u);
+    }
+    a[g] = acc;
+  }
+  // byte k of a[0..3] -> the word of variable i + k
+  const uint32_t t0 = __byte_perm(a[0], a[1], 0x5140u), t1 = __byte_perm(a[2], a[3], 0x5140u);
+  const uint32_t t2 = __byte_perm(a[0], a[1], 0x7362u), t3 = __byte_perm(a[2], a[3], 0x7362u);
+  return make_uint4(__byte_perm(t0, t1, 0x5410u), __byte_perm(t0, t1, 0x7632u),
+                    __byte_perm(t2, t3, 0x5410u), __byte_perm(t2, t3, 0x7632u));
+}
+
 template <bool A>
 __global__ void __launch_bounds__(256) k_pack_bits(const uint8_t* __restrict__ assign, int B,
                                                    int n, int W, int nstride,
@@ -73,36 +106,10 @@ __global__ void __launch_bounds__(256) k_pack_bits(const uint8_t* __restrict__ a
   const uint8_t* end = assign + (size_t)B * n;
   for (size_t task = self / 32; task < tasks; task += warps) {
     const int w = (int)(task / groups), i = (int)(task % groups) * 128 + lane * 4;
-    const int rows = min(32, B - w * 32);
-    const uint8_t* p = assign + (size_t)w * 32 * n + i;
-    uint32_t a[4];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      uint32_t v[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        v[r] = 0u;
-        if (i < n && g * 8 + r < rows) {
-          const uint8_t* q = p + (size_t)(g * 8 + r) * n;
-          v[r] = A ? __ldg(reinterpret_cast<const uint32_t*>(q)) : load4(q, assign, end);
-        }
-      }
-      // bit r of byte k: row r's byte k is nonzero
-      uint32_t acc = 0u;
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const uint32_t nz = ((v[r] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | v[r];
-        acc = ((acc >> 1) & 0x7F7F7F7Fu) | (nz & 0x80808080u);
-      }
-      a[g] = acc;
-    }
-    // byte k of a[0..3] -> the word of variable i + k
-    const uint32_t t0 = __byte_perm(a[0], a[1], 0x5140u), t1 = __byte_perm(a[2], a[3], 0x5140u);
-    const uint32_t t2 = __byte_perm(a[0], a[1], 0x7362u), t3 = __byte_perm(a[2], a[3], 0x7362u);
+    const uint4 words =
+        pack4<A>(assign + (size_t)w * 32 * n, min(32, B - w * 32), i, n, assign, end);
     if (i < nstride)  // variables n .. nstride - 1 are padding, never read
-      *reinterpret_cast<uint4*>(X + (size_t)w * nstride + i) =
-          make_uint4(__byte_perm(t0, t1, 0x5410u), __byte_perm(t0, t1, 0x7632u),
-                     __byte_perm(t2, t3, 0x5410u), __byte_perm(t2, t3, 0x7632u));
+      *reinterpret_cast<uint4*>(X + (size_t)w * nstride + i) = words;
   }
 }
 
@@ -173,9 +180,12 @@ __global__ void __launch_bounds__(256) k_bits_slabs(BitsFormula F, int n_pos) {
 
 // V: int32_t when every 32 clauses of a slab weigh less than 2^31, else
 // int64_t. RAW: a caller's DIMACS arrays, not checked before.
-template <typename V, bool RAW, int WARPS>
+// PACK (one formula, one block per word): the block packs its 32 assignments
+// itself and writes their costs; assign stands for X.
+template <typename V, bool RAW, int WARPS, bool PACK>
 __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawFormula R,
                                                           const uint32_t* __restrict__ X,
+                                                          const uint8_t* __restrict__ assign,
                                                           int nstride, int B,
                                                           unsigned long long* __restrict__ out) {
   extern __shared__ __align__(16) uint32_t s_row[];
@@ -203,7 +213,14 @@ __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawForm
   }
   pdl_wait();
   const uint32_t* row = X + (size_t)word * nstride + v0;
-  if ((v0 & 3) == 0) {
+  if constexpr (PACK) {
+    const uint8_t *rows = assign + (size_t)word * 32 * nv, *end = assign + (size_t)B * nv;
+    const bool aligned = ((reinterpret_cast<uintptr_t>(assign) | (uintptr_t)nv) & 3u) == 0;
+    for (int k = threadIdx.x * 4; k < nv; k += 128 * WARPS)
+      *reinterpret_cast<uint4*>(s_row + k) =
+          aligned ? pack4<true>(rows, min(32, B - word * 32), k, nv, assign, end)
+                  : pack4<false>(rows, min(32, B - word * 32), k, nv, assign, end);
+  } else if ((v0 & 3) == 0) {
 #pragma unroll 8
     for (int k = threadIdx.x * 4; k < nv; k += 128 * WARPS)
       *reinterpret_cast<uint4*>(s_row + k) = __ldg(reinterpret_cast<const uint4*>(row + k));
@@ -262,7 +279,11 @@ __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawForm
 #pragma unroll
     for (int k = 0; k < WARPS; ++k) c += s_sum[k][lane];
     const int b = word * 32 + lane;
-    if (b < B && c != 0) atomicAdd(out + (size_t)inst * B + b, (unsigned long long)c);
+    if (PACK) {
+      if (b < B) out[b] = (unsigned long long)c;
+    } else if (b < B && c != 0) {
+      atomicAdd(out + (size_t)inst * B + b, (unsigned long long)c);
+    }
   }
 }
 
@@ -280,6 +301,13 @@ int sms() {
 
 int row_bytes(int nv) { return 4 * ((nv + 3) / 4 * 4) + 16; }  // with the zero word
 
+// Formulas scored by one launch: a block packs its own 32 assignments (32 n
+// bytes) and its 8 warps take all runs of 32 clauses, at most 4 each. Back to
+// back, one / two launches: m = 420, 16 assignments 3.2 / 5.0 us; m = 1280, 16 to
+// 2048 assignments 4.8-5.1 / 4.9-5.8, 4096 7.6 / 7.4; m = 2048, 16 to 8192
+// assignments 6.4-12.3 / 5.0-11.3. The start of a launch bounds both.
+constexpr int kOneLaunchVars = 1024, kOneLaunchClauses = 1024;
+
 // blocks of 8 warps that share an SM: room for the staged rows
 int cost_blocks_per_sm(int nv) { return 226 * 1024 / (row_bytes(nv) + 11 * 1024); }
 
@@ -291,15 +319,18 @@ int cost_chunks(int W, int runs, int nv) {
   return std::max(1, std::min(std::min(want, fit), (runs + 15) / 16));
 }
 
-template <typename V, bool RAW, int WARPS>
-cudaError_t cost_variant(const BitsFormula& F, const RawFormula& R, const uint32_t* X, int nstride,
-                         int B, int nv, int chunks, int64_t* cost, cudaStream_t st) {
-  auto kern = k_bits_cost<V, RAW, WARPS>;
-  const int smem = row_bytes(nv);
-  const cudaError_t e = allow_dynamic_smem(kern, smem);
-  if (e != cudaSuccess) return e;
+template <typename V, bool RAW, int WARPS, bool PACK>
+cudaError_t cost_variant(const BitsFormula& F, const RawFormula& R, const uint32_t* X,
+                         const uint8_t* assign, int nstride, int B, int nv, int chunks,
+                         int64_t* cost, cudaStream_t st) {
+  auto kern = k_bits_cost<V, RAW, WARPS, PACK>;
+  const int smem = row_bytes(nv), fixed = WARPS * (128 * (int)sizeof(V) + 256);
+  if (smem + fixed > 48 * 1024) {
+    const cudaError_t e = allow_dynamic_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+  }
   return launch_pdl(kern, dim3((unsigned)((B + 31) / 32), (unsigned)chunks), 32 * WARPS, smem, st,
-                      F, R, X, nstride, B, reinterpret_cast<unsigned long long*>(cost));
+                    F, R, X, assign, nstride, B, reinterpret_cast<unsigned long long*>(cost));
 }
 
 // rows so long that at most two blocks share an SM get blocks of 16 warps
@@ -307,8 +338,8 @@ template <typename V, bool RAW>
 cudaError_t cost_launch(const BitsFormula& F, const RawFormula& R, const uint32_t* X, int nstride,
                         int B, int nv, int chunks, int64_t* cost, cudaStream_t st) {
   return cost_blocks_per_sm(nv) <= 2
-             ? cost_variant<V, RAW, 16>(F, R, X, nstride, B, nv, chunks, cost, st)
-             : cost_variant<V, RAW, 8>(F, R, X, nstride, B, nv, chunks, cost, st);
+             ? cost_variant<V, RAW, 16, false>(F, R, X, nullptr, nstride, B, nv, chunks, cost, st)
+             : cost_variant<V, RAW, 8, false>(F, R, X, nullptr, nstride, B, nv, chunks, cost, st);
 }
 
 }  // namespace
@@ -343,6 +374,22 @@ cudaError_t launch_bits_cost(const BitsFormula& F, const uint32_t* X, int nstrid
   const int chunks = F.items ? F.n_items : cost_chunks((B + 31) / 32, F.n_slabs, F.n);
   return F.wide ? cost_launch<int64_t, false>(F, RawFormula{}, X, nstride, B, F.n, chunks, cost, st)
                 : cost_launch<int32_t, false>(F, RawFormula{}, X, nstride, B, F.n, chunks, cost, st);
+}
+
+bool bits_one_launch(int n, int64_t m) { return n <= kOneLaunchVars && m <= kOneLaunchClauses; }
+
+cudaError_t launch_bits_eval(const BitsFormula& F, const uint8_t* assign, int B, int64_t* cost,
+                             cudaStream_t st) {
+  return F.wide ? cost_variant<int64_t, false, 8, true>(F, RawFormula{}, nullptr, assign, 0, B, F.n,
+                                                        1, cost, st)
+                : cost_variant<int32_t, false, 8, true>(F, RawFormula{}, nullptr, assign, 0, B, F.n,
+                                                        1, cost, st);
+}
+
+cudaError_t launch_bits_eval_raw(const RawFormula& R, const uint8_t* assign, int B, int64_t* cost,
+                                 cudaStream_t st) {
+  return cost_variant<int64_t, true, 8, true>(BitsFormula{}, R, nullptr, assign, 0, B, R.n, 1, cost,
+                                              st);
 }
 
 cudaError_t launch_bits_cost_raw(const RawFormula& R, const uint32_t* X, int nstride, int B,

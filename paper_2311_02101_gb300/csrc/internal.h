@@ -243,6 +243,13 @@ cudaError_t launch_bits_slabs(const BitsFormula& F, cudaStream_t st);
 // adds the costs of B assignments to cost (n_inst x B, zeroed)
 cudaError_t launch_bits_cost(const BitsFormula& F, const uint32_t* X, int nstride, int B,
                              int64_t* cost, cudaStream_t st);
+// whether one formula is small enough for a launch that packs and scores
+bool bits_one_launch(int n, int64_t m);
+// writes the costs of B assignments (B x n bytes) of one formula
+cudaError_t launch_bits_eval(const BitsFormula& F, const uint8_t* assign, int B, int64_t* cost,
+                             cudaStream_t st);
+cudaError_t launch_bits_eval_raw(const RawFormula& R, const uint8_t* assign, int B, int64_t* cost,
+                                 cudaStream_t st);
 cudaError_t launch_bits_cost_raw(const RawFormula& R, const uint32_t* X, int nstride, int B,
                                  int64_t* cost, cudaStream_t st);
 

@@ -171,13 +171,9 @@ extern "C" int maxsat_eval_noalloc(int32_t n, int64_t m, int64_t n_lits,
   int64_t* part = reinterpret_cast<int64_t*>(scratch + xt_bytes);
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   if (n <= kBitsMaxVars) {
-    // assignments packed to bits (eval_bits.cu): two launches; the packed words
-    // take an eighth of the scratch that the byte form needs
-    uint32_t* X = reinterpret_cast<uint32_t*>(scratch);
-    const int stride = (n + 3) / 4 * 4;
-    cudaError_t e = launch_pack_bits(assign_dev, B, n, stride, X, cost_dev, (size_t)B, st);
-    if (e != cudaSuccess)
-      return noalloc_fail(MAXSAT_ECUDA, std::string("pack launch: ") + cudaGetErrorString(e));
+    // assignments packed to bits (eval_bits.cu): one launch for small formulas,
+    // else two; the packed words take an eighth of the scratch that the byte form
+    // needs
     RawFormula R;
     R.m = (int32_t)m;
     R.n = n;
@@ -185,7 +181,17 @@ extern "C" int maxsat_eval_noalloc(int32_t n, int64_t m, int64_t n_lits,
     R.off = off_dev;
     R.lits = lits_dev;
     R.w = w_dev;
-    e = launch_bits_cost_raw(R, X, stride, B, cost_dev, st);
+    cudaError_t e = cudaSuccess;
+    if (bits_one_launch(n, m)) {
+      e = launch_bits_eval_raw(R, assign_dev, B, cost_dev, st);
+    } else {
+      uint32_t* X = reinterpret_cast<uint32_t*>(scratch);
+      const int stride = (n + 3) / 4 * 4;
+      e = launch_pack_bits(assign_dev, B, n, stride, X, cost_dev, (size_t)B, st);
+      if (e != cudaSuccess)
+        return noalloc_fail(MAXSAT_ECUDA, std::string("pack launch: ") + cudaGetErrorString(e));
+      e = launch_bits_cost_raw(R, X, stride, B, cost_dev, st);
+    }
     if (e != cudaSuccess)
       return noalloc_fail(MAXSAT_ECUDA, std::string("cost launch: ") + cudaGetErrorString(e));
     return MAXSAT_OK;

@@ -58,7 +58,8 @@ def costs(ms, table, insts, X, offset):
 @pytest.mark.parametrize("n,m,kmax,wmax,B,offset", [
     (1, 1, 1, 2, 1, 0), (37, 33, 3, 9, 31, 1), (128, 512, 3, 1000, 32, 0),
     (129, 513, 6, 2 ** 40, 33, 3), (1000, 6000, 3, 1000, 100, 0), (1003, 777, 6, 5, 1025, 2),
-    (4, 0, 3, 5, 70, 0)])
+    (4, 0, 3, 5, 70, 0), (1024, 1024, 6, 9, 64, 0), (1025, 1024, 3, 9, 33, 1),
+    (1023, 1025, 3, 2 ** 33, 31, 2), (300, 1024, 3, 2 ** 40, 95, 3)])
 def test_packed_costs(ms, table, n, m, kmax, wmax, B, offset):
     inst = random_formula(n, m, kmax, wmax, n + B)
     X = np.random.default_rng(B).integers(0, 2, size=(B, n), dtype=np.uint8)
