@@ -432,6 +432,12 @@ int plan_blocks(const maxsat_ctx* ctx, int cb) {
   return (int)std::min<int64_t>(nb, INT32_MAX);
 }
 
+// The 256-byte record blocks of every (group, temperature) are built (T.rec3;
+// larger ensembles, up to 64 temperatures, read T.rec instead).
+bool record_blocks_fit(const DevTables& T) {
+  return T.one_chunk && (int64_t)T.n_groups * T.n_temps * 256 <= 32 * 1024;
+}
+
 // Clauses per gather block for `tiles` chain tiles. A batch's formulas are split
 // one by one, so that the rule for one formula gives some blocks more than fit
 // at once (96 formulas, 500 blocks on 456 places: the 44 left over cost a launch
@@ -1530,11 +1536,12 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
           slots[s] = make_int4(i, ioff[i], ioff[i + 1] - ioff[i], k);
         }
       UP(slots, F.var_slot);
-      // lists of the local rounds: 16-bit indices, all weights together below
-      // 2^31 - 1, and (28 bytes a clause, 52 a variable) within an SM
+      // lists of the local rounds: record blocks built, 16-bit indices, all
+      // weights together below 2^31 - 1, and (28 bytes a clause, 52 a variable)
+      // within an SM
       int64_t weight = 0;
       for (int64_t c = 0; c < m; ++c) weight += cl_w[c];
-      if (T.one_chunk && n_inst == 1 && n_rows <= 65535 && 28 * m + 52 * (int64_t)n <= 220 * 1024 &&
+      if (record_blocks_fit(T) && n_inst == 1 && n_rows <= 65535 && 28 * m + 52 * (int64_t)n <= 220 * 1024 &&
           weight < (int64_t)INT32_MAX) {
         std::vector<uint2> lcl(m);
         std::vector<uint32_t> linc((size_t)nnz);
@@ -1634,7 +1641,7 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   }
   T.rec3 = nullptr;
   T.rec3_words = 0;
-  if (T.one_chunk && (int64_t)T.n_groups * T.n_temps * 256 <= 32 * 1024) {
+  if (record_blocks_fit(T)) {
     // one 256-byte block per (group, temperature): the group's 2^K records at
     // that temperature, then from word 32 those at the next one (for octets of
     // chains that lie across two temperatures)

@@ -300,10 +300,11 @@ LocalFn local_kernel(const LocalPlan& P, bool plain3) {
 
 }  // namespace
 
-// Shape of the local rounds, threads = 0 when the formula does not fit or the
-// resident rounds would be faster.
+// Shape of the local rounds, threads = 0 when the tables they read are not
+// built, the formula does not fit or the resident rounds would be faster.
 LocalPlan local_plan(const DevFormula& F, const DevTables& T, int Bp) {
   LocalPlan P;
+  if (!T.rec3 || !T.ptab || !T.pva) return P;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)

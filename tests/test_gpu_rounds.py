@@ -154,3 +154,32 @@ def test_contexts_side_by_side_match_oracle(ms):
         assert np.array_equal(g["nu"], st.nu32)
         for name in ("cost", "best_cost", "best_x"):
             assert np.array_equal(g[name], getattr(st, name)), name
+
+
+def test_many_temperatures_match_oracle(ms):
+    """64 temperatures and 6 clause groups: more (group, temperature) pairs than
+    the 256-byte record blocks are built for, in steps of eight rounds and more
+    and in shorter ones."""
+    import torch
+    temps, B, seed, alpha = 64, 520, 23, 0.05
+    table = oracle.make_table([1, 2, 3], list(np.linspace(0.05, 0.5, temps)), n_buckets=2, Q=4,
+                              iters=50)
+    for s in table.sets:
+        s["W"] = 6.0 * np.asarray(s["W"])
+    inst = short_clauses(23, 90, 15)
+    p = ms.maxsat_default_params(sets=table.sets, n_temps=temps, n_buckets=2, alpha=alpha,
+                                 quant_bits=4, path=ms.MAXSAT_PATH_SPARSE)
+    ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, torch.cuda.Stream())
+    ms.maxsat_reset(ctx, B, seed)
+    for steps in (8, 1, 11):
+        ms.maxsat_step(ctx, steps)
+    g = ms.maxsat_get_state(ctx)
+    ms.maxsat_destroy(ctx)
+    st = oracle.init_chains(inst.n, B, seed)
+    oracle.gibbs(inst, table, st, 20, seed, n_temps=temps, n_buckets=2, alpha=alpha,
+                 threads=os.cpu_count() or 4)
+    assert np.array_equal(g["x"], st.x)
+    assert np.array_equal(g["nu"], st.nu32)
+    for k in ("cost", "best_cost", "best_x"):
+        assert np.array_equal(g[k], getattr(st, k)), k
+    np.testing.assert_allclose(g["free_energy"], st.free_energy, rtol=1e-3, atol=1e-6)
