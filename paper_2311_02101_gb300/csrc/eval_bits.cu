@@ -11,7 +11,8 @@
 //                assignments x 128 variables: rows read 128 bytes at a time,
 //                8 rows folded into the bytes of one register by shifts, a
 //                4 x 4 byte transpose, one 16-byte store per lane.
-//   k_pack_rows  the same from variable-major bytes (n x Bp, 0 / 1).
+//   k_pack_rows  the same from variable-major bytes (n x Bp, 0 / 1; columns past
+//                the last assignment may hold anything).
 //   k_bits_cost  one block = one word of assignments x a run of clauses. The
 //                word's row of X (4 bytes per variable) is staged in shared
 //                memory; a warp takes 32 consecutive clauses, one per lane, so
@@ -113,9 +114,11 @@ __global__ void __launch_bounds__(256) k_pack_bits(const uint8_t* __restrict__ a
   }
 }
 
-// the four 0 / 1 bytes of v as 4 bits (byte k -> bit k)
+// the low bits of the four bytes of v as 4 bits (byte k -> bit k). The mask keeps
+// the other bits of bytes that nobody wrote (columns past the last assignment)
+// out of the products of their neighbours.
 __device__ __forceinline__ uint32_t bytes_to_bits(uint32_t v) {
-  return (v * 0x10204080u) >> 28;
+  return ((v & 0x01010101u) * 0x10204080u) >> 28;
 }
 
 __global__ void __launch_bounds__(256) k_pack_rows(const uint8_t* __restrict__ xt, int Bp, int n,

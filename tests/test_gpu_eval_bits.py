@@ -78,3 +78,46 @@ def test_packed_costs_of_a_batch(ms, table):
     for k, i in enumerate(insts):
         assert np.array_equal(got[k], oracle.evaluate(i, X[:, at:at + i.n].copy())), k
         at += i.n
+
+
+@pytest.mark.parametrize("B", [65, 257, 301])
+def test_merges_of_odd_chain_counts(ms, B):
+    """2 B candidates, two of them in the last group of four bytes that are
+    packed together; the other two bytes are columns that nobody writes, in
+    memory where earlier contexts kept floats."""
+    import os
+    import torch
+    tab = oracle.make_table([1, 2, 3], [0.068, 0.528], n_buckets=1, iters=300)
+    seed, alpha, tau = 31 + B, 0.05, 0.2
+    p = ms.maxsat_default_params(sets=tab.sets, n_temps=2, n_buckets=1, alpha=alpha,
+                                 path=ms.MAXSAT_PATH_SPARSE)
+    p.fstar = None
+    inst = random_formula(400, 1700, 3, 9, B)
+    bp2 = (2 * B + 255) // 256 * 256
+    # blocks of the candidates' size that held nu: n Bp floats
+    olds = [random_formula(400 * bp2 // 1024, 900, 3, 9, k) for k in range(12)]
+    held = [ms.maxsat_create(i.n, i.off, i.lits, i.w, p, torch.cuda.Stream()) for i in olds]
+    for c in held:
+        ms.maxsat_reset(c, 256, 5)
+        ms.maxsat_step(c, 20)
+    torch.cuda.synchronize()
+    for c in held:
+        ms.maxsat_destroy(c)
+    ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, torch.cuda.Stream())
+    prob = np.random.default_rng(B).random(inst.n).astype(np.float32)
+    st = oracle.init_chains(inst.n, B, seed)
+    kw = dict(n_temps=2, n_buckets=1, alpha=alpha, threads=os.cpu_count() or 4)
+    ms.maxsat_reset(ctx, B, seed)
+    for _ in range(3):
+        ms.maxsat_step(ctx, 2)
+        ms.maxsat_up(ctx)
+        ms.maxsat_step(ctx, 1)
+        ms.maxsat_propose_flips(ctx, prob, tau)
+        oracle.gibbs(inst, tab, st, 2, seed, **kw)
+        oracle.up_merge(inst, st, oracle.unit_prop(inst, st.x, st.nu32))
+        oracle.gibbs(inst, tab, st, 1, seed, **kw)
+        oracle.up_merge(inst, st, oracle.flip_proposals(st.x, prob, tau))
+    g = ms.maxsat_get_state(ctx)
+    ms.maxsat_destroy(ctx)
+    assert np.array_equal(g["x"], st.x)
+    assert np.array_equal(g["nu"], st.nu32)
