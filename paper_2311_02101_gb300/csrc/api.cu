@@ -1668,7 +1668,8 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   int64_t slab_rows = 0;
   {
     // the packed evaluation's slabs of 32 clauses, by length within a formula; a
-    // batch gets a list of runs of slabs of one formula (fewer than 65536 runs)
+    // batch gets a list of runs of slabs of one formula, each one grid row of a
+    // launch: at most 65535 (upload_plan likewise)
     BitsFormula& E = ctx->bits;
     E.m = (int32_t)m;
     for (int k = 0; k < n_inst; ++k) E.n = std::max(E.n, var_base[k + 1] - var_base[k]);
@@ -1678,7 +1679,16 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
     std::vector<int4> slabs, items;
     std::vector<int2> vars;
     int64_t& rows = slab_rows;
-    const int64_t run = std::max<int64_t>(64, m / 1048576 + 1);
+    int64_t run = 64;
+    auto runs = [&]() {
+      int64_t count = 0;
+      for (int k = 0; k < n_inst; ++k) {
+        const int64_t in = (cl_base[k + 1] - cl_base[k] + 31) / 32;
+        count += (in + run - 1) / run;
+      }
+      return count;
+    };
+    while (n_inst > 1 && runs() > 65535) run *= 2;  // n_inst <= 65535: ends
     bool one_length = true;  // of every clause: they keep their order
     for (int64_t c = 1; c < m && one_length; ++c)
       one_length = cl_off[c + 1] - cl_off[c] == cl_off[1];

@@ -121,3 +121,29 @@ def test_merges_of_odd_chain_counts(ms, B):
     ms.maxsat_destroy(ctx)
     assert np.array_equal(g["x"], st.x)
     assert np.array_equal(g["nu"], st.nu32)
+
+
+def test_packed_costs_of_the_largest_batch(ms, table):
+    """65535 formulas, one of them with more than 64 slabs of 32 clauses: one
+    run of slabs per formula at least, more would not fit a launch's grid."""
+    import torch
+    n_inst, B, at = 65535, 3, 40000
+    big = random_formula(50, 2100, 3, 9, 1)
+    w = np.arange(1, n_inst + 1, dtype=np.int64)
+    insts = [(1, np.array([0, 1]), np.array([1], np.int32), w[k:k + 1]) for k in range(n_inst)]
+    insts[at] = (big.n, big.off, big.lits, big.w)
+    p = ms.maxsat_default_params(sets=table.sets, n_temps=1, n_buckets=1)
+    p.fstar = None
+    ctx = ms.maxsat_create_batch(insts, p, torch.cuda.Stream())
+    X = np.random.default_rng(2).integers(0, 2, size=(B, n_inst - 1 + big.n), dtype=np.uint8)
+    out = torch.full((n_inst, B), -1, dtype=torch.int64, device="cuda")
+    xd = torch.from_numpy(X).cuda()
+    torch.cuda.synchronize()
+    ms.maxsat_eval(ctx, xd, out)
+    torch.cuda.synchronize()
+    ms.maxsat_destroy(ctx)
+    got = out.cpu().numpy()
+    first = np.where(np.arange(n_inst) <= at, np.arange(n_inst), np.arange(n_inst) - 1 + big.n)
+    unit = (w[:, None] * (1 - X[:, first].T)).astype(np.int64)
+    unit[at] = oracle.evaluate(big, X[:, at:at + big.n].copy())
+    assert np.array_equal(got, unit)
