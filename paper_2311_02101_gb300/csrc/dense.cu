@@ -403,19 +403,11 @@ cudaError_t launch_gemm1_eval(const CUtensorMap& tmA, const CUtensorMap& tmB, in
                               int n_pad, int B, int Bp, bool e5m2, const int32_t* row_len,
                               const int64_t* row_w, const uint8_t* grp_small, int64_t* out,
                               int* err, cudaStream_t st) {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_gemm1_eval<kEpiWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kGemm1Smem);
-    if (e != cudaSuccess) {
-      sms = 0;
-      return e;
-    }
-  }
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = allow_dynamic_smem(k_gemm1_eval<kEpiWarps>, kGemm1Smem);
+  if (e != cudaSuccess) return e;
   const uint32_t fmt = e5m2 ? 1u : 0u;
   const uint32_t idesc = tc::instr_desc(kBM, kBN, fmt, fmt);
   const int tiles_m = m_pad / kBM, tiles_n = Bp / kBN;

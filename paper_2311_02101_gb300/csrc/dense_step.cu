@@ -1319,8 +1319,7 @@ __global__ void k_keep_copy_dense(const DevChains C, const uint8_t* X, uint8_t* 
 template <typename... P, typename... Q>
 cudaError_t launch_step(void (*kern)(P...), int grid, int threads, int smem, cudaStream_t st,
                         const Q&... args) {
-  const cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  const cudaError_t e = allow_dynamic_smem(kern, smem);
   return e != cudaSuccess ? e : launch_pdl(kern, dim3((unsigned)grid), threads, smem, st, args...);
 }
 

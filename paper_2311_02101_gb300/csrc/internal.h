@@ -127,14 +127,26 @@ struct DevTables {
 
 // Lets kernel `kern` launch with `dyn` bytes of dynamic shared memory: when
 // dynamic plus the kernel's static shared memory exceed the default 48 KB per
-// block, the launch needs the opt-in attribute.
+// block, the launch needs the opt-in attribute. The attribute belongs to the
+// kernel, not to the launch: contexts on other host threads use it too. So it is
+// raised once, to all that a block may have, and never lowered (set to each
+// launch's own size, a smaller formula's launch between another thread's set and
+// launch made that launch fail). A launch still takes only the bytes it asks for.
 template <typename K>
 cudaError_t allow_dynamic_smem(K kern, int dyn) {
   cudaFuncAttributes fa;
-  const cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+  cudaError_t e = cudaFuncGetAttributes(&fa, kern);
   if (e != cudaSuccess) return e;
-  if ((size_t)dyn + fa.sharedSizeBytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
+  if ((size_t)dyn + fa.sharedSizeBytes <= 48 * 1024 || dyn <= fa.maxDynamicSharedSizeBytes)
+    return cudaSuccess;
+  int dev = 0, most = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) !=
+      cudaSuccess)
+    return e;
+  most -= (int)fa.sharedSizeBytes;
+  if (dyn > most) return cudaErrorInvalidValue;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 // Philox round keys of one seed (computed on the host, read by the kernels
