@@ -415,8 +415,7 @@ __global__ void __launch_bounds__(64 + 32 * kEpi1, 1)
 
 // ---------------------------------------------------------------- keep
 __global__ void __launch_bounds__(64, 1)
-    k_keep_dense(const int64_t* __restrict__ cost_part, const float* __restrict__ fe_part,
-                 int tiles_m, DevChains C) {
+    k_keep_dense(const int64_t* cost_part, const float* fe_part, int tiles_m, DevChains C) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait();
   pdl_release();
@@ -574,7 +573,7 @@ __global__ void __launch_bounds__(64 + 32 * (kBld + kEpi2), 1)
     uint8_t* __restrict__ Xs = a.X;
     float* __restrict__ nus = a.nu;
     uint8_t* __restrict__ bxs = a.best_x;
-    const uint8_t* __restrict__ impv = C.improved;
+    const uint8_t* impv = C.improved;
     const int quarter = warp & 3;
     const int i = tv * kBM + quarter * 32 + lane;
     const bool valid = i < a.n;
@@ -979,7 +978,7 @@ __global__ void __launch_bounds__(64 + 32 * (kBld + kEpi2), 1)
     uint8_t* __restrict__ Xs = a.X;
     float* __restrict__ nus = a.nu;
     uint8_t* __restrict__ bxs = a.best_x;
-    const uint8_t* __restrict__ impv = C.improved;
+    const uint8_t* impv = C.improved;
     const int quarter = warp & 3;
     const int i = tv * kBM + quarter * 32 + lane;
     const bool valid = i < a.n;

@@ -45,14 +45,14 @@ namespace {
 __device__ __forceinline__ uint32_t load4(const uint8_t* p, const uint8_t* lo, const uint8_t* hi) {
   const uint8_t* a = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(p) & ~(uintptr_t)3);
   if (a >= lo && a + 8 <= hi) {
-    const uint32_t w0 = __ldg(reinterpret_cast<const uint32_t*>(a));
-    const uint32_t w1 = __ldg(reinterpret_cast<const uint32_t*>(a) + 1);
+    const uint32_t w0 = reinterpret_cast<const uint32_t*>(a)[0];
+    const uint32_t w1 = reinterpret_cast<const uint32_t*>(a)[1];
     return __funnelshift_r(w0, w1, 8u * (uint32_t)(p - a));
   }
   uint32_t v = 0;
 #pragma unroll
   for (int k = 0; k < 4; ++k)
-    if (p + k < hi) v |= (uint32_t)__ldg(p + k) << (8 * k);
+    if (p + k < hi) v |= (uint32_t)p[k] << (8 * k);
   return v;
 }
 
@@ -71,7 +71,7 @@ __device__ __forceinline__ uint4 pack4(const uint8_t* row, int rows, int i, int 
       v[r] = 0u;
       if (i < n && g * 8 + r < rows) {
         const uint8_t* q = row + i + (size_t)(g * 8 + r) * n;
-        v[r] = A ? __ldg(reinterpret_cast<const uint32_t*>(q)) : load4(q, lo, hi);
+        v[r] = A ? *reinterpret_cast<const uint32_t*>(q) : load4(q, lo, hi);
       }
     }
     // bit r of byte k: row r's byte k is nonzero
@@ -91,10 +91,9 @@ __device__ __forceinline__ uint4 pack4(const uint8_t* row, int rows, int i, int 
 }
 
 template <bool A>
-__global__ void __launch_bounds__(256) k_pack_bits(const uint8_t* __restrict__ assign, int B,
-                                                   int n, int W, int nstride,
-                                                   uint32_t* __restrict__ X,
-                                                   int64_t* __restrict__ cost, size_t n_cost) {
+__global__ void __launch_bounds__(256) k_pack_bits(const uint8_t* assign, int B, int n, int W,
+                                                   int nstride, uint32_t* X, int64_t* cost,
+                                                   size_t n_cost) {
   pdl_release();
   // X and the costs may still be read or added into by the launch before
   pdl_wait();
@@ -187,10 +186,9 @@ __global__ void __launch_bounds__(256) k_bits_slabs(BitsFormula F, int n_pos) {
 // itself and writes their costs; assign stands for X.
 template <typename V, bool RAW, int WARPS, bool PACK>
 __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawFormula R,
-                                                          const uint32_t* __restrict__ X,
-                                                          const uint8_t* __restrict__ assign,
-                                                          int nstride, int B,
-                                                          unsigned long long* __restrict__ out) {
+                                                          const uint32_t* X,
+                                                          const uint8_t* assign, int nstride,
+                                                          int B, unsigned long long* out) {
   extern __shared__ __align__(16) uint32_t s_row[];
   __shared__ V s_lut[WARPS][128];
   __shared__ long long s_sum[WARPS][32];
@@ -226,9 +224,9 @@ __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawForm
   } else if ((v0 & 3) == 0) {
 #pragma unroll 8
     for (int k = threadIdx.x * 4; k < nv; k += 128 * WARPS)
-      *reinterpret_cast<uint4*>(s_row + k) = __ldg(reinterpret_cast<const uint4*>(row + k));
+      *reinterpret_cast<uint4*>(s_row + k) = *reinterpret_cast<const uint4*>(row + k);
   } else {
-    for (int k = threadIdx.x; k < nv; k += 32 * WARPS) s_row[k] = __ldg(row + k);
+    for (int k = threadIdx.x; k < nv; k += 32 * WARPS) s_row[k] = row[k];
   }
   if (threadIdx.x == 0) s_row[(nv + 3) / 4 * 4] = 0u;
   __syncthreads();
@@ -240,15 +238,19 @@ __global__ void __launch_bounds__(32 * WARPS) k_bits_cost(BitsFormula F, RawForm
     if constexpr (RAW) {
       const int c = 32 * k + lane;
       if (c < R.m) {
-        w = R.w ? (V)__ldg(R.w + c) : V(1);
-        const int64_t o0 = min(max(__ldg(R.off + c), (int64_t)0), R.n_lits);
-        const int64_t o1 = min(max(__ldg(R.off + c + 1), o0), R.n_lits);
-        for (int64_t j = o0; j < o1; ++j) {
-          const int32_t l = __ldg(R.lits + j);
-          // |INT32_MIN| does not fit an int: such a literal is out of range
-          const int64_t v = (l > 0 ? (int64_t)l : -(int64_t)l) - 1;
-          if (l == 0 || v < 0 || v >= nv) continue;
-          sat |= s_row[v] ^ (uint32_t)(l >> 31);
+        w = R.w ? (V)R.w[c] : V(1);
+        const int64_t o0 = min(max(R.off[c], (int64_t)0), R.n_lits);
+        const int64_t o1 = min(max(R.off[c + 1], o0), R.n_lits);
+        for (int64_t j = o0; j < o1; j += 4) {
+          int32_t l[4];  // four literals in flight
+#pragma unroll
+          for (int u = 0; u < 4; ++u) l[u] = j + u < o1 ? R.lits[j + u] : 0;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            // |INT32_MIN| does not fit an int: such a literal is out of range
+            const int64_t v = (l[u] > 0 ? (int64_t)l[u] : -(int64_t)l[u]) - 1;
+            if (l[u] != 0 && v < nv) sat |= s_row[v] ^ (uint32_t)(l[u] >> 31);
+          }
         }
       }
     } else {

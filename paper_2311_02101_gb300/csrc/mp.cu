@@ -255,8 +255,8 @@ __device__ __forceinline__ void gather_pair(const DevFormula& F, const float* sr
           if (base + u + v < (q ? L1.cnt : L0.cnt)) {
             const int o = e & 0x7FFFFFFF;
             s[q][v] = e < 0 ? -1.f : 1.f;
-            if (scale) s[q][v] *= __ldg(scale + o);
-            x[q][v] = __ldg(reinterpret_cast<const float4*>(src + (size_t)o * kH) + c);
+            if (scale) s[q][v] *= scale[o];
+            x[q][v] = *(reinterpret_cast<const float4*>(src + (size_t)o * kH) + c);
           }
         }
 #pragma unroll
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(256, 3) k_mp_fwd(DevFormula F, const float* sr
       for (int q = 0; q < 2; ++q) {
         const int r = tile * kTile + hr + 16 * (k + q);
         own[q] = row4(self, r, r < rows, c);
-        sc[q] = r < rows ? __ldg(out_scale + r) : 0.f;
+        sc[q] = r < rows ? out_scale[r] : 0.f;
       }
       gather_pair<CL>(F, src, nullptr, lists[k], lists[k + 1], c, v);
 #pragma unroll
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int r = tile * kTile + hr + 16 * (k + q);
-          const float z = r < rows ? __ldg(dz + r) : 0.f;
+          const float z = r < rows ? dz[r] : 0.f;
           d[q] = make_float4(z * __ldg(wo + 4 * c), z * __ldg(wo + 4 * c + 1),
                              z * __ldg(wo + 4 * c + 2), z * __ldg(wo + 4 * c + 3));
         }
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(256) k_mp_embed_bwd(DevFormula F, int nbv, con
     const float d0 = h.x > 0.f ? d.x : 0.f, d1 = h.y > 0.f ? d.y : 0.f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const float xk = __ldg(x + k);
+      const float xk = x[k];
       acc[k] = fmaf(d0, xk, acc[k]);
       acc[3 + k] = fmaf(d1, xk, acc[3 + k]);
     }
@@ -612,8 +612,8 @@ __global__ void __launch_bounds__(256) k_mp_embed_bwd(DevFormula F, int nbv, con
 #pragma unroll 4
       for (int j = j0; j < j1; ++j) {
         const int2 inc = __ldg(reinterpret_cast<const int2*>(F.var_inc + j));
-        const float sc = (inc.y < 0 ? -1.f : 1.f) * __ldg(in_scale + inc.x);
-        const float2 x = __ldg(reinterpret_cast<const float2*>(src + (size_t)inc.x * kH) + lane);
+        const float sc = (inc.y < 0 ? -1.f : 1.f) * in_scale[inc.x];
+        const float2 x = reinterpret_cast<const float2*>(src + (size_t)inc.x * kH)[lane];
         a.x = fmaf(sc, x.x, a.x);
         a.y = fmaf(sc, x.y, a.y);
       }

@@ -2,7 +2,11 @@
 // the stream finishes, sets itself up from data that no kernel in flight
 // writes (formula, tables), and waits for the predecessor's results before it
 // touches them. Every block of such a kernel waits, so a finished kernel means
-// that all before it are finished too.
+// that all before it are finished too. What a predecessor or the caller's work
+// before it writes is read by plain loads after the wait, never by __ldg or
+// through a const __restrict__ parameter: read-only loads are for data that does
+// not change while the kernel is in flight (formula, tables, weights), and may
+// be moved across the wait.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -108,7 +108,7 @@ template <int MODE, bool SM, typename HT, bool ONE>
 // 3-SAT n = 1000, m = 6000, 4096 chains); 3 for longer records, which spill
 // far more at 64 registers
 __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTables T, DevChains C,
-                                                const uint8_t* __restrict__ xt, int B, int Bp,
+                                                const uint8_t* xt, int B, int Bp,
                                                 GatherPlan P, const uint32_t* tdev,
                                                 uint32_t t_rel, int64_t* cost_part,
                                                 float* fe_part, int32_t* tickets,
@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
         uint2 x8[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-          x8[k] = k < len ? __ldg(reinterpret_cast<const uint2*>(xt + (size_t)lv[k] * Bp + b0))
+          x8[k] = k < len ? *reinterpret_cast<const uint2*>(xt + (size_t)lv[k] * Bp + b0)
                           : make_uint2(0u, 0u);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
           uint2 x8[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            x8[k] = k < len ? __ldg(reinterpret_cast<const uint2*>(
-                                  xt + (size_t)(lv[k] & 0x7FFFFFFF) * Bp + b0))
+            x8[k] = k < len ? *reinterpret_cast<const uint2*>(
+                                  xt + (size_t)(lv[k] & 0x7FFFFFFF) * Bp + b0)
                             : make_uint2(0u, 0u);
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(256, ONE ? 4 : 3) k_gather(DevFormula F, DevTa
           for (int k = 0; k < len; ++k) {
             const int32_t lv = __ldg(F.lit_var + o + k);
             const uint2 x8 =
-                __ldg(reinterpret_cast<const uint2*>(xt + (size_t)(lv & 0x7FFFFFFF) * Bp + b0));
+                *reinterpret_cast<const uint2*>(xt + (size_t)(lv & 0x7FFFFFFF) * Bp + b0);
             const uint32_t flip = lv < 0 ? 0x01010101u : 0u;
             if (k < 8) {
               lo0 |= (x8.x ^ flip) << k;
@@ -424,15 +424,15 @@ __device__ __forceinline__ void l2_prefetch(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// A load of chain state: through the read-only path when the state cannot
-// change during the launch, else from the L2 (CG: a persistent launch whose
-// other phase writes it; read-only cache lines could be stale there).
+// A load of chain state: a plain one after pdl_wait (not __ldg: the kernel is in
+// flight while its predecessor still writes), or from the L2 (CG: a launch whose
+// other phase writes it; L1 lines could be stale there).
 template <bool CG, typename V>
 __device__ __forceinline__ V ld_state(const V* p) {
   if constexpr (CG)
     return __ldcg(p);
   else
-    return __ldg(p);
+    return *p;
 }
 
 // The 8 state bytes of the thread's chains for each literal of clause record
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(256, 2) k_gather_nib(DevFormula F, DevTables T
   };
   const uint8_t* xtb = C.xt + b0;
   auto state_of = [&](int32_t l) {
-    return __ldg(reinterpret_cast<const uint2*>(xtb + (size_t)(l & 0x7FFFFFFF) * Bp));
+    return ld_state<false>(reinterpret_cast<const uint2*>(xtb + (size_t)(l & 0x7FFFFFFF) * Bp));
   };
   auto load_states = [&](const int4& r, const int32_t (&l)[4], uint2 (&x)[4]) {
 #pragma unroll

@@ -147,3 +147,24 @@ def test_packed_costs_of_the_largest_batch(ms, table):
     unit = (w[:, None] * (1 - X[:, first].T)).astype(np.int64)
     unit[at] = oracle.evaluate(big, X[:, at:at + big.n].copy())
     assert np.array_equal(got, unit)
+
+
+def test_evaluations_in_flight_together(ms, table):
+    """Evaluations of several assignment blocks launched one after another into
+    the same packed words, each overlapping the end of the one before."""
+    import torch
+    inst = random_formula(1000, 6000, 3, 9, 3)
+    stream = torch.cuda.Stream()
+    p = ms.maxsat_default_params(sets=table.sets, n_temps=1, n_buckets=1)
+    p.fstar = None
+    ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, stream)
+    X = np.random.default_rng(4).integers(0, 2, size=(5, 2048, inst.n), dtype=np.uint8)
+    xd = torch.from_numpy(X).cuda()
+    out = torch.full((60, X.shape[1]), -1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    for k in range(len(out)):
+        ms.maxsat_eval(ctx, xd[k % 5], out[k])
+    stream.synchronize()
+    ms.maxsat_destroy(ctx)
+    want = np.stack([oracle.evaluate(inst, x) for x in X])
+    assert np.array_equal(out.cpu().numpy(), want[np.arange(len(out)) % 5])
