@@ -132,9 +132,9 @@ typedef struct {
                             resident, the gather's and the visible update's
                             blocks walked by the same CTAs, grid barriers
                             between the phases (bounded waits: a wait that
-                            gives up after about 2 s makes the next
-                            maxsat_solve / maxsat_get_state fail with
-                            MAXSAT_ECUDA). Only for clauses of at most 3
+                            gives up after about 2 s makes maxsat_get_state,
+                            and the maxsat_solve that ran it, fail with
+                            MAXSAT_ECUDA until the chains are reset). Only for clauses of at most 3
                             literals on single-temperature chain octets,
                             without profiling and while no GPU unit
                             propagation is pending; otherwise the two-launch

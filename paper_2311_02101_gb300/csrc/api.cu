@@ -244,7 +244,8 @@ struct maxsat_ctx {
   int dev_Bp = 0;
   CUtensorMap tmXe[2] = {};
   int ev_buf = 0;                 // state buffer of the next evaluation
-  int* d_err = nullptr;           // device wait-timeout code (0 = none)
+  int* d_err = nullptr;           // device wait-timeout codes (0 = none): tensor-core pipelines;
+                                  // rounds of many per launch (cleared with the chains)
   uint32_t* d_bar = nullptr;      // persistent round: grid-barrier arrivals and give-up flag
   // resident rounds (k_rounds) of the current chains: blocks per chain tile (0:
   // not used), its buffers, and what the next launch starts from
@@ -254,7 +255,7 @@ struct maxsat_ctx {
   LocalPlan local_shape;          // for the current chains (threads 0: not used)
   int rounds_slot_count = -1;     // resident blocks of k_rounds (-1: not queried)
   int rounds_per_sm = 0;
-  bool persist_ran = false;       // some maxsat_step ran persistent launches (read d_err)
+  bool persist_ran = false;       // some maxsat_step ran many rounds per launch (read d_err)
   // dense scatter-add (GEMM2): block-diagonal variable x incidence matrix
   int tiles_v = 0, kmax = 0;
   bool g_bf16 = true;             // G operand BF16 (else FP16)
@@ -578,21 +579,21 @@ int plan_rounds(maxsat_ctx* ctx, DevAllocs& A, int Bp) {
   CK(ctx, A.alloc(&R.bar, (size_t)tiles * 2 * kBarStride));
   CK(ctx, A.alloc(&R.best, (size_t)Bp));
   CK(ctx, A.alloc(&R.acc, (size_t)6 * Bp));
-  R.err = ctx->d_err;
+  R.err = ctx->d_err + 1;
   R.S = S;
   return MAXSAT_OK;
 }
 
-// Fresh barrier counts and accumulators for the resident rounds.
+// Fresh barrier counts, accumulators and wait code for new chains' rounds (what
+// a launch that gave up left behind goes with the chains it left unfinished).
 int clear_rounds(maxsat_ctx* ctx) {
   RoundsArgs& R = ctx->rounds;
+  if (ctx->persist_ran) CK(ctx, cudaMemsetAsync(ctx->d_err + 1, 0, sizeof(int), ctx->stream));
   if (R.S == 0) return MAXSAT_OK;
   const int Bp = ctx->C.Bp;
   CK(ctx, cudaMemsetAsync(R.bar, 0, 4 * (size_t)(Bp / kChainTile) * 2 * kBarStride,
                           ctx->stream));
   CK(ctx, cudaMemsetAsync(R.acc, 0, 8 * (size_t)6 * Bp, ctx->stream));
-  R.done0 = R.ticket0 = 0;
-  R.acc0 = 0;
   return MAXSAT_OK;
 }
 
@@ -667,10 +668,11 @@ int alloc_chains(maxsat_ctx* ctx, int32_t B) {
 
 // Copies h to a new device buffer padded with zeros to a multiple of 16 bytes
 // (kernels stage tables into shared memory 16 bytes at a time).
-// Reads the kernels' wait-timeout code (call after synchronising the stream).
+// Reads the kernels' wait-timeout codes (call after synchronising the stream).
 int check_device_error(maxsat_ctx* ctx) {
-  int code = 0;
-  CK(ctx, cudaMemcpy(&code, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost));
+  int codes[2] = {0, 0};
+  CK(ctx, cudaMemcpy(codes, ctx->d_err, sizeof(codes), cudaMemcpyDeviceToHost));
+  const int code = codes[0] != 0 ? codes[0] : codes[1];
   if (code != 0)
     return fail(ctx, MAXSAT_ECUDA,
                 std::string(code == 16 ? "a block barrier of the resident or persistent rounds"
@@ -1777,9 +1779,9 @@ static int create_impl(maxsat_ctx** out, int32_t n, int64_t m, const int64_t* of
   }
   {
     cudaError_t e = A.alloc(&ctx->d_t, 1);
-    if (e == cudaSuccess) e = A.alloc(&ctx->d_err, 1);
+    if (e == cudaSuccess) e = A.alloc(&ctx->d_err, 2);
     if (e == cudaSuccess) e = A.alloc(&ctx->d_bar, 2);
-    if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, 2 * sizeof(int));
     if (e != cudaSuccess) {
       delete ctx;
       return cuda_fail(nullptr, e, "cudaMalloc");
@@ -1889,17 +1891,6 @@ static bool persistent_round_active(const maxsat_ctx* ctx) {
          persistent_round_supported(ctx->T, ctx->C, ctx->F, ctx->wide_h);
 }
 
-// The caller is capturing the context's stream: a resident launch carries the
-// barrier counts it starts from, so it cannot be replayed.
-static bool stream_capturing(cudaStream_t st) {
-  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) {
-    cudaGetLastError();
-    return true;
-  }
-  return s != cudaStreamCaptureStatusNone;
-}
-
 // rounds per launch of the resident rounds
 static constexpr int64_t kMaxResidentRounds = 1000;
 
@@ -1910,7 +1901,7 @@ static constexpr int64_t kMinLocalRounds = 8;
 // maxsat_step runs local rounds (local.cu)
 static bool local_rounds_active(const maxsat_ctx* ctx) {
   return ctx->have_chains && !ctx->dense && ctx->local_shape.threads > 0 && ctx->C.nib &&
-         !ctx->profiling && !stream_capturing(ctx->stream);
+         !ctx->profiling;
 }
 
 // maxsat_step runs resident rounds (k_rounds): planned for these chains, no
@@ -1918,7 +1909,7 @@ static bool local_rounds_active(const maxsat_ctx* ctx) {
 // rounds on a side stream; blocks that wait would hold the SMs it could use)
 static bool resident_rounds_active(const maxsat_ctx* ctx) {
   return ctx->have_chains && !ctx->dense && ctx->rounds.S > 0 && ctx->C.nib && !ctx->profiling &&
-         !(ctx->up_pending && ctx->up_on_gpu) && !stream_capturing(ctx->stream);
+         !(ctx->up_pending && ctx->up_on_gpu);
 }
 
 int maxsat_get_persistent_round(const maxsat_ctx* ctx) {
@@ -2002,10 +1993,6 @@ int maxsat_step(maxsat_ctx* ctx, int64_t steps) {
       CK(ctx, launch_rounds(ctx->F, ctx->T, ctx->C, R, ctx->rounds_cost16, (float)ctx->prm.alpha,
                             ctx->stream));
       ctx->persist_ran = true;
-      // every share finished; every block drew one ticket past the last
-      R.done0 += 2u * (uint32_t)R.rounds * (uint32_t)R.S;
-      R.ticket0 += (2u * (uint32_t)R.rounds + 1u) * (uint32_t)R.S;
-      R.acc0 = (R.acc0 + R.rounds) % 3;
       ctx->t += (uint32_t)R.rounds;
       ctx->d_t_synced = false;
       steps -= R.rounds;
@@ -2017,7 +2004,7 @@ int maxsat_step(maxsat_ctx* ctx, int64_t steps) {
     while (steps > 0) {
       const int r = (int)std::min(steps, chunk);
       CK(ctx, launch_round_persistent(ctx->F, ctx->T, ctx->C, ctx->plan, ctx->t, r,
-                                      (float)ctx->prm.alpha, ctx->d_bar, ctx->d_err,
+                                      (float)ctx->prm.alpha, ctx->d_bar, ctx->d_err + 1,
                                       ctx->stream));
       ctx->persist_ran = true;
       ctx->t += (uint32_t)r;

@@ -437,15 +437,14 @@ cudaError_t launch_visible(const DevFormula& F, const DevTables& T, const DevCha
 bool nib_patterns_supported(const DevTables& T, int B_total);
 // Resident rounds of one formula (k_rounds): `rounds` rounds from t0 in one
 // launch of S blocks per tile of 256 chains. bar: per tile the count of finished
-// shares, done0 at the launch's start, and kBarStride words on the count of
-// tickets, ticket0 (a launch adds 2 rounds S and (2 rounds + 1) S); acc: 3
-// buffers of 2 Bp 64-bit sums, buffer acc0 % 3 zero; err: device error code (16 =
-// a wait gave up after about 2 s).
+// shares and, kBarStride words on, of tickets; acc: 3 buffers of 2 Bp 64-bit
+// sums. Both counts and the first buffer are zero at a launch's start and end.
+// err: device error code (16 = a wait gave up after about 2 s; set at its start,
+// a launch does nothing).
 constexpr int kBarStride = 32;
 struct RoundsArgs {
   uint32_t t0 = 0;
-  int rounds = 0, S = 0, acc0 = 0;
-  uint32_t done0 = 0, ticket0 = 0;  // the counters at the launch's start
+  int rounds = 0, S = 0;
   uint32_t* bar = nullptr;
   int64_t* best = nullptr;  // Bp: best costs after odd rounds of a launch
   unsigned long long* acc = nullptr;

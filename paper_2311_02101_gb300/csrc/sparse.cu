@@ -1386,7 +1386,11 @@ __global__ void __launch_bounds__(256, BLOCKS)
 //  - State that another block wrote is read from the L2 (ld.global.cg,
 //    cp.async.cg); the barrier's release and acquire order it.
 // Every barrier wait is bounded (about 2 s): a block that gives up records
-// kErrGridBarrier and leaves, and so do the others of its tile.
+// kErrGridBarrier and leaves, and so do the others of its tile; launches after it
+// leave at once until the counters and the code are cleared for new chains.
+// A launch that ends leaves its counters and the accumulators of its first round
+// at zero, so that a launch depends on nothing the host would have to carry from
+// one to the next (a reset that is captured, but not run, changes no counter).
 // ---------------------------------------------------------------------------
 constexpr long long kBarrierWaitCycles = 4000000000LL;  // ~2 s at 2 GHz
 constexpr int kErrGridBarrier = 16;                    // device error code of a barrier timeout
@@ -1403,8 +1407,8 @@ __device__ __forceinline__ uint32_t ld_relaxed_gpu(const uint32_t* p) {
   return v;
 }
 
-// The end of a share, and the block's next ticket: done counts finished shares
-// and is never cleared; *s_seen receives the count with this one.
+// The end of a share, and the block's next ticket: done counts finished shares;
+// *s_seen receives the count with this one.
 // The block's next ticket is drawn only now: drawn at a share's start, two of
 // one phase can fall to one block and none to another, and that repeats.
 __device__ __forceinline__ uint32_t tile_next(uint32_t* done, uint32_t* tickets, int* s_seen,
@@ -1494,8 +1498,9 @@ __global__ void __launch_bounds__(256, 3)
     nib_copy_rows(win, cnt, H, hstride, rows_s + (uint32_t)(buf * kRowBuf), s_off[warp][buf], lane);
   };
   if (tid == 0) {
-    s_ticket = atomicAdd(tickets, 1u) - A.ticket0;
-    s_go = (int)A.done0;
+    s_go = 0;
+    // (no share for anyone once an earlier launch gave up)
+    s_ticket = *reinterpret_cast<const volatile int*>(A.err) == 0 ? atomicAdd(tickets, 1u) : ~0u;
   }
   __syncthreads();
 
@@ -1504,10 +1509,10 @@ __global__ void __launch_bounds__(256, 3)
   while (cur < items) {
     const uint32_t phase = cur / (uint32_t)S;
     const int share = (int)(cur - phase * (uint32_t)S), r = (int)(phase >> 1);
-    const uint32_t target = A.done0 + phase * (uint32_t)S;
+    const uint32_t target = phase * (uint32_t)S;
     const uint32_t t = A.t0 + (uint32_t)r;
     const bool last = r + 1 == A.rounds;
-    const int buf = (A.acc0 + r) % 3, clear = (A.acc0 + r + 1) % 3;
+    const int buf = r % 3, clear = (r + 1) % 3;
     unsigned long long* acc_cost = A.acc + (size_t)buf * 2 * C.Bp + b;
     unsigned long long* acc_fe = acc_cost + C.Bp;
     if ((phase & 1u) == 0) {
@@ -1626,12 +1631,21 @@ __global__ void __launch_bounds__(256, 3)
         n1 = m1;
       }
     }
-    cur = tile_next(done, tickets, &s_go, &s_ticket) - A.ticket0;
+    cur = tile_next(done, tickets, &s_go, &s_ticket);
   }
-  // an odd number of rounds leaves the best costs in the second buffer: the
-  // block that finished the tile's last share moves them
+  // The block that drew the tile's last ticket (each of the S blocks draws one
+  // past the shares) clears the ticket counter: no block draws after it.
+  if (tid == 0 && cur == items + (uint32_t)S - 1u) *tickets = 0u;
+  // The block that finished the tile's last share clears the count of finished
+  // shares, which no block waits for any more, and the first round's
+  // accumulators; an odd number of rounds leaves the best costs in the second
+  // buffer, and it moves them. (s_go: 0 in a block that had no share.)
+  if (s_go != (int)items) return;
   __threadfence();
-  if ((A.rounds & 1) && s_go == (int)(A.done0 + items)) C.best[b] = __ldcg(A.best + b);
+  if (tid == 0) *done = 0u;
+  A.acc[b] = 0ull;
+  A.acc[C.Bp + b] = 0ull;
+  if (A.rounds & 1) C.best[b] = __ldcg(A.best + b);
 }
 
 // ---------------------------------------------------------------------------
