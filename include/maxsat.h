@@ -126,26 +126,30 @@ typedef struct {
                             another. Same results for every value; no effect
                             where hidden patterns take 4 bits (that update
                             copies whole windows ahead). Default 0 */
-  int32_t persistent_round; /* 1: maxsat_step runs its sparse rounds as one
-                            persistent cooperative launch per
-                            max(1, steps_per_graph) rounds: every block
-                            resident, the gather's and the visible update's
-                            blocks walked by the same CTAs, grid barriers
-                            between the phases (bounded waits: a wait that
-                            gives up after about 2 s makes maxsat_get_state,
-                            and the maxsat_solve that ran it, fail with
-                            MAXSAT_ECUDA until the chains are reset). Only for clauses of at most 3
-                            literals on single-temperature chain octets,
-                            without profiling and while no GPU unit
-                            propagation is pending; otherwise the two-launch
-                            round runs (maxsat_get_persistent_round tells).
-                            Same results bit for bit. Default 0: one formula
-                            of clauses of at most 3 literals with 4-bit hidden
-                            patterns runs many rounds per launch too (each
-                            tile of 256 chains with barriers of its own, or
-                            small formulas one block per 8 chains); the rest
-                            takes two launches per round with programmatic
-                            dependent launch, replayed from CUDA graphs */
+  int32_t persistent_round; /* 1: maxsat_step runs its sparse rounds in launches
+                            of up to max(1, steps_per_graph) rounds. One formula
+                            with 4-bit hidden patterns takes the launches of
+                            many rounds that it takes by default (below), cut
+                            to that length; else one cooperative launch has
+                            every block resident, the gather's and the visible
+                            update's blocks walked by the same CTAs, grid
+                            barriers between the phases. Only for clauses of
+                            at most 3 literals on single-temperature chain
+                            octets, without profiling and while no GPU unit
+                            propagation is pending; otherwise as by default
+                            (maxsat_get_persistent_round tells). Same results
+                            bit for bit, the free energy up to its summation
+                            order. Default 0: one formula of clauses of at most
+                            3 literals with 4-bit hidden patterns runs up to
+                            1000 rounds per launch (each tile of 256 chains
+                            with barriers of its own, or small formulas one
+                            block per 8 chains); the rest takes two launches
+                            per round with programmatic dependent launch,
+                            replayed from CUDA graphs. Waits between blocks of
+                            a launch are bounded: one that gives up after about
+                            2 s makes maxsat_get_state, and the maxsat_solve
+                            that ran it, fail with MAXSAT_ECUDA until the
+                            chains are reset */
 } maxsat_params;
 
 typedef struct maxsat_ctx maxsat_ctx;
@@ -221,9 +225,9 @@ int maxsat_get_clause_block(const maxsat_ctx* ctx);
  * params.tune_blocks); a negative code for a NULL context. */
 int maxsat_get_visible_batch(const maxsat_ctx* ctx);
 
-/* 1 when maxsat_step runs the current chains' rounds as persistent launches
- * (params.persistent_round and the context qualifies), 0 when it runs the
- * two-launch round; a negative code for a NULL context. */
+/* 1 when params.persistent_round is set and covers the current chains' rounds
+ * (see there), 0 when they run as by default; a negative code for a NULL
+ * context. */
 int maxsat_get_persistent_round(const maxsat_ctx* ctx);
 
 /* Starts B fresh chains (Fig. code initialisation): every variable drawn
