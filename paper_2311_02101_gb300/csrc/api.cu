@@ -830,6 +830,125 @@ void set_ensemble(maxsat_ctx* ctx, int32_t g8_off, int32_t B_total) {
                    : 0;
 }
 
+// params.persistent_round covers maxsat_step's rounds: requested, sparse chains
+// that the cooperative launch covers, no per-kernel profiling, no GPU unit
+// propagation pending (its side-stream kernel shares the SMs that launch must
+// hold). Where local or resident rounds apply they run instead (weighted 3-SAT
+// n = 1000, m = 6000, 4096 chains: 54.9 us a round against 74.9).
+bool persistent_round_active(const maxsat_ctx* ctx) {
+  return ctx->prm.persistent_round && ctx->have_chains && !ctx->dense && !ctx->profiling &&
+         !(ctx->up_pending && ctx->up_on_gpu) &&
+         persistent_round_supported(ctx->T, ctx->C, ctx->F, ctx->wide_h);
+}
+
+// rounds per launch of the local and resident rounds
+constexpr int64_t kMaxResidentRounds = 1000;
+int64_t rounds_per_launch(const maxsat_ctx* ctx) {
+  return ctx->prm.persistent_round
+             ? std::min<int64_t>(kMaxResidentRounds, std::max(1, ctx->prm.steps_per_graph))
+             : kMaxResidentRounds;
+}
+
+// rounds of a call from which the local rounds pay for loading the formula into
+// every block
+constexpr int64_t kMinLocalRounds = 8;
+
+// maxsat_step runs local rounds (local.cu)
+bool local_rounds_active(const maxsat_ctx* ctx) {
+  return ctx->have_chains && !ctx->dense && ctx->local_shape.threads > 0 && ctx->C.nib &&
+         !ctx->profiling;
+}
+
+// maxsat_step runs resident rounds (k_rounds): planned for these chains, no
+// per-kernel profiling, no GPU unit propagation pending (it runs beside the
+// rounds on a side stream; blocks that wait would hold the SMs it could use)
+bool resident_rounds_active(const maxsat_ctx* ctx) {
+  return ctx->have_chains && !ctx->dense && ctx->rounds.S > 0 && ctx->C.nib && !ctx->profiling &&
+         !(ctx->up_pending && ctx->up_on_gpu);
+}
+
+// maxsat_step runs `steps` rounds in launches of many
+bool many_rounds_apply(const maxsat_ctx* ctx, int64_t steps) {
+  return (steps >= kMinLocalRounds && local_rounds_active(ctx)) || resident_rounds_active(ctx) ||
+         persistent_round_active(ctx);
+}
+
+// (where many_rounds_apply)
+int run_many_rounds(maxsat_ctx* ctx, int64_t steps) {
+  if (steps >= kMinLocalRounds && local_rounds_active(ctx)) {
+    while (steps > 0) {
+      const int r = (int)std::min<int64_t>(steps, rounds_per_launch(ctx));
+      CK(ctx, launch_rounds_local(ctx->F, ctx->T, ctx->C, ctx->local, ctx->local_shape, ctx->t, r,
+                                  (float)ctx->prm.alpha, ctx->stream));
+      ctx->t += (uint32_t)r;
+      ctx->d_t_synced = false;
+      steps -= r;
+    }
+    return MAXSAT_OK;
+  }
+  if (resident_rounds_active(ctx)) {
+    while (steps > 0) {
+      RoundsArgs& R = ctx->rounds;
+      R.t0 = ctx->t;
+      R.rounds = (int)std::min<int64_t>(steps, rounds_per_launch(ctx));
+      CK(ctx, launch_rounds(ctx->F, ctx->T, ctx->C, R, ctx->rounds_cost16, (float)ctx->prm.alpha,
+                            ctx->stream));
+      ctx->persist_ran = true;
+      ctx->t += (uint32_t)R.rounds;
+      ctx->d_t_synced = false;
+      steps -= R.rounds;
+    }
+    return MAXSAT_OK;
+  }
+  while (steps > 0) {
+    const int r = (int)std::min<int64_t>(steps, std::max(1, ctx->prm.steps_per_graph));
+    CK(ctx, launch_round_persistent(ctx->F, ctx->T, ctx->C, ctx->plan, ctx->t, r,
+                                    (float)ctx->prm.alpha, ctx->d_bar, ctx->d_err + 1,
+                                    ctx->stream));
+    ctx->persist_ran = true;
+    ctx->t += (uint32_t)r;
+    ctx->d_t_synced = false;
+    steps -= r;
+  }
+  return MAXSAT_OK;
+}
+
+// Times new chains' rounds in the form that maxsat_step will run (two launches a
+// round without a graph): `warm` rounds, then `rounds` more (where local rounds
+// apply, as many as they start from); ms per round. Leaves no valid chains.
+int time_rounds(maxsat_ctx* ctx, int32_t B, int warm, int rounds, cudaEvent_t e0, cudaEvent_t e1,
+                float* ms_per_round) {
+  int rc = alloc_chains(ctx, B);
+  if (rc != MAXSAT_OK) return rc;
+  ctx->C.keys = philox_keys(0x5EEDu, 0u);
+  set_ensemble(ctx, 0, B);
+  CK(ctx, ctx->dense ? launch_init_dense(ctx->C, ctx->dX, ctx->dnu, ctx->dbest_x, ctx->n,
+                                         ctx->n_pad, ctx->e5m2, ctx->stream)
+                     : launch_init_sparse(ctx->F, ctx->C, ctx->n, ctx->stream));
+  if ((rc = clear_rounds(ctx)) != MAXSAT_OK) return rc;
+  ctx->have_chains = true;
+  ctx->t = 0;
+  if (local_rounds_active(ctx)) warm = rounds = (int)kMinLocalRounds;
+  for (int part = 0; part < 2 && rc == MAXSAT_OK; ++part) {
+    const int n = part == 0 ? warm : rounds;
+    if (part == 1) cudaEventRecord(e0, ctx->stream);
+    if (many_rounds_apply(ctx, n)) {
+      rc = run_many_rounds(ctx, n);
+    } else {
+      for (int r = 0; r < n && rc == MAXSAT_OK; ++r)
+        rc = launch_round(ctx, ctx->stream, nullptr, ctx->t++);
+    }
+  }
+  ctx->have_chains = false;
+  if (rc != MAXSAT_OK) return rc;
+  cudaEventRecord(e1, ctx->stream);
+  CK(ctx, cudaEventSynchronize(e1));
+  float ms = 0.f;
+  CK(ctx, cudaEventElapsedTime(&ms, e0, e1));
+  *ms_per_round = ms / (float)rounds;
+  return MAXSAT_OK;
+}
+
 // Measured path choice (MAXSAT_PATH_AUTO): times a few Gibbs rounds of B
 // chains on the sparse path, then on the dense path unless its tensor-core
 // products alone (at nominal peaks) would take longer than the measured
@@ -867,32 +986,7 @@ int choose_path(maxsat_ctx* ctx, int32_t B) {
       if (!ctx->dense_built) break;
     }
     ctx->dense = d == 1;
-    rc = alloc_chains(ctx, B);
-    if (rc != MAXSAT_OK) break;
-    ctx->C.keys = philox_keys(0x5EEDu, 0u);
-    set_ensemble(ctx, 0, B);
-    cudaError_t e = ctx->dense ? launch_init_dense(ctx->C, ctx->dX, ctx->dnu, ctx->dbest_x, ctx->n,
-                                                   ctx->n_pad, ctx->e5m2, ctx->stream)
-                               : launch_init_sparse(ctx->F, ctx->C, ctx->n, ctx->stream);
-    if (e != cudaSuccess) {
-      rc = cuda_fail(ctx, e, "init");
-      break;
-    }
-    constexpr int kRounds = 3;
-    for (int r = 0; r <= kRounds && rc == MAXSAT_OK; ++r) {
-      if (r == 1) cudaEventRecord(e0, ctx->stream);
-      rc = launch_round(ctx, ctx->stream, nullptr, (uint32_t)r);
-    }
-    if (rc != MAXSAT_OK) break;
-    cudaEventRecord(e1, ctx->stream);
-    e = cudaEventSynchronize(e1);
-    if (e != cudaSuccess) {
-      rc = cuda_fail(ctx, e, "cudaEventSynchronize");
-      break;
-    }
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    ctx->auto_ms[d] = ms / kRounds;
+    rc = time_rounds(ctx, B, 1, 3, e0, e1, &ctx->auto_ms[d]);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -933,28 +1027,10 @@ int tune_blocks(maxsat_ctx* ctx, int32_t B) {
   ctx->profiling = false;
   ctx->tune_ms.clear();
   ctx->tune_vis_ms.clear();
-  // ms per round of the current shape (fresh chains, 2 warm-up rounds)
-  auto time_rounds = [&](float* ms_out) -> int {
+  // ms per round of the current shape (new chains, 2 warm-up rounds)
+  auto time_shape = [&](float* ms_out) -> int {
     ctx->have_chains = false;
-    int r0 = alloc_chains(ctx, B);
-    if (r0 != MAXSAT_OK) return r0;
-    ctx->C.keys = philox_keys(0x5EEDu, 0u);
-    set_ensemble(ctx, 0, B);
-    cudaError_t e = launch_init_sparse(ctx->F, ctx->C, ctx->n, ctx->stream);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "init");
-    constexpr int kWarm = 2, kRounds = 6;
-    for (int r = 0; r < kWarm + kRounds; ++r) {
-      if (r == kWarm) cudaEventRecord(e0, ctx->stream);
-      r0 = launch_round(ctx, ctx->stream, nullptr, (uint32_t)r);
-      if (r0 != MAXSAT_OK) return r0;
-    }
-    cudaEventRecord(e1, ctx->stream);
-    e = cudaEventSynchronize(e1);
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaEventSynchronize");
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
-    *ms_out = ms / kRounds;
-    return MAXSAT_OK;
+    return time_rounds(ctx, B, 2, 6, e0, e1, ms_out);
   };
   std::map<int, float> best_of;  // clause block actually used -> fastest ms per round
   int rc = MAXSAT_OK;
@@ -962,7 +1038,7 @@ int tune_blocks(maxsat_ctx* ctx, int32_t B) {
     for (int cb : cand) {
       ctx->cb_force = cb;
       float ms = 0.f;
-      rc = time_rounds(&ms);
+      rc = time_shape(&ms);
       if (rc != MAXSAT_OK) break;
       ctx->tune_ms.emplace_back(ctx->gather_cb, ms);
       auto it = best_of.find(ctx->gather_cb);
@@ -984,7 +1060,7 @@ int tune_blocks(maxsat_ctx* ctx, int32_t B) {
     for (int vb : {2, 4, 8}) {
       ctx->vis_batch = vb;
       float ms = 0.f;
-      rc = time_rounds(&ms);
+      rc = time_shape(&ms);
       if (rc != MAXSAT_OK) break;
       ctx->tune_vis_ms.emplace_back(vb, ms);
       auto it = vis_of.find(vb);
@@ -1882,43 +1958,6 @@ int maxsat_get_visible_batch(const maxsat_ctx* ctx) {
   return ctx->vis_batch;
 }
 
-// params.persistent_round covers maxsat_step's rounds: requested, sparse chains
-// that the cooperative launch covers, no per-kernel profiling, no GPU unit
-// propagation pending (its side-stream kernel shares the SMs that launch must
-// hold). Where local or resident rounds apply they run instead (weighted 3-SAT
-// n = 1000, m = 6000, 4096 chains: 54.9 us a round against 74.9).
-static bool persistent_round_active(const maxsat_ctx* ctx) {
-  return ctx->prm.persistent_round && ctx->have_chains && !ctx->dense && !ctx->profiling &&
-         !(ctx->up_pending && ctx->up_on_gpu) &&
-         persistent_round_supported(ctx->T, ctx->C, ctx->F, ctx->wide_h);
-}
-
-// rounds per launch of the local and resident rounds
-static constexpr int64_t kMaxResidentRounds = 1000;
-static int64_t rounds_per_launch(const maxsat_ctx* ctx) {
-  return ctx->prm.persistent_round
-             ? std::min<int64_t>(kMaxResidentRounds, std::max(1, ctx->prm.steps_per_graph))
-             : kMaxResidentRounds;
-}
-
-// rounds of a call from which the local rounds pay for loading the formula into
-// every block
-static constexpr int64_t kMinLocalRounds = 8;
-
-// maxsat_step runs local rounds (local.cu)
-static bool local_rounds_active(const maxsat_ctx* ctx) {
-  return ctx->have_chains && !ctx->dense && ctx->local_shape.threads > 0 && ctx->C.nib &&
-         !ctx->profiling;
-}
-
-// maxsat_step runs resident rounds (k_rounds): planned for these chains, no
-// per-kernel profiling, no GPU unit propagation pending (it runs beside the
-// rounds on a side stream; blocks that wait would hold the SMs it could use)
-static bool resident_rounds_active(const maxsat_ctx* ctx) {
-  return ctx->have_chains && !ctx->dense && ctx->rounds.S > 0 && ctx->C.nib && !ctx->profiling &&
-         !(ctx->up_pending && ctx->up_on_gpu);
-}
-
 int maxsat_get_persistent_round(const maxsat_ctx* ctx) {
   if (!ctx) return MAXSAT_EINVAL;
   return persistent_round_active(ctx) ? 1 : 0;
@@ -1981,45 +2020,7 @@ int maxsat_step(maxsat_ctx* ctx, int64_t steps) {
   if (!ctx->have_chains) return fail(ctx, MAXSAT_ESTATE, "maxsat_step before maxsat_reset");
   if (steps < 0) return fail(ctx, MAXSAT_EINVAL, "steps must be >= 0");
   if ((uint64_t)ctx->t + (uint64_t)steps > 0xFFFFFFFFull) return fail(ctx, MAXSAT_EINVAL, "round index would exceed 2^32");
-  if (steps >= kMinLocalRounds && local_rounds_active(ctx)) {
-    while (steps > 0) {
-      const int r = (int)std::min<int64_t>(steps, rounds_per_launch(ctx));
-      CK(ctx, launch_rounds_local(ctx->F, ctx->T, ctx->C, ctx->local, ctx->local_shape, ctx->t, r,
-                                  (float)ctx->prm.alpha, ctx->stream));
-      ctx->t += (uint32_t)r;
-      ctx->d_t_synced = false;
-      steps -= r;
-    }
-    return MAXSAT_OK;
-  }
-  if (resident_rounds_active(ctx)) {
-    while (steps > 0) {
-      RoundsArgs& R = ctx->rounds;
-      R.t0 = ctx->t;
-      R.rounds = (int)std::min<int64_t>(steps, rounds_per_launch(ctx));
-      CK(ctx, launch_rounds(ctx->F, ctx->T, ctx->C, R, ctx->rounds_cost16, (float)ctx->prm.alpha,
-                            ctx->stream));
-      ctx->persist_ran = true;
-      ctx->t += (uint32_t)R.rounds;
-      ctx->d_t_synced = false;
-      steps -= R.rounds;
-    }
-    return MAXSAT_OK;
-  }
-  if (persistent_round_active(ctx)) {
-    const int64_t chunk = std::max(1, ctx->prm.steps_per_graph);
-    while (steps > 0) {
-      const int r = (int)std::min(steps, chunk);
-      CK(ctx, launch_round_persistent(ctx->F, ctx->T, ctx->C, ctx->plan, ctx->t, r,
-                                      (float)ctx->prm.alpha, ctx->d_bar, ctx->d_err + 1,
-                                      ctx->stream));
-      ctx->persist_ran = true;
-      ctx->t += (uint32_t)r;
-      ctx->d_t_synced = false;
-      steps -= r;
-    }
-    return MAXSAT_OK;
-  }
+  if (many_rounds_apply(ctx, steps)) return run_many_rounds(ctx, steps);
   const int S = ctx->profiling ? 0 : ctx->prm.steps_per_graph;
   while (steps > 0) {
     if (S > 0 && steps >= S) {

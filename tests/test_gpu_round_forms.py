@@ -92,3 +92,23 @@ def test_many_rounds_a_launch_equal_two_launches_at_full_size(ms):
         for k in EXACT:
             assert np.array_equal(two[k], many[k]), (persist, k)
         np.testing.assert_allclose(many["free_energy"], two["free_energy"], rtol=1e-3, atol=1e-6)
+
+
+@pytest.mark.parametrize("n,m,B", [(50, 215, 300), (60, 300, 1300), (600, 3600, 1024)])
+def test_rounds_after_measured_choices(ms, n, m, B):
+    """The path choice and the tuner run the forms they choose between (one block
+    per octet, shares by ticket) on the chains' own buffers before the reset."""
+    import torch
+    table, seed, rounds = table_of(4), 64, 13
+    inst = oracle.Instance(*workloads.random_ksat(n, m, 3, 64, 50))
+    p = ms.maxsat_default_params(sets=table.sets, n_temps=2, n_buckets=1, alpha=ALPHA,
+                                 quant_bits=4, path=ms.MAXSAT_PATH_AUTO, tune_blocks=1)
+    p.fstar = None
+    ctx = ms.maxsat_create(inst.n, inst.off, inst.lits, inst.w, p, torch.cuda.Stream())
+    for b in (B // 2, B):
+        ms.maxsat_reset(ctx, b, seed)
+    ms.maxsat_step(ctx, 3)
+    ms.maxsat_step(ctx, rounds - 3)
+    g = ms.maxsat_get_state(ctx)
+    ms.maxsat_destroy(ctx)
+    same_as_oracle(g, table, inst, B, seed, rounds)
