@@ -1499,8 +1499,9 @@ __global__ void __launch_bounds__(256, 3)
   };
   if (tid == 0) {
     s_go = 0;
-    // (no share for anyone once an earlier launch gave up)
-    s_ticket = *reinterpret_cast<const volatile int*>(A.err) == 0 ? atomicAdd(tickets, 1u) : ~0u;
+    // no share for anyone once an earlier launch gave up (both in flight together)
+    const uint32_t ticket = atomicAdd(tickets, 1u);
+    s_ticket = *reinterpret_cast<const volatile int*>(A.err) == 0 ? ticket : ~0u;
   }
   __syncthreads();
 
@@ -1976,10 +1977,6 @@ cudaError_t visible_nib(const DevFormula& F, const DevTables& T, const DevChains
 
 }  // namespace
 
-// Nibble patterns: the contribution rows were built (every chunk's |2^Q G| <=
-// 1023, so a window of 32 incidences fits 16 bits) and fit shared memory with
-// two blocks per SM, and no octet of chains spans more than
-// two temperatures (temperature blocks of at least 8 chains).
 cudaError_t launch_inc_rows(const DevFormula& F, const int4* groups, int gq_len, bool one_chunk,
                             int2* inc8, cudaStream_t st) {
   if (F.n <= 0) return cudaSuccess;
@@ -1987,6 +1984,10 @@ cudaError_t launch_inc_rows(const DevFormula& F, const int4* groups, int gq_len,
   return cudaGetLastError();
 }
 
+// Nibble patterns: the contribution rows were built (every chunk's |2^Q G| <=
+// 1023, so a window of 32 incidences fits 16 bits) and fit shared memory with
+// two blocks per SM, and no octet of chains spans more than
+// two temperatures (temperature blocks of at least 8 chains).
 bool nib_patterns_supported(const DevTables& T, int B_total) {
   return (T.one_chunk || T.recn) && T.ptab && nib_smem_bytes(T) <= kNibSmemLimit &&
          (T.n_temps == 1 || B_total / T.n_temps >= 8);
@@ -2045,8 +2046,8 @@ int gather_blocks_per_sm(const DevTables& T, bool wide) {
   const bool use_sm = sm <= kSmemLimit;
   const bool one = T.one_chunk && !wide;
   if (use_sm && one && T.rec3) {
-    // k_gather3 runs whenever the chains' octets have single temperatures
-    // (the variant with the most registers stands for all four)
+    // k_gather3 runs whenever no octet of chains has more than two temperatures
+    // (the variant with the most registers stands for all eight)
     const int sm3 = gather3_smem_bytes(T);
     auto kern = k_gather3<false, false, true>;
     if (allow_dynamic_smem(kern, sm3) != cudaSuccess) return 1;
