@@ -443,12 +443,15 @@ int maxsat_get_path(const maxsat_ctx* ctx);
  *                   the caller's buffers when the sizes given are theirs
  *   weights_dev     n_clauses device int64 weights, or NULL for all 1
  *   assign_dev      B x n_vars device bytes (nonzero = true); cost_dev: B int64
- * Its scratch memory (the assignments transposed to variable-major,
- * n_vars x B' bytes rounded up to 256, plus int64 cost partials,
- * ceil(n_clauses / max(64, ceil(n_clauses / 256))) x B' x 8 bytes, with B'
- * = B rounded up to 256) is one file-scope device array of
+ * Its scratch memory is one file-scope device array of
  * MAXSAT_NOALLOC_SCRATCH_BYTES that every GPU loading the library holds
- * until exit; larger requests fail with MAXSAT_EINVAL before any launch. The
+ * until exit. Up to 50000 variables it holds the assignments packed to one
+ * bit per variable (nothing when n_vars and n_clauses are at most 1024);
+ * beyond that, transposed to variable-major bytes (n_vars x B' rounded up to
+ * 256) and int64 cost partials (ceil(n_clauses / max(64, ceil(n_clauses /
+ * 256))) x B' x 8 bytes), with B' = B rounded up to 256. The limit is that of
+ * the byte form for every size: requests for which it would be larger than
+ * the array fail with MAXSAT_EINVAL before any launch. The
  * first call on each device looks the array's address up
  * (cudaGetSymbolAddress), so make that first call before any stream capture.
  * Every call overwrites all of the scratch it reads, but all calls share the

@@ -666,8 +666,6 @@ int alloc_chains(maxsat_ctx* ctx, int32_t B) {
   return plan_rounds(ctx, A, Bp);
 }
 
-// Copies h to a new device buffer padded with zeros to a multiple of 16 bytes
-// (kernels stage tables into shared memory 16 bytes at a time).
 // Reads the kernels' wait-timeout codes (call after synchronising the stream).
 int check_device_error(maxsat_ctx* ctx) {
   int codes[2] = {0, 0};
@@ -681,6 +679,8 @@ int check_device_error(maxsat_ctx* ctx) {
   return MAXSAT_OK;
 }
 
+// Copies h to a new device buffer padded with zeros to a multiple of 16 bytes
+// (kernels stage tables into shared memory 16 bytes at a time).
 template <class T>
 int upload(maxsat_ctx* ctx, DevAllocs& A, std::vector<T> h, const T** out) {
   while ((h.size() * sizeof(T)) % 16 != 0 || h.empty()) h.push_back(T{});

@@ -289,8 +289,11 @@ __device__ __forceinline__ void stage_weights(__nv_bfloat16* Ws, const __nv_bflo
 // tile's rows hang on a chain of three loads (where the lists begin, their
 // entries, the rows those name): the first two are made one and two tiles ahead,
 // in registers, so that only the rows themselves are waited for. At 318000
-// clauses and 53000 variables a clause layer takes 103 us forward and 173
-// backward (290 with the chain in turn), a variable layer 61 and 90. (16 warps
+// clauses and 53000 variables a clause layer takes 105 us forward and 174
+// backward (290 with the chain in turn), a variable layer 68 and 75, with events
+// around each launch. (The rows are read by plain loads, as a launch in flight may
+// still write them; by read-only loads the backward layers took 194 and 93: the
+// compiler then keeps fewer values in flight, 24 bytes of spills against 72. 16 warps
 // of which half fetched and half multiplied were slower, 131 and 262 us; rows of
 // the whole next tile in registers no faster, 115 us forward.) A launch stages
 // its weights and first lists while its predecessor ends: eight launches of a
