@@ -19,6 +19,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <shared_mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -42,6 +43,20 @@ struct NvtxRange {
   NvtxRange(const NvtxRange&) = delete;
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
+
+// While a stream of this process is being captured, cudaDeviceSynchronize fails
+// and invalidates the capture. Contexts belong to different host threads, so the
+// library's captures (shared) and waits for the whole device (exclusive) take
+// turns.
+std::shared_mutex& capture_gate() {
+  static std::shared_mutex* m = new std::shared_mutex();  // kept until exit, as the cache below
+  return *m;
+}
+
+cudaError_t wait_for_device() {
+  std::unique_lock<std::shared_mutex> lock(capture_gate());
+  return cudaDeviceSynchronize();
+}
 
 // Device blocks freed by contexts, kept per device for later contexts:
 // cudaMalloc and cudaFree take tens of microseconds each (and cudaFree waits
@@ -101,8 +116,15 @@ struct DevAllocs {
   // wait): work still queued on any stream may use them
   void release() {
     if (blocks.empty()) return;
-    cudaDeviceSynchronize();
-    for (const Block& b : blocks) block_cache().put(b.dev, b.p, b.bytes);
+    if (wait_for_device() == cudaSuccess) {
+      for (const Block& b : blocks) block_cache().put(b.dev, b.p, b.bytes);
+    } else {
+      // refused (the application is capturing): not known to be idle, so not for
+      // another context; cudaFree waits by itself
+      cudaGetLastError();
+      for (const Block& b : blocks) cudaFree(b.p);
+      cudaGetLastError();
+    }
     blocks.clear();
   }
   template <class T>
@@ -395,6 +417,7 @@ int launch_round(maxsat_ctx* ctx, cudaStream_t st, const uint32_t* tdev, uint32_
 int capture_graph(maxsat_ctx* ctx, int S) {
   destroy_graph(ctx);
   if (!ctx->cap_stream) CK(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
+  std::shared_lock<std::shared_mutex> capturing(capture_gate());
   CK(ctx, cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
   int rc = MAXSAT_OK;
   for (int s = 0; s < S && rc == MAXSAT_OK; ++s) rc = launch_round(ctx, ctx->cap_stream, ctx->d_t, (uint32_t)s);
@@ -404,6 +427,7 @@ int capture_graph(maxsat_ctx* ctx, int S) {
   }
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(ctx->cap_stream, &g);
+  capturing.unlock();
   if (rc != MAXSAT_OK) {
     if (g) cudaGraphDestroy(g);
     return rc;
@@ -2021,12 +2045,16 @@ int maxsat_step(maxsat_ctx* ctx, int64_t steps) {
   if (steps < 0) return fail(ctx, MAXSAT_EINVAL, "steps must be >= 0");
   if ((uint64_t)ctx->t + (uint64_t)steps > 0xFFFFFFFFull) return fail(ctx, MAXSAT_EINVAL, "round index would exceed 2^32");
   if (many_rounds_apply(ctx, steps)) return run_many_rounds(ctx, steps);
-  const int S = ctx->profiling ? 0 : ctx->prm.steps_per_graph;
+  int S = ctx->profiling ? 0 : ctx->prm.steps_per_graph;
   while (steps > 0) {
     if (S > 0 && steps >= S) {
-      if (!ctx->graph || ctx->graph_steps != S) {
-        int rc = capture_graph(ctx, S);
-        if (rc != MAXSAT_OK) return rc;
+      if ((!ctx->graph || ctx->graph_steps != S) && capture_graph(ctx, S) != MAXSAT_OK) {
+        // (an application's own wait for the device, in another thread, invalidates
+        // a capture): these rounds as plain launches
+        cudaGetLastError();
+        ctx->err.clear();
+        S = 0;
+        continue;
       }
       if (!ctx->d_t_synced) {
         CK(ctx, launch_set_u32(ctx->d_t, ctx->t, ctx->stream));
@@ -2875,7 +2903,7 @@ int maxsat_mp_create(maxsat_mp** out, int32_t n_layers, uint64_t seed) {
   if (e == cudaSuccess) e = cudaMemset(mp->M, 0, 4 * (size_t)T);
   if (e == cudaSuccess) e = cudaMemset(mp->V, 0, 4 * (size_t)T);
   if (e == cudaSuccess) e = mp_launch_to_bf16(mp->P, mp->Pb, T, nullptr);
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (e == cudaSuccess) e = wait_for_device();
   if (e != cudaSuccess) {
     delete mp;
     return mp_fail(nullptr, MAXSAT_ECUDA, std::string("mp create: ") + cudaGetErrorString(e));
@@ -2893,13 +2921,13 @@ int maxsat_mp_set_params(maxsat_mp* mp, const float* theta) {
   MPCK(mp, cudaMemset(mp->M, 0, 4 * (size_t)mp->lay.total));
   MPCK(mp, cudaMemset(mp->V, 0, 4 * (size_t)mp->lay.total));
   mp->step = 0;
-  MPCK(mp, cudaDeviceSynchronize());
+  MPCK(mp, wait_for_device());
   return MAXSAT_OK;
 }
 
 int maxsat_mp_get_params(maxsat_mp* mp, float* theta, float* grad) {
   if (!mp) return MAXSAT_EINVAL;
-  MPCK(mp, cudaDeviceSynchronize());
+  MPCK(mp, wait_for_device());
   if (theta) MPCK(mp, cudaMemcpy(theta, mp->P, 4 * (size_t)mp->lay.total, cudaMemcpyDeviceToHost));
   if (grad) MPCK(mp, cudaMemcpy(grad, mp->G, 4 * (size_t)mp->lay.total, cudaMemcpyDeviceToHost));
   return MAXSAT_OK;
@@ -2983,7 +3011,7 @@ const char* maxsat_mp_last_error(const maxsat_mp* mp) {
 
 void maxsat_mp_destroy(maxsat_mp* mp) {
   if (!mp) return;
-  cudaDeviceSynchronize();
+  wait_for_device();
   delete mp;
 }
 
@@ -3026,7 +3054,7 @@ void maxsat_destroy(maxsat_ctx* ctx) {
   if (ctx->up_ev_snap) cudaEventDestroy(ctx->up_ev_snap);
   if (ctx->up_ev_done) cudaEventDestroy(ctx->up_ev_done);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  else cudaDeviceSynchronize();
+  else wait_for_device();
   drain_marks(ctx);
   destroy_graph(ctx);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
